@@ -66,7 +66,7 @@ constexpr int kMaxCpt = 256;
 // Direct-mode hash output per chunk: its length, and this bit when dirty.
 constexpr uint64_t kAccDirty = 1ull << 63;
 
-__device__ __forceinline__ uint64_t umin64(uint64_t a, uint64_t b) { return a < b ? a : b; }
+__host__ __device__ __forceinline__ uint64_t umin64(uint64_t a, uint64_t b) { return a < b ? a : b; }
 
 __device__ __forceinline__ uint64_t mixw(uint64_t w, uint64_t key) {
     const uint64_t y = (w ^ key) * kM1;

@@ -205,7 +205,10 @@ struct RestoreParams {
     uint32_t log2_chunk;
     uint64_t n_entries;
     const ScatterDesc *desc;      // all images' descriptors, RestorePiece::desc_off into it
-    uint32_t *owner;              // per target chunk: newest chain position + 1 (0 = none)
+    const ScatterDesc *tgt;       // the target image's descriptors (in `desc`)
+    uint32_t n_tgt;
+    uint32_t log2_part;           // log2 of the bytes one warp copies (set by the scatter's launch)
+    unsigned long long *owner;    // per target chunk: newest chain position + 1 and its entry (0 = none)
     uint64_t n_owner;
     unsigned int *err;
     // Incremental restore: current and target fingerprints per target chunk.
@@ -213,10 +216,11 @@ struct RestoreParams {
     uint32_t coded;               // some piece has a zlen table (coded image)
 };
 // Multi-image restore: mark owners for every entry of every piece (atomicMax,
-// so the newest image wins in any order), check coverage, scatter owned chunks.
+// so the newest image wins in any order), check coverage, scatter every target
+// chunk from its owner (the scatter's grid follows the work, up to max_grid).
 cudaError_t launch_restore_mark(const RestoreParams &p, int grid, cudaStream_t s);
 cudaError_t launch_restore_check(const RestoreParams &p, int grid, cudaStream_t s);
-cudaError_t launch_restore_scatter(const RestoreParams &p, int grid, cudaStream_t s);
+cudaError_t launch_restore_scatter(const RestoreParams &p, uint64_t max_grid, cudaStream_t s);
 // Incremental restore, between check and scatter: clears the owner of every
 // chunk whose current fingerprint equals the target's, so it is not written.
 cudaError_t launch_restore_unmark(const RestoreParams &p, int grid, cudaStream_t s);

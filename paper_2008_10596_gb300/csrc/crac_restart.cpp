@@ -72,7 +72,7 @@ crac_status_t img_offsets(crac_image *im) {
 crac_status_t reserve_restart(crac_ctx *c, uint64_t nt, size_t descs, size_t pieces) {
     const size_t bytes = round_up(descs * sizeof(ScatterDesc), 256) +
                          round_up(std::max<size_t>(pieces, 1) * sizeof(RestorePiece), 256);
-    TRY(ensure_dev(c->owner, std::max<uint64_t>(nt, 1) * 4));
+    TRY(ensure_dev(c->owner, std::max<uint64_t>(nt, 1) * 8));
     TRY(ensure_dev(c->sdesc, bytes));
     TRY(ensure_host(c->sdesc_h, bytes));
     TRY(ensure_dev(c->serr, 256));
@@ -144,7 +144,7 @@ crac_status_t restart_device(crac_ctx *c, crac_image *img, const std::vector<cra
         if (im->done) CK(cudaStreamWaitEvent(s, im->done, 0));
     CK(cudaStreamWaitEvent(s, c->ev_last, 0));
     CK(cudaMemsetAsync(c->serr.p, 0, 256, s));
-    if (nt) CK(cudaMemsetAsync(c->owner.p, 0, nt * 4, s));
+    if (nt) CK(cudaMemsetAsync(c->owner.p, 0, nt * 8, s));
     CK(link_copy(c, c->sdesc.p, c->sdesc_h.p, desc_bytes + ppos * sizeof(RestorePiece), cudaMemcpyHostToDevice, s));
     crac_restart_info_t ri{};
     ri.chain_length = ri.images_used = (uint32_t)chain.size();
@@ -157,7 +157,9 @@ crac_status_t restart_device(crac_ctx *c, crac_image *img, const std::vector<cra
     P.log2_chunk = c->log2S;
     P.n_entries = entries;
     P.desc = (const ScatterDesc *)c->sdesc.p;
-    P.owner = (uint32_t *)c->owner.p;
+    P.tgt = P.desc + (total_desc - img->allocs.size());   // the chain ends with the target
+    P.n_tgt = (uint32_t)img->allocs.size();
+    P.owner = (unsigned long long *)c->owner.p;
     P.n_owner = nt;
     P.err = (unsigned int *)c->serr.p;
     for (const crac_image *im : chain) P.coded |= (im->flags & CRAC_IMAGE_CODED) ? 1u : 0u;
@@ -182,7 +184,7 @@ crac_status_t restart_device(crac_ctx *c, crac_image *img, const std::vector<cra
     CK(launch_restore_check(P, (int)std::max<uint64_t>(1, std::min<uint64_t>((nt + 255) / 256, grid)), s));
     if (incremental)
         CK(launch_restore_unmark(P, (int)std::max<uint64_t>(1, std::min<uint64_t>((nt + 255) / 256, grid)), s));
-    CK(launch_restore_scatter(P, (int)std::max<uint64_t>(1, std::min<uint64_t>((entries + 7) / 8, grid)), s));
+    CK(launch_restore_scatter(P, any_host || incremental || P.coded ? grid : UINT64_MAX, s));
     CK(cudaEventRecord(c->ev_r1, s));
     if (incremental) CK(launch_report(vctrl, sizeof(CkptCtrl) / 8, nullptr, c->ctrl_h.p, s));
     if (nt) {

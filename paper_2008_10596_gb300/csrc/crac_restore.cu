@@ -58,26 +58,22 @@ __device__ __forceinline__ uint32_t find_piece(const RestorePiece *__restrict__ 
     return lo;
 }
 
-// Target chunk of entry e, or ~0 when its allocation is not restored.
-__device__ __forceinline__ uint64_t restore_target(const RestoreParams &P, const RestorePiece &pc, uint64_t e,
-                                                   uint64_t *c_out, ScatterDesc *d_out) {
-    const uint64_t c = reinterpret_cast<const uint64_t *>(pc.idx)[e - pc.entry_base];
-    const ScatterDesc *dd = P.desc + pc.desc_off;
-    const ScatterDesc d = dd[find_scatter(dd, pc.n_desc, c)];
-    *c_out = c;
-    *d_out = d;
-    if (d.dst == 0) return ~0ull;
-    return d.tgt_first + (c - d.img_first);
-}
+// An owner word: the newest image holding a target chunk, as chain position + 1
+// (bits 40 and up), and the entry that holds it (bits 0-39); 0: none, or
+// nothing to restore.  atomicMax over the entries that mark a chunk leaves the
+// newest image's, whatever the order of execution.
+constexpr int kOwnerShift = 40;
+constexpr uint64_t kOwnerEntry = (1ull << kOwnerShift) - 1;
 
 __global__ void __launch_bounds__(256) restore_mark_kernel(const RestoreParams P) {
     for (uint64_t e = (uint64_t)blockIdx.x * 256 + threadIdx.x; e < P.n_entries; e += (uint64_t)gridDim.x * 256) {
         const RestorePiece pc = P.pieces[find_piece(P.pieces, P.n_pieces, e)];
-        uint64_t c;
-        ScatterDesc d;
-        const uint64_t tc = restore_target(P, pc, e, &c, &d);
-        if (tc == ~0ull) continue;
-        if (tc < P.n_owner) atomicMax(P.owner + tc, pc.image_index + 1u);
+        const uint64_t c = reinterpret_cast<const uint64_t *>(pc.idx)[e - pc.entry_base];
+        const ScatterDesc *dd = P.desc + pc.desc_off;
+        const ScatterDesc d = dd[find_scatter(dd, pc.n_desc, c)];
+        if (d.dst == 0) continue;   // its allocation is not restored
+        const uint64_t tc = d.tgt_first + (c - d.img_first);
+        if (tc < P.n_owner) atomicMax(P.owner + tc, ((unsigned long long)(pc.image_index + 1u) << kOwnerShift) | e);
         else atomicOr(P.err, kErrBounds);
     }
 }
@@ -94,45 +90,84 @@ __global__ void __launch_bounds__(256) restore_unmark_kernel(const RestoreParams
         if (P.fp_now[i] == P.fp_img[i]) P.owner[i] = 0;
 }
 
-// kCoded: some piece of the chain is coded (its decoder needs registers the
-// plain copy does not, so chains without coded images keep the lean build,
-// restore_scatter_kernel; coded chains run restore_scatter_coded_kernel).
+// The scatter: every target chunk's bytes from the entry that owns it, so each
+// byte is read once and written once, in the order of the target's memory.  An
+// item is 1 << P.log2_part bytes of a target chunk (or a whole short chunk), a
+// warp each.  The grid covers the items once with ordinary CTAs, so that the
+// hardware hands them to whichever SM is free: HBM serves the SMs unevenly, and
+// a copy cut into equal shares for one wave of resident CTAs waits for the
+// slowest (4 GiB in 64 KiB chunks: 1.32 ms in one wave of 5 CTAs per SM, 1.22 ms
+// with a CTA for every 64 KiB).  With a smaller grid (host images, whose link
+// one CTA per SM already paces; incremental restores, where most items are
+// skipped) a warp strides over the items, 32 at a time, a lane looking up each.
+struct RestoreItem {
+    uint64_t dst, src;
+    uint32_t len, z;   // bytes to write (0: nothing), bytes stored
+};
+
 template <bool kCoded>
-__device__ __forceinline__ void restore_scatter_body(const RestoreParams &P, uint8_t *scratch) {
-    if (*(volatile unsigned int *)P.err) return;   // uncovered or out of range: memory untouched
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint64_t S = 1ull << P.log2_chunk;
-    for (uint64_t e = (uint64_t)blockIdx.x * (kScatterNT / 32) + warp; e < P.n_entries;
-         e += (uint64_t)gridDim.x * (kScatterNT / 32)) {
-        const RestorePiece pc = P.pieces[find_piece(P.pieces, P.n_pieces, e)];
-        uint64_t c;
-        ScatterDesc d;
-        const uint64_t tc = restore_target(P, pc, e, &c, &d);
-        if (tc >= P.n_owner || P.owner[tc] != pc.image_index + 1u) continue;
-        const uint64_t local = c - d.img_first;
-        const uint64_t len = min(S, d.bytes - (local << P.log2_chunk));
-        const uint64_t o = reinterpret_cast<const uint64_t *>(pc.off)[e - pc.entry_base];
-        // Coded image: the entry's stream length (equal to len when stored raw).
-        const uint64_t z = (kCoded && pc.zlen) ? reinterpret_cast<const uint64_t *>(pc.zlen)[e - pc.entry_base] : len;
-        if (o > pc.bytes || z > pc.bytes - o) {
-            if (lane == 0) atomicOr(P.err, kErrBounds);
-            continue;
-        }
-        uint8_t *dst = reinterpret_cast<uint8_t *>(d.dst) + (local << P.log2_chunk);
-        const uint8_t *src = reinterpret_cast<const uint8_t *>(pc.payload) + o;
-        if (!kCoded || z == len) copy_group<32>(dst, src, len, lane);
-        else if (!crz_decode_warp(dst, src, len, z, lane, scratch + kCrzDecodeScratch * warp) && lane == 0)
-            atomicOr(P.err, kErrCodec);
+__device__ __forceinline__ RestoreItem restore_item(const RestoreParams &P, uint64_t it) {
+    RestoreItem r{0, 0, 0, 0};
+    const uint32_t parts = P.log2_chunk - P.log2_part;   // log2 of the items per chunk
+    const uint64_t tc = it >> parts;
+    const uint64_t po = (it & ((1ull << parts) - 1)) << P.log2_part;   // the item's offset in its chunk
+    const uint64_t own = P.owner[tc];
+    const ScatterDesc *d = P.tgt + find_scatter(P.tgt, P.n_tgt, tc);
+    const uint64_t at = (tc - d->img_first) << P.log2_chunk;
+    const uint64_t clen = umin64(1ull << P.log2_chunk, d->bytes - at);
+    if (!own || po >= clen) return r;   // a short last chunk has fewer items
+    const uint64_t e = own & kOwnerEntry;
+    const RestorePiece *pc = P.pieces + find_piece(P.pieces, P.n_pieces, e);
+    const uint64_t o = reinterpret_cast<const uint64_t *>(pc->off)[e - pc->entry_base];
+    // Coded image: the entry's stream length (equal to clen when stored raw).
+    const uint64_t ez = (kCoded && pc->zlen) ? reinterpret_cast<const uint64_t *>(pc->zlen)[e - pc->entry_base] : clen;
+    if (o > pc->bytes || ez > pc->bytes - o) {
+        atomicOr(P.err, kErrBounds);
+        return r;
     }
+    r.dst = d->dst + at + po;
+    r.src = pc->payload + o + po;
+    r.len = (uint32_t)umin64(1ull << P.log2_part, clen - po);
+    r.z = (kCoded && ez != clen) ? (uint32_t)ez : r.len;
+    return r;
 }
 
 __global__ void __launch_bounds__(kScatterNT) restore_scatter_kernel(const RestoreParams P) {
-    restore_scatter_body<false>(P, nullptr);
+    if (*(volatile unsigned int *)P.err) return;   // uncovered or out of range: memory untouched
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint64_t n_items = P.n_owner << (P.log2_chunk - P.log2_part);
+    const uint64_t nw = (uint64_t)gridDim.x * (kScatterNT / 32);
+    for (uint64_t i0 = (uint64_t)blockIdx.x * (kScatterNT / 32) + warp; i0 < n_items; i0 += 32 * nw) {
+        RestoreItem r{0, 0, 0, 0};
+        if (i0 + lane * nw < n_items) r = restore_item<false>(P, i0 + lane * nw);
+        unsigned todo = __ballot_sync(kFull, r.len != 0);
+        while (todo) {   // warp-uniform
+            const int i = __ffs(todo) - 1;
+            todo &= todo - 1;
+            copy_group<32>(reinterpret_cast<uint8_t *>(__shfl_sync(kFull, r.dst, i)),
+                           reinterpret_cast<const uint8_t *>(__shfl_sync(kFull, r.src, i)),
+                           __shfl_sync(kFull, r.len, i), lane);
+        }
+    }
 }
 
+// Chains with a coded image: the decoder needs registers that the plain copy
+// does not (hence two kernels), and an item is a whole chunk, looked up by the
+// whole warp: its decoding takes far longer than the look-up.
 __global__ void __launch_bounds__(kScatterNT, 4) restore_scatter_coded_kernel(const RestoreParams P) {
     __shared__ __align__(16) uint8_t scratch[kCrzDecodeScratch * (kScatterNT / 32)];
-    restore_scatter_body<true>(P, scratch);
+    if (*(volatile unsigned int *)P.err) return;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint64_t nw = (uint64_t)gridDim.x * (kScatterNT / 32);
+    for (uint64_t it = (uint64_t)blockIdx.x * (kScatterNT / 32) + warp; it < P.n_owner; it += nw) {
+        const RestoreItem r = restore_item<true>(P, it);
+        if (r.len == 0) continue;
+        uint8_t *dst = reinterpret_cast<uint8_t *>(r.dst);
+        const uint8_t *src = reinterpret_cast<const uint8_t *>(r.src);
+        if (r.z == r.len) copy_group<32>(dst, src, r.len, lane);
+        else if (!crz_decode_warp(dst, src, r.len, r.z, lane, scratch + kCrzDecodeScratch * warp) && lane == 0)
+            atomicOr(P.err, kErrCodec);
+    }
 }
 
 }  // namespace
@@ -161,10 +196,18 @@ cudaError_t launch_restore_unmark(const RestoreParams &p, int grid, cudaStream_t
     return e;
 }
 
-cudaError_t launch_restore_scatter(const RestoreParams &p, int grid, cudaStream_t s) {
-    if (p.n_entries == 0) return cudaSuccess;
-    if (p.coded) restore_scatter_coded_kernel<<<grid, kScatterNT, 0, s>>>(p);
-    else restore_scatter_kernel<<<grid, kScatterNT, 0, s>>>(p);
+cudaError_t launch_restore_scatter(const RestoreParams &p, uint64_t max_grid, cudaStream_t s) {
+    if (p.n_entries == 0 || p.n_owner == 0) return cudaSuccess;
+    constexpr uint64_t kWarps = kScatterNT / 32;
+    RestoreParams q = p;
+    // A coded entry is decoded whole, by one warp; a plain chunk is cut into
+    // parts of 8 KiB, and a warp takes about 8 KiB of short chunks.
+    q.log2_part = p.coded || p.log2_chunk < 13 ? p.log2_chunk : 13;
+    uint64_t warps = p.n_owner << (p.log2_chunk - q.log2_part);
+    if (p.log2_chunk < 13) warps = ((warps - 1) >> (13 - (p.log2_chunk < 8 ? 8 : p.log2_chunk))) + 1;
+    const uint64_t ctas = umin64((warps + kWarps - 1) / kWarps, umin64(max_grid, 0x7fffffffull));
+    if (p.coded) restore_scatter_coded_kernel<<<(unsigned)ctas, kScatterNT, 0, s>>>(q);
+    else restore_scatter_kernel<<<(unsigned)ctas, kScatterNT, 0, s>>>(q);
     const cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) count_launches(1);
     return e;
