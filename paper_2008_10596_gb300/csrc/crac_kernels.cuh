@@ -156,7 +156,8 @@ const void *split_hash_fn(bool crz_headers = false);
 // it finalizes every chunk itself, so finalize runs with log2Seg = log2_chunk.
 const void *split_hash_small_fn(int lanes_per_chunk);
 const void *split_finalize_fn();
-const void *split_gather_fn(bool crz_headers);
+// aligned: every allocation's size is a multiple of 16 bytes.
+const void *split_gather_fn(bool crz_headers, bool aligned);
 int split_hash_threads();
 int split_finalize_threads();
 int split_gather_threads();
@@ -214,6 +215,7 @@ struct RestoreParams {
     // Incremental restore: current and target fingerprints per target chunk.
     const uint64_t *fp_now, *fp_img;
     uint32_t coded;               // some piece has a zlen table (coded image)
+    uint32_t ragged;              // some allocation's size is not a multiple of 16 bytes
 };
 // Multi-image restore: mark owners for every entry of every piece (atomicMax,
 // so the newest image wins in any order), check coverage, scatter every target

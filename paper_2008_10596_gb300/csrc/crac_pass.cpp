@@ -250,9 +250,7 @@ crac_status_t launch_fused_graph(crac_ctx *c, const CkptParams &P, size_t work_b
 crac_status_t launch_split_graph(crac_ctx *c, const CkptParams &P, size_t work_bytes, unsigned long long *acc,
                                  uint32_t log2Seg, const void *hash_fn, size_t hash_smem, const int grids[3],
                                  void *ctrl_dst, cudaStream_t s) {
-    // The gather instance follows P.crz_hdr, which only the hash instance
-    // split_hash_kernel<true> runs with: hash_fn alone keys the cached graph.
-    const void *fns[3] = {hash_fn, split_finalize_fn(), split_gather_fn(P.crz_hdr != nullptr)};
+    const void *fns[3] = {hash_fn, split_finalize_fn(), split_gather_fn(P.crz_hdr != nullptr, c->all16)};
     const int thr[3] = {split_hash_threads(), split_finalize_threads(), split_gather_threads()};
     CkptParams Pc = P;
     unsigned long long *accv = acc;
@@ -274,7 +272,7 @@ crac_status_t launch_split_graph(crac_ctx *c, const CkptParams &P, size_t work_b
     mp.width = work_bytes / 4;
     mp.height = 1;
     ReportNode rep(P.ctrl, ctrl_dst);
-    bool ok = c->sgexec != nullptr && c->s_hash_fn == hash_fn;
+    bool ok = c->sgexec != nullptr && c->s_hash_fn == hash_fn && c->s_gather_fn == fns[2];
     if (ok) {
         ok = cudaGraphExecMemsetNodeSetParams(c->sgexec, c->s_memset, &mp) == cudaSuccess;
         for (int i = 0; ok && i < 3; ++i)
@@ -307,6 +305,7 @@ crac_status_t launch_split_graph(crac_ctx *c, const CkptParams &P, size_t work_b
         CK(cudaGraphAddKernelNode(&c->s_copy, c->sgraph, &c->s_k[2], 1, &rep.kp));
         CK(cudaGraphInstantiate(&c->sgexec, c->sgraph, 0));
         c->s_hash_fn = hash_fn;
+        c->s_gather_fn = fns[2];
     }
     CK(cudaEventRecord(c->ev_t0, s));
     CK(cudaGraphLaunch(c->sgexec, s));
@@ -1269,6 +1268,7 @@ crac_status_t ctx_checkpoint(crac_ctx *c, cudaStream_t s, crac_image_t **out) {
             prefix_h[a] = pre;
             pre += c->allocs[a].bytes;
         }
+        c->all16 = all16;
         c->full_copy_ok = !any_base && all16;
         c->pass_now = resolve_pass_kernel(c, dev_res, all16);
         c->sparse_ok = c->pass_now == CRAC_PASS_SPARSE && dev_res && all16 &&
@@ -1459,6 +1459,7 @@ crac_status_t ctx_trial_pass(crac_ctx *c, cudaStream_t s, bool commit, float *ms
         prefix_h[a] = pre;
         pre += c->allocs[a].bytes;
     }
+    c->all16 = all16;
     c->full_copy_ok = !any_base && all16;
     // Trial passes run the configured kernel; AUTO is the split pass here, so
     // that the tuner's observations of different sizes are comparable.

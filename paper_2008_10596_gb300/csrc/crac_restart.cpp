@@ -162,7 +162,10 @@ crac_status_t restart_device(crac_ctx *c, crac_image *img, const std::vector<cra
     P.owner = (unsigned long long *)c->owner.p;
     P.n_owner = nt;
     P.err = (unsigned int *)c->serr.p;
-    for (const crac_image *im : chain) P.coded |= (im->flags & CRAC_IMAGE_CODED) ? 1u : 0u;
+    for (const crac_image *im : chain) {
+        P.coded |= (im->flags & CRAC_IMAGE_CODED) ? 1u : 0u;
+        for (const ImgAlloc &a : im->allocs) P.ragged |= (a.bytes & 15) ? 1u : 0u;
+    }
     // Reads of host images are paced by the host link, which one CTA per SM
     // already saturates (4 KiB in flight per warp); a bigger grid would only
     // keep SMs from other streams' work for the length of the transfer.

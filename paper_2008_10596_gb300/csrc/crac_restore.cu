@@ -12,7 +12,7 @@ namespace {
 // ---------------------------------------------------------------------------
 constexpr int kScatterNT = 256;
 
-__global__ void __launch_bounds__(kScatterNT) scatter_kernel(const ScatterParams P) {
+__global__ void __launch_bounds__(kScatterNT, 4) scatter_kernel(const ScatterParams P) {
     constexpr int GT = 32;
     // A resolution or bounds error found earlier on this stream (chain not
     // covering the target, index out of range) leaves memory untouched.
@@ -132,7 +132,9 @@ __device__ __forceinline__ RestoreItem restore_item(const RestoreParams &P, uint
     return r;
 }
 
-__global__ void __launch_bounds__(kScatterNT) restore_scatter_kernel(const RestoreParams P) {
+// kAligned: every allocation's size is a multiple of 16 bytes.
+template <bool kAligned>
+__device__ __forceinline__ void restore_scatter_body(const RestoreParams &P) {
     if (*(volatile unsigned int *)P.err) return;   // uncovered or out of range: memory untouched
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint64_t n_items = P.n_owner << (P.log2_chunk - P.log2_part);
@@ -144,11 +146,19 @@ __global__ void __launch_bounds__(kScatterNT) restore_scatter_kernel(const Resto
         while (todo) {   // warp-uniform
             const int i = __ffs(todo) - 1;
             todo &= todo - 1;
-            copy_group<32>(reinterpret_cast<uint8_t *>(__shfl_sync(kFull, r.dst, i)),
-                           reinterpret_cast<const uint8_t *>(__shfl_sync(kFull, r.src, i)),
-                           __shfl_sync(kFull, r.len, i), lane);
+            copy_group<32, kAligned>(reinterpret_cast<uint8_t *>(__shfl_sync(kFull, r.dst, i)),
+                                     reinterpret_cast<const uint8_t *>(__shfl_sync(kFull, r.src, i)),
+                                     __shfl_sync(kFull, r.len, i), lane);
         }
     }
+}
+
+__global__ void __launch_bounds__(kScatterNT, 4) restore_scatter_kernel(const RestoreParams P) {
+    restore_scatter_body<true>(P);
+}
+
+__global__ void __launch_bounds__(kScatterNT, 4) restore_scatter_ragged_kernel(const RestoreParams P) {
+    restore_scatter_body<false>(P);
 }
 
 // Chains with a coded image: the decoder needs registers that the plain copy
@@ -207,6 +217,7 @@ cudaError_t launch_restore_scatter(const RestoreParams &p, uint64_t max_grid, cu
     if (p.log2_chunk < 13) warps = ((warps - 1) >> (13 - (p.log2_chunk < 8 ? 8 : p.log2_chunk))) + 1;
     const uint64_t ctas = umin64((warps + kWarps - 1) / kWarps, umin64(max_grid, 0x7fffffffull));
     if (p.coded) restore_scatter_coded_kernel<<<(unsigned)ctas, kScatterNT, 0, s>>>(q);
+    else if (p.ragged) restore_scatter_ragged_kernel<<<(unsigned)ctas, kScatterNT, 0, s>>>(q);
     else restore_scatter_kernel<<<(unsigned)ctas, kScatterNT, 0, s>>>(q);
     const cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) count_launches(1);

@@ -445,9 +445,10 @@ struct crac_ctx {
     cudaGraphExec_t sgexec = nullptr;
     cudaGraphNode_t s_memset = nullptr, s_k[3] = {nullptr, nullptr, nullptr}, s_copy = nullptr;
     cudaEvent_t sev[4] = {nullptr, nullptr, nullptr, nullptr};   // around each split-pass kernel
-    const void *s_hash_fn = nullptr;
+    const void *s_hash_fn = nullptr, *s_gather_fn = nullptr;   // the instances in it
     crac_pass_info_t last{};
     crac_restart_info_t last_restart{};
+    bool all16 = false;          // current pass: every size a multiple of 16 bytes
     bool full_copy_ok = false;   // current pass: no baseline anywhere and 16-byte sizes
     bool sparse_ok = false;      // current pass: CRAC_PASS_SPARSE, device images, 16-byte sizes
     bool dense_now = false;      // ... and, on 512 B - 4 KiB chunks, dense placement of the dirty chunks

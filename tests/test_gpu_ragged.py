@@ -1,0 +1,42 @@
+"""Payloads off the 16-byte grid (GPU): allocations of any byte size shift every
+later chunk's payload offset, so the copies into the payload and back out of it
+run between differently aligned addresses.  Byte for byte against the oracle."""
+import numpy as np
+import pytest
+
+import paper_2008_10596_gb300 as C
+from tests.gpu_harness import Harness, pattern_mutations
+
+pytestmark = [pytest.mark.gpu, pytest.mark.usefixtures("oracle_lib")]
+
+KIB = 1024
+
+# Every residue of the payload offset mod 16, and lengths around one vector, one
+# warp's 512-byte row and its 2 KiB strip; then chunks cut into 8 KiB parts.
+SHORT = [1, 15, 16, 17, 31, 33, 47, 62, 63, 64, 511, 512, 513, 527, 2047, 2048, 2049, 2063, 2064, 4095, 4111]
+LONG = [64 * KIB + 1, 3, 64 * KIB - 1, 8 * KIB + 7, 16 * KIB - 5, 200001, 64 * KIB * 3, 24 * KIB + 2, 131072 + 13]
+
+
+@pytest.mark.parametrize("S,sizes", [(4 * KIB, SHORT), (64 * KIB, LONG + SHORT), (256 * KIB, LONG + [700001, 5, 262144])])
+@pytest.mark.parametrize("kern", [C.CRAC_PASS_SPLIT, C.CRAC_PASS_LDG, C.CRAC_PASS_AUTO])
+@pytest.mark.parametrize("residency", [C.CRAC_RESIDENCY_DEVICE, C.CRAC_RESIDENCY_HOST])
+def test_ragged_sizes(S, sizes, kern, residency):
+    flags = C.CRAC_FLAG_STAGED_RESTORE if residency == C.CRAC_RESIDENCY_HOST and kern == C.CRAC_PASS_LDG else 0
+    h = Harness(S, lineage=1500 + S % 97 + kern, pass_kernel=kern, image_residency=residency, flags=flags)
+    try:
+        for i, n in enumerate(sizes):
+            h.add(n, seed=400 + i)
+        img, lib, ora = h.checkpoint()
+        assert lib == ora
+        for pattern in ("alternating", "alternating", "random10", "all"):   # repeated: the predicted chunks too
+            h.mutate(pattern_mutations(h.first(), sizes, S, pattern, seed=7))
+            img, lib, ora = h.checkpoint()
+            assert lib == ora
+        want = h.host()
+        for b in h.bufs:
+            b.zero()
+        h.restart(img)
+        for b, w in zip(h.bufs, want):
+            assert np.array_equal(b.read(), w)
+    finally:
+        h.close()
