@@ -272,6 +272,20 @@ __device__ __forceinline__ uint32_t find_alloc(const CkptDesc *__restrict__ d, u
     return lo;
 }
 
+// The same search by one full warp (c warp-uniform): 32 pivots at a time, so
+// two or three dependent loads for a few hundred or thousand allocations.
+__device__ __forceinline__ uint32_t find_alloc_warp(const CkptDesc *__restrict__ d, uint32_t n, uint64_t c, int lane) {
+    uint32_t lo = 0, span = n;
+    while (span > 1) {
+        const uint32_t step = (span + 31) >> 5, i = lane * step;
+        const unsigned m = __ballot_sync(kFull, i < span && (i == 0 || d[lo + i].first_chunk <= c));
+        const uint32_t k = (31u - __clz(m)) * step;
+        lo += k;
+        span = span - k < step ? span - k : step;
+    }
+    return lo;
+}
+
 __device__ __forceinline__ uint32_t find_scatter(const ScatterDesc *__restrict__ d, uint32_t n,
                                                  uint64_t c) {
     uint32_t lo = 0, hi = n;

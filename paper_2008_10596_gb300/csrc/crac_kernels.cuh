@@ -71,6 +71,9 @@ struct CkptParams {
     // dirty entry's offset points there, ctrl->D counts the segment's bytes
     // and ctrl->payload the dirty ones; nothing is gathered.
     uint32_t sparse;
+    // Split pass, hash kernel on chunks below 512 B and from 8 KiB: segments per
+    // warp.
+    uint32_t slots_per_warp;
     // TMA pass: the allocations' first_chunk column fits in the CTA's shared
     // memory (n_allocs <= ckpt_tma_cached_allocs()) and is searched there.
     uint32_t first_cached;
@@ -152,7 +155,7 @@ cudaError_t ckpt_tma_prepare();   // raise the dynamic shared memory limit (once
 // must be zero before H; F uses cpt = split_finalize_threads() chunks per
 // tile and the look-back status words; G reads k from ctrl.
 const void *split_hash_fn(bool crz_headers = false);
-// Hash kernel for 512 B <= chunk < 8 KiB: lanes_per_chunk = 32 * chunk / 8192;
+// Hash kernel for 512 B <= chunk < 8 KiB: lanes_per_chunk = chunk / 128;
 // it finalizes every chunk itself, so finalize runs with log2Seg = log2_chunk.
 const void *split_hash_small_fn(int lanes_per_chunk);
 const void *split_finalize_fn();
@@ -161,7 +164,14 @@ const void *split_gather_fn(bool crz_headers, bool aligned);
 int split_hash_threads();
 int split_finalize_threads();
 int split_gather_threads();
-int split_max_ctas_per_sm(const void *fn, int threads);
+// log2 of the hash kernel's segment (at most the chunk) for `bytes` tracked
+// bytes; copy: every chunk is also written.  Not for chunks of 512 B - 4 KiB.
+uint32_t split_hash_seg(uint64_t bytes, uint32_t log2_chunk, bool copy);
+// Grid of the hash kernel over n_chunks chunks holding `bytes` bytes, and
+// CkptParams::slots_per_warp of that grid.
+uint32_t split_hash_grid(uint64_t n_chunks, uint64_t bytes, uint32_t log2_chunk, uint32_t log2_seg,
+                         uint32_t *slots_per_warp);
+const void *split_hash_small_dense_fn(int lanes_per_chunk);
 
 cudaError_t launch_fp_range(const CkptDesc *d, uint64_t c0, uint64_t c1, uint32_t log2_chunk,
                             const uint64_t *fp_old, uint64_t *fp_new, uint32_t *lens,

@@ -248,7 +248,7 @@ crac_status_t launch_fused_graph(crac_ctx *c, const CkptParams &P, size_t work_b
 
 // Build (or update) the split-pass graph and launch it.
 crac_status_t launch_split_graph(crac_ctx *c, const CkptParams &P, size_t work_bytes, unsigned long long *acc,
-                                 uint32_t log2Seg, const void *hash_fn, size_t hash_smem, const int grids[3],
+                                 uint32_t log2Seg, const void *hash_fn, const int grids[3],
                                  void *ctrl_dst, cudaStream_t s) {
     const void *fns[3] = {hash_fn, split_finalize_fn(), split_gather_fn(P.crz_hdr != nullptr, c->all16)};
     const int thr[3] = {split_hash_threads(), split_finalize_threads(), split_gather_threads()};
@@ -262,7 +262,6 @@ crac_status_t launch_split_graph(crac_ctx *c, const CkptParams &P, size_t work_b
         kp[i].func = const_cast<void *>(fns[i]);
         kp[i].gridDim = dim3(grids[i]);
         kp[i].blockDim = dim3(thr[i]);
-        kp[i].sharedMemBytes = i == 0 ? (unsigned)hash_smem : 0u;
         kp[i].kernelParams = args;
     }
     cudaMemsetParams mp{};
@@ -339,18 +338,17 @@ crac_status_t launch_segment(crac_ctx *c, const Segment &sg, const CkptDesc *des
         TRY(ensure_dev(c->work, work_bytes));
         // 512 B..4 KiB chunks: several whole chunks per warp iteration.
         const bool small = c->log2S >= 9 && c->log2S < 13;
-        const uint32_t log2Seg = std::min<uint32_t>(c->log2S, 13);
+        const bool copies = staging && (c->full_copy_ok || c->sparse_ok);   // the hash kernel writes every chunk
+        const uint32_t log2Seg = small ? c->log2S : split_hash_seg(sg.bytes, c->log2S, copies);
         // Coded contexts with chunks of 8 KiB and more: the kernel that writes a
         // chunk to staging (hash or gather) also writes its CRZ1 block headers
         // for the encoder.
         uint64_t *crz_hdr = c->crz_hdr_now ? (uint64_t *)c->chdr.p : nullptr;
         // The sparse pass on 512 B - 4 KiB chunks may place the dirty chunks
-        // densely (a bulk store per warp iteration from shared memory).
+        // densely.
         const bool dense = small && c->sparse_ok && staging && c->dense_now;
-        const void *hash_fn = dense ? split_hash_small_dense_fn(1 << (c->log2S - 8))
-                              : small ? split_hash_small_fn(1 << (c->log2S - 8)) : split_hash_fn(crz_hdr != nullptr);
-        const size_t hash_smem = dense ? split_dense_smem() : 0;
-        if (dense) CK(split_dense_prepare(hash_fn));
+        const void *hash_fn = dense ? split_hash_small_dense_fn(1 << (c->log2S - 7))
+                              : small ? split_hash_small_fn(1 << (c->log2S - 7)) : split_hash_fn(crz_hdr != nullptr);
         CkptParams P{};
         P.crz_hdr = crz_hdr;
         P.desc = desc_dev;
@@ -388,15 +386,11 @@ crac_status_t launch_segment(crac_ctx *c, const Segment &sg, const CkptDesc *des
             P.seg_base = pre + ((sg.c0 - first[a0]) << c->log2S);
         }
         unsigned long long *acc = (unsigned long long *)((uint8_t *)c->work.p + status_bytes);
-        const uint64_t n_slots = small ? (nseg + (8192u >> c->log2S) - 1) / (8192u >> c->log2S)
-                                       : nseg << (c->log2S - log2Seg);
-        const int gh = (int)std::max<uint64_t>(1, std::min<uint64_t>(
-                           (n_slots + 7) / 8,
-                           (uint64_t)c->sm_count * split_max_ctas_per_sm_smem(hash_fn, split_hash_threads(), hash_smem)));
+        const int gh = (int)split_hash_grid(nseg, sg.bytes, c->log2S, log2Seg, &P.slots_per_warp);
         const int gf = (int)std::min<uint64_t>(n_tiles, (uint64_t)c->sm_count * 2);
         const int gg = c->sm_count * 8;
         const int grids[3] = {gh, gf, gg};
-        TRY(launch_split_graph(c, P, work_bytes, acc, log2Seg, hash_fn, hash_smem, grids, ctrl_dst, s));
+        TRY(launch_split_graph(c, P, work_bytes, acc, log2Seg, hash_fn, grids, ctrl_dst, s));
         if (c->spec_now) {   // this pass's offsets predict the next one's
             c->ppos_cur ^= 1;
             c->ppos_ok = true;
@@ -1512,7 +1506,11 @@ crac_status_t fingerprint_against(crac_ctx *c, const uint64_t *fp_ref, cudaStrea
     const uint32_t log2S = c->log2S;
     const uint64_t S = 1ull << log2S;
     std::vector<uint64_t> first(na + 1, 0);
-    for (size_t a = 0; a < na; ++a) first[a + 1] = first[a] + ((c->allocs[a].bytes + S - 1) >> log2S);
+    uint64_t bytes = 0;
+    for (size_t a = 0; a < na; ++a) {
+        first[a + 1] = first[a] + ((c->allocs[a].bytes + S - 1) >> log2S);
+        bytes += c->allocs[a].bytes;
+    }
     const uint64_t n = first[na];
     const uint32_t cptF = (uint32_t)split_finalize_threads();
     const uint64_t n_tiles = (n + cptF - 1) / cptF;
@@ -1531,8 +1529,8 @@ crac_status_t fingerprint_against(crac_ctx *c, const uint64_t *fp_ref, cudaStrea
     CK(link_copy(c, c->vdesc.p, dh, na * sizeof(CkptDesc), cudaMemcpyHostToDevice, s));
     CK(cudaMemsetAsync(c->vwork.p, 0, work_bytes, s));
     const bool small = log2S >= 9 && log2S < 13;
-    uint32_t log2Seg = std::min<uint32_t>(log2S, 13);
-    const void *hash_fn = small ? split_hash_small_fn(1 << (log2S - 8)) : split_hash_fn();
+    uint32_t log2Seg = small ? log2S : split_hash_seg(bytes, log2S, false);
+    const void *hash_fn = small ? split_hash_small_fn(1 << (log2S - 7)) : split_hash_fn();
     CkptParams P{};
     P.desc = (const CkptDesc *)c->vdesc.p;
     P.n_allocs = (uint32_t)na;
@@ -1551,9 +1549,7 @@ crac_status_t fingerprint_against(crac_ctx *c, const uint64_t *fp_ref, cudaStrea
     P.tile_bytes = P.tile_cnt + n_tiles;
     P.timeout_ns = c->cfg.timeout_ns;
     unsigned long long *acc = (unsigned long long *)((uint8_t *)c->vwork.p + status_bytes);
-    const uint64_t n_slots = small ? (n + (8192u >> log2S) - 1) / (8192u >> log2S) : n << (log2S - log2Seg);
-    const int gh = (int)std::max<uint64_t>(1, std::min<uint64_t>(
-                       (n_slots + 7) / 8, (uint64_t)c->sm_count * split_max_ctas_per_sm(hash_fn, split_hash_threads())));
+    const int gh = (int)split_hash_grid(n, bytes, log2S, log2Seg, &P.slots_per_warp);
     const int gf = (int)std::max<uint64_t>(1, std::min<uint64_t>(n_tiles, (uint64_t)c->sm_count * 2));
     void *args[] = {&P, &acc, &log2Seg};
     CK(cudaLaunchKernel(hash_fn, dim3(gh), dim3(split_hash_threads()), args, 0, s));

@@ -6,11 +6,18 @@ namespace crac {
 
 namespace {
 
+// Out of line, so that the registers of the unaligned copy do not cost the
+// fused kernel a resident CTA.
+template <int GT>
+__device__ __noinline__ void copy_shifted_call(uint8_t *dst, const uint8_t *src, uint64_t len, int gl) {
+    copy_shifted<GT>(dst, src, len, gl);
+}
+
 // ---------------------------------------------------------------------------
 // Fused batched checkpoint pass: K1 + K2 + K3 in one persistent kernel.
 // ---------------------------------------------------------------------------
 template <int NT, int WPC>
-__global__ void __launch_bounds__(NT) ckpt_fused_kernel(const CkptParams P) {
+__global__ void __launch_bounds__(NT, 5) ckpt_fused_kernel(const CkptParams P) {
     constexpr int W = NT / 32;
     constexpr int G = W / WPC;        // chunk groups per CTA
     constexpr int GT = WPC * 32;      // threads per group
@@ -147,8 +154,11 @@ __global__ void __launch_bounds__(NT) ckpt_fused_kernel(const CkptParams P) {
                 if (gl == 0) atomicOr(&P.ctrl->err, kErrBounds);
                 continue;
             }
-            copy_group<GT>(P.staging + dst,
-                           reinterpret_cast<const uint8_t *>(d.ptr) + (local << log2S), len, gl);
+            const uint8_t *src = reinterpret_cast<const uint8_t *>(d.ptr) + (local << log2S);
+            if ((((uintptr_t)(P.staging + dst) | (uintptr_t)src) & 15u) == 0)
+                copy_group<GT, true>(P.staging + dst, src, len, gl);
+            else
+                copy_shifted_call<GT>(P.staging + dst, src, len, gl);
         }
         __syncthreads();
     }

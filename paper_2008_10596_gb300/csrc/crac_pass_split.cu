@@ -10,11 +10,16 @@ namespace {
 // Split pass: H (hash) -> F (finalize + dirty test + compaction) -> G (gather).
 //
 // H streams the tracked bytes with no inter-CTA dependency: every warp takes
-// a contiguous range of segments (8 KiB, or the chunk if smaller), issues all
-// of a segment's 128-bit loads at once (16 per lane), sums the per-word
-// terms, and adds the warp's sum into the chunk's accumulator with one 64-bit
-// atomicAdd.  The CRAC-FP64 sum is taken mod 2^64, so the order of these
-// additions does not change a bit.  F turns each accumulator into the
+// one segment (8 or 16 KiB, or several short chunks), in rounds of eight
+// 128-bit loads per lane, sums the per-word terms, and adds the warp's sum into
+// the chunk's accumulator with one 64-bit atomicAdd.  The CRAC-FP64 sum is
+// taken mod 2^64, so the order of these additions does not change a bit.  The
+// grid covers the segments once with ordinary CTAs: HBM serves the SMs unevenly,
+// and the hardware hands CTAs to whichever SM is free, where equal shares for
+// one wave of resident CTAs wait for the slowest (4 GiB in 64 KiB chunks, one
+// wave of two CTAs per SM with sixteen loads per lane -> this grid with three
+// CTAs per SM: 1350 -> 1207 us with every chunk written, 640 -> 591 us read only;
+// of the measured copy rate 0.94 -> 1.05).  F turns each accumulator into the
 // fingerprint, tests it against the baseline, and compacts the dirty chunks
 // (ballot + block scan per 1024-chunk tile, decoupled look-back across
 // tiles).  G copies the listed chunks into staging.  HBM traffic: B + 2D plus
@@ -41,51 +46,51 @@ __device__ __forceinline__ bool spec_ok(const CkptParams &P, uint64_t po, uint64
 }
 
 // Partial CRAC-FP64 sum of a segment (<= 8 KiB) whose first word is word j0
-// of its chunk, over the lanes of one warp; with copy_to, the segment's bytes
-// are also stored there, and then (kHdr) the CRZ1 header word of each whole
-// 512-byte block of the segment goes to hdr[block] (lane l holds bytes
-// 16l .. 16l+15 of block u in q[u], the encoder's layout of a block).  Only
-// chunks written to staging get headers, so their cost follows the dirty bytes.
-template <bool kHdr = false>
-__device__ __forceinline__ uint64_t hash_seg(const uint8_t *__restrict__ src, uint32_t len, uint64_t j0,
-                                             int lane, uint4 *__restrict__ copy_to = nullptr,
-                                             uint64_t *__restrict__ hdr = nullptr) {
+// of its chunk, over the lanes of one warp.  dest(), asked for once the first
+// loads are on their way, says where the segment's bytes are also stored (null:
+// nowhere); then (kHdr) the CRZ1 header word of each whole 512-byte block of
+// the segment goes to hdr[block] (lane l holds bytes 16l .. 16l+15 of block u
+// in q[u], the encoder's layout of a block).  Only chunks written to staging
+// get headers, so their cost follows the dirty bytes.
+template <bool kHdr, class Dest>
+__device__ __forceinline__ uint64_t hash_seg(const uint8_t *__restrict__ src, uint32_t len, uint32_t j0, int lane,
+                                             Dest &&dest, uint64_t *__restrict__ hdr) {
     const uint4 *p = reinterpret_cast<const uint4 *>(src);
     const uint32_t nv = len >> 4;
-    constexpr int U = 16;
-    uint4 q[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-        const uint32_t v = lane + 32u * u;
-        if (v < nv) q[u] = __ldg(p + v);
-    }
-    if (copy_to) {   // FULL checkpoint: the vectors also go straight to staging
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const uint32_t v = lane + 32u * u;
-            if (v < nv) __stcs(copy_to + v, q[u]);
-        }
-    }
+    constexpr int U = 8;
     uint64_t acc = 0;
-    uint64_t key = (j0 + 2ull * (uint64_t)lane + 1ull) * kK1;
+    uint64_t key = (uint64_t)(j0 + 2u * lane + 1u) * kK1;
     constexpr uint64_t kStep = 64ull * kK1;
+    uint4 *copy_to = nullptr;
+#pragma unroll 1
+    for (uint32_t v0 = 0; v0 < nv || v0 == 0; v0 += 32 * U) {   // warp-uniform
+        uint4 q[U];
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-        const uint32_t v = lane + 32u * u;
-        if (v < nv) {
-            acc += mixw(((uint64_t)q[u].y << 32) | q[u].x, key);
-            acc += mixw(((uint64_t)q[u].w << 32) | q[u].z, key + kK1);
+        for (int u = 0; u < U; ++u)
+            if (v0 + 32u * u + lane < nv) q[u] = __ldg(p + v0 + 32u * u + lane);
+        if (v0 == 0) copy_to = dest();
+        if (copy_to) {   // the vectors also go straight to staging
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (v0 + 32u * u + lane < nv) __stcs(copy_to + v0 + 32u * u + lane, q[u]);
         }
-        key += kStep;
-    }
-    if (kHdr && copy_to) {
-        const uint32_t nb = len >> 9;   // whole blocks (warp-uniform)
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            if ((uint32_t)u < nb) {
-                const uint32_t r[4] = {crz_rot(q[u].x), crz_rot(q[u].y), crz_rot(q[u].z), crz_rot(q[u].w)};
-                const uint64_t h = crz_block_header(r);
-                if (lane == 0) hdr[u] = h;
+            if (v0 + 32u * u + lane < nv) {
+                acc += mixw(((uint64_t)q[u].y << 32) | q[u].x, key);
+                acc += mixw(((uint64_t)q[u].w << 32) | q[u].z, key + kK1);
+            }
+            key += kStep;
+        }
+        if (kHdr && copy_to) {
+            const uint32_t b0 = v0 >> 5, nb = len >> 9;   // this round's first block, whole blocks
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (b0 + u < nb) {
+                    const uint32_t r[4] = {crz_rot(q[u].x), crz_rot(q[u].y), crz_rot(q[u].z), crz_rot(q[u].w)};
+                    const uint64_t h = crz_block_header(r);
+                    if (lane == 0) hdr[b0 + u] = h;
+                }
             }
         }
     }
@@ -99,7 +104,7 @@ __device__ __forceinline__ uint64_t hash_seg(const uint8_t *__restrict__ src, ui
             else w1 |= byte << (8 * (b - 8));
             if (copy_to) reinterpret_cast<uint8_t *>(copy_to + nv)[b] = (uint8_t)byte;
         }
-        const uint64_t kt = (j0 + 2ull * nv + 1ull) * kK1;
+        const uint64_t kt = (uint64_t)(j0 + 2u * nv + 1u) * kK1;
         acc += mixw(w0, kt);
         if (rem > 8) acc += mixw(w1, kt + kK1);
     }
@@ -142,57 +147,53 @@ __device__ __forceinline__ void copy_with_headers(uint8_t *__restrict__ dst, con
 }
 
 template <bool kHdr>
-__global__ void __launch_bounds__(kHashNT, 2)
+__global__ void __launch_bounds__(kHashNT, 3)
 split_hash_kernel(const CkptParams P, unsigned long long *__restrict__ acc, uint32_t log2Seg) {
-    const int lane = threadIdx.x & 31;
-    const uint64_t warp_g = ((uint64_t)blockIdx.x * kHashNT + threadIdx.x) >> 5;
-    const uint64_t n_warps = ((uint64_t)gridDim.x * kHashNT) >> 5;
+    constexpr uint32_t kWarps = kHashNT / 32;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t log2S = P.log2_chunk;
     const uint32_t spc = log2S - log2Seg;   // log2 of segments per chunk
-    const uint64_t n_slots = (P.c_end - P.c_begin) << spc;
-    const uint64_t per = (n_slots + n_warps - 1) / n_warps;
-    uint64_t q = warp_g * per;
-    const uint64_t q_end = umin64(q + per, n_slots);
-    CkptDesc d{};
-    uint64_t a_next = 0;
+    // The CTA's segments in turn to its warps, so that it streams through them.
+    const uint64_t per_cta = (uint64_t)kWarps * P.slots_per_warp;
+    const uint64_t q_end = umin64((blockIdx.x + 1) * per_cta, (P.c_end - P.c_begin) << spc);
     uint32_t a = 0;
-    bool have = false;
-    uint32_t writes = 0;   // chunks this warp wrote speculatively (lane 0)
-    for (; q < q_end; ++q) {
+    uint64_t a_next = 0;   // first chunk after allocation a
+    CkptDesc d{};
+    uint32_t writes = 0;   // chunks this warp wrote speculatively
+    for (uint64_t q = blockIdx.x * per_cta + warp; q < q_end; q += kWarps) {
         const uint64_t c = P.c_begin + (q >> spc);
-        if (!have || c >= a_next) {
-            a = find_alloc(P.desc, P.n_allocs, c);
+        if (c >= a_next) {
+            a = find_alloc_warp(P.desc, P.n_allocs, c, lane);
             d = P.desc[a];
-            a_next = a + 1 < P.n_allocs ? P.desc[a + 1].first_chunk : ~0ull;
-            have = true;
+            a_next = d.first_chunk + ((d.bytes - 1) >> log2S) + 1;
         }
         const uint64_t local = c - d.first_chunk;
-        const uint64_t rest = d.bytes - (local << log2S);
-        const uint64_t clen = rest < (1ull << log2S) ? rest : (1ull << log2S);
-        const uint64_t off = (q & ((1ull << spc) - 1)) << log2Seg;
+        const uint32_t clen = (uint32_t)umin64(d.bytes - (local << log2S), 1ull << log2S);
+        const uint32_t off = (uint32_t)(q & ((1ull << spc) - 1)) << log2Seg;
         if (off >= clen) continue;   // beyond the end of a short last chunk (warp-uniform)
-        const uint32_t len = (uint32_t)umin64(1ull << log2Seg, clen - off);
+        const uint32_t len = min(1u << log2Seg, clen - off);
         // Direct mode (S <= 8 KiB, the warp sees the whole chunk): the baseline
         // fingerprint is loaded before the chunk so that both latencies overlap.
         uint64_t fo = 0;
         const bool has = d.base_first != kNoBase;
         if (spc == 0 && lane == 0 && has) fo = __ldg(P.fp_old + d.base_first + local);
-        const uint8_t *src = reinterpret_cast<const uint8_t *>(d.ptr) + (local << log2S) + off;
-        uint4 *copy_to = nullptr;
-        if (P.full_copy) {   // FULL checkpoint: the segment's final staging offset is known
-            const uint64_t o = P.alloc_prefix[a] + (local << log2S) + off - P.seg_base;
-            if (o + len <= P.staging_cap) copy_to = reinterpret_cast<uint4 *>(P.staging + o);
-            else if (lane == 0) atomicOr(&P.ctrl->err, kErrBounds);
-        } else if (P.ppos) {   // predicted dirty: written to the offset it had last time
-            const uint64_t po = __ldg(P.ppos + (c - P.c_begin));
-            if (spec_ok(P, po, clen)) {
-                copy_to = reinterpret_cast<uint4 *>(P.staging + po + off);
-                writes += off == 0 ? 1u : 0u;
+        auto dest = [&]() -> uint4 * {
+            if (P.full_copy) {   // FULL checkpoint: the segment's final staging offset is known
+                const uint64_t o = P.alloc_prefix[a] + (local << log2S) + off - P.seg_base;
+                if (o + len <= P.staging_cap) return reinterpret_cast<uint4 *>(P.staging + o);
+                if (lane == 0) atomicOr(&P.ctrl->err, kErrBounds);
+            } else if (P.ppos) {   // predicted dirty: written to the offset it had last time
+                const uint64_t po = __ldg(P.ppos + (c - P.c_begin));
+                if (spec_ok(P, po, clen)) {
+                    writes += off == 0 ? 1u : 0u;
+                    return reinterpret_cast<uint4 *>(P.staging + po + off);
+                }
             }
-        }
-        uint64_t sum = kHdr ? hash_seg<true>(src, len, off >> 3, lane, copy_to,
-                                             P.crz_hdr + (c << (log2S - 9)) + (off >> 9))
-                            : hash_seg(src, len, off >> 3, lane, copy_to);
+            return nullptr;
+        };
+        const uint8_t *src = reinterpret_cast<const uint8_t *>(d.ptr) + (local << log2S) + off;
+        uint64_t sum = hash_seg<kHdr>(src, len, off >> 3, lane, dest,
+                                      kHdr ? P.crz_hdr + (c << (log2S - 9)) + (off >> 9) : nullptr);
         sum = warp_sum(sum);
         if (lane == 0) {
             if (spc == 0) {
@@ -209,13 +210,17 @@ split_hash_kernel(const CkptParams P, unsigned long long *__restrict__ acc, uint
     if (lane == 0 && writes) atomicAdd(&P.ctrl->spec_writes, (unsigned long long)writes);
 }
 
-// When log2Seg == log2_chunk the hash kernel has already finalized every
-// chunk and left its length and dirty bit in acc; only the compaction remains.
-// Hash kernel for chunks of 512 B..4 KiB: one warp iteration covers 8 KiB,
-// i.e. 8192/S whole chunks, one group of LPC = 32*S/8192 lanes per chunk (16
-// vectors per lane), so a warp keeps 8 KiB in flight whatever the chunk size.
+// Hash kernel for chunks of 512 B..4 KiB: one warp iteration covers 4 KiB,
+// i.e. 4096/S whole chunks, one group of LPC = S/128 lanes per chunk (8
+// vectors per lane), so a warp keeps 4 KiB in flight whatever the chunk size; a
+// warp makes two iterations, a CTA 64 KiB, in the grid of split_hash_kernel
+// (8 GiB in 4 KiB chunks, every chunk written: 2741 -> 2407 us against one wave
+// of resident CTAs; one iteration per warp gives 2397, four 2453).
 // Every chunk is finalized in place (direct mode: acc receives the dirty
-// length).
+// length, and finalize only compacts).
+constexpr int kSmallVecs = 8;     // vectors per lane of one iteration
+constexpr int kSmallIters = 2;    // iterations per warp
+
 template <int LPC>
 __device__ __forceinline__ void hash_small_iter(const CkptParams &P, unsigned long long *__restrict__ acc,
                                                 uint64_t c, const CkptDesc &d_warp, uint32_t a_warp,
@@ -227,7 +232,7 @@ __device__ __forceinline__ void hash_small_iter(const CkptParams &P, unsigned lo
     CkptDesc d = d_warp;
     uint32_t a = a_warp;
     uint64_t local = 0;
-    uint4 q[16];
+    uint4 q[kSmallVecs];
     // Sparse delta pass: the group holds its whole chunk in q until the
     // fingerprint is known and stores it only if it is dirty (B + D of HBM
     // traffic instead of B + B); clean chunks' bytes are never referenced.
@@ -246,14 +251,14 @@ __device__ __forceinline__ void hash_small_iter(const CkptParams &P, unsigned lo
         const uint4 *p = reinterpret_cast<const uint4 *>(reinterpret_cast<const uint8_t *>(d.ptr) + (local << log2S));
         nv = len >> 4;
 #pragma unroll
-        for (int u = 0; u < 16; ++u) {
+        for (int u = 0; u < kSmallVecs; ++u) {
             const uint32_t v = li + LPC * u;
             if (v < nv) q[u] = __ldg(p + v);
         }
         uint64_t key = (2ull * (uint64_t)li + 1ull) * kK1;
         constexpr uint64_t kStep = 2ull * LPC * kK1;
 #pragma unroll
-        for (int u = 0; u < 16; ++u) {
+        for (int u = 0; u < kSmallVecs; ++u) {
             const uint32_t v = li + LPC * u;
             if (v < nv) {
                 sum += mixw(((uint64_t)q[u].y << 32) | q[u].x, key);
@@ -266,7 +271,7 @@ __device__ __forceinline__ void hash_small_iter(const CkptParams &P, unsigned lo
             if (o + len <= P.staging_cap) {
                 uint4 *dst = reinterpret_cast<uint4 *>(P.staging + o);
 #pragma unroll
-                for (int u = 0; u < 16; ++u) {
+                for (int u = 0; u < kSmallVecs; ++u) {
                     const uint32_t v = li + LPC * u;
                     if (v < nv) __stcs(dst + v, q[u]);
                 }
@@ -279,7 +284,7 @@ __device__ __forceinline__ void hash_small_iter(const CkptParams &P, unsigned lo
                 writes += li == 0 ? 1u : 0u;
                 uint8_t *dst = P.staging + po;
 #pragma unroll
-                for (int u = 0; u < 16; ++u) {
+                for (int u = 0; u < kSmallVecs; ++u) {
                     const uint32_t v = li + LPC * u;
                     if (v < nv) __stcs(reinterpret_cast<uint4 *>(dst) + v, q[u]);
                 }
@@ -320,7 +325,7 @@ __device__ __forceinline__ void hash_small_iter(const CkptParams &P, unsigned lo
         if (o + len <= P.staging_cap) {
             uint4 *dst = reinterpret_cast<uint4 *>(P.staging + o);
 #pragma unroll
-            for (int u = 0; u < 16; ++u) {
+            for (int u = 0; u < kSmallVecs; ++u) {
                 const uint32_t v = li + LPC * u;
                 if (v < nv) __stcs(dst + v, q[u]);
             }
@@ -331,28 +336,24 @@ __device__ __forceinline__ void hash_small_iter(const CkptParams &P, unsigned lo
 }
 
 template <int LPC>
-__global__ void __launch_bounds__(kHashNT, 2)
+__global__ void __launch_bounds__(kHashNT, 3)
 split_hash_small_kernel(const CkptParams P, unsigned long long *__restrict__ acc, uint32_t) {
-    constexpr int CPS = 32 / LPC;   // chunks per 8 KiB segment
+    constexpr int CPS = 32 / LPC;   // chunks per iteration
     const int lane = threadIdx.x & 31;
     const uint64_t warp_g = ((uint64_t)blockIdx.x * kHashNT + threadIdx.x) >> 5;
-    const uint64_t n_warps = ((uint64_t)gridDim.x * kHashNT) >> 5;
     const uint64_t n_slots = (P.c_end - P.c_begin + CPS - 1) / CPS;
-    const uint64_t per = (n_slots + n_warps - 1) / n_warps;
-    uint64_t q = warp_g * per;
-    const uint64_t q_end = umin64(q + per, n_slots);
+    uint64_t q = warp_g * kSmallIters;
+    const uint64_t q_end = umin64(q + kSmallIters, n_slots);
     CkptDesc d{};
     uint64_t a_next = 0;
     uint32_t a = 0;
-    bool have = false;
     uint32_t writes = 0;   // chunks this lane's groups wrote speculatively (group leaders)
     for (; q < q_end; ++q) {
         const uint64_t c0 = P.c_begin + q * CPS;
-        if (!have || c0 >= a_next) {
-            a = find_alloc(P.desc, P.n_allocs, c0);
+        if (c0 >= a_next) {
+            a = find_alloc_warp(P.desc, P.n_allocs, c0, lane);
             d = P.desc[a];
-            a_next = a + 1 < P.n_allocs ? P.desc[a + 1].first_chunk : ~0ull;
-            have = true;
+            a_next = d.first_chunk + ((d.bytes - 1) >> P.log2_chunk) + 1;
         }
         hash_small_iter<LPC>(P, acc, c0 + lane / LPC, d, a, a_next, lane % LPC, writes);
     }
@@ -362,109 +363,65 @@ split_hash_small_kernel(const CkptParams P, unsigned long long *__restrict__ acc
 
 // ---------------------------------------------------------------------------
 // Sparse pass on 512 B - 4 KiB chunks with dense placement (P.sparse == 2).
-// Each warp iteration hashes 8 KiB of whole chunks as split_hash_small_kernel
-// does, then stages its dirty chunks back to back in the warp's 8 KiB of
-// shared memory and takes their room in the image from a running byte
-// counter (P.ctrl->pad[0], one atomicAdd per iteration with dirty bytes).
-// The counter's answer is used one iteration later: after the next
-// iteration's loads are issued, one lane stores the staged bytes with a bulk
-// copy (shared -> global) and the group leaders record each chunk's offset
-// in its accumulator word, so neither the atomic's round trip nor the store
-// holds the loads up.  The image's span is then exactly its dirty bytes.
-// Sizes are multiples of 16 (a sparse pass requires it), so every staged
-// chunk and every offset is 16-byte aligned.
+// A warp hashes 4 KiB of whole chunks as split_hash_small_kernel does, holding
+// them in registers, takes the room of its dirty chunks in the image from a
+// running byte counter (P.ctrl->pad[0], one atomicAdd where any is dirty) and
+// stores them there, back to back; the SM's other warps cover the atomic's
+// round trip.  The image's span is then exactly its dirty bytes, and the group
+// leaders record each chunk's offset in its accumulator word.  Sizes are
+// multiples of 16 (a sparse pass requires it), so every offset is 16-byte
+// aligned.  8 GiB in 4 KiB chunks, 10% dirty: 1400 -> 1330 us against a form
+// that staged the dirty chunks in shared memory in one wave of resident CTAs;
+// one atomic per CTA, with two barriers for it, took 1505.
 // ---------------------------------------------------------------------------
-constexpr uint32_t kDenseWarpBytes = 8192;   // shared memory per warp
 constexpr uint64_t kAccLenMask = (1ull << 24) - 1;   // accumulator word: length in bits 0-23,
 constexpr int kAccPosShift = 24;                     // the chunk's offset in bits 24-62 (dense
 constexpr uint64_t kAccPosMask = (1ull << 39) - 1;   // sparse placement), kAccDirty in bit 63
 
-__device__ __forceinline__ void dense_bulk_store(void *dst, const void *src_smem, uint32_t bytes) {
-    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst),
-                 "r"((uint32_t)__cvta_generic_to_shared(src_smem)), "r"(bytes)
-                 : "memory");
-    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-}
-__device__ __forceinline__ void dense_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
-__device__ __forceinline__ void dense_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
-__device__ __forceinline__ void dense_fence() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-
 template <int LPC>
-__global__ void __launch_bounds__(kHashNT, 2)
+__global__ void __launch_bounds__(kHashNT, 4)
 split_hash_small_dense_kernel(const CkptParams P, unsigned long long *__restrict__ acc, uint32_t) {
-    extern __shared__ __align__(128) uint8_t dense_smem[];
-    constexpr int CPS = 32 / LPC;   // chunks per 8 KiB iteration
+    constexpr int CPS = 32 / LPC;   // chunks per iteration
     const int lane = threadIdx.x & 31;
     const int li = lane % LPC;
-    uint8_t *buf = dense_smem + (threadIdx.x >> 5) * kDenseWarpBytes;
-    const uint64_t warp_g = ((uint64_t)blockIdx.x * kHashNT + threadIdx.x) >> 5;
-    const uint64_t n_warps = ((uint64_t)gridDim.x * kHashNT) >> 5;
-    const uint64_t n_slots = (P.c_end - P.c_begin + CPS - 1) / CPS;
-    const uint64_t per = (n_slots + n_warps - 1) / n_warps;
-    uint64_t q = warp_g * per;
-    const uint64_t q_end = umin64(q + per, n_slots);
     const uint32_t log2S = P.log2_chunk;
-    CkptDesc dw{};
+    const uint64_t warp_g = ((uint64_t)blockIdx.x * kHashNT + threadIdx.x) >> 5;
+    uint32_t a = 0;
     uint64_t a_next = 0;
-    uint32_t aw = 0;
-    bool have = false;
-    // the previous iteration's staged chunks: warp-uniform byte count, the
-    // counter's answer (lane 0), and each group's chunk, length and offset
-    uint32_t pend_total = 0;
-    unsigned long long pend_base = 0;
-    uint64_t pend_c = 0;
-    uint32_t pend_len = 0, pend_loc = 0;
-    bool pend_dirty = false;
-    auto flush = [&]() {
-        if (!pend_total) return;   // warp-uniform
-        const uint64_t base = __shfl_sync(kFull, (uint64_t)pend_base, 0);
-        const bool fits = base + pend_total <= P.staging_cap;
-        if (lane == 0) {
-            if (fits) dense_bulk_store(P.staging + base, buf, pend_total);
-            else atomicOr(&P.ctrl->err, kErrBounds);
-        }
-        if (li == 0 && pend_dirty)
-            acc[pend_c - P.c_begin] = pend_len | kAccDirty | ((fits ? base + pend_loc : 0ull) << kAccPosShift);
-        pend_total = 0;
-    };
-    for (; q < q_end; ++q) {
-        const uint64_t c0 = P.c_begin + q * CPS;
-        if (!have || c0 >= a_next) {
-            aw = find_alloc(P.desc, P.n_allocs, c0);
-            dw = P.desc[aw];
-            a_next = aw + 1 < P.n_allocs ? P.desc[aw + 1].first_chunk : ~0ull;
-            have = true;
+    CkptDesc dw{};
+#pragma unroll 1
+    for (int it = 0; it < kSmallIters; ++it) {
+        const uint64_t c0 = P.c_begin + (warp_g * kSmallIters + it) * CPS;
+        if (c0 >= P.c_end) break;   // warp-uniform
+        if (c0 >= a_next) {
+            a = find_alloc_warp(P.desc, P.n_allocs, c0, lane);
+            dw = P.desc[a];
+            a_next = dw.first_chunk + ((dw.bytes - 1) >> log2S) + 1;
         }
         const uint64_t c = c0 + lane / LPC;
         uint64_t sum = 0, fo = 0;
         uint32_t len = 0, nv = 0;
         bool has = false;
-        uint4 v16[16];
+        uint4 q[kSmallVecs];
         if (c < P.c_end) {
             CkptDesc d = dw;
             if (c >= a_next) d = P.desc[find_alloc(P.desc, P.n_allocs, c)];   // the iteration crosses an allocation end
             const uint64_t local = c - d.first_chunk;
             len = (uint32_t)umin64(d.bytes - (local << log2S), 1ull << log2S);
             has = d.base_first != kNoBase;
-            if (li == 0 && has) fo = __ldg(P.fp_old + d.base_first + local);
             const uint4 *p = reinterpret_cast<const uint4 *>(reinterpret_cast<const uint8_t *>(d.ptr) + (local << log2S));
             nv = len >> 4;
 #pragma unroll
-            for (int u = 0; u < 16; ++u) {
-                const uint32_t v = li + LPC * u;
-                if (v < nv) v16[u] = __ldg(p + v);
-            }
-        }
-        flush();   // the previous iteration's chunks leave shared memory while these loads are in flight
-        if (c < P.c_end) {
+            for (int u = 0; u < kSmallVecs; ++u)
+                if ((uint32_t)(li + LPC * u) < nv) q[u] = __ldg(p + li + LPC * u);
+            if (li == 0 && has) fo = __ldg(P.fp_old + d.base_first + local);
             uint64_t key = (2ull * (uint64_t)li + 1ull) * kK1;
             constexpr uint64_t kStep = 2ull * LPC * kK1;
 #pragma unroll
-            for (int u = 0; u < 16; ++u) {
-                const uint32_t v = li + LPC * u;
-                if (v < nv) {
-                    sum += mixw(((uint64_t)v16[u].y << 32) | v16[u].x, key);
-                    sum += mixw(((uint64_t)v16[u].w << 32) | v16[u].z, key + kK1);
+            for (int u = 0; u < kSmallVecs; ++u) {
+                if ((uint32_t)(li + LPC * u) < nv) {
+                    sum += mixw(((uint64_t)q[u].y << 32) | q[u].x, key);
+                    sum += mixw(((uint64_t)q[u].w << 32) | q[u].z, key + kK1);
                 }
                 key += kStep;
             }
@@ -478,34 +435,33 @@ split_hash_small_dense_kernel(const CkptParams P, unsigned long long *__restrict
             P.fp_new[c] = fp;
             if (!dirty) acc[c - P.c_begin] = len;
         }
-        // stage the dirty chunks back to back in the warp's buffer
-        const uint64_t mine = (li == 0 && dirty) ? len : 0u;
-        const uint64_t incl = warp_incl_scan(mine, lane);
-        const uint32_t total = (uint32_t)__shfl_sync(kFull, incl, 31);
-        const uint32_t loc = (uint32_t)__shfl_sync(kFull, incl - mine, lane - li);
-        if (total) {   // warp-uniform
-            if (lane == 0) dense_wait_read();   // the previous bulk store has read the buffer
-            __syncwarp();
-            if (dirty) {
-                uint4 *dst = reinterpret_cast<uint4 *>(buf + loc);
+        if (!__any_sync(kFull, dirty)) continue;
+        const uint32_t mine = (li == 0 && dirty) ? len : 0u;
+        uint32_t incl = mine;
+        if (LPC < 32) {
 #pragma unroll
-                for (int u = 0; u < 16; ++u) {
-                    const uint32_t v = li + LPC * u;
-                    if (v < nv) dst[v] = v16[u];
-                }
+            for (int o = LPC; o < 32; o <<= 1) {   // only the leaders hold a length
+                const uint32_t t = __shfl_up_sync(kFull, incl, o);
+                if (lane >= o) incl += t;
             }
-            dense_fence();   // the staged bytes are visible to the bulk copy
-            __syncwarp();
-            if (lane == 0) pend_base = atomicAdd(&P.ctrl->pad[0], (unsigned long long)total);
         }
-        pend_total = total;
-        pend_c = c;
-        pend_len = len;
-        pend_loc = loc;
-        pend_dirty = dirty;
+        const uint32_t total = __shfl_sync(kFull, incl, 32 - LPC);   // the last leader
+        const uint32_t loc = __shfl_sync(kFull, incl - mine, lane - li);
+        uint64_t base = 0;
+        if (lane == 0) base = atomicAdd(&P.ctrl->pad[0], (unsigned long long)total);
+        base = __shfl_sync(kFull, base, 0);
+        const bool fits = base + total <= P.staging_cap;
+        if (!fits && lane == 0) atomicOr(&P.ctrl->err, kErrBounds);
+        if (dirty) {
+            if (li == 0) acc[c - P.c_begin] = len | kAccDirty | ((fits ? base + loc : 0ull) << kAccPosShift);
+            if (fits) {
+                uint4 *dst = reinterpret_cast<uint4 *>(P.staging + base + loc);
+#pragma unroll
+                for (int u = 0; u < kSmallVecs; ++u)
+                    if ((uint32_t)(li + LPC * u) < nv) __stcs(dst + li + LPC * u, q[u]);
+            }
+        }
     }
-    flush();
-    if (lane == 0) dense_wait_all();   // shared memory stays until the bulk stores have finished
 }
 
 constexpr uint32_t kFinCachedAllocs = 4096;   // first_chunk columns the finalize keeps on chip
@@ -727,10 +683,10 @@ const void *split_hash_fn(bool crz_headers) {
 }
 const void *split_hash_small_fn(int lanes_per_chunk) {
     switch (lanes_per_chunk) {
-    case 2: return reinterpret_cast<const void *>(&split_hash_small_kernel<2>);
     case 4: return reinterpret_cast<const void *>(&split_hash_small_kernel<4>);
     case 8: return reinterpret_cast<const void *>(&split_hash_small_kernel<8>);
     case 16: return reinterpret_cast<const void *>(&split_hash_small_kernel<16>);
+    case 32: return reinterpret_cast<const void *>(&split_hash_small_kernel<32>);
     default: return nullptr;
     }
 }
@@ -747,26 +703,39 @@ int split_finalize_threads() { return kFinNT; }
 int split_gather_threads() { return kGatherNT; }
 const void *split_hash_small_dense_fn(int lanes_per_chunk) {
     switch (lanes_per_chunk) {
-    case 2: return reinterpret_cast<const void *>(&split_hash_small_dense_kernel<2>);
     case 4: return reinterpret_cast<const void *>(&split_hash_small_dense_kernel<4>);
     case 8: return reinterpret_cast<const void *>(&split_hash_small_dense_kernel<8>);
     case 16: return reinterpret_cast<const void *>(&split_hash_small_dense_kernel<16>);
+    case 32: return reinterpret_cast<const void *>(&split_hash_small_dense_kernel<32>);
     default: return nullptr;
     }
 }
-size_t split_dense_smem() { return (size_t)(kHashNT / 32) * kDenseWarpBytes; }
-cudaError_t split_dense_prepare(const void *fn) {
-    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)split_dense_smem());
+// Bytes of a segment: 8 KiB; 16 KiB where the pass mostly reads and is large
+// enough that every SM still gets dozens of CTAs (4 GiB, read only: 623 -> 600
+// us), not where it writes every chunk (1211 -> 1234 us).
+uint32_t split_hash_seg(uint64_t bytes, uint32_t log2S, bool copy) {
+    const uint32_t m = copy || (bytes >> 14) < 32768 ? 13 : 14;
+    return log2S < m ? log2S : m;
 }
-int split_max_ctas_per_sm_smem(const void *fn, int threads, size_t smem) {
-    int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, threads, smem) != cudaSuccess) return 1;
-    return n > 0 ? n : 1;
-}
-int split_max_ctas_per_sm(const void *fn, int threads) {
-    int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, threads, 0) != cudaSuccess) return 1;
-    return n > 0 ? n : 1;
+
+// A warp takes one segment, or as many as hold a segment's bytes on average
+// (chunks below 512 B; allocations mostly much shorter than a chunk, whose
+// segments past their end are empty).
+uint32_t split_hash_grid(uint64_t n_chunks, uint64_t bytes, uint32_t log2S, uint32_t log2Seg,
+                         uint32_t *slots_per_warp) {
+    constexpr uint64_t kWarps = kHashNT / 32;
+    uint64_t per, n = n_chunks;   // items per warp, items
+    if (log2S >= 9 && log2S < 13) {   // chunks
+        per = (4096ull >> log2S) * kSmallIters;
+    } else {                          // segments
+        n <<= log2S - log2Seg;
+        const uint32_t m = log2Seg < 13 ? 13 : log2Seg;
+        per = n / ((bytes >> m) + 1);
+        per = per < 1 ? 1 : umin64(per, 1u << 20);
+    }
+    *slots_per_warp = (uint32_t)per;
+    const uint64_t g = (n + per * kWarps - 1) / (per * kWarps);
+    return (uint32_t)(g < 1 ? 1 : umin64(g, 0x7fffffffull));
 }
 
 }  // namespace crac

@@ -532,10 +532,6 @@ cudaError_t launch_link_copy(void *dst, const void *src, uint64_t bytes, int max
 // (lanes_per_chunk = chunk bytes / 256), the dynamic shared memory it runs
 // with, the attribute that allows it (before its first launch or graph
 // node), and occupancy with dynamic shared memory (crac_pass_split.cu).
-const void *split_hash_small_dense_fn(int lanes_per_chunk);
-size_t split_dense_smem();
-cudaError_t split_dense_prepare(const void *fn);
-int split_max_ctas_per_sm_smem(const void *fn, int threads, size_t smem);
 
 // Entries [0, n) of a sparse device piece packed back to back into device
 // memory dst: entry j's cum[j+1] - cum[j] bytes from span + off[j] to
