@@ -63,6 +63,7 @@ struct CkptParams {
     // skipped.
     uint32_t full_copy;
     const uint64_t *alloc_prefix;   // payload bytes of all allocations before each one
+    const uint32_t *full_flag;      // null, or a device word that can still take full_copy back
     uint64_t seg_base;              // payload offset of the segment's first chunk
     // Sparse split pass (with full_copy, on delta checkpoints too): chunks
     // are written at their uncompacted offsets (on a delta with chunks of
@@ -131,8 +132,6 @@ struct PerAllocCarry {
 };
 
 // ---- launchers (return cudaGetLastError() of the launch) ----------------
-cudaError_t launch_ckpt_fused(const CkptParams &p, int threads, int warps_per_chunk, int grid,
-                              cudaStream_t s);
 // Kernel entry of the fused pass for a (threads, warps_per_chunk) variant, for
 // building a graph kernel node; nullptr if the variant does not exist.
 const void *ckpt_fused_fn(int threads, int warps_per_chunk);

@@ -5,9 +5,11 @@
 //
 // For callers that must not allocate (an interposed cudaMalloc/cudaFree
 // wrapper, an allocator hook, a preemption-time checkpoint, a process out of
-// memory): the same fused kernel, with its scratch -- the control block and
-// the look-back status words -- in a fixed array of this library's device
-// memory instead of a buffer obtained from cudaMalloc.
+// memory): the kernels of the split pass (hash, finalize, gather), with their
+// scratch -- the control block, the look-back status words and the regions'
+// payload offsets -- in a fixed array of this library's device memory instead
+// of a buffer obtained from cudaMalloc, and the caller's fingerprint table as
+// the chunks' accumulators.
 // ---------------------------------------------------------------------------
 
 namespace {
@@ -18,8 +20,55 @@ constexpr size_t kNoAllocScratchBytes =
 constexpr int kNoAllocMaxDevices = 64;
 std::mutex g_noalloc_mu;
 void *g_noalloc_addr[kNoAllocMaxDevices];     // device address of the scratch, per device
-int g_noalloc_grid[kNoAllocMaxDevices][2];   // SMs x occupancy for warps-per-chunk 1 and 8
+int g_noalloc_grid[kNoAllocMaxDevices][2];   // SMs x occupancy of the fused kernel for warps-per-chunk 1 and 8
+int g_noalloc_sms[kNoAllocMaxDevices];
 
+constexpr int kPrefixNT = 1024;
+
+// One CTA, before a pass without a baseline: the payload bytes before each
+// region, and the flag that the hash kernel may write every chunk there as it
+// reads it (every size a multiple of 16 bytes, and room for them all).
+__global__ void __launch_bounds__(kPrefixNT)
+noalloc_prefix_kernel(const crac::CkptDesc *__restrict__ d, uint32_t n, uint64_t cap, uint64_t *__restrict__ prefix,
+                      uint32_t *__restrict__ flag) {
+    using namespace crac;
+    __shared__ uint64_t s_sum[kPrefixNT / 32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t per = (n + kPrefixNT - 1) / kPrefixNT;
+    const uint32_t i0 = threadIdx.x * per, i1 = min(n, i0 + per);
+    uint64_t sum = 0;
+    bool odd = false;
+    for (uint32_t i = i0; i < i1; ++i) {
+        sum += d[i].bytes;
+        odd |= (d[i].bytes & 15u) != 0;
+    }
+    uint64_t incl = warp_incl_scan(sum, lane);
+    if (lane == 31) s_sum[warp] = incl;
+    odd = __syncthreads_or(odd);
+    uint64_t before = 0, total = 0;
+    for (int w = 0; w < kPrefixNT / 32; ++w) {
+        if (w < warp) before += s_sum[w];
+        total += s_sum[w];
+    }
+    uint64_t at = before + incl - sum;
+    for (uint32_t i = i0; i < i1; ++i) {
+        prefix[i] = at;
+        at += d[i].bytes;
+    }
+    if (threadIdx.x == 0) *flag = !odd && total <= cap ? 1u : 0u;
+}
+
+// The pass's results (a crac_pass_totals_t at any address) from its control
+// block.  `reserved` keeps the value that earlier versions left in that word
+// (tiles and CTAs of a ticket-driven pass).
+__global__ void noalloc_totals_kernel(const crac::CkptCtrl *ctrl, uint8_t *out, uint32_t reserved) {
+    const uint32_t t = threadIdx.x;
+    if (t >= sizeof(crac_pass_totals_t)) return;
+    const uint64_t w = t < 8 ? (uint64_t)ctrl->err << 32 | reserved : t < 16 ? ctrl->k : ctrl->D;
+    out[t] = (uint8_t)(w >> (8 * (t & 7u)));
+}
+
+// Tile of the pass's limit (CRAC_NOALLOC_MAX_TILES), in chunks.
 uint32_t noalloc_split(uint32_t chunk_bytes, int *wpc) {
     *wpc = chunk_bytes >= 16384u ? 8 : 1;
     uint32_t cpt = (128u << 10) / chunk_bytes;
@@ -79,6 +128,7 @@ extern "C" crac_status_t crac_pass_noalloc(const crac_region_t *regions_dev, uin
                 note_cuda_error((int)e);
                 return CRAC_ERR_CUDA;
             }
+            g_noalloc_sms[dev] = sms;
             g_noalloc_grid[dev][0] = sms * (ckpt_fused_max_ctas_per_sm(256, 1) > 0 ? ckpt_fused_max_ctas_per_sm(256, 1) : 1);
             g_noalloc_grid[dev][1] = sms * (ckpt_fused_max_ctas_per_sm(256, 8) > 0 ? ckpt_fused_max_ctas_per_sm(256, 8) : 1);
             g_noalloc_addr[dev] = p;
@@ -87,9 +137,12 @@ extern "C" crac_status_t crac_pass_noalloc(const crac_region_t *regions_dev, uin
         grid_per[0] = g_noalloc_grid[dev][0];
         grid_per[1] = g_noalloc_grid[dev][1];
     }
-    const size_t used = sizeof(CkptCtrl) + 16 * n_tiles;
+    const uint32_t fin_tiles = (uint32_t)((n_chunks + split_finalize_threads() - 1) / split_finalize_threads());
+    const size_t used = sizeof(CkptCtrl) + 16 * (size_t)fin_tiles;   // at most 128 KiB + 64 B of the scratch
     e = cudaMemsetAsync(scratch, 0, used, s);   // control block + status words start at zero
+    uint32_t reserved = 0;
     if (e == cudaSuccess && n_tiles) {
+        unsigned char *sc = static_cast<unsigned char *>(scratch);
         CkptParams P{};
         P.desc = reinterpret_cast<const CkptDesc *>(regions_dev);
         P.n_allocs = n_regions;
@@ -98,8 +151,8 @@ extern "C" crac_status_t crac_pass_noalloc(const crac_region_t *regions_dev, uin
         P.log2_chunk = l;
         P.c_begin = 0;
         P.c_end = n_chunks;
-        P.cpt = cpt;
-        P.n_tiles = (uint32_t)n_tiles;
+        P.cpt = (uint32_t)split_finalize_threads();
+        P.n_tiles = fin_tiles;
         P.fp_old = fp_old_dev;
         P.fp_new = fp_new_dev;
         P.idx_out = idx_dev;
@@ -108,15 +161,52 @@ extern "C" crac_status_t crac_pass_noalloc(const crac_region_t *regions_dev, uin
         P.staging = staging_dev;
         P.staging_cap = staging_dev ? staging_cap : 0;
         P.ctrl = reinterpret_cast<CkptCtrl *>(scratch);
-        P.tile_cnt = reinterpret_cast<uint64_t *>(static_cast<unsigned char *>(scratch) + sizeof(CkptCtrl));
-        P.tile_bytes = P.tile_cnt + n_tiles;
+        P.tile_cnt = reinterpret_cast<uint64_t *>(sc + sizeof(CkptCtrl));
+        P.tile_bytes = P.tile_cnt + fin_tiles;
         P.timeout_ns = 2000000000ull;
-        P.skip_first_ticket = 0;
+        // Without a baseline every chunk is dirty and its payload offset known
+        // beforehand: the hash kernel writes it there as it reads it, unless a
+        // region's size turns out not to be a multiple of 16 bytes (1 GiB in
+        // 64 KiB chunks: 486 us with the fused kernel, which reads every chunk
+        // twice, 340 us this way; with a baseline and 10% dirty 263 and 205 us).
+        const size_t at = (used + 255) / 256 * 256;
+        if (!fp_old_dev && staging_dev && ((uintptr_t)staging_dev & 15u) == 0 &&
+            n_regions <= (kNoAllocScratchBytes - at) / 8 - 1) {
+            uint64_t *prefix = reinterpret_cast<uint64_t *>(sc + at);
+            P.full_copy = 1;
+            P.full_flag = reinterpret_cast<const uint32_t *>(prefix + n_regions);
+            P.alloc_prefix = prefix;
+            noalloc_prefix_kernel<<<1, kPrefixNT, 0, s>>>(P.desc, n_regions, P.staging_cap, prefix,
+                                                          reinterpret_cast<uint32_t *>(prefix + n_regions));
+            e = cudaGetLastError();
+            count_launches(1);
+        }
+        const bool small = l >= 9 && l < 13;
+        const uint64_t most = n_chunks << l;   // the regions' bytes are in device memory only
+        uint32_t log2Seg = small ? l : split_hash_seg(most, l, P.full_copy != 0);
+        const uint32_t grid = split_hash_grid(n_chunks, most, l, log2Seg, &P.slots_per_warp);
+        // Segmented chunks are summed up in the caller's table, in place.
+        unsigned long long *acc = log2Seg < l ? reinterpret_cast<unsigned long long *>(fp_new_dev) : nullptr;
+        if (e == cudaSuccess && acc) e = cudaMemsetAsync(fp_new_dev, 0, n_chunks * 8, s);
+        void *args[] = {&P, &acc, &log2Seg};
+        const int sms = g_noalloc_sms[dev];
+        if (e == cudaSuccess)
+            e = cudaLaunchKernel(small ? split_hash_small_fn(1 << (l - 7)) : split_hash_fn(), dim3(grid),
+                                 dim3(split_hash_threads()), args, 0, s);
+        if (e == cudaSuccess)
+            e = cudaLaunchKernel(split_finalize_fn(), dim3(fin_tiles < 2u * sms ? fin_tiles : 2u * sms),
+                                 dim3(split_finalize_threads()), args, 0, s);
+        if (e == cudaSuccess)
+            e = cudaLaunchKernel(split_gather_fn(false, false), dim3(8 * sms), dim3(split_gather_threads()), args, 0, s);
+        if (e == cudaSuccess) count_launches(3);
         const uint64_t g = grid_per[wpc == 8 ? 1 : 0];
-        e = launch_ckpt_fused(P, 256, wpc, (int)(n_tiles < g ? n_tiles : g), s);
+        reserved = (uint32_t)(n_tiles + (n_tiles < g ? n_tiles : g));
     }
-    // totals = {reserved, err, k, payload_bytes}: the control block's layout from byte 0
-    if (e == cudaSuccess) e = cudaMemcpyAsync(totals_dev, scratch, sizeof(crac_pass_totals_t), cudaMemcpyDeviceToDevice, s);
+    if (e == cudaSuccess) {
+        noalloc_totals_kernel<<<1, 32, 0, s>>>(reinterpret_cast<const CkptCtrl *>(scratch), reinterpret_cast<uint8_t *>(totals_dev), reserved);
+        e = cudaGetLastError();
+        if (e == cudaSuccess) count_launches(1);
+    }
     if (e != cudaSuccess) {
         note_cuda_error((int)e);
         return CRAC_ERR_CUDA;

@@ -164,13 +164,6 @@ __global__ void __launch_bounds__(NT, 5) ckpt_fused_kernel(const CkptParams P) {
     }
 }
 
-
-template <int NT, int WPC>
-cudaError_t launch_fused_t(const CkptParams &p, int grid, cudaStream_t s) {
-    ckpt_fused_kernel<NT, WPC><<<grid, NT, 0, s>>>(p);
-    return cudaGetLastError();
-}
-
 }  // namespace
 
 static uint64_t g_launches = 0;   // guarded by the callers' context lock is not enough
@@ -191,16 +184,6 @@ int ckpt_fused_max_ctas_per_sm(int threads, int wpc) {
     int n = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, threads, 0) != cudaSuccess) return 0;
     return n;
-}
-
-cudaError_t launch_ckpt_fused(const CkptParams &p, int threads, int wpc, int grid,
-                              cudaStream_t s) {
-    if (p.cpt == 0 || p.cpt > (uint32_t)kMaxCpt || grid <= 0) return cudaErrorInvalidValue;
-    cudaError_t e = cudaErrorInvalidValue;
-    if (threads == 256 && wpc == 1) e = launch_fused_t<256, 1>(p, grid, s);
-    else if (threads == 256 && wpc == 8) e = launch_fused_t<256, 8>(p, grid, s);
-    if (e == cudaSuccess) count_launches(1);
-    return e;
 }
 
 }  // namespace crac

@@ -45,7 +45,12 @@ __device__ __forceinline__ bool spec_ok(const CkptParams &P, uint64_t po, uint64
     return po != ~0ull && (po & 15u) == 0 && po <= P.staging_cap && len <= P.staging_cap - po;
 }
 
-// Partial CRAC-FP64 sum of a segment (<= 8 KiB) whose first word is word j0
+// Whether the hash kernel writes every chunk at its uncompacted offset.
+__device__ __forceinline__ bool copies_all(const CkptParams &P) {
+    return P.full_copy && (P.full_flag == nullptr || *P.full_flag);
+}
+
+// Partial CRAC-FP64 sum of a segment (<= 16 KiB) whose first word is word j0
 // of its chunk, over the lanes of one warp.  dest(), asked for once the first
 // loads are on their way, says where the segment's bytes are also stored (null:
 // nowhere); then (kHdr) the CRZ1 header word of each whole 512-byte block of
@@ -175,10 +180,10 @@ split_hash_kernel(const CkptParams P, unsigned long long *__restrict__ acc, uint
         // Direct mode (S <= 8 KiB, the warp sees the whole chunk): the baseline
         // fingerprint is loaded before the chunk so that both latencies overlap.
         uint64_t fo = 0;
-        const bool has = d.base_first != kNoBase;
+        const bool has = d.base_first != kNoBase && P.fp_old;
         if (spc == 0 && lane == 0 && has) fo = __ldg(P.fp_old + d.base_first + local);
         auto dest = [&]() -> uint4 * {
-            if (P.full_copy) {   // FULL checkpoint: the segment's final staging offset is known
+            if (copies_all(P)) {   // FULL checkpoint: the segment's final staging offset is known
                 const uint64_t o = P.alloc_prefix[a] + (local << log2S) + off - P.seg_base;
                 if (o + len <= P.staging_cap) return reinterpret_cast<uint4 *>(P.staging + o);
                 if (lane == 0) atomicOr(&P.ctrl->err, kErrBounds);
@@ -201,7 +206,7 @@ split_hash_kernel(const CkptParams P, unsigned long long *__restrict__ acc, uint
                 // the length and the dirty bit for the compaction kernel.
                 const uint64_t fp = fp_finalize(sum, len);
                 P.fp_new[c] = fp;
-                acc[c - P.c_begin] = len | ((!has || fo != fp) ? kAccDirty : 0ull);
+                if (acc) acc[c - P.c_begin] = len | ((!has || fo != fp) ? kAccDirty : 0ull);
             } else {
                 atomicAdd(acc + (c - P.c_begin), (unsigned long long)sum);
             }
@@ -245,7 +250,7 @@ __device__ __forceinline__ void hash_small_iter(const CkptParams &P, unsigned lo
         local = c - d.first_chunk;
         const uint64_t rest = d.bytes - (local << log2S);
         len = (uint32_t)umin64(rest, 1ull << log2S);
-        has = d.base_first != kNoBase;
+        has = d.base_first != kNoBase && P.fp_old;
         hold = P.sparse && has;
         if (li == 0 && has) fo = __ldg(P.fp_old + d.base_first + local);
         const uint4 *p = reinterpret_cast<const uint4 *>(reinterpret_cast<const uint8_t *>(d.ptr) + (local << log2S));
@@ -266,7 +271,7 @@ __device__ __forceinline__ void hash_small_iter(const CkptParams &P, unsigned lo
             }
             key += kStep;
         }
-        if (P.full_copy && !hold) {   // FULL checkpoint: the chunk goes straight to its staging offset
+        if (!hold && copies_all(P)) {   // FULL checkpoint: the chunk goes straight to its staging offset
             const uint64_t o = P.alloc_prefix[a] + (local << log2S) - P.seg_base;
             if (o + len <= P.staging_cap) {
                 uint4 *dst = reinterpret_cast<uint4 *>(P.staging + o);
@@ -318,7 +323,7 @@ __device__ __forceinline__ void hash_small_iter(const CkptParams &P, unsigned lo
     const bool dirty = !has || fo != fp;
     if (li == 0 && c < P.c_end) {
         P.fp_new[c] = fp;
-        acc[c - P.c_begin] = len | (dirty ? kAccDirty : 0ull);
+        if (acc) acc[c - P.c_begin] = len | (dirty ? kAccDirty : 0ull);
     }
     if (hold && dirty) {   // sparse delta pass: sizes are multiples of 16 (no tail bytes)
         const uint64_t o = P.alloc_prefix[a] + (local << log2S) - P.seg_base;
@@ -468,8 +473,11 @@ constexpr uint32_t kFinCachedAllocs = 4096;   // first_chunk columns the finaliz
 
 __global__ void __launch_bounds__(kFinNT)
 split_finalize_kernel(const CkptParams P, unsigned long long *__restrict__ acc, uint32_t log2Seg) {
-    const bool direct = log2Seg == P.log2_chunk;
-    // Segmented chunks need their allocation: searched in an on-chip copy of
+    // Whole: the hash kernel saw whole chunks and has finalized them; direct: it
+    // also left each one's length and dirty bit in acc (the allocation-free
+    // pass has no room for that).
+    const bool whole = log2Seg == P.log2_chunk, direct = whole && acc;
+    // Other chunks need their allocation: searched in an on-chip copy of
     // the first_chunk column when it fits (a search in global memory is a
     // chain of dependent loads per chunk).
     __shared__ uint64_t s_first[kFinCachedAllocs];
@@ -518,9 +526,14 @@ split_finalize_kernel(const CkptParams P, unsigned long long *__restrict__ acc, 
             const CkptDesc d = P.desc[a];
             const uint64_t local = c - d.first_chunk;
             len = (uint32_t)min(S, d.bytes - (local << log2S));
-            const uint64_t fp = fp_finalize(acc[c - P.c_begin], len);
-            P.fp_new[c] = fp;
-            const bool dirty = d.base_first == kNoBase || P.fp_old[d.base_first + local] != fp;
+            uint64_t fp;
+            if (whole) {
+                fp = P.fp_new[c];
+            } else {
+                fp = fp_finalize(acc[c - P.c_begin], len);
+                P.fp_new[c] = fp;
+            }
+            const bool dirty = d.base_first == kNoBase || !P.fp_old || P.fp_old[d.base_first + local] != fp;
             dl = dirty ? len : 0u;
         }
         if (P.ppos_next && c < P.c_end) P.ppos_next[c - P.c_begin] = ~0ull;   // the gather sets the dirty ones
@@ -607,8 +620,8 @@ split_finalize_kernel(const CkptParams P, unsigned long long *__restrict__ acc, 
 template <bool kHdr, bool kAligned>
 __global__ void __launch_bounds__(kGatherNT, kHdr ? 2 : 4)
 split_gather_kernel(const CkptParams P, unsigned long long *, uint32_t) {
-    if (P.full_copy) return;   // the hash kernel has already written every chunk
-    wait_for_producer();       // the finalize kernel's list and counts
+    if (copies_all(P)) return;   // the hash kernel has already written every chunk
+    wait_for_producer();         // the finalize kernel's list and counts
     const int lane = threadIdx.x & 31;
     const uint64_t kd = (uint64_t)P.ctrl->k;
     const uint64_t k = kd < P.idx_cap ? kd : P.idx_cap;
