@@ -116,7 +116,6 @@ crac_status_t crac_ctx_free(crac_ctx_t *ctx, void *ptr) {
     const uint64_t p = (uint64_t)(uintptr_t)ptr;
     for (size_t i = 0; i < ctx->allocs.size(); ++i) {
         if (ctx->allocs[i].ptr == p) {
-            ctx->base_first.erase(ctx->allocs[i].id);
             ctx->allocs.erase(ctx->allocs.begin() + i);
             ctx->layout_version++;
             return CRAC_OK;
@@ -152,7 +151,7 @@ crac_status_t crac_ctx_invalidate(crac_ctx_t *ctx) {
     std::lock_guard<std::mutex> lk(ctx->mu);
     settle_all(ctx);
     ctx->base_valid = false;
-    ctx->base_first.clear();
+    ctx->base_first.reset();
     return CRAC_OK;
 }
 

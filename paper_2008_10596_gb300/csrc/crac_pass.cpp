@@ -136,6 +136,12 @@ void pick_split(const crac_ctx *c, int *wpc, uint32_t *cpt) {
     *cpt = t;
 }
 
+BaseLayout layout_of(const std::vector<AllocRec> &allocs, const std::vector<uint64_t> &first) {
+    auto t = std::make_shared<std::vector<std::pair<uint64_t, uint64_t>>>(allocs.size());
+    for (size_t a = 0; a < allocs.size(); ++a) (*t)[a] = {allocs[a].id, first[a]};
+    return t;
+}
+
 struct Segment {
     uint64_t c0, c1, bytes;
 };
@@ -859,8 +865,7 @@ void settle_front(crac_ctx *c) {
     if (st == CRAC_OK) {
         sd.fp = im->out_fp;
         sd.valid = true;
-        sd.first.clear();
-        for (const ImgAlloc &a : im->allocs) sd.first[a.id] = a.first_chunk;
+        sd.first = im->layout;
         img_ref(im);
         img_unref(sd.parent);
         sd.parent = im;
@@ -1165,13 +1170,17 @@ crac_status_t ctx_checkpoint(crac_ctx *c, cudaStream_t s, crac_image_t **out) {
     TRY(ctx_settle(c, false));
     while (c->pending.size() >= 2) settle_front(c);
     // Which chunks have a baseline (no settling after this point may move it).
-    auto base_of = [&](size_t a) {
-        if (!c->base_valid) return kNoBase;
-        auto it = c->base_first.find(c->allocs[a].id);
-        return it == c->base_first.end() ? kNoBase : it->second;
-    };
+    std::vector<uint64_t> base(na);
     bool any_base = false;
-    for (size_t a = 0; a < na; ++a) any_base |= base_of(a) != kNoBase;
+    auto find_bases = [&] {
+        BaseLookup of(c->base_valid ? c->base_first : nullptr);
+        any_base = false;
+        for (size_t a = 0; a < na; ++a) {
+            base[a] = of(c->allocs[a].id);
+            any_base |= base[a] != kNoBase;
+        }
+    };
+    find_bases();
     // A host image's payload block is taken before the pass: the whole
     // segment for a FULL pass (its size is known), else the worst case from
     // the pinned regions as they are (growing them mid-loop would stall the
@@ -1187,8 +1196,7 @@ crac_status_t ctx_checkpoint(crac_ctx *c, cudaStream_t s, crac_image_t **out) {
     if (!defer) {
         pa.free(dpc.host);
         TRY(ctx_settle(c, true));
-        any_base = false;
-        for (size_t a = 0; a < na; ++a) any_base |= base_of(a) != kNoBase;
+        find_bases();
     }
     c->last = crac_pass_info_t{};
     c->last.tracked_bytes = tracked;
@@ -1258,7 +1266,7 @@ crac_status_t ctx_checkpoint(crac_ctx *c, cudaStream_t s, crac_image_t **out) {
         uint64_t pre = 0;
         for (size_t a = 0; a < na; ++a) {
             all16 &= (c->allocs[a].bytes & 15) == 0;
-            dh[a] = CkptDesc{c->allocs[a].ptr, c->allocs[a].bytes, first[a], base_of(a)};
+            dh[a] = CkptDesc{c->allocs[a].ptr, c->allocs[a].bytes, first[a], base[a]};
             prefix_h[a] = pre;
             pre += c->allocs[a].bytes;
         }
@@ -1385,8 +1393,8 @@ crac_status_t ctx_checkpoint(crac_ctx *c, cudaStream_t s, crac_image_t **out) {
         im->had_base = any_base;
     }
     c->fp_cur = out_fp;
-    c->base_first.clear();
-    for (size_t a = 0; a < na; ++a) c->base_first[c->allocs[a].id] = first[a];
+    c->base_first = layout_of(c->allocs, first);
+    if (im->deferred) im->layout = c->base_first;
     c->base_valid = true;
     c->epoch_max = im->epoch;
     c->parent_epoch = im->epoch;
@@ -1441,12 +1449,9 @@ crac_status_t ctx_trial_pass(crac_ctx *c, cudaStream_t s, bool commit, float *ms
     uint64_t *prefix_h = (uint64_t *)(dh + na);
     bool any_base = false, all16 = true;
     uint64_t pre = 0;
+    BaseLookup base_of(c->base_valid ? c->base_first : nullptr);
     for (size_t a = 0; a < na; ++a) {
-        uint64_t bf = kNoBase;
-        if (c->base_valid) {
-            auto it = c->base_first.find(c->allocs[a].id);
-            if (it != c->base_first.end()) bf = it->second;
-        }
+        const uint64_t bf = base_of(c->allocs[a].id);
         any_base |= bf != kNoBase;
         all16 &= (c->allocs[a].bytes & 15) == 0;
         dh[a] = CkptDesc{c->allocs[a].ptr, c->allocs[a].bytes, first[a], bf};
@@ -1487,8 +1492,7 @@ crac_status_t ctx_trial_pass(crac_ctx *c, cudaStream_t s, bool commit, float *ms
         c->prev_base_valid = c->base_valid;
         c->prev_fp = c->fp_cur;
         c->fp_cur = out_fp;
-        c->base_first.clear();
-        for (size_t a = 0; a < na; ++a) c->base_first[c->allocs[a].id] = first[a];
+        c->base_first = layout_of(c->allocs, first);
         c->base_valid = true;
     }
     return CRAC_OK;

@@ -8,12 +8,13 @@ namespace crac {
 // After a successful restore: the registry takes the image's identities and
 // its fingerprints (already in fp[fp_cur]) become the baseline.
 void restart_commit(crac_ctx *c, crac_image *img) {
-    c->base_first.clear();
+    auto t = std::make_shared<std::vector<std::pair<uint64_t, uint64_t>>>(img->allocs.size());
     for (size_t a = 0; a < img->allocs.size(); ++a) {
         c->allocs[a].id = img->allocs[a].id;
         c->next_id = std::max(c->next_id, img->allocs[a].id + 1);
-        c->base_first[img->allocs[a].id] = img->allocs[a].first_chunk;
+        (*t)[a] = {img->allocs[a].id, img->allocs[a].first_chunk};
     }
+    c->base_first = std::move(t);
     c->base_valid = true;
     c->lineage = img->lineage;
     c->epoch_max = std::max(c->epoch_max, img->epoch);
@@ -24,15 +25,37 @@ void restart_commit(crac_ctx *c, crac_image *img) {
 }
 
 // Image allocation -> target allocation (-1: not restored), by allocation id.
-std::vector<int64_t> map_allocs(const crac_image *im, const crac_image *tgt,
-                                const std::unordered_map<uint64_t, size_t> &tpos) {
-    std::vector<int64_t> m(im->allocs.size());
-    for (size_t a = 0; a < im->allocs.size(); ++a) {
-        auto it = tpos.find(im->allocs[a].id);
-        m[a] = (it == tpos.end() || tgt->allocs[it->second].bytes != im->allocs[a].bytes) ? -1 : (int64_t)it->second;
+// Ids ascend in registry order, so an image's allocations are usually the
+// target's, position by position; the others are looked up in an index made
+// on the first miss.
+class AllocMap {
+  public:
+    explicit AllocMap(const crac_image *tgt) : tgt_(tgt) {
+        for (size_t a = 1; a < tgt->allocs.size() && ascending_; ++a)
+            ascending_ = tgt->allocs[a - 1].id < tgt->allocs[a].id;
     }
-    return m;
-}
+    std::vector<int64_t> of(const crac_image *im) {
+        const std::vector<ImgAlloc> &t = tgt_->allocs;
+        std::vector<int64_t> m(im->allocs.size());
+        for (size_t a = 0; a < im->allocs.size(); ++a) {
+            const ImgAlloc &r = im->allocs[a];
+            int64_t p = ascending_ && a < t.size() && t[a].id == r.id ? (int64_t)a : find(r.id);
+            m[a] = p >= 0 && t[p].bytes == r.bytes ? p : -1;
+        }
+        return m;
+    }
+
+  private:
+    int64_t find(uint64_t id) {
+        if (index_.empty())
+            for (size_t a = 0; a < tgt_->allocs.size(); ++a) index_[tgt_->allocs[a].id] = a;
+        const auto it = index_.find(id);
+        return it == index_.end() ? -1 : (int64_t)it->second;
+    }
+    const crac_image *tgt_;
+    bool ascending_ = true;
+    std::unordered_map<uint64_t, size_t> index_;
+};
 
 // Offset of every entry's bytes inside its piece's payload, for a host image
 // (its payload is compact: the prefix of the entries' chunk lengths, or of a
@@ -95,8 +118,7 @@ crac_status_t restart_device(crac_ctx *c, crac_image *img, const std::vector<cra
         TRY(img_offsets(im));
     }
     const uint64_t nt = img->n_chunks;
-    std::unordered_map<uint64_t, size_t> tpos;
-    for (size_t a = 0; a < img->allocs.size(); ++a) tpos[img->allocs[a].id] = a;
+    AllocMap allocs(img);
     if (fault_hit(CRAC_FAULT_H2D)) {
         t_last_cuda = (int)cudaErrorLaunchFailure;
         return CRAC_ERR_CUDA;
@@ -118,7 +140,7 @@ crac_status_t restart_device(crac_ctx *c, crac_image *img, const std::vector<cra
     uint64_t entries = 0;
     for (size_t i = 0; i < chain.size(); ++i) {
         const crac_image *im = chain[i];
-        const std::vector<int64_t> m = map_allocs(im, img, tpos);
+        const std::vector<int64_t> m = allocs.of(im);
         const size_t d0 = dpos;
         for (size_t a = 0; a < im->allocs.size(); ++a, ++dpos)
             sdh[dpos] = ScatterDesc{im->allocs[a].first_chunk, im->allocs[a].bytes,
@@ -267,8 +289,7 @@ crac_status_t ctx_restart(crac_ctx *c, crac_image *img, cudaStream_t s) {
     const uint32_t log2S = c->log2S;
     const size_t na = img->allocs.size();
     const uint64_t nt = img->n_chunks;
-    std::unordered_map<uint64_t, size_t> tpos;
-    for (size_t a = 0; a < na; ++a) tpos[img->allocs[a].id] = a;
+    AllocMap allocs(img);
 
     // Owner map: for every target chunk, the newest chain image holding it.
     TRY(ensure_host(c->owner_h, std::max<uint64_t>(nt, 1) * 2));
@@ -279,12 +300,7 @@ crac_status_t ctx_restart(crac_ctx *c, crac_image *img, cudaStream_t s) {
     std::vector<std::vector<int64_t>> img_map(chain.size());   // image alloc -> target alloc or -1
     for (size_t i = 0; i < chain.size(); ++i) {
         crac_image *im = chain[i];
-        std::vector<int64_t> &m = img_map[i];
-        m.resize(im->allocs.size());
-        for (size_t a = 0; a < im->allocs.size(); ++a) {
-            auto it = tpos.find(im->allocs[a].id);
-            m[a] = (it == tpos.end() || img->allocs[it->second].bytes != im->allocs[a].bytes) ? -1 : (int64_t)it->second;
-        }
+        const std::vector<int64_t> &m = img_map[i] = allocs.of(im);
         if (im->flags & CRAC_IMAGE_FULL) {
             for (size_t a = 0; a < im->allocs.size(); ++a) {
                 if (m[a] < 0) continue;

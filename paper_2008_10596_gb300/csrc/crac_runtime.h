@@ -321,6 +321,35 @@ struct AllocRec {
     uint32_t kind;
 };
 
+// A baseline's chunk layout: allocation id and its first chunk, in registry
+// order.  Shared between the context, its unsettled images and the settled
+// state, and never changed once made (a registry of a thousand allocations
+// would otherwise be copied several times per checkpoint).
+using BaseLayout = std::shared_ptr<const std::vector<std::pair<uint64_t, uint64_t>>>;
+
+// First chunks in a layout, asked for in registry order: the registry usually
+// still holds the layout's allocations in the same order, so each one is found
+// at the cursor; others (after frees) through an index made on the first miss.
+class BaseLookup {
+  public:
+    explicit BaseLookup(BaseLayout t) : t_(std::move(t)) {}
+    uint64_t operator()(uint64_t id) {
+        if (!t_) return kNoBase;
+        if (at_ < t_->size() && (*t_)[at_].first == id) return (*t_)[at_++].second;
+        if (index_.empty())
+            for (size_t i = 0; i < t_->size(); ++i) index_[(*t_)[i].first] = i;
+        const auto it = index_.find(id);
+        if (it == index_.end()) return kNoBase;
+        at_ = it->second + 1;
+        return (*t_)[it->second].second;
+    }
+
+  private:
+    BaseLayout t_;
+    size_t at_ = 0;
+    std::unordered_map<uint64_t, size_t> index_;
+};
+
 }  // namespace crac
 
 using crac::AllocRec;
@@ -363,6 +392,7 @@ struct crac_image {
     Block ctrl_b;                   // pinned landing of the pass's control block
     crac_image *dep = nullptr;
     int out_fp = -1;                // fingerprint table of the context the pass wrote
+    crac::BaseLayout layout;        // ... and its chunk layout
     bool had_base = false;          // some chunk had a baseline (the pass measured a dirty fraction)
     bool lost = false;              // its kernel reported kErrLostCopy
     uint64_t seq = 0;               // the context's pass counter at this pass
@@ -415,8 +445,8 @@ struct crac_ctx {
     int fp_cur = 0;
     int prev_fp = 1;             // autotuner shadows: the table before the last committed trial pass
     bool base_valid = false;
-    std::unordered_map<uint64_t, uint64_t> base_first;   // alloc id -> first chunk in fp[fp_cur]
-    std::unordered_map<uint64_t, uint64_t> prev_base_first;   // autotuner shadows: the baseline before the last
+    crac::BaseLayout base_first;        // first chunk of each allocation in fp[fp_cur] (null: no baseline)
+    crac::BaseLayout prev_base_first;   // autotuner shadows: the baseline before the last
     bool prev_base_valid = false;                             // committed trial pass (still in fp[1 - fp_cur])
     // pass scratch
     DevBuf desc, work, idx, off, staging, lens, carry;
@@ -481,7 +511,7 @@ struct crac_ctx {
     struct Settled {
         int fp = 0;
         bool valid = false;
-        std::unordered_map<uint64_t, uint64_t> first;
+        crac::BaseLayout first;
         crac_image *parent = nullptr;   // strong reference
         uint64_t parent_epoch = kNoParent, epoch_max = 0;
     } settled;

@@ -240,7 +240,7 @@ crac_status_t ctx_tune_apply(crac_ctx *c, cudaStream_t s, double link_gbs, crac_
         c->log2S = t->log2S;
         c->layout_version++;
         c->base_valid = false;
-        c->base_first.clear();
+        c->base_first.reset();
     }
     c->cfg.pass_kernel = win_vt.best_v;
     tune_clear(c);
