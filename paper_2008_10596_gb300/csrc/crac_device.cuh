@@ -68,6 +68,14 @@ constexpr uint64_t kAccDirty = 1ull << 63;
 
 __host__ __device__ __forceinline__ uint64_t umin64(uint64_t a, uint64_t b) { return a < b ? a : b; }
 
+// Kernels that hang off their producer by a programmatic dependency are
+// launched while it drains: each waits here until the producing grid has
+// completed and its writes are visible before touching what it (or a grid
+// before it) wrote.  In an ordinary stream launch this returns at once.
+__device__ __forceinline__ void wait_for_producer() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 __device__ __forceinline__ uint64_t mixw(uint64_t w, uint64_t key) {
     const uint64_t y = (w ^ key) * kM1;
     return y ^ (y >> 32);

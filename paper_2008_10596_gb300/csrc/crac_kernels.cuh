@@ -193,9 +193,20 @@ cudaError_t prepare_drain();
 // null) zero-extended, to dst (pinned host memory, through its device
 // mapping), by a one-warp kernel on s rather than by a copy engine.
 cudaError_t launch_report(const void *words, uint32_t n, const uint32_t *word32, void *dst, cudaStream_t s);
-const void *report_fn();   // the kernel, for graph nodes: args (words, n, word32, dst)
+// the kernel, for graph nodes: args (words, n, word32, dst, table_dst, table_src, table_words)
+const void *report_fn();
+// zero16 16-byte words at `zero` set to zero and copy16 of them copied from src
+// (pinned host memory) to dst, in one launch; the kernel and grid for graph nodes.
+cudaError_t launch_prologue(void *zero, uint64_t zero16, void *dst, const void *src, uint64_t copy16, int sm_count,
+                            cudaStream_t s);
+const void *prologue_fn();
+int prologue_threads();
+uint32_t prologue_grid(uint64_t zero16, uint64_t copy16, int sm_count);
+// Launch on s with a programmatic dependency on the launch before it.
+cudaError_t launch_chained(const void *fn, uint32_t grid, uint32_t threads, void **args, cudaStream_t s);
 cudaError_t launch_drain(const CkptCtrl *ctrl, const uint8_t *src, uint8_t *dst, uint64_t cap,
-                         const uint64_t *idx_src, uint64_t *idx_dst, uint64_t idx_cap, int grid, cudaStream_t s);
+                         const uint64_t *idx_src, uint64_t *idx_dst, uint64_t idx_cap, const uint64_t *fp_src,
+                         uint64_t *fp_dst, uint64_t fp_words, int grid, cudaStream_t s);
 // One piece of a device-resident image in a multi-image restore: its chunk
 // list, offsets and payload, where its entries start in the combined entry
 // space, its image's position in the chain and its descriptor range.
@@ -208,6 +219,7 @@ struct RestorePiece {
     uint32_t desc_off, n_desc, pad;
     uint64_t zlen;                // coded image: device address of each entry's
                                   // stream length (0: entries are raw chunks)
+    uint64_t pad1;                // copied in 16-byte words
 };
 struct RestoreParams {
     const RestorePiece *pieces;
@@ -223,6 +235,7 @@ struct RestoreParams {
     unsigned int *err;
     // Incremental restore: current and target fingerprints per target chunk.
     const uint64_t *fp_now, *fp_img;
+    uint64_t *fp_out;             // the check also copies the target's fingerprints here
     uint32_t coded;               // some piece has a zlen table (coded image)
     uint32_t ragged;              // some allocation's size is not a multiple of 16 bytes
 };

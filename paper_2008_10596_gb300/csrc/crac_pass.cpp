@@ -180,26 +180,33 @@ std::vector<Segment> make_segments(const std::vector<AllocRec> &allocs, const st
     return out;
 }
 
-// Kernel-node parameters of the control block's report to the host (args
-// must outlive the node's add or update call).
+// Kernel-node parameters of the control block's report to the host, with a
+// device table copied beside it (args must outlive the node's add or update
+// call).
 struct ReportNode {
     const void *words;
     uint32_t n = sizeof(CkptCtrl) / 8;
     const uint32_t *word32 = nullptr;
     void *dst;
-    void *args[4];
+    void *table_dst;
+    const void *table_src;
+    uint64_t table_words;
+    void *args[7];
     cudaKernelNodeParams kp{};
-    ReportNode(const void *src, void *to) : words(src), dst(to) {
-        args[0] = &words;
-        args[1] = &n;
-        args[2] = &word32;
-        args[3] = &dst;
+    ReportNode(const void *src, void *to, void *tdst = nullptr, const void *tsrc = nullptr, uint64_t twords = 0,
+               int sm_count = 1)
+        : words(src), dst(to), table_dst(tdst), table_src(tsrc), table_words(twords),
+          args{&words, &n, &word32, &dst, &table_dst, &table_src, &table_words} {
         kp.func = const_cast<void *>(report_fn());
-        kp.gridDim = dim3(1);
-        kp.blockDim = dim3(32);
+        kp.gridDim = dim3(twords ? (unsigned)std::min<uint64_t>((twords + 255) / 256, 2ull * sm_count) : 1u);
+        kp.blockDim = dim3(twords ? 256 : 32);
         kp.kernelParams = args;
     }
 };
+
+// Bytes of the descriptor table per allocation: its descriptor, and the payload
+// bytes before it.
+constexpr size_t kDescBytes = sizeof(CkptDesc) + 8;
 
 // Build (or update) the graph memset -> fused kernel -> ctrl report and launch it.
 crac_status_t launch_fused_graph(crac_ctx *c, const CkptParams &P, size_t work_bytes, const void *fn,
@@ -270,16 +277,21 @@ crac_status_t launch_split_graph(crac_ctx *c, const CkptParams &P, size_t work_b
         kp[i].blockDim = dim3(thr[i]);
         kp[i].kernelParams = args;
     }
-    cudaMemsetParams mp{};
-    mp.dst = c->work.p;
-    mp.value = 0;
-    mp.elementSize = 4;
-    mp.width = work_bytes / 4;
-    mp.height = 1;
-    ReportNode rep(P.ctrl, ctrl_dst);
+    // The prologue zeroes the work area and brings the descriptors in.
+    void *zero = c->work.p, *desc = c->desc.p;
+    const void *desc_h = c->desc_src;
+    uint64_t zero16 = (work_bytes + 15) / 16, desc16 = c->uva ? (c->allocs.size() * kDescBytes + 15) / 16 : 0;
+    void *pro_args[] = {&zero, &zero16, &desc, &desc_h, &desc16};
+    cudaKernelNodeParams pro{};
+    pro.func = const_cast<void *>(prologue_fn());
+    pro.gridDim = dim3(prologue_grid(zero16, desc16, c->sm_count));
+    pro.blockDim = dim3(prologue_threads());
+    pro.kernelParams = pro_args;
+    ReportNode rep(P.ctrl, ctrl_dst, c->fp_copy_dst, c->fp_copy_dst ? P.fp_new : nullptr,
+                   c->fp_copy_dst ? P.c_end : 0, c->sm_count);
     bool ok = c->sgexec != nullptr && c->s_hash_fn == hash_fn && c->s_gather_fn == fns[2];
     if (ok) {
-        ok = cudaGraphExecMemsetNodeSetParams(c->sgexec, c->s_memset, &mp) == cudaSuccess;
+        ok = cudaGraphExecKernelNodeSetParams(c->sgexec, c->s_pro, &pro) == cudaSuccess;
         for (int i = 0; ok && i < 3; ++i)
             ok = cudaGraphExecKernelNodeSetParams(c->sgexec, c->s_k[i], &kp[i]) == cudaSuccess;
         if (ok) ok = cudaGraphExecKernelNodeSetParams(c->sgexec, c->s_copy, &rep.kp) == cudaSuccess;
@@ -290,31 +302,34 @@ crac_status_t launch_split_graph(crac_ctx *c, const CkptParams &P, size_t work_b
         if (c->sgraph) cudaGraphDestroy(c->sgraph);
         c->sgexec = nullptr;
         c->sgraph = nullptr;
-        // memset -> event 0 -> hash => finalize => gather -> control block report,
-        // where => is a programmatic edge (the consumer is launched as its
-        // producer drains and waits in-kernel for its completion); events 1-3
-        // record each kernel's end on side branches, off the critical path.
+        // prologue => hash => finalize => gather => control block report, where
+        // => is a programmatic edge (the consumer is launched as its producer
+        // drains and waits in-kernel for its completion); events 0-3 record the
+        // ends of the first four on side branches, off the critical path.
         CK(cudaGraphCreate(&c->sgraph, 0));
-        CK(cudaGraphAddMemsetNode(&c->s_memset, c->sgraph, nullptr, 0, &mp));
-        cudaGraphNode_t ev;
-        CK(cudaGraphAddEventRecordNode(&ev, c->sgraph, &c->s_memset, 1, c->sev[0]));
-        CK(cudaGraphAddKernelNode(&c->s_k[0], c->sgraph, &ev, 1, &kp[0]));
         cudaGraphEdgeData pe{};
         pe.from_port = cudaGraphKernelNodePortProgrammatic;
         pe.type = cudaGraphDependencyTypeProgrammatic;
-        for (int i = 1; i < 3; ++i) {
+        CK(cudaGraphAddKernelNode(&c->s_pro, c->sgraph, nullptr, 0, &pro));
+        const cudaGraphNode_t *last = &c->s_pro;
+        cudaGraphNode_t ev;
+        CK(cudaGraphAddEventRecordNode(&ev, c->sgraph, last, 1, c->sev[0]));
+        for (int i = 0; i < 3; ++i) {
             CK(cudaGraphAddKernelNode(&c->s_k[i], c->sgraph, nullptr, 0, &kp[i]));
-            CK(cudaGraphAddDependencies(c->sgraph, &c->s_k[i - 1], &c->s_k[i], &pe, 1));
+            CK(cudaGraphAddDependencies(c->sgraph, last, &c->s_k[i], &pe, 1));
+            last = &c->s_k[i];
+            CK(cudaGraphAddEventRecordNode(&ev, c->sgraph, last, 1, c->sev[i + 1]));
         }
-        for (int i = 0; i < 3; ++i) CK(cudaGraphAddEventRecordNode(&ev, c->sgraph, &c->s_k[i], 1, c->sev[i + 1]));
-        CK(cudaGraphAddKernelNode(&c->s_copy, c->sgraph, &c->s_k[2], 1, &rep.kp));
+        CK(cudaGraphAddKernelNode(&c->s_copy, c->sgraph, nullptr, 0, &rep.kp));
+        CK(cudaGraphAddDependencies(c->sgraph, last, &c->s_copy, &pe, 1));
         CK(cudaGraphInstantiate(&c->sgexec, c->sgraph, 0));
         c->s_hash_fn = hash_fn;
         c->s_gather_fn = fns[2];
     }
+    if (!c->uva) CK(link_copy(c, c->desc.p, c->desc_src, c->allocs.size() * kDescBytes, cudaMemcpyHostToDevice, s));
     CK(cudaEventRecord(c->ev_t0, s));
     CK(cudaGraphLaunch(c->sgexec, s));
-    count_launches(4);
+    count_launches(5);
     return CRAC_OK;
 }
 
@@ -335,13 +350,15 @@ crac_status_t launch_segment(crac_ctx *c, const Segment &sg, const CkptDesc *des
     }
     const bool split = c->cfg.launch_mode == CRAC_LAUNCH_BATCHED &&
                        (c->pass_now == CRAC_PASS_SPLIT || c->pass_now == CRAC_PASS_SPARSE);
+    if (!split)   // the split pass's prologue does this
+        CK(link_copy(c, c->desc.p, c->desc_src, c->allocs.size() * kDescBytes, cudaMemcpyHostToDevice, s));
     if (split) {
         const uint32_t cptF = (uint32_t)split_finalize_threads();
         const uint64_t n_tiles = (nseg + cptF - 1) / cptF;
         if (n_tiles > 0x7fffffffull) return CRAC_ERR_UNSUPPORTED;
         const size_t status_bytes = sizeof(CkptCtrl) + 16 * n_tiles;
         const size_t work_bytes = status_bytes + 8 * nseg;
-        TRY(ensure_dev(c->work, work_bytes));
+        TRY(ensure_dev(c->work, work_bytes + 16));   // zeroed in 16-byte words
         // 512 B..4 KiB chunks: several whole chunks per warp iteration.
         const bool small = c->log2S >= 9 && c->log2S < 13;
         const bool copies = staging && (c->full_copy_ok || c->sparse_ok);   // the hash kernel writes every chunk
@@ -405,7 +422,7 @@ crac_status_t launch_segment(crac_ctx *c, const Segment &sg, const CkptDesc *des
         c->last.grid = (uint32_t)gh;
         c->last.chunks_per_tile = cptF;
         c->last.warps_per_chunk = 0;
-        c->last.kernel_launches += 4;   // hash, finalize, gather, control-block report
+        c->last.kernel_launches += 5;   // prologue, hash, finalize, gather, control-block report
         c->last.pass_kernel = P.sparse ? CRAC_PASS_SPARSE : CRAC_PASS_SPLIT;
     } else if (c->cfg.launch_mode == CRAC_LAUNCH_BATCHED) {
         const uint64_t S = 1ull << c->log2S;
@@ -1089,6 +1106,9 @@ crac_status_t checkpoint_enqueue(crac_ctx *c, crac_image *im, const Segment &sg,
     }
     TRY(pa.alloc(sizeof(CkptCtrl), &im->ctrl_b));
     CK(cudaStreamWaitEvent(s, c->ev_last, 0));
+    // The split pass's report also copies a device image's fingerprint table.
+    if (!host_res && (c->pass_now == CRAC_PASS_SPLIT || c->pass_now == CRAC_PASS_SPARSE))
+        c->fp_copy_dst = im->fp_dev.p;
     TRY(launch_segment(c, sg, (const CkptDesc *)c->desc.p, first, idx_d, off_d, n, stg, sg.bytes, out_fp,
                        im->ctrl_b.p, s));
     if (fault_hit(CRAC_FAULT_DRAIN)) {
@@ -1102,12 +1122,12 @@ crac_status_t checkpoint_enqueue(crac_ctx *c, crac_image *im, const Segment &sg,
         // bytes cross by SM stores into the pinned blocks (this path requires
         // the device mapping of pinned memory)
         CK(launch_drain((const CkptCtrl *)c->work.p, direct ? nullptr : (const uint8_t *)c->staging.p, pc.host.p,
-                        sg.bytes, idx_d, (uint64_t *)im->idx_h.p, n, c->sm_count * 2, c->side));
-        CK(link_copy(c, im->fp_h.p, c->fp[out_fp].p, n * 8, cudaMemcpyDeviceToHost, c->side));
+                        sg.bytes, idx_d, (uint64_t *)im->idx_h.p, n, (const uint64_t *)c->fp[out_fp].p,
+                        (uint64_t *)im->fp_h.p, n, c->sm_count * 2, c->side));
         CK(cudaEventRecord(im->done, c->side));
         CK(cudaEventRecord(c->ev_last, c->side));
     } else {
-        CK(cudaMemcpyAsync(im->fp_dev.p, c->fp[out_fp].p, n * 8, cudaMemcpyDeviceToDevice, s));
+        if (!c->fp_copy_dst) CK(cudaMemcpyAsync(im->fp_dev.p, c->fp[out_fp].p, n * 8, cudaMemcpyDeviceToDevice, s));
         CK(cudaEventRecord(im->done, s));
         CK(cudaEventRecord(c->ev_last, s));
     }
@@ -1256,9 +1276,9 @@ crac_status_t ctx_checkpoint(crac_ctx *c, cudaStream_t s, crac_image_t **out) {
         for (int t = 0; t < 3 && st == CRAC_OK; ++t)
             if (t == out_fp || !c->fp[t].p || (t != c->fp_cur && (c->pending.empty() || t != c->settled.fp)))
                 st = ensure_dev(c->fp[t], n * 8);   // (a table never allocated holds nothing either)
-        if (st == CRAC_OK) st = ensure_dev(c->desc, na * (sizeof(CkptDesc) + 8));
-        if (st == CRAC_OK) st = ensure_host(c->desc_h, na * (sizeof(CkptDesc) + 8));
-        if (st == CRAC_OK) st = ensure_host(c->desc_h2, na * (sizeof(CkptDesc) + 8));
+        if (st == CRAC_OK) st = ensure_dev(c->desc, na * kDescBytes + 16);
+        if (st == CRAC_OK) st = ensure_host(c->desc_h, na * kDescBytes + 16);
+        if (st == CRAC_OK) st = ensure_host(c->desc_h2, na * kDescBytes + 16);
         if (st != CRAC_OK) return fail(st);
         CkptDesc *dh = (CkptDesc *)dbuf.p;
         uint64_t *prefix_h = (uint64_t *)(dh + na);   // payload bytes before each allocation
@@ -1281,8 +1301,8 @@ crac_status_t ctx_checkpoint(crac_ctx *c, cudaStream_t s, crac_image_t **out) {
         c->dense_now = c->sparse_ok && any_base && c->delta_frac_valid && c->delta_frac < 0.25f;
         // Order after the previous operation of this context (drain / restore).
         if (cudaStreamWaitEvent(s, c->ev_last, 0) != cudaSuccess) return fail(cuda_status(cudaGetLastError()));
-        if (link_copy(c, c->desc.p, dh, na * (sizeof(CkptDesc) + 8), cudaMemcpyHostToDevice, s) != cudaSuccess)
-            return fail(cuda_status(cudaGetLastError()));
+        c->desc_src = dh;   // copied by the pass
+        c->fp_copy_dst = nullptr;
         // Managed regions migrate to the device before they are read.
         bool any_managed = false;
         for (const AllocRec &r : c->allocs) any_managed |= r.kind == CRAC_KIND_MANAGED;
@@ -1443,8 +1463,8 @@ crac_status_t ctx_trial_pass(crac_ctx *c, cudaStream_t s, bool commit, float *ms
     if (n == 0) return CRAC_OK;
     const int out_fp = spare_fp(c);
     TRY(ensure_dev(c->fp[out_fp], n * 8));
-    TRY(ensure_dev(c->desc, na * (sizeof(CkptDesc) + 8)));
-    TRY(ensure_host(c->desc_h, na * (sizeof(CkptDesc) + 8)));
+    TRY(ensure_dev(c->desc, na * kDescBytes + 16));
+    TRY(ensure_host(c->desc_h, na * kDescBytes + 16));
     CkptDesc *dh = (CkptDesc *)c->desc_h.p;
     uint64_t *prefix_h = (uint64_t *)(dh + na);
     bool any_base = false, all16 = true;
@@ -1467,7 +1487,8 @@ crac_status_t ctx_trial_pass(crac_ctx *c, cudaStream_t s, bool commit, float *ms
                    all16 && c->cfg.launch_mode == CRAC_LAUNCH_BATCHED;
     c->dense_now = c->sparse_ok && any_base && c->dense_hint;
     CK(cudaStreamWaitEvent(s, c->ev_last, 0));
-    CK(link_copy(c, c->desc.p, dh, na * (sizeof(CkptDesc) + 8), cudaMemcpyHostToDevice, s));
+    c->desc_src = dh;
+    c->fp_copy_dst = nullptr;
     uint64_t cap = c->cfg.staging_bytes ? c->cfg.staging_bytes : std::min(tracked, kDefaultStagingMax);
     cap = std::max(round_up(cap, 256), S);
     const std::vector<Segment> segs = make_segments(c->allocs, first, log2S, cap);
@@ -1523,15 +1544,17 @@ crac_status_t fingerprint_against(crac_ctx *c, const uint64_t *fp_ref, cudaStrea
     const size_t work_bytes = status_bytes + 8 * n;
     TRY(ensure_dev(c->vdesc, std::max<size_t>(na, 1) * sizeof(CkptDesc)));
     TRY(ensure_host(c->vdesc_h, std::max<size_t>(na, 1) * sizeof(CkptDesc)));
-    TRY(ensure_dev(c->vwork, work_bytes));
+    TRY(ensure_dev(c->vwork, work_bytes + 16));
     TRY(ensure_dev(c->vfp, std::max<uint64_t>(n, 1) * 8));
     TRY(ensure_dev(c->vidx, std::max<uint64_t>(n, 1) * 8));
     TRY(ensure_dev(c->voff, (n + 1) * 8));
     CkptDesc *dh = (CkptDesc *)c->vdesc_h.p;
     for (size_t a = 0; a < na; ++a)   // the reference table has the same chunk layout
         dh[a] = CkptDesc{c->allocs[a].ptr, c->allocs[a].bytes, first[a], first[a]};
-    CK(link_copy(c, c->vdesc.p, dh, na * sizeof(CkptDesc), cudaMemcpyHostToDevice, s));
-    CK(cudaMemsetAsync(c->vwork.p, 0, work_bytes, s));
+    static_assert(sizeof(CkptDesc) % 16 == 0, "copied in 16-byte words");
+    if (!c->uva) CK(link_copy(c, c->vdesc.p, dh, na * sizeof(CkptDesc), cudaMemcpyHostToDevice, s));
+    CK(launch_prologue(c->vwork.p, (work_bytes + 15) / 16, c->vdesc.p, dh, c->uva ? na * sizeof(CkptDesc) / 16 : 0,
+                       c->sm_count, s));
     const bool small = log2S >= 9 && log2S < 13;
     uint32_t log2Seg = small ? log2S : split_hash_seg(bytes, log2S, false);
     const void *hash_fn = small ? split_hash_small_fn(1 << (log2S - 7)) : split_hash_fn();
@@ -1556,9 +1579,8 @@ crac_status_t fingerprint_against(crac_ctx *c, const uint64_t *fp_ref, cudaStrea
     const int gh = (int)split_hash_grid(n, bytes, log2S, log2Seg, &P.slots_per_warp);
     const int gf = (int)std::max<uint64_t>(1, std::min<uint64_t>(n_tiles, (uint64_t)c->sm_count * 2));
     void *args[] = {&P, &acc, &log2Seg};
-    CK(cudaLaunchKernel(hash_fn, dim3(gh), dim3(split_hash_threads()), args, 0, s));
-    CK(cudaLaunchKernel(split_finalize_fn(), dim3(gf), dim3(split_finalize_threads()), args, 0, s));
-    count_launches(2);
+    CK(launch_chained(hash_fn, gh, split_hash_threads(), args, s));
+    CK(launch_chained(split_finalize_fn(), gf, split_finalize_threads(), args, s));
     *fp_out = (const uint64_t *)c->vfp.p;
     *ctrl_out = P.ctrl;
     return CRAC_OK;

@@ -30,14 +30,6 @@ constexpr int kHashNT = 256;
 constexpr int kFinNT = 1024;
 constexpr int kGatherNT = 256;
 
-// In the pass graph, finalize and gather hang off their producer by a
-// programmatic edge, so they are launched while it drains: each waits here
-// until the producing grid has completed and its writes are visible before
-// touching what it wrote.  In an ordinary stream launch this returns at once.
-__device__ __forceinline__ void wait_for_producer() {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-}
-
 // A chunk of len bytes predicted at staging offset po is written there by the
 // hash kernels (and then found in place by the gather) when the offset is
 // 16-byte aligned (vector stores) and the chunk fits the staging buffer.
@@ -155,6 +147,7 @@ template <bool kHdr>
 __global__ void __launch_bounds__(kHashNT, 3)
 split_hash_kernel(const CkptParams P, unsigned long long *__restrict__ acc, uint32_t log2Seg) {
     constexpr uint32_t kWarps = kHashNT / 32;
+    wait_for_producer();   // the descriptors and zeroed accumulators
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t log2S = P.log2_chunk;
     const uint32_t spc = log2S - log2Seg;   // log2 of segments per chunk
@@ -344,6 +337,7 @@ template <int LPC>
 __global__ void __launch_bounds__(kHashNT, 3)
 split_hash_small_kernel(const CkptParams P, unsigned long long *__restrict__ acc, uint32_t) {
     constexpr int CPS = 32 / LPC;   // chunks per iteration
+    wait_for_producer();   // the descriptors and zeroed accumulators
     const int lane = threadIdx.x & 31;
     const uint64_t warp_g = ((uint64_t)blockIdx.x * kHashNT + threadIdx.x) >> 5;
     const uint64_t n_slots = (P.c_end - P.c_begin + CPS - 1) / CPS;
@@ -387,6 +381,7 @@ template <int LPC>
 __global__ void __launch_bounds__(kHashNT, 4)
 split_hash_small_dense_kernel(const CkptParams P, unsigned long long *__restrict__ acc, uint32_t) {
     constexpr int CPS = 32 / LPC;   // chunks per iteration
+    wait_for_producer();   // the descriptors and zeroed accumulators
     const int lane = threadIdx.x & 31;
     const int li = lane % LPC;
     const uint32_t log2S = P.log2_chunk;
@@ -482,9 +477,9 @@ split_finalize_kernel(const CkptParams P, unsigned long long *__restrict__ acc, 
     // chain of dependent loads per chunk).
     __shared__ uint64_t s_first[kFinCachedAllocs];
     const bool cached = !direct && P.n_allocs <= kFinCachedAllocs;
-    if (cached)   // the descriptors were copied before the pass
-        for (uint32_t a = threadIdx.x; a < P.n_allocs; a += kFinNT) s_first[a] = P.desc[a].first_chunk;
     wait_for_producer();   // the hash kernel's accumulators
+    if (cached)
+        for (uint32_t a = threadIdx.x; a < P.n_allocs; a += kFinNT) s_first[a] = P.desc[a].first_chunk;
     __shared__ uint32_t s_wcnt[32];
     __shared__ uint64_t s_wbytes[32];
     __shared__ uint64_t s_wdirty[32];

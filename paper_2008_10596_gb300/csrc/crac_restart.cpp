@@ -95,10 +95,9 @@ crac_status_t img_offsets(crac_image *im) {
 crac_status_t reserve_restart(crac_ctx *c, uint64_t nt, size_t descs, size_t pieces) {
     const size_t bytes = round_up(descs * sizeof(ScatterDesc), 256) +
                          round_up(std::max<size_t>(pieces, 1) * sizeof(RestorePiece), 256);
-    TRY(ensure_dev(c->owner, std::max<uint64_t>(nt, 1) * 8));
+    TRY(ensure_dev(c->owner, nt * 8 + 32));   // + the error word
     TRY(ensure_dev(c->sdesc, bytes));
     TRY(ensure_host(c->sdesc_h, bytes));
-    TRY(ensure_dev(c->serr, 256));
     return CRAC_OK;
 }
 
@@ -165,9 +164,13 @@ crac_status_t restart_device(crac_ctx *c, crac_image *img, const std::vector<cra
     for (crac_image *im : chain)   // deserialized images have no event: complete from the start
         if (im->done) CK(cudaStreamWaitEvent(s, im->done, 0));
     CK(cudaStreamWaitEvent(s, c->ev_last, 0));
-    CK(cudaMemsetAsync(c->serr.p, 0, 256, s));
-    if (nt) CK(cudaMemsetAsync(c->owner.p, 0, nt * 8, s));
-    CK(link_copy(c, c->sdesc.p, c->sdesc_h.p, desc_bytes + ppos * sizeof(RestorePiece), cudaMemcpyHostToDevice, s));
+    // The owner map, zeroed, with the error word behind it, and the descriptors.
+    static_assert(sizeof(ScatterDesc) % 16 == 0 && sizeof(RestorePiece) % 16 == 0, "copied in 16-byte words");
+    const uint64_t owner16 = (nt * 8 + 15) / 16, sdesc16 = (desc_bytes + ppos * sizeof(RestorePiece)) / 16;
+    CK(cudaEventRecord(c->ev_r0, s));
+    if (!c->uva)
+        CK(cudaMemcpyAsync(c->sdesc.p, c->sdesc_h.p, sdesc16 * 16, cudaMemcpyHostToDevice, s));
+    CK(launch_prologue(c->owner.p, owner16 + 1, c->sdesc.p, c->sdesc_h.p, c->uva ? sdesc16 : 0, c->sm_count, s));
     crac_restart_info_t ri{};
     ri.chain_length = ri.images_used = (uint32_t)chain.size();
     for (const ImgAlloc &a : img->allocs) ri.restored_bytes += a.bytes;
@@ -183,7 +186,7 @@ crac_status_t restart_device(crac_ctx *c, crac_image *img, const std::vector<cra
     P.n_tgt = (uint32_t)img->allocs.size();
     P.owner = (unsigned long long *)c->owner.p;
     P.n_owner = nt;
-    P.err = (unsigned int *)c->serr.p;
+    P.err = (unsigned int *)((uint8_t *)c->owner.p + owner16 * 16);
     for (const crac_image *im : chain) {
         P.coded |= (im->flags & CRAC_IMAGE_CODED) ? 1u : 0u;
         for (const ImgAlloc &a : im->allocs) P.ragged |= (a.bytes & 15) ? 1u : 0u;
@@ -202,9 +205,9 @@ crac_status_t restart_device(crac_ctx *c, crac_image *img, const std::vector<cra
     const uint64_t *fp_img = img->residency == CRAC_RESIDENCY_DEVICE ? (const uint64_t *)img->fp_dev.p
                                                                       : (const uint64_t *)img->fp_h.p;
     const CkptCtrl *vctrl = nullptr;
-    CK(cudaEventRecord(c->ev_r0, s));
     if (incremental) TRY(fingerprint_against(c, fp_img, s, &P.fp_now, &vctrl));
     P.fp_img = fp_img;
+    P.fp_out = (uint64_t *)c->fp[spare].p;
     CK(launch_restore_mark(P, (int)std::max<uint64_t>(1, std::min<uint64_t>((entries + 255) / 256, grid)), s));
     CK(launch_restore_check(P, (int)std::max<uint64_t>(1, std::min<uint64_t>((nt + 255) / 256, grid)), s));
     if (incremental)
@@ -212,11 +215,7 @@ crac_status_t restart_device(crac_ctx *c, crac_image *img, const std::vector<cra
     CK(launch_restore_scatter(P, any_host || incremental || P.coded ? grid : UINT64_MAX, s));
     CK(cudaEventRecord(c->ev_r1, s));
     if (incremental) CK(launch_report(vctrl, sizeof(CkptCtrl) / 8, nullptr, c->ctrl_h.p, s));
-    if (nt) {
-        const void *fp = img->residency == CRAC_RESIDENCY_DEVICE ? (const void *)img->fp_dev.p : (const void *)img->fp_h.p;
-        CK(link_copy(c, c->fp[spare].p, fp, nt * 8, cudaMemcpyDefault, s));
-    }
-    CK(launch_report(nullptr, 0, (const uint32_t *)c->serr.p, c->serr_h.p, s));
+    CK(launch_report(nullptr, 0, P.err, c->serr_h.p, s));
     CK(cudaEventRecord(c->ev_last, s));
     CK(cudaEventSynchronize(c->ev_last));
     const unsigned err = *(const unsigned *)c->serr_h.p;

@@ -66,6 +66,7 @@ constexpr int kOwnerShift = 40;
 constexpr uint64_t kOwnerEntry = (1ull << kOwnerShift) - 1;
 
 __global__ void __launch_bounds__(256) restore_mark_kernel(const RestoreParams P) {
+    wait_for_producer();
     for (uint64_t e = (uint64_t)blockIdx.x * 256 + threadIdx.x; e < P.n_entries; e += (uint64_t)gridDim.x * 256) {
         const RestorePiece pc = P.pieces[find_piece(P.pieces, P.n_pieces, e)];
         const uint64_t c = reinterpret_cast<const uint64_t *>(pc.idx)[e - pc.entry_base];
@@ -78,14 +79,20 @@ __global__ void __launch_bounds__(256) restore_mark_kernel(const RestoreParams P
     }
 }
 
+// Every target chunk needs an owner; the target's fingerprints go to the
+// context's spare table on the way (adopted only if the restore succeeds).
 __global__ void __launch_bounds__(256) restore_check_kernel(const RestoreParams P) {
-    for (uint64_t i = (uint64_t)blockIdx.x * 256 + threadIdx.x; i < P.n_owner; i += (uint64_t)gridDim.x * 256)
+    wait_for_producer();
+    for (uint64_t i = (uint64_t)blockIdx.x * 256 + threadIdx.x; i < P.n_owner; i += (uint64_t)gridDim.x * 256) {
+        P.fp_out[i] = P.fp_img[i];
         if (P.owner[i] == 0) atomicOr(P.err, kErrUncovered);
+    }
 }
 
 // Incremental restore: a target chunk that already holds the image's bytes
 // (same fingerprint) keeps them; clearing its owner makes the scatter skip it.
 __global__ void __launch_bounds__(256) restore_unmark_kernel(const RestoreParams P) {
+    wait_for_producer();
     for (uint64_t i = (uint64_t)blockIdx.x * 256 + threadIdx.x; i < P.n_owner; i += (uint64_t)gridDim.x * 256)
         if (P.fp_now[i] == P.fp_img[i]) P.owner[i] = 0;
 }
@@ -135,6 +142,7 @@ __device__ __forceinline__ RestoreItem restore_item(const RestoreParams &P, uint
 // kAligned: every allocation's size is a multiple of 16 bytes.
 template <bool kAligned>
 __device__ __forceinline__ void restore_scatter_body(const RestoreParams &P) {
+    wait_for_producer();
     if (*(volatile unsigned int *)P.err) return;   // uncovered or out of range: memory untouched
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint64_t n_items = P.n_owner << (P.log2_chunk - P.log2_part);
@@ -166,6 +174,7 @@ __global__ void __launch_bounds__(kScatterNT, 4) restore_scatter_ragged_kernel(c
 // whole warp: its decoding takes far longer than the look-up.
 __global__ void __launch_bounds__(kScatterNT, 4) restore_scatter_coded_kernel(const RestoreParams P) {
     __shared__ __align__(16) uint8_t scratch[kCrzDecodeScratch * (kScatterNT / 32)];
+    wait_for_producer();
     if (*(volatile unsigned int *)P.err) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint64_t nw = (uint64_t)gridDim.x * (kScatterNT / 32);
@@ -182,28 +191,25 @@ __global__ void __launch_bounds__(kScatterNT, 4) restore_scatter_coded_kernel(co
 
 }  // namespace
 
+// The restore kernels are chained: each is launched while the one before it
+// drains (mark -> check -> scatter by ordinary launches left 2-3 us between them).
+template <class K>
+static cudaError_t chain(K *kernel, const RestoreParams &p, uint64_t grid, uint32_t threads, cudaStream_t s) {
+    RestoreParams q = p;
+    void *args[] = {&q};
+    return launch_chained(reinterpret_cast<const void *>(kernel), (uint32_t)grid, threads, args, s);
+}
+
 cudaError_t launch_restore_mark(const RestoreParams &p, int grid, cudaStream_t s) {
-    if (p.n_entries == 0) return cudaSuccess;
-    restore_mark_kernel<<<grid, 256, 0, s>>>(p);
-    const cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) count_launches(1);
-    return e;
+    return p.n_entries ? chain(restore_mark_kernel, p, grid, 256, s) : cudaSuccess;
 }
 
 cudaError_t launch_restore_check(const RestoreParams &p, int grid, cudaStream_t s) {
-    if (p.n_owner == 0) return cudaSuccess;
-    restore_check_kernel<<<grid, 256, 0, s>>>(p);
-    const cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) count_launches(1);
-    return e;
+    return p.n_owner ? chain(restore_check_kernel, p, grid, 256, s) : cudaSuccess;
 }
 
 cudaError_t launch_restore_unmark(const RestoreParams &p, int grid, cudaStream_t s) {
-    if (p.n_owner == 0) return cudaSuccess;
-    restore_unmark_kernel<<<grid, 256, 0, s>>>(p);
-    const cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) count_launches(1);
-    return e;
+    return p.n_owner ? chain(restore_unmark_kernel, p, grid, 256, s) : cudaSuccess;
 }
 
 cudaError_t launch_restore_scatter(const RestoreParams &p, uint64_t max_grid, cudaStream_t s) {
@@ -216,12 +222,10 @@ cudaError_t launch_restore_scatter(const RestoreParams &p, uint64_t max_grid, cu
     uint64_t warps = p.n_owner << (p.log2_chunk - q.log2_part);
     if (p.log2_chunk < 13) warps = ((warps - 1) >> (13 - (p.log2_chunk < 8 ? 8 : p.log2_chunk))) + 1;
     const uint64_t ctas = umin64((warps + kWarps - 1) / kWarps, umin64(max_grid, 0x7fffffffull));
-    if (p.coded) restore_scatter_coded_kernel<<<(unsigned)ctas, kScatterNT, 0, s>>>(q);
-    else if (p.ragged) restore_scatter_ragged_kernel<<<(unsigned)ctas, kScatterNT, 0, s>>>(q);
-    else restore_scatter_kernel<<<(unsigned)ctas, kScatterNT, 0, s>>>(q);
-    const cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) count_launches(1);
-    return e;
+    return chain(p.coded    ? restore_scatter_coded_kernel
+                 : p.ragged ? restore_scatter_ragged_kernel
+                            : restore_scatter_kernel,
+                 q, ctas, kScatterNT, s);
 }
 
 cudaError_t launch_scatter(const ScatterParams &p, int grid, cudaStream_t s) {

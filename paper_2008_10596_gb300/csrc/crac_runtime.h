@@ -452,6 +452,8 @@ struct crac_ctx {
     DevBuf desc, work, idx, off, staging, lens, carry;
     HostBuf desc_h, desc_h2, ctrl_h;
     int desc_flip = 0;           // which of desc_h / desc_h2 the next pass fills
+    const void *desc_src = nullptr;   // the current pass's descriptors (pinned), copied to desc as it starts
+    void *fp_copy_dst = nullptr;      // ... and where its report also copies the fingerprints (device image)
     DevBuf cstage, zwork, zoff, zlen;   // CRAC_FLAG_COMPRESS: streams, encoder scratch, tables
     // restart scratch
     DevBuf owner, sdesc, sidx, soff, serr;
@@ -470,10 +472,10 @@ struct crac_ctx {
     int g_threads = 0, g_wpc = 0;
     const void *g_fn = nullptr;
     bool tma_ready = false;
-    // graph for the split pass: memset -> hash -> finalize -> gather -> ctrl D2H
+    // graph for the split pass: prologue -> hash -> finalize -> gather -> ctrl report
     cudaGraph_t sgraph = nullptr;
     cudaGraphExec_t sgexec = nullptr;
-    cudaGraphNode_t s_memset = nullptr, s_k[3] = {nullptr, nullptr, nullptr}, s_copy = nullptr;
+    cudaGraphNode_t s_pro = nullptr, s_k[3] = {nullptr, nullptr, nullptr}, s_copy = nullptr;
     cudaEvent_t sev[4] = {nullptr, nullptr, nullptr, nullptr};   // around each split-pass kernel
     const void *s_hash_fn = nullptr, *s_gather_fn = nullptr;   // the instances in it
     crac_pass_info_t last{};
@@ -557,11 +559,6 @@ double now_s();
 // device mapping (or both device memory), by SM loads and stores on s with at
 // most max_grid CTAs, instead of a copy engine (crac_drain.cu).
 cudaError_t launch_link_copy(void *dst, const void *src, uint64_t bytes, int max_grid, cudaStream_t s);
-
-// The sparse pass's dense-placement hash kernel for 512 B - 4 KiB chunks
-// (lanes_per_chunk = chunk bytes / 256), the dynamic shared memory it runs
-// with, the attribute that allows it (before its first launch or graph
-// node), and occupancy with dynamic shared memory (crac_pass_split.cu).
 
 // Entries [0, n) of a sparse device piece packed back to back into device
 // memory dst: entry j's cum[j+1] - cum[j] bytes from span + off[j] to
