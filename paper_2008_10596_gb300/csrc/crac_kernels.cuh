@@ -57,10 +57,9 @@ struct CkptParams {
     CkptCtrl *ctrl;
     uint64_t timeout_ns;
     uint32_t skip_first_ticket;  // fault injection: tile 0 is never processed
-    // Split pass, FULL checkpoints only (no chunk has a baseline, every size a
-    // multiple of 16): the hash kernels write each chunk straight to its final
-    // staging offset alloc_prefix[a] + local*S - seg_base, and the gather is
-    // skipped.
+    // Split pass, FULL checkpoints only (no chunk has a baseline): the hash
+    // kernels write each chunk straight to its final staging offset
+    // alloc_prefix[a] + local*S - seg_base, and the gather is skipped.
     uint32_t full_copy;
     const uint64_t *alloc_prefix;   // payload bytes of all allocations before each one
     const uint32_t *full_flag;      // null, or a device word that can still take full_copy back
@@ -153,12 +152,13 @@ cudaError_t ckpt_tma_prepare();   // raise the dynamic shared memory limit (once
 // run in order H -> F -> G.  acc holds one u64 per chunk of the segment and
 // must be zero before H; F uses cpt = split_finalize_threads() chunks per
 // tile and the look-back status words; G reads k from ctrl.
-const void *split_hash_fn(bool crz_headers = false);
+// aligned: every allocation's size is a multiple of 16 bytes (the other
+// instances store chunks at payload offsets of any alignment).
+const void *split_hash_fn(bool crz_headers, bool aligned);
 // Hash kernel for 512 B <= chunk < 8 KiB: lanes_per_chunk = chunk / 128;
 // it finalizes every chunk itself, so finalize runs with log2Seg = log2_chunk.
-const void *split_hash_small_fn(int lanes_per_chunk);
+const void *split_hash_small_fn(int lanes_per_chunk, bool aligned);
 const void *split_finalize_fn();
-// aligned: every allocation's size is a multiple of 16 bytes.
 const void *split_gather_fn(bool crz_headers, bool aligned);
 int split_hash_threads();
 int split_finalize_threads();

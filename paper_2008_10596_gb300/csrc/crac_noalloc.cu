@@ -27,7 +27,7 @@ constexpr int kPrefixNT = 1024;
 
 // One CTA, before a pass without a baseline: the payload bytes before each
 // region, and the flag that the hash kernel may write every chunk there as it
-// reads it (every size a multiple of 16 bytes, and room for them all).
+// reads it (there is room for them all).
 __global__ void __launch_bounds__(kPrefixNT)
 noalloc_prefix_kernel(const crac::CkptDesc *__restrict__ d, uint32_t n, uint64_t cap, uint64_t *__restrict__ prefix,
                       uint32_t *__restrict__ flag) {
@@ -37,14 +37,10 @@ noalloc_prefix_kernel(const crac::CkptDesc *__restrict__ d, uint32_t n, uint64_t
     const uint32_t per = (n + kPrefixNT - 1) / kPrefixNT;
     const uint32_t i0 = threadIdx.x * per, i1 = min(n, i0 + per);
     uint64_t sum = 0;
-    bool odd = false;
-    for (uint32_t i = i0; i < i1; ++i) {
-        sum += d[i].bytes;
-        odd |= (d[i].bytes & 15u) != 0;
-    }
-    uint64_t incl = warp_incl_scan(sum, lane);
+    for (uint32_t i = i0; i < i1; ++i) sum += d[i].bytes;
+    const uint64_t incl = warp_incl_scan(sum, lane);
     if (lane == 31) s_sum[warp] = incl;
-    odd = __syncthreads_or(odd);
+    __syncthreads();
     uint64_t before = 0, total = 0;
     for (int w = 0; w < kPrefixNT / 32; ++w) {
         if (w < warp) before += s_sum[w];
@@ -55,7 +51,7 @@ noalloc_prefix_kernel(const crac::CkptDesc *__restrict__ d, uint32_t n, uint64_t
         prefix[i] = at;
         at += d[i].bytes;
     }
-    if (threadIdx.x == 0) *flag = !odd && total <= cap ? 1u : 0u;
+    if (threadIdx.x == 0) *flag = total <= cap ? 1u : 0u;
 }
 
 // The pass's results (a crac_pass_totals_t at any address) from its control
@@ -165,13 +161,12 @@ extern "C" crac_status_t crac_pass_noalloc(const crac_region_t *regions_dev, uin
         P.tile_bytes = P.tile_cnt + fin_tiles;
         P.timeout_ns = 2000000000ull;
         // Without a baseline every chunk is dirty and its payload offset known
-        // beforehand: the hash kernel writes it there as it reads it, unless a
-        // region's size turns out not to be a multiple of 16 bytes (1 GiB in
-        // 64 KiB chunks: 486 us with the fused kernel, which reads every chunk
-        // twice, 340 us this way; with a baseline and 10% dirty 263 and 205 us).
+        // beforehand: the hash kernel writes it there as it reads it, if they
+        // all fit (1 GiB in 64 KiB chunks: 486 us with the fused kernel, which
+        // reads every chunk twice, 340 us this way; with a baseline and 10%
+        // dirty 263 and 205 us).
         const size_t at = (used + 255) / 256 * 256;
-        if (!fp_old_dev && staging_dev && ((uintptr_t)staging_dev & 15u) == 0 &&
-            n_regions <= (kNoAllocScratchBytes - at) / 8 - 1) {
+        if (!fp_old_dev && staging_dev && n_regions <= (kNoAllocScratchBytes - at) / 8 - 1) {
             uint64_t *prefix = reinterpret_cast<uint64_t *>(sc + at);
             P.full_copy = 1;
             P.full_flag = reinterpret_cast<const uint32_t *>(prefix + n_regions);
@@ -191,7 +186,7 @@ extern "C" crac_status_t crac_pass_noalloc(const crac_region_t *regions_dev, uin
         void *args[] = {&P, &acc, &log2Seg};
         const int sms = g_noalloc_sms[dev];
         if (e == cudaSuccess)
-            e = cudaLaunchKernel(small ? split_hash_small_fn(1 << (l - 7)) : split_hash_fn(), dim3(grid),
+            e = cudaLaunchKernel(small ? split_hash_small_fn(1 << (l - 7), false) : split_hash_fn(false, false), dim3(grid),
                                  dim3(split_hash_threads()), args, 0, s);
         if (e == cudaSuccess)
             e = cudaLaunchKernel(split_finalize_fn(), dim3(fin_tiles < 2u * sms ? fin_tiles : 2u * sms),

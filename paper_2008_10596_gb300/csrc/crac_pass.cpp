@@ -371,7 +371,8 @@ crac_status_t launch_segment(crac_ctx *c, const Segment &sg, const CkptDesc *des
         // densely.
         const bool dense = small && c->sparse_ok && staging && c->dense_now;
         const void *hash_fn = dense ? split_hash_small_dense_fn(1 << (c->log2S - 7))
-                              : small ? split_hash_small_fn(1 << (c->log2S - 7)) : split_hash_fn(crz_hdr != nullptr);
+                              : small ? split_hash_small_fn(1 << (c->log2S - 7), c->all16)
+                                      : split_hash_fn(crz_hdr != nullptr, c->all16);
         CkptParams P{};
         P.crz_hdr = crz_hdr;
         P.desc = desc_dev;
@@ -1291,7 +1292,7 @@ crac_status_t ctx_checkpoint(crac_ctx *c, cudaStream_t s, crac_image_t **out) {
             pre += c->allocs[a].bytes;
         }
         c->all16 = all16;
-        c->full_copy_ok = !any_base && all16;
+        c->full_copy_ok = !any_base;
         c->pass_now = resolve_pass_kernel(c, dev_res, all16);
         c->sparse_ok = c->pass_now == CRAC_PASS_SPARSE && dev_res && all16 &&
                        c->cfg.launch_mode == CRAC_LAUNCH_BATCHED;
@@ -1479,7 +1480,7 @@ crac_status_t ctx_trial_pass(crac_ctx *c, cudaStream_t s, bool commit, float *ms
         pre += c->allocs[a].bytes;
     }
     c->all16 = all16;
-    c->full_copy_ok = !any_base && all16;
+    c->full_copy_ok = !any_base;
     // Trial passes run the configured kernel; AUTO is the split pass here, so
     // that the tuner's observations of different sizes are comparable.
     c->pass_now = c->cfg.pass_kernel == CRAC_PASS_AUTO ? (uint32_t)CRAC_PASS_SPLIT : c->cfg.pass_kernel;
@@ -1557,7 +1558,7 @@ crac_status_t fingerprint_against(crac_ctx *c, const uint64_t *fp_ref, cudaStrea
                        c->sm_count, s));
     const bool small = log2S >= 9 && log2S < 13;
     uint32_t log2Seg = small ? log2S : split_hash_seg(bytes, log2S, false);
-    const void *hash_fn = small ? split_hash_small_fn(1 << (log2S - 7)) : split_hash_fn();
+    const void *hash_fn = small ? split_hash_small_fn(1 << (log2S - 7), true) : split_hash_fn(false, true);
     CkptParams P{};
     P.desc = (const CkptDesc *)c->vdesc.p;
     P.n_allocs = (uint32_t)na;

@@ -481,7 +481,7 @@ struct crac_ctx {
     crac_pass_info_t last{};
     crac_restart_info_t last_restart{};
     bool all16 = false;          // current pass: every size a multiple of 16 bytes
-    bool full_copy_ok = false;   // current pass: no baseline anywhere and 16-byte sizes
+    bool full_copy_ok = false;   // current pass: no baseline anywhere
     bool sparse_ok = false;      // current pass: CRAC_PASS_SPARSE, device images, 16-byte sizes
     bool dense_now = false;      // ... and, on 512 B - 4 KiB chunks, dense placement of the dirty chunks
     bool dense_hint = false;     // trial passes: dense placement (set by the tuner for a sparse timing)

@@ -40,3 +40,34 @@ def test_ragged_sizes(S, sizes, kern, residency):
             assert np.array_equal(b.read(), w)
     finally:
         h.close()
+
+
+@pytest.mark.parametrize("S", [64, 256, 512, 1 * KIB, 2 * KIB, 4 * KIB, 8 * KIB, 16 * KIB, 64 * KIB])
+@pytest.mark.parametrize("flags", [0, C.CRAC_FLAG_DIRECT_DRAIN, C.CRAC_FLAG_COMPRESS])
+def test_ragged_write_through(S, flags):
+    """The hash kernels write FULL and predicted chunks to payload offsets of any
+    alignment: chunks of every length mod 16, each at every offset mod 16 across
+    the list, in every lane layout of the hash kernels."""
+    rng = np.random.default_rng(S + flags)
+    sizes = [S + 1, 1, 15, 16, 17, S - 1, 3 * S + 7] + [int(x) for x in rng.integers(1, 3 * S, 40)] + [2 * S, 5]
+    h = Harness(S, lineage=1700 + S % 97 + flags, flags=flags)
+    try:
+        for i, n in enumerate(sizes):
+            h.add(n, seed=800 + i)
+        img, lib, ora = h.checkpoint()
+        assert lib == ora
+        muts = pattern_mutations(h.first(), sizes, S, "random10", seed=11)
+        for _ in range(3):   # the same chunks: found in place from the second pass on
+            h.mutate(muts)
+            img, lib, ora = h.checkpoint()
+            assert lib == ora
+        if not flags:
+            assert C.crac_ctx_last_pass(h.ctx)["in_place"] == len(muts)
+        want = h.host()
+        for b in h.bufs:
+            b.zero()
+        h.restart(img)
+        for b, w in zip(h.bufs, want):
+            assert np.array_equal(b.read(), w)
+    finally:
+        h.close()
