@@ -140,6 +140,22 @@ __device__ bool load_window(const CodecParams &P, uint8_t *sdata, uint64_t *bar,
     return true;
 }
 
+// 16 bytes from any address of a window.
+__device__ __forceinline__ uint4 load16_any(const uint8_t *p) {
+    const uintptr_t a = (uintptr_t)p;
+    if ((a & 15u) == 0) return *reinterpret_cast<const uint4 *>(p);
+    if ((a & 3u) == 0) {
+        const uint32_t *q = reinterpret_cast<const uint32_t *>(p);
+        return make_uint4(q[0], q[1], q[2], q[3]);
+    }
+    uint32_t w[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        w[i] = (uint32_t)p[4 * i] | ((uint32_t)p[4 * i + 1] << 8) | ((uint32_t)p[4 * i + 2] << 16) |
+               ((uint32_t)p[4 * i + 3] << 24);
+    return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
 // 16 bytes at p (generic, any alignment) to a 16-byte aligned q.
 __device__ __forceinline__ void copy_bytes_cta(uint8_t *q, const uint8_t *p, uint64_t len, int tid) {
     const uint64_t nv = len >> 4;
@@ -251,9 +267,13 @@ __global__ void __launch_bounds__(kCodecNT, 3) crz_encode_kernel(const CodecPara
                 const uint32_t lo = n_win == 1 ? s_bent[fb] : 0u;
                 const uint32_t b = fb - s_nbp[lo];
                 const uint64_t o = s_off[lo];
-                const uint4 v = load16_any(sb + (o - wa) + 512ull * b + 16u * lane);
-                const uint32_t r[4] = {crz_rot(v.x), crz_rot(v.y), crz_rot(v.z), crz_rot(v.w)};
-                const uint64_t h = crz_block_header(r);
+                uint32_t r[4];
+                crz_load_words(sb + (o - wa) + 512ull * b, lane, r);
+#pragma unroll
+                for (int g = 0; g < 4; ++g) r[g] = crz_rot(r[g]);
+                uint32_t mins, maxs;
+                crz_block_range(r, &mins, &maxs);
+                const uint64_t h = crz_header(mins, maxs);
                 if (lane == 0) {
                     s_hdr[fb - f0] = h;
                     if (n_win > 1) P.hdr[(o >> 9) + b] = h;   // for the second pass over the windows
@@ -348,12 +368,11 @@ __global__ void __launch_bounds__(kCodecNT, 3) crz_encode_kernel(const CodecPara
                 const uint32_t b = fb - s_nbp[lo];
                 // units before this block within its entry
                 const uint32_t before = n_win == 1 ? s_boff[fb] - s_boff[s_nbp[lo]] : carry + s_boff[fb - f0];
-                const uint4 v = load16_any(sb + (o - wa) + 512ull * b + 16u * lane);
-                const uint32_t r[4] = {crz_rot(v.x), crz_rot(v.y), crz_rot(v.z), crz_rot(v.w)};
-                uint32_t pw[4];
-                crz_bytes_transpose(r, pw);
+                uint32_t words[4];
+                crz_load_words(sb + (o - wa) + 512ull * b, lane, words);
                 uint8_t *d = P.dst + base + s_zpre[lo] + crz_head_bytes(L >> 9) + 16ull * before;
-                crz_block_units(s_hdr[fb - f0], pw, d, lane, LT, s_units[warp]);
+                const uint64_t h = s_hdr[fb - f0];
+                crz_block_units<true>((uint32_t)h, crz_ends(h), words, d, lane, LT, s_units[warp]);
             }
             carry += wcount;
             // raw entries, and the tails of coded ones, where they overlap the window
@@ -381,9 +400,10 @@ __global__ void __launch_bounds__(kCodecNT, 3) crz_encode_kernel(const CodecPara
 // With every block's header word already in P.chdr, a stream's length needs
 // only its headers' widths: crz_size_kernel sizes and places every stream
 // first, and crz_encode_sized_kernel then codes without any wait between
-// CTAs, one warp per 64 KiB segment of an entry, straight from staging.
-constexpr uint32_t kSizeTile = kCodecNT;   // entries per tile of the sizing kernel
-constexpr uint32_t kSegBlocks = 128;       // blocks per work item of the sized encoder
+// CTAs, one warp per 16 KiB segment of an entry, straight from staging.
+constexpr uint32_t kSizeTile = 64;         // entries per tile of the sizing kernel: eight a warp (with 256,
+                                           // 2 GiB of 64 KiB entries kept 128 CTAs busy for 36 us)
+constexpr uint32_t kSegBlocks = 32;        // blocks per work item of the sized encoder: 16 KiB
 
 // zlen and zoff of every entry (and zoff[k]) from the header widths: one warp
 // per entry sums them; a tile's padded lengths are scanned and placed by a
@@ -454,24 +474,24 @@ __global__ void __launch_bounds__(kCodecNT) crz_size_kernel(const CodecParams P)
     }
 }
 
-// Bytes [x0, x1) of a raw entry (src, any alignment) to d (16-byte aligned),
-// one warp.
-__device__ __forceinline__ void copy_raw_warp(uint8_t *d, const uint8_t *src, uint64_t x0, uint64_t x1, int lane) {
-    const uint64_t nv = (x1 - x0) >> 4;
-    for (uint64_t v = lane; v < nv; v += 32)
-        *reinterpret_cast<uint4 *>(d + x0 + 16 * v) = load16_any(src + x0 + 16 * v);
-    for (uint64_t i = x0 + 16 * nv + lane; i < x1; i += 32) d[i] = src[i];
-}
-
 // Entries [e_begin, e_end) -> their streams at zoff (made by crz_size_kernel):
-// work item = (entry, 64 KiB segment), one warp each, in entry order.  A
-// coded segment writes its blocks' header words and units (unit offsets: the
-// widths of the entry's earlier blocks, then a warp scan over the segment's),
-// and the segment holding the entry's last block also the header pad, the
-// raw tail and the stream pad; a raw entry is copied segment by segment.
+// work item = (entry, segment of kSegBlocks blocks), one warp each, in entry
+// order.  A coded segment writes its blocks' header words and units (unit
+// offsets: the widths of the entry's earlier blocks, then a warp scan over the
+// segment's, a lane per block), and the segment holding the entry's last block
+// also the header pad, the raw tail and the stream pad; a raw entry is copied
+// segment by segment.  Coding is integer work (about 146 warp instructions per
+// block, 76% of the issue slots used), so the raw blocks arrive in a ring of
+// shared memory by asynchronous copies, kAhead blocks a step, three steps
+// ahead, without registers or waits for loads.  2 GiB of fp32: 1071 -> 620 us
+// (32x32 transposes from 16-byte loads, 213 instructions per block, one block
+// ahead in registers -> 8x8 transposes; blocks ahead in registers took 728).
+constexpr int kAhead = 2;
+
+template <bool kScratch>
 __global__ void __launch_bounds__(kCodecNT, 4) crz_encode_sized_kernel(const CodecParams P) {
-    __shared__ __align__(16) uint8_t s_units[kCodecWarps][512];
-    __shared__ uint32_t s_boff[kCodecWarps][kSegBlocks];
+    __shared__ __align__(16) uint8_t s_units[kScratch ? kCodecWarps : 1][512];
+    __shared__ __align__(16) uint8_t s_ring[kCodecWarps][512 * kAhead * 4];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const CrzLane LT = crz_lane(lane);
     const uint32_t spe = P.segs_per_entry;
@@ -488,69 +508,85 @@ __global__ void __launch_bounds__(kCodecNT, 4) crz_encode_sized_kernel(const Cod
             const uint64_t x0 = (uint64_t)sg * (512ull * kSegBlocks);
             if (x0 >= L) continue;
             const uint64_t x1 = umin64(L, x0 + 512ull * kSegBlocks);
-            copy_raw_warp(d, src, x0, x1, lane);
+            copy_group<32>(d + x0, src + x0, x1 - x0, lane);
             if (x1 == L)
                 for (uint64_t i = L + lane; i < ((L + 15) & ~15ull); i += 32) d[i] = 0;
             continue;
         }
-        const uint64_t nb = L >> 9;   // >= 1: a coded stream is shorter than its entry
-        const uint32_t last = (uint32_t)((nb - 1) / kSegBlocks);
+        const uint32_t nb = (uint32_t)(L >> 9);   // >= 1: a coded stream is shorter than its entry
+        const uint32_t last = (nb - 1) / kSegBlocks;
         if (sg > last) continue;
-        const uint64_t b0 = (uint64_t)sg * kSegBlocks;
-        const uint32_t nseg = (uint32_t)umin64(kSegBlocks, nb - b0);
+        const uint32_t b0 = sg * kSegBlocks;
+        const uint32_t nseg = min(kSegBlocks, nb - b0);
         const uint64_t *h = P.chdr + (P.idx[e] << P.log2_bpc);
         uint64_t *dh = reinterpret_cast<uint64_t *>(d);
+        src += 512ull * b0;
         // units of the entry's blocks before this segment
         uint32_t before = 0;
-        for (uint64_t b = lane; b < b0; b += 32) before += crz_width_sum(h[b]);
+        for (uint32_t b = lane; b < b0; b += 32) before += crz_width_sum(h[b]);
         before = __reduce_add_sync(kFull, before);
-        // lane l: blocks b0 + 4l .. 4l + 3 of the segment -> header words, unit offsets
-        uint32_t wq[4], sum = 0;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const uint32_t j = 4u * lane + q;
-            wq[q] = 0;
-            if (j < nseg) {
-                const uint64_t hw = h[b0 + j];
-                dh[b0 + j] = hw;
-                wq[q] = crz_width_sum(hw);
-            }
-            sum += wq[q];
+        // lane l: block b0 + l's header word, and its units' place in the stream
+        uint64_t hw = 0;
+        if ((uint32_t)lane < nseg) {
+            hw = h[b0 + lane];
+            dh[b0 + lane] = hw;
         }
-        uint32_t inc = sum;
+        const uint32_t ends = crz_ends(hw), mine = ends >> 24;
+        uint32_t inc = mine;
 #pragma unroll
         for (int s = 1; s < 32; s <<= 1) {
             const uint32_t t = __shfl_up_sync(kFull, inc, s);
             if (lane >= s) inc += t;
         }
-        uint32_t run = before + inc - sum;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const uint32_t j = 4u * lane + q;
-            if (j < nseg) s_boff[warp][j] = run;
-            run += wq[q];
-        }
-        const uint64_t head = crz_head_bytes(nb);
+        const uint32_t first = before + inc - mine;
+        uint8_t *units = d + crz_head_bytes(nb);
         if (sg == last && lane == 0 && (nb & 1)) dh[nb] = 0;   // header pad
-        __syncwarp();
-        // blocks, the next one's 16 bytes loaded while this one is coded
-        uint4 v = load16_any(src + 512ull * b0 + 16u * lane);
-        for (uint32_t j = 0; j < nseg; ++j) {
-            const uint64_t b = b0 + j;
-            uint4 nx = v;
-            if (j + 1 < nseg) nx = load16_any(src + 512ull * (b + 1) + 16u * lane);
-            const uint32_t r[4] = {crz_rot(v.x), crz_rot(v.y), crz_rot(v.z), crz_rot(v.w)};
-            uint32_t pw[4];
-            crz_bytes_transpose(r, pw);
-            crz_block_units(__ldg(h + b), pw, d + head + 16ull * s_boff[warp][j], lane, LT, s_units[warp]);
-            v = nx;
+        auto code = [&](uint32_t j, const uint32_t w[4]) {
+            const uint32_t mins = __shfl_sync(kFull, (uint32_t)hw, j);
+            const uint32_t be = __shfl_sync(kFull, ends, j);
+            const uint32_t u = __shfl_sync(kFull, first, j);
+            crz_block_units<kScratch>(mins, be, w, units + 16ull * u, lane, LT, s_units[kScratch ? warp : 0]);
+        };
+        if (((uintptr_t)src & 15u) == 0) {
+            constexpr int kG = kAhead, kN = 4;   // blocks a step, steps in the ring
+            uint8_t *ring = s_ring[warp];
+            auto fetch = [&](uint32_t j) {
+#pragma unroll
+                for (int g = 0; g < kG; ++g)
+                    if (j + g < nseg)
+                        cp_async16(ring + 512 * ((j + g) % (kG * kN)) + 16 * lane, src + 512ull * (j + g) + 16 * lane);
+                cp_async_commit();
+            };
+            __syncwarp();
+#pragma unroll
+            for (int i = 0; i < kG * (kN - 1); i += kG) fetch(i);
+            const uint32_t *rd = reinterpret_cast<const uint32_t *>(ring) + 4 * (lane & 7) + (lane >> 3);
+#pragma unroll 1
+            for (uint32_t j = 0; j < nseg; j += kG) {
+                fetch(j + kG * (kN - 1));
+                cp_async_wait<kN - 1>();
+                __syncwarp();
+#pragma unroll
+                for (int g = 0; g < kG; ++g) {
+                    if (j + g >= nseg) break;   // warp-uniform
+                    const uint32_t *n = rd + 128 * ((j + g) % (kG * kN));
+                    const uint32_t v[4] = {n[0], n[32], n[64], n[96]};
+                    code(j + g, v);
+                }
+                __syncwarp();
+            }
+        } else {   // a payload off the 16-byte grid (allocations of any byte size)
+            for (uint32_t j = 0; j < nseg; ++j) {
+                uint32_t w[4];
+                crz_load_words(src + 512 * j, lane, w);
+                code(j, w);
+            }
         }
         if (sg == last) {   // the raw tail, then the stream pad
             const uint64_t tl = L & 511u;
-            copy_raw_warp(d + z - tl - 512ull * nb, src, 512ull * nb, L, lane);
+            copy_group<32>(d + z - tl, src + 512ull * nseg, tl, lane);
             for (uint64_t i = z + lane; i < ((z + 15) & ~15ull); i += 32) d[i] = 0;
         }
-        __syncwarp();   // s_boff is rewritten by the warp's next item
     }
 }
 
@@ -558,7 +594,9 @@ __global__ void __launch_bounds__(kCodecNT, 4) crz_encode_sized_kernel(const Cod
 
 uint32_t crz_tile_max() { return kCodecTileMax; }
 
-uint32_t crz_sized_segs(uint32_t log2S) { return log2S > 16 ? 1u << (log2S - 16) : 1u; }
+uint64_t crz_size_tiles(uint64_t k) { return (k + kSizeTile - 1) / kSizeTile; }
+
+uint32_t crz_sized_segs(uint32_t log2S) { return log2S > 14 ? 1u << (log2S - 14) : 1u; }
 
 cudaError_t launch_crz_size(const CodecParams &p, int grid, cudaStream_t s) {
     if (p.k == 0) return cudaSuccess;
@@ -568,25 +606,20 @@ cudaError_t launch_crz_size(const CodecParams &p, int grid, cudaStream_t s) {
     return e;
 }
 
-cudaError_t launch_crz_encode_sized(const CodecParams &p, int grid, cudaStream_t s) {
+// A CTA for every eight items, handed out by the hardware (a wave of resident
+// CTAs with equal shares waits for the slowest SM); where the streams go
+// straight to mapped host memory, whose link paces the stores, one wave of
+// three CTAs per SM, and 16-byte stores.
+cudaError_t launch_crz_encode_sized(const CodecParams &p, bool to_host, int sm_count, cudaStream_t s) {
     if (p.e_end <= p.e_begin) return cudaSuccess;
-    crz_encode_sized_kernel<<<grid, kCodecNT, 0, s>>>(p);
+    const uint64_t want = ((p.e_end - p.e_begin) * p.segs_per_entry + kCodecWarps - 1) / kCodecWarps;
+    if (to_host)
+        crz_encode_sized_kernel<true><<<(unsigned)umin64(want, 3ull * sm_count), kCodecNT, 0, s>>>(p);
+    else
+        crz_encode_sized_kernel<false><<<(unsigned)umin64(want, 0x7fffffffull), kCodecNT, 0, s>>>(p);
     const cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) count_launches(1);
     return e;
-}
-
-int crz_sized_max_ctas_per_sm() {
-    static int v = 0;
-    static std::once_flag once;
-    std::call_once(once, [] {
-        int n = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, crz_encode_sized_kernel, kCodecNT, 0) != cudaSuccess)
-            n = 1;
-        cudaGetLastError();
-        v = n > 0 ? n : 1;
-    });
-    return v;
 }
 
 int crz_encode_max_ctas_per_sm() {

@@ -149,10 +149,12 @@ cudaError_t launch_prologue(void *zero, uint64_t zero16, void *dst, const void *
 
 // A kernel launch that may start while the one before it on s drains; the
 // kernel waits for that one itself (wait_for_producer).
-cudaError_t launch_chained(const void *fn, uint32_t grid, uint32_t threads, void **args, cudaStream_t s) {
+cudaError_t launch_chained(const void *fn, uint32_t grid, uint32_t threads, void **args, cudaStream_t s,
+                           uint32_t smem) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute at{};
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;

@@ -203,7 +203,8 @@ const void *prologue_fn();
 int prologue_threads();
 uint32_t prologue_grid(uint64_t zero16, uint64_t copy16, int sm_count);
 // Launch on s with a programmatic dependency on the launch before it.
-cudaError_t launch_chained(const void *fn, uint32_t grid, uint32_t threads, void **args, cudaStream_t s);
+cudaError_t launch_chained(const void *fn, uint32_t grid, uint32_t threads, void **args, cudaStream_t s,
+                           uint32_t smem = 0);
 cudaError_t launch_drain(const CkptCtrl *ctrl, const uint8_t *src, uint8_t *dst, uint64_t cap,
                          const uint64_t *idx_src, uint64_t *idx_dst, uint64_t idx_cap, const uint64_t *fp_src,
                          uint64_t *fp_dst, uint64_t fp_words, int grid, cudaStream_t s);
@@ -237,6 +238,7 @@ struct RestoreParams {
     const uint64_t *fp_now, *fp_img;
     uint64_t *fp_out;             // the check also copies the target's fingerprints here
     uint32_t coded;               // some piece has a zlen table (coded image)
+    uint32_t host;                // some piece is in pinned host memory
     uint32_t ragged;              // some allocation's size is not a multiple of 16 bytes
 };
 // Multi-image restore: mark owners for every entry of every piece (atomicMax,
@@ -283,7 +285,7 @@ struct CodecParams {
     // With chdr, the streams are sized and placed first (crz_size_kernel:
     // zlen, zoff; piece_off[i] = zoff[k * i / pieces], i = 0 .. pieces), then
     // coded by crz_encode_sized_kernel over entries [e_begin, e_end), each
-    // entry as segs_per_entry work items of 64 KiB.
+    // entry as segs_per_entry work items of 16 KiB.
     uint64_t *piece_off;
     uint32_t pieces;
     uint32_t segs_per_entry;
@@ -291,8 +293,8 @@ struct CodecParams {
 };
 cudaError_t launch_crz_encode(const CodecParams &p, int grid, cudaStream_t s);
 cudaError_t launch_crz_size(const CodecParams &p, int grid, cudaStream_t s);
-cudaError_t launch_crz_encode_sized(const CodecParams &p, int grid, cudaStream_t s);
-int crz_sized_max_ctas_per_sm();
+uint64_t crz_size_tiles(uint64_t k);   // look-back words it needs
+cudaError_t launch_crz_encode_sized(const CodecParams &p, bool to_host, int sm_count, cudaStream_t s);
 uint32_t crz_sized_segs(uint32_t log2S);   // work items per entry of the sized encoder
 uint32_t crz_tile_max();
 int crz_encode_max_ctas_per_sm();

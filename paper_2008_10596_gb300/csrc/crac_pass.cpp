@@ -596,9 +596,8 @@ crac_status_t encode_segment_sized(crac_ctx *c, Piece &pc, const CkptCtrl &ctrl,
     *zplaced = false;
     TRY(ensure_dev(c->zwork, crz_work_bytes(k, D, c->log2S)));
     uint8_t *w = (uint8_t *)c->zwork.p;
-    const uint64_t size_tiles = (k + 255) / 256;
+    const uint64_t size_tiles = crz_size_tiles(k);
     const uint32_t spe = crz_sized_segs(c->log2S);
-    const uint64_t warps = (uint64_t)c->sm_count * crz_sized_max_ctas_per_sm() * 8;
     // staged host images: launches of at least 32 MiB of raw payload each (the
     // copy of a piece's streams takes far longer than its encoding)
     uint32_t pieces = 1;
@@ -654,13 +653,12 @@ crac_status_t encode_segment_sized(crac_ctx *c, Piece &pc, const CkptCtrl &ctrl,
         TRY(device_arena(c->device).alloc(std::max<uint64_t>(z_all, 16), &pc.dev));
         P.dst = pc.dev.p;
     }
-    const int grid = (int)std::max<uint64_t>(1, warps / 8);
     CK(cudaEventRecord(c->ev_z1, s));
     for (uint32_t i = 0; i < pieces; ++i) {
         CodecParams Q = P;
         Q.e_begin = k * i / pieces;
         Q.e_end = k * (i + 1) / pieces;
-        CK(launch_crz_encode_sized(Q, grid, s));
+        CK(launch_crz_encode_sized(Q, host_res && P.dst == pc.host.p, c->sm_count, s));
         if (piped) {
             CK(cudaEventRecord(c->ev_piece[i], s));
             if (poff[i + 1] > poff[i]) {

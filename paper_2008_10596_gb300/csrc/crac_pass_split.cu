@@ -66,6 +66,24 @@ __device__ __forceinline__ bool copies_all(const CkptParams &P) {
     return P.full_copy && (P.full_flag == nullptr || *P.full_flag);
 }
 
+// CRZ1 header words of the first n (at most 8) blocks of q (block u: q[u]
+// across the warp) to hdr[0 .. n).  Lane u keeps block u's ranges, so that the
+// header words are put together once for the eight, and stored together
+// (a FULL pass that makes them, 2 GiB: 739 -> 662 us, against 600 without).
+__device__ __forceinline__ void block_headers(const uint4 q[8], uint32_t n, int lane, uint64_t *__restrict__ hdr) {
+    uint32_t mins = 0, maxs = 0;
+#pragma unroll
+    for (uint32_t u = 0; u < 8; ++u) {
+        if (u < n) {   // warp-uniform
+            const uint32_t r[4] = {crz_rot(q[u].x), crz_rot(q[u].y), crz_rot(q[u].z), crz_rot(q[u].w)};
+            uint32_t m, M;
+            crz_block_range(r, &m, &M);
+            if (lane == (int)u) mins = m, maxs = M;
+        }
+    }
+    if (lane < 8 && (uint32_t)lane < n) hdr[lane] = crz_header(mins, maxs);
+}
+
 // Partial CRAC-FP64 sum of a segment (<= 16 KiB) whose first word is word j0
 // of its chunk, over the lanes of one warp.  dest(), asked for once the first
 // loads are on their way, says where the segment's bytes are also stored (null:
@@ -118,15 +136,7 @@ __device__ __forceinline__ uint64_t hash_seg(const uint8_t *__restrict__ src, ui
             key += kStep;
         }
         if (kHdr && copy_to) {
-            const uint32_t b0 = v0 >> 5, nb = len >> 9;   // this round's first block, whole blocks
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                if (b0 + u < nb) {
-                    const uint32_t r[4] = {crz_rot(q[u].x), crz_rot(q[u].y), crz_rot(q[u].z), crz_rot(q[u].w)};
-                    const uint64_t h = crz_block_header(r);
-                    if (lane == 0) hdr[b0 + u] = h;
-                }
-            }
+            block_headers(q, (len >> 9) - (v0 >> 5), lane, hdr + (v0 >> 5));
         }
     }
     const uint32_t rem = len & 15u;
@@ -168,14 +178,7 @@ __device__ __forceinline__ void copy_with_headers(uint8_t *__restrict__ dst, con
             for (int u = 0; u < U; ++u)
                 if (b + u < nb) __stcs(d + 32 * (b + u) + lane, q[u]);
         }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            if (b + u < nb) {
-                const uint32_t r[4] = {crz_rot(q[u].x), crz_rot(q[u].y), crz_rot(q[u].z), crz_rot(q[u].w)};
-                const uint64_t h = crz_block_header(r);
-                if (lane == 0) hdr[b + u] = h;
-            }
-        }
+        block_headers(q, (uint32_t)(nb - b), lane, hdr + b);
     }
     if (vec) copy_group<32, true>(dst + (nb << 9), src + (nb << 9), len - (nb << 9), lane);
     else copy_group<32>(dst, src, len, lane);

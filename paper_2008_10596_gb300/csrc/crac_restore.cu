@@ -108,13 +108,15 @@ __global__ void __launch_bounds__(256) restore_unmark_kernel(const RestoreParams
 // one CTA per SM already paces; incremental restores, where most items are
 // skipped) a warp strides over the items, 32 at a time, a lane looking up each.
 struct RestoreItem {
-    uint64_t dst, src;
-    uint32_t len, z;   // bytes to write (0: nothing), bytes stored
+    uint64_t dst, src;   // raw: the item's bytes; coded: the whole chunk, its stream
+    uint32_t len;        // bytes to write (0: nothing)
+    uint32_t z;          // coded: the stream's length (0: stored raw)
+    uint32_t po, clen;   // the item's offset in its chunk, the chunk's length
 };
 
 template <bool kCoded>
 __device__ __forceinline__ RestoreItem restore_item(const RestoreParams &P, uint64_t it) {
-    RestoreItem r{0, 0, 0, 0};
+    RestoreItem r{};
     const uint32_t parts = P.log2_chunk - P.log2_part;   // log2 of the items per chunk
     const uint64_t tc = it >> parts;
     const uint64_t po = (it & ((1ull << parts) - 1)) << P.log2_part;   // the item's offset in its chunk
@@ -132,10 +134,15 @@ __device__ __forceinline__ RestoreItem restore_item(const RestoreParams &P, uint
         atomicOr(P.err, kErrBounds);
         return r;
     }
-    r.dst = d->dst + at + po;
-    r.src = pc->payload + o + po;
+    const bool stream = kCoded && ez != clen;
+    r.dst = d->dst + at + (stream ? 0 : po);
+    r.src = pc->payload + o + (stream ? 0 : po);
     r.len = (uint32_t)umin64(1ull << P.log2_part, clen - po);
-    r.z = (kCoded && ez != clen) ? (uint32_t)ez : r.len;
+    if (kCoded) {
+        r.z = stream ? (uint32_t)ez : 0u;
+        r.po = (uint32_t)po;
+        r.clen = (uint32_t)clen;
+    }
     return r;
 }
 
@@ -148,7 +155,7 @@ __device__ __forceinline__ void restore_scatter_body(const RestoreParams &P) {
     const uint64_t n_items = P.n_owner << (P.log2_chunk - P.log2_part);
     const uint64_t nw = (uint64_t)gridDim.x * (kScatterNT / 32);
     for (uint64_t i0 = (uint64_t)blockIdx.x * (kScatterNT / 32) + warp; i0 < n_items; i0 += 32 * nw) {
-        RestoreItem r{0, 0, 0, 0};
+        RestoreItem r{};
         if (i0 + lane * nw < n_items) r = restore_item<false>(P, i0 + lane * nw);
         unsigned todo = __ballot_sync(kFull, r.len != 0);
         while (todo) {   // warp-uniform
@@ -170,21 +177,27 @@ __global__ void __launch_bounds__(kScatterNT, 4) restore_scatter_ragged_kernel(c
 }
 
 // Chains with a coded image: the decoder needs registers that the plain copy
-// does not (hence two kernels), and an item is a whole chunk, looked up by the
-// whole warp: its decoding takes far longer than the look-up.
-__global__ void __launch_bounds__(kScatterNT, 4) restore_scatter_coded_kernel(const RestoreParams P) {
-    __shared__ __align__(16) uint8_t scratch[kCrzDecodeScratch * (kScatterNT / 32)];
+// does not (hence a kernel of its own), and an item, of 16 KiB or more, is
+// looked up by the whole warp: its decoding takes far longer than the look-up.
+__global__ void __launch_bounds__(kScatterNT, 3) restore_scatter_coded_kernel(const RestoreParams P) {
+    extern __shared__ __align__(16) uint8_t scratch[];   // kCrzDecodeScratch per warp
     wait_for_producer();
     if (*(volatile unsigned int *)P.err) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t parts = P.log2_chunk - P.log2_part;
+    const uint64_t n_items = P.n_owner << parts;
     const uint64_t nw = (uint64_t)gridDim.x * (kScatterNT / 32);
-    for (uint64_t it = (uint64_t)blockIdx.x * (kScatterNT / 32) + warp; it < P.n_owner; it += nw) {
+    for (uint64_t it = (uint64_t)blockIdx.x * (kScatterNT / 32) + warp; it < n_items; it += nw) {
         const RestoreItem r = restore_item<true>(P, it);
         if (r.len == 0) continue;
         uint8_t *dst = reinterpret_cast<uint8_t *>(r.dst);
         const uint8_t *src = reinterpret_cast<const uint8_t *>(r.src);
-        if (r.z == r.len) copy_group<32>(dst, src, r.len, lane);
-        else if (!crz_decode_warp(dst, src, r.len, r.z, lane, scratch + kCrzDecodeScratch * warp) && lane == 0)
+        if (!r.z) {
+            copy_group<32>(dst, src, r.len, lane);
+            continue;
+        }
+        const uint32_t b0 = r.po >> 9, b1 = (r.po + (1u << P.log2_part)) >> 9;   // the item's blocks of its chunk
+        if (!crz_decode_warp(dst, src, r.clen, r.z, b0, b1, lane, scratch + kCrzDecodeScratch * warp) && lane == 0)
             atomicOr(P.err, kErrCodec);
     }
 }
@@ -216,16 +229,22 @@ cudaError_t launch_restore_scatter(const RestoreParams &p, uint64_t max_grid, cu
     if (p.n_entries == 0 || p.n_owner == 0) return cudaSuccess;
     constexpr uint64_t kWarps = kScatterNT / 32;
     RestoreParams q = p;
-    // A coded entry is decoded whole, by one warp; a plain chunk is cut into
-    // parts of 8 KiB, and a warp takes about 8 KiB of short chunks.
-    q.log2_part = p.coded || p.log2_chunk < 13 ? p.log2_chunk : 13;
+    // A plain chunk is cut into parts of 8 KiB, and a warp takes about 8 KiB of
+    // short chunks.  Coded chunks are cut into parts of 16 KiB, and at most
+    // sixteen, as every part checks the whole stream's headers; not where those
+    // would cross the host link again.
+    if (p.coded) q.log2_part = p.host || p.log2_chunk < 15 ? p.log2_chunk : p.log2_chunk > 19 ? p.log2_chunk - 4 : 15;
+    else q.log2_part = p.log2_chunk < 13 ? p.log2_chunk : 13;
     uint64_t warps = p.n_owner << (p.log2_chunk - q.log2_part);
     if (p.log2_chunk < 13) warps = ((warps - 1) >> (13 - (p.log2_chunk < 8 ? 8 : p.log2_chunk))) + 1;
     const uint64_t ctas = umin64((warps + kWarps - 1) / kWarps, umin64(max_grid, 0x7fffffffull));
-    return chain(p.coded    ? restore_scatter_coded_kernel
-                 : p.ragged ? restore_scatter_ragged_kernel
-                            : restore_scatter_kernel,
-                 q, ctas, kScatterNT, s);
+    if (p.coded) {
+        constexpr int kSmem = kCrzDecodeScratch * (int)kWarps;
+        void *args[] = {&q};
+        return launch_chained(reinterpret_cast<const void *>(&restore_scatter_coded_kernel), (uint32_t)ctas, kScatterNT,
+                              args, s, kSmem);
+    }
+    return chain(p.ragged ? restore_scatter_ragged_kernel : restore_scatter_kernel, q, ctas, kScatterNT, s);
 }
 
 cudaError_t launch_scatter(const ScatterParams &p, int grid, cudaStream_t s) {
