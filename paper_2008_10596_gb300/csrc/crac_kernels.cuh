@@ -150,15 +150,16 @@ cudaError_t ckpt_tma_prepare();   // raise the dynamic shared memory limit (once
 
 // Split pass: three kernels with the signature (CkptParams, u64 *acc, u32 log2Seg),
 // run in order H -> F -> G.  acc holds one u64 per chunk of the segment and
-// must be zero before H; F uses cpt = split_finalize_threads() chunks per
-// tile and the look-back status words; G reads k from ctrl.
+// must be zero before H; F uses cpt = split_finalize_tile() chunks per tile
+// and the look-back status words; G reads k from ctrl.
 // aligned: every allocation's size is a multiple of 16 bytes (the other
 // instances store chunks at payload offsets of any alignment).
 const void *split_hash_fn(bool crz_headers, bool aligned);
 // Hash kernel for 512 B <= chunk < 8 KiB: lanes_per_chunk = chunk / 128;
 // it finalizes every chunk itself, so finalize runs with log2Seg = log2_chunk.
 const void *split_hash_small_fn(int lanes_per_chunk, bool aligned);
-const void *split_finalize_fn();
+uint32_t split_finalize_tile(uint64_t n_chunks, int sm_count);   // chunks per tile of the finalize kernel
+const void *split_finalize_fn(uint32_t tile);
 const void *split_gather_fn(bool crz_headers, bool aligned);
 int split_hash_threads();
 int split_finalize_threads();

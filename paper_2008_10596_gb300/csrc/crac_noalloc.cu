@@ -133,7 +133,8 @@ extern "C" crac_status_t crac_pass_noalloc(const crac_region_t *regions_dev, uin
         grid_per[0] = g_noalloc_grid[dev][0];
         grid_per[1] = g_noalloc_grid[dev][1];
     }
-    const uint32_t fin_tiles = (uint32_t)((n_chunks + split_finalize_threads() - 1) / split_finalize_threads());
+    const uint32_t fin_tile = split_finalize_tile(n_chunks, g_noalloc_sms[dev]);
+    const uint32_t fin_tiles = (uint32_t)((n_chunks + fin_tile - 1) / fin_tile);
     const size_t used = sizeof(CkptCtrl) + 16 * (size_t)fin_tiles;   // at most 128 KiB + 64 B of the scratch
     e = cudaMemsetAsync(scratch, 0, used, s);   // control block + status words start at zero
     uint32_t reserved = 0;
@@ -147,7 +148,7 @@ extern "C" crac_status_t crac_pass_noalloc(const crac_region_t *regions_dev, uin
         P.log2_chunk = l;
         P.c_begin = 0;
         P.c_end = n_chunks;
-        P.cpt = (uint32_t)split_finalize_threads();
+        P.cpt = fin_tile;
         P.n_tiles = fin_tiles;
         P.fp_old = fp_old_dev;
         P.fp_new = fp_new_dev;
@@ -189,7 +190,7 @@ extern "C" crac_status_t crac_pass_noalloc(const crac_region_t *regions_dev, uin
             e = cudaLaunchKernel(small ? split_hash_small_fn(1 << (l - 7), false) : split_hash_fn(false, false), dim3(grid),
                                  dim3(split_hash_threads()), args, 0, s);
         if (e == cudaSuccess)
-            e = cudaLaunchKernel(split_finalize_fn(), dim3(fin_tiles < 2u * sms ? fin_tiles : 2u * sms),
+            e = cudaLaunchKernel(split_finalize_fn(fin_tile), dim3(fin_tiles < 2u * sms ? fin_tiles : 2u * sms),
                                  dim3(split_finalize_threads()), args, 0, s);
         if (e == cudaSuccess)
             e = cudaLaunchKernel(split_gather_fn(false, false), dim3(8 * sms), dim3(split_gather_threads()), args, 0, s);

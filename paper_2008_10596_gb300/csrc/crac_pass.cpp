@@ -263,7 +263,7 @@ crac_status_t launch_fused_graph(crac_ctx *c, const CkptParams &P, size_t work_b
 crac_status_t launch_split_graph(crac_ctx *c, const CkptParams &P, size_t work_bytes, unsigned long long *acc,
                                  uint32_t log2Seg, const void *hash_fn, const int grids[3],
                                  void *ctrl_dst, cudaStream_t s) {
-    const void *fns[3] = {hash_fn, split_finalize_fn(), split_gather_fn(P.crz_hdr != nullptr, c->all16)};
+    const void *fns[3] = {hash_fn, split_finalize_fn(P.cpt), split_gather_fn(P.crz_hdr != nullptr, c->all16)};
     const int thr[3] = {split_hash_threads(), split_finalize_threads(), split_gather_threads()};
     CkptParams Pc = P;
     unsigned long long *accv = acc;
@@ -289,7 +289,7 @@ crac_status_t launch_split_graph(crac_ctx *c, const CkptParams &P, size_t work_b
     pro.kernelParams = pro_args;
     ReportNode rep(P.ctrl, ctrl_dst, c->fp_copy_dst, c->fp_copy_dst ? P.fp_new : nullptr,
                    c->fp_copy_dst ? P.c_end : 0, c->sm_count);
-    bool ok = c->sgexec != nullptr && c->s_hash_fn == hash_fn && c->s_gather_fn == fns[2];
+    bool ok = c->sgexec != nullptr && c->s_fns[0] == fns[0] && c->s_fns[1] == fns[1] && c->s_fns[2] == fns[2];
     if (ok) {
         ok = cudaGraphExecKernelNodeSetParams(c->sgexec, c->s_pro, &pro) == cudaSuccess;
         for (int i = 0; ok && i < 3; ++i)
@@ -323,8 +323,7 @@ crac_status_t launch_split_graph(crac_ctx *c, const CkptParams &P, size_t work_b
         CK(cudaGraphAddKernelNode(&c->s_copy, c->sgraph, nullptr, 0, &rep.kp));
         CK(cudaGraphAddDependencies(c->sgraph, last, &c->s_copy, &pe, 1));
         CK(cudaGraphInstantiate(&c->sgexec, c->sgraph, 0));
-        c->s_hash_fn = hash_fn;
-        c->s_gather_fn = fns[2];
+        std::copy(fns, fns + 3, c->s_fns);
     }
     if (!c->uva) CK(link_copy(c, c->desc.p, c->desc_src, c->allocs.size() * kDescBytes, cudaMemcpyHostToDevice, s));
     CK(cudaEventRecord(c->ev_t0, s));
@@ -353,7 +352,7 @@ crac_status_t launch_segment(crac_ctx *c, const Segment &sg, const CkptDesc *des
     if (!split)   // the split pass's prologue does this
         CK(link_copy(c, c->desc.p, c->desc_src, c->allocs.size() * kDescBytes, cudaMemcpyHostToDevice, s));
     if (split) {
-        const uint32_t cptF = (uint32_t)split_finalize_threads();
+        const uint32_t cptF = split_finalize_tile(nseg, c->sm_count);
         const uint64_t n_tiles = (nseg + cptF - 1) / cptF;
         if (n_tiles > 0x7fffffffull) return CRAC_ERR_UNSUPPORTED;
         const size_t status_bytes = sizeof(CkptCtrl) + 16 * n_tiles;
@@ -1536,7 +1535,7 @@ crac_status_t fingerprint_against(crac_ctx *c, const uint64_t *fp_ref, cudaStrea
         bytes += c->allocs[a].bytes;
     }
     const uint64_t n = first[na];
-    const uint32_t cptF = (uint32_t)split_finalize_threads();
+    const uint32_t cptF = split_finalize_tile(n, c->sm_count);
     const uint64_t n_tiles = (n + cptF - 1) / cptF;
     if (n_tiles > 0x7fffffffull) return CRAC_ERR_UNSUPPORTED;
     const size_t status_bytes = sizeof(CkptCtrl) + 16 * n_tiles;
@@ -1579,7 +1578,7 @@ crac_status_t fingerprint_against(crac_ctx *c, const uint64_t *fp_ref, cudaStrea
     const int gf = (int)std::max<uint64_t>(1, std::min<uint64_t>(n_tiles, (uint64_t)c->sm_count * 2));
     void *args[] = {&P, &acc, &log2Seg};
     CK(launch_chained(hash_fn, gh, split_hash_threads(), args, s));
-    CK(launch_chained(split_finalize_fn(), gf, split_finalize_threads(), args, s));
+    CK(launch_chained(split_finalize_fn(cptF), gf, split_finalize_threads(), args, s));
     *fp_out = (const uint64_t *)c->vfp.p;
     *ctrl_out = P.ctrl;
     return CRAC_OK;

@@ -477,7 +477,7 @@ struct crac_ctx {
     cudaGraphExec_t sgexec = nullptr;
     cudaGraphNode_t s_pro = nullptr, s_k[3] = {nullptr, nullptr, nullptr}, s_copy = nullptr;
     cudaEvent_t sev[4] = {nullptr, nullptr, nullptr, nullptr};   // around each split-pass kernel
-    const void *s_hash_fn = nullptr, *s_gather_fn = nullptr;   // the instances in it
+    const void *s_fns[3] = {nullptr, nullptr, nullptr};   // the kernels in it
     crac_pass_info_t last{};
     crac_restart_info_t last_restart{};
     bool all16 = false;          // current pass: every size a multiple of 16 bytes
