@@ -230,6 +230,10 @@ __device__ __forceinline__ void cp_async_wait() {
 // partly written when a plane value overflows a byte.  Bound by issue slots and
 // the latency of the shuffles, hence four blocks at a time: 2 GiB of fp32 in
 // device images 1264 -> 760 us (one block at a time 997, two 876 us).
+// kHost: the stream is in mapped host memory, where asynchronous copies into
+// shared memory reach 120 GB/s, ordinary loads the link's rate (190-200): the
+// units then come through registers, one step ahead of their use.
+template <bool kHost>
 __device__ __forceinline__ bool crz_decode_warp(uint8_t *dst, const uint8_t *src, uint64_t len, uint64_t z,
                                                 uint32_t b_begin, uint32_t b_end, int lane, uint8_t *scratch) {
     const uint32_t nb = (uint32_t)(len >> 9), tl = (uint32_t)len & 511u;   // chunks are at most 2^24 bytes
@@ -276,23 +280,34 @@ __device__ __forceinline__ bool crz_decode_warp(uint8_t *dst, const uint8_t *src
             tight |= ((uint32_t)(h >> (8 * p)) & 255u) + (1u << crz_width(h, p)) - 1u > 255u;
         const unsigned checked = __ballot_sync(kFull, tight);
         const int nblk = (int)min(32u, b_end - b0);
-        // The units arrive in shared memory a few groups of blocks ahead of
-        // their use: one 16-byte copy per lane and block (lane k: unit k).
+        // The units arrive in shared memory ahead of their use: one 16-byte
+        // copy (kHost: load) per lane and block, lane k unit k.
+        uint4 raw[kHost ? kG : 1];
         auto fetch = [&](int i) {
 #pragma unroll
             for (int g = 0; g < kG; ++g) {
                 const uint32_t n = __shfl_sync(kFull, ws, (i + g) & 31), u = __shfl_sync(kFull, first, (i + g) & 31);
-                if (i + g < nblk && (uint32_t)lane < n)
-                    cp_async16(scratch + 512 * ((i + g) % (kG * kN)) + 16 * lane, units + 16ull * (u + lane));
+                if (i + g < nblk && (uint32_t)lane < n) {
+                    const uint8_t *from = units + 16ull * (u + lane);
+                    if (kHost) raw[kHost ? g : 0] = *reinterpret_cast<const uint4 *>(from);
+                    else cp_async16(scratch + 512 * ((i + g) % (kG * kN)) + 16 * lane, from);
+                }
             }
-            cp_async_commit();
+            if (!kHost) cp_async_commit();
         };
 #pragma unroll
-        for (int i = 0; i < kG * (kN - 1); i += kG) fetch(i);
+        for (int i = 0; i < (kHost ? kG : kG * (kN - 1)); i += kG) fetch(i);
 #pragma unroll 1
         for (int i = 0; i < nblk; i += kG) {
-            fetch(i + kG * (kN - 1));   // (an empty group past the end)
-            cp_async_wait<kN - 1>();    // this step's units have landed
+            if (kHost) {
+#pragma unroll
+                for (int g = 0; g < kG; ++g)   // whatever lies past a block's units is not read
+                    *reinterpret_cast<uint4 *>(scratch + 512 * ((i + g) % (kG * kN)) + 16 * lane) = raw[kHost ? g : 0];
+                fetch(i + kG);
+            } else {
+                fetch(i + kG * (kN - 1));   // (an empty group past the end)
+                cp_async_wait<kN - 1>();    // this step's units have landed
+            }
             __syncwarp();
             // The group's blocks step by step together, so that their chains of
             // shuffles overlap (past the end: a block of width 0, not stored).

@@ -179,6 +179,7 @@ __global__ void __launch_bounds__(kScatterNT, 4) restore_scatter_ragged_kernel(c
 // Chains with a coded image: the decoder needs registers that the plain copy
 // does not (hence a kernel of its own), and an item, of 16 KiB or more, is
 // looked up by the whole warp: its decoding takes far longer than the look-up.
+template <bool kHost>
 __global__ void __launch_bounds__(kScatterNT, 3) restore_scatter_coded_kernel(const RestoreParams P) {
     extern __shared__ __align__(16) uint8_t scratch[];   // kCrzDecodeScratch per warp
     wait_for_producer();
@@ -197,7 +198,8 @@ __global__ void __launch_bounds__(kScatterNT, 3) restore_scatter_coded_kernel(co
             continue;
         }
         const uint32_t b0 = r.po >> 9, b1 = (r.po + (1u << P.log2_part)) >> 9;   // the item's blocks of its chunk
-        if (!crz_decode_warp(dst, src, r.clen, r.z, b0, b1, lane, scratch + kCrzDecodeScratch * warp) && lane == 0)
+        if (!crz_decode_warp<kHost>(dst, src, r.clen, r.z, b0, b1, lane, scratch + kCrzDecodeScratch * warp) &&
+            lane == 0)
             atomicOr(P.err, kErrCodec);
     }
 }
@@ -241,8 +243,9 @@ cudaError_t launch_restore_scatter(const RestoreParams &p, uint64_t max_grid, cu
     if (p.coded) {
         constexpr int kSmem = kCrzDecodeScratch * (int)kWarps;
         void *args[] = {&q};
-        return launch_chained(reinterpret_cast<const void *>(&restore_scatter_coded_kernel), (uint32_t)ctas, kScatterNT,
-                              args, s, kSmem);
+        const void *fn = p.host ? reinterpret_cast<const void *>(&restore_scatter_coded_kernel<true>)
+                                : reinterpret_cast<const void *>(&restore_scatter_coded_kernel<false>);
+        return launch_chained(fn, (uint32_t)ctas, kScatterNT, args, s, kSmem);
     }
     return chain(p.ragged ? restore_scatter_ragged_kernel : restore_scatter_kernel, q, ctas, kScatterNT, s);
 }
