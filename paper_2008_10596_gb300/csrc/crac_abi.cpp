@@ -28,6 +28,8 @@ bool fault_hit(int step) {
     return false;
 }
 
+bool fault_armed(int step) { return g_fault_step.load() == step && g_fault_count.load() > 0; }
+
 void note_cuda_error(int e) { t_last_cuda = e; }
 
 namespace {

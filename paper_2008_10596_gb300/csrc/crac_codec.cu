@@ -405,6 +405,13 @@ constexpr uint32_t kSizeTile = 64;         // entries per tile of the sizing ker
                                            // 2 GiB of 64 KiB entries kept 128 CTAs busy for 36 us)
 constexpr uint32_t kSegBlocks = 32;        // blocks per work item of the sized encoder: 16 KiB
 
+// The entries to code: P.k, or in the pass's graph what the pass found (none
+// after an error, whose tables may have holes).
+__device__ __forceinline__ uint64_t entry_count(const CodecParams &P) {
+    if (!P.ctrl) return P.k;
+    return P.ctrl->err ? 0 : (uint64_t)P.ctrl->k;
+}
+
 // zlen and zoff of every entry (and zoff[k]) from the header widths: one warp
 // per entry sums them; a tile's padded lengths are scanned and placed by a
 // decoupled look-back over the earlier tiles (tiles are taken in ticket
@@ -416,6 +423,8 @@ __global__ void __launch_bounds__(kCodecNT) crz_size_kernel(const CodecParams P)
     __shared__ uint64_t s_w64[kCodecWarps];
     __shared__ uint64_t s_base;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    wait_for_producer();   // in the pass's graph: its list, counts and headers
+    const uint64_t k = entry_count(P);
     for (;;) {
         __syncthreads();   // the previous tile's shared state is consumed
         if (tid == 0) {
@@ -427,12 +436,16 @@ __global__ void __launch_bounds__(kCodecNT) crz_size_kernel(const CodecParams P)
         }
         __syncthreads();
         const uint64_t e0 = (uint64_t)s_tile * kSizeTile;
-        if (e0 >= P.k) return;
-        const uint32_t ne = (uint32_t)umin64(kSizeTile, P.k - e0);
+        if (e0 >= k) return;
+        const uint32_t ne = (uint32_t)umin64(kSizeTile, k - e0);
         for (uint32_t t = warp; t < ne; t += kCodecWarps) {
             const uint64_t e = e0 + t;
-            const uint64_t L = P.off[e + 1] - P.off[e], nb = L >> 9;
-            const uint64_t *h = P.chdr + (P.idx[e] << P.log2_bpc);
+            const uint64_t L = P.off[e + 1] - P.off[e], nb = L >> 9, c = P.idx[e];
+            const uint64_t *h = P.chdr + (c << P.log2_bpc);
+            if (P.srcs) {   // where the encoder finds the entry
+                const CkptDesc a = P.desc[find_alloc_warp(P.desc, P.n_allocs, c, lane)];
+                if (lane == 0) P.srcs[e] = a.ptr + ((c - a.first_chunk) << (P.log2_bpc + 9));
+            }
             uint32_t w = 0;
             for (uint64_t b = lane; b < nb; b += 32) w += crz_width_sum(h[b]);
             w = __reduce_add_sync(kFull, w);   // <= 32 per block, nb <= 2^15
@@ -464,11 +477,11 @@ __global__ void __launch_bounds__(kCodecNT) crz_size_kernel(const CodecParams P)
             const uint64_t e = e0 + tid, zo = base + ex;
             P.zoff[e] = zo;
             // entries that start a piece: k * i / pieces == e for some i
-            const uint64_t i = (e * P.pieces + P.k - 1) / P.k;   // smallest i with k * i / pieces >= e
-            if (i < P.pieces && P.k * i / P.pieces == e) P.piece_off[i] = zo;
+            const uint64_t i = (e * P.pieces + k - 1) / k;   // smallest i with k * i / pieces >= e
+            if (i < P.pieces && k * i / P.pieces == e) P.piece_off[i] = zo;
         }
-        if (tid == 0 && e0 + ne == P.k) {
-            P.zoff[P.k] = base + tile_bytes;
+        if (tid == 0 && e0 + ne == k) {
+            P.zoff[k] = base + tile_bytes;
             P.piece_off[P.pieces] = base + tile_bytes;
         }
     }
@@ -494,8 +507,14 @@ __global__ void __launch_bounds__(kCodecNT, 4) crz_encode_sized_kernel(const Cod
     __shared__ __align__(16) uint8_t s_ring[kCodecWarps][512 * kAhead * 4];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const CrzLane LT = crz_lane(lane);
+    wait_for_producer();   // in the pass's graph: the sizing kernel
     const uint32_t spe = P.segs_per_entry;
-    const uint64_t items = (P.e_end - P.e_begin) * spe;
+    uint64_t items = (P.e_end - P.e_begin) * spe;
+    if (P.ctrl) {
+        const unsigned int err = *P.err;   // of the sizing: offsets are missing
+        if (err && blockIdx.x == 0 && tid == 0) atomicOr(&P.ctrl->err, err);
+        items = err ? 0 : entry_count(P) * spe;
+    }
     const uint64_t nw = ((uint64_t)gridDim.x * kCodecNT) >> 5;
     for (uint64_t it = ((uint64_t)blockIdx.x * kCodecNT + tid) >> 5; it < items; it += nw) {
         const uint64_t e = P.e_begin + it / spe;
@@ -503,7 +522,7 @@ __global__ void __launch_bounds__(kCodecNT, 4) crz_encode_sized_kernel(const Cod
         const uint64_t o = P.off[e], L = P.off[e + 1] - o;
         const uint64_t z = P.zlen[e];
         uint8_t *d = P.dst + P.zoff[e];
-        const uint8_t *src = P.src + o;
+        const uint8_t *src = P.srcs ? reinterpret_cast<const uint8_t *>(P.srcs[e]) : P.src + o;
         if (z == L) {   // stored raw
             const uint64_t x0 = (uint64_t)sg * (512ull * kSegBlocks);
             if (x0 >= L) continue;
@@ -597,6 +616,10 @@ uint32_t crz_tile_max() { return kCodecTileMax; }
 uint64_t crz_size_tiles(uint64_t k) { return (k + kSizeTile - 1) / kSizeTile; }
 
 uint32_t crz_sized_segs(uint32_t log2S) { return log2S > 14 ? 1u << (log2S - 14) : 1u; }
+
+const void *crz_size_fn() { return reinterpret_cast<const void *>(&crz_size_kernel); }
+const void *crz_encode_sized_fn() { return reinterpret_cast<const void *>(&crz_encode_sized_kernel<false>); }
+int crz_threads() { return kCodecNT; }
 
 cudaError_t launch_crz_size(const CodecParams &p, int grid, cudaStream_t s) {
     if (p.k == 0) return cudaSuccess;

@@ -92,8 +92,11 @@ struct CkptParams {
     // (c << (log2_chunk - 9)) + block, written by whichever kernel writes the
     // chunk (hash: FULL or predicted; gather: the rest) from the vectors it
     // holds (laid out across the warp as the encoder lays out a block), so
-    // that the encoder does not compute them again.
+    // that the encoder does not compute them again.  hdr_only: the encoder
+    // reads the allocations themselves (CodecParams::srcs); nothing is written
+    // to staging, and offsets in it only tell where the chunks would be.
     uint64_t *crz_hdr;
+    uint32_t hdr_only;
 };
 
 // Restore: one image allocation mapped onto the target layout.
@@ -291,7 +294,18 @@ struct CodecParams {
     uint32_t pieces;
     uint32_t segs_per_entry;
     uint64_t e_begin, e_end;
+    // Coded in the pass's own graph, straight from the allocations (the pass
+    // then writes block headers but no payload): the entry count and the pass's
+    // error bits are in *ctrl, which also receives this coder's, and the sizing
+    // kernel leaves every entry's address in srcs.  Null: src, k.
+    CkptCtrl *ctrl;
+    uint64_t *srcs;
+    const CkptDesc *desc;
+    uint32_t n_allocs;
 };
+const void *crz_size_fn();
+const void *crz_encode_sized_fn();   // streams to device memory
+int crz_threads();
 cudaError_t launch_crz_encode(const CodecParams &p, int grid, cudaStream_t s);
 cudaError_t launch_crz_size(const CodecParams &p, int grid, cudaStream_t s);
 uint64_t crz_size_tiles(uint64_t k);   // look-back words it needs

@@ -105,7 +105,7 @@ void ctx_free_all(crac_ctx *c) {
     if (c->sgexec) cudaGraphExecDestroy(c->sgexec);
     if (c->sgraph) cudaGraphDestroy(c->sgraph);
     for (cudaEvent_t e : {c->ev_last, c->ev_pass, c->ev_t0, c->ev_t1, c->ev_p0, c->ev_p1, c->sev[0], c->sev[1],
-                          c->sev[2], c->sev[3], c->ev_r0, c->ev_r1})
+                          c->sev[2], c->sev[3], c->sev[4], c->ev_r0, c->ev_r1})
         if (e) cudaEventDestroy(e);
     for (cudaEvent_t e : c->ev_piece)
         if (e) cudaEventDestroy(e);
@@ -259,10 +259,12 @@ crac_status_t launch_fused_graph(crac_ctx *c, const CkptParams &P, size_t work_b
     return CRAC_OK;
 }
 
-// Build (or update) the split-pass graph and launch it.
+// Build (or update) the split-pass graph and launch it; with `enc`, the coder
+// runs in it after the gather, so that a coded image too is of one point in the
+// stream's order.
 crac_status_t launch_split_graph(crac_ctx *c, const CkptParams &P, size_t work_bytes, unsigned long long *acc,
                                  uint32_t log2Seg, const void *hash_fn, const int grids[3],
-                                 void *ctrl_dst, cudaStream_t s) {
+                                 const CodecParams *enc, void *ctrl_dst, cudaStream_t s) {
     const void *fns[3] = {hash_fn, split_finalize_fn(P.cpt), split_gather_fn(P.crz_hdr != nullptr, c->all16)};
     const int thr[3] = {split_hash_threads(), split_finalize_threads(), split_gather_threads()};
     CkptParams Pc = P;
@@ -287,13 +289,34 @@ crac_status_t launch_split_graph(crac_ctx *c, const CkptParams &P, size_t work_b
     pro.gridDim = dim3(prologue_grid(zero16, desc16, c->sm_count));
     pro.blockDim = dim3(prologue_threads());
     pro.kernelParams = pro_args;
+    CodecParams Ec{};
+    void *enc_args[] = {&Ec};
+    cudaKernelNodeParams ek[2] = {};
+    if (enc) {
+        Ec = *enc;
+        const uint64_t n = P.c_end - P.c_begin, items = n * Ec.segs_per_entry, warps = crz_threads() / 32;
+        ek[0].func = const_cast<void *>(crz_size_fn());
+        ek[0].gridDim = dim3((unsigned)std::min<uint64_t>(crz_size_tiles(n), (uint64_t)c->sm_count * 4));
+        // A FULL pass codes every item: a CTA for every eight.  A delta's count
+        // is not known yet: up to four waves of resident CTAs stride over it.
+        ek[1].func = const_cast<void *>(crz_encode_sized_fn());
+        ek[1].gridDim = dim3((unsigned)std::min<uint64_t>(
+            (items + warps - 1) / warps, c->full_copy_ok ? 0x7fffffffull : (uint64_t)c->sm_count * 16));
+        for (cudaKernelNodeParams &k : ek) {
+            k.blockDim = dim3(crz_threads());
+            k.kernelParams = enc_args;
+        }
+    }
     ReportNode rep(P.ctrl, ctrl_dst, c->fp_copy_dst, c->fp_copy_dst ? P.fp_new : nullptr,
                    c->fp_copy_dst ? P.c_end : 0, c->sm_count);
-    bool ok = c->sgexec != nullptr && c->s_fns[0] == fns[0] && c->s_fns[1] == fns[1] && c->s_fns[2] == fns[2];
+    bool ok = c->sgexec != nullptr && c->s_fns[0] == fns[0] && c->s_fns[1] == fns[1] && c->s_fns[2] == fns[2] &&
+              c->s_codes == (enc != nullptr);
     if (ok) {
         ok = cudaGraphExecKernelNodeSetParams(c->sgexec, c->s_pro, &pro) == cudaSuccess;
         for (int i = 0; ok && i < 3; ++i)
             ok = cudaGraphExecKernelNodeSetParams(c->sgexec, c->s_k[i], &kp[i]) == cudaSuccess;
+        for (int i = 0; ok && enc && i < 2; ++i)
+            ok = cudaGraphExecKernelNodeSetParams(c->sgexec, c->s_enc[i], &ek[i]) == cudaSuccess;
         if (ok) ok = cudaGraphExecKernelNodeSetParams(c->sgexec, c->s_copy, &rep.kp) == cudaSuccess;
         if (!ok) cudaGetLastError();
     }
@@ -302,10 +325,11 @@ crac_status_t launch_split_graph(crac_ctx *c, const CkptParams &P, size_t work_b
         if (c->sgraph) cudaGraphDestroy(c->sgraph);
         c->sgexec = nullptr;
         c->sgraph = nullptr;
-        // prologue => hash => finalize => gather => control block report, where
-        // => is a programmatic edge (the consumer is launched as its producer
+        // prologue => hash => finalize => gather [=> size => code] => control block
+        // report, where => is a programmatic edge (the consumer is launched as its producer
         // drains and waits in-kernel for its completion); events 0-3 record the
-        // ends of the first four on side branches, off the critical path.
+        // ends of the first four and of the coding on side branches, off the
+        // critical path.
         CK(cudaGraphCreate(&c->sgraph, 0));
         cudaGraphEdgeData pe{};
         pe.from_port = cudaGraphKernelNodePortProgrammatic;
@@ -320,25 +344,34 @@ crac_status_t launch_split_graph(crac_ctx *c, const CkptParams &P, size_t work_b
             last = &c->s_k[i];
             CK(cudaGraphAddEventRecordNode(&ev, c->sgraph, last, 1, c->sev[i + 1]));
         }
+        for (int i = 0; enc && i < 2; ++i) {
+            CK(cudaGraphAddKernelNode(&c->s_enc[i], c->sgraph, nullptr, 0, &ek[i]));
+            CK(cudaGraphAddDependencies(c->sgraph, last, &c->s_enc[i], &pe, 1));
+            last = &c->s_enc[i];
+        }
+        if (enc) CK(cudaGraphAddEventRecordNode(&ev, c->sgraph, last, 1, c->sev[4]));
         CK(cudaGraphAddKernelNode(&c->s_copy, c->sgraph, nullptr, 0, &rep.kp));
         CK(cudaGraphAddDependencies(c->sgraph, last, &c->s_copy, &pe, 1));
         CK(cudaGraphInstantiate(&c->sgexec, c->sgraph, 0));
         std::copy(fns, fns + 3, c->s_fns);
+        c->s_codes = enc != nullptr;
     }
     if (!c->uva) CK(link_copy(c, c->desc.p, c->desc_src, c->allocs.size() * kDescBytes, cudaMemcpyHostToDevice, s));
     CK(cudaEventRecord(c->ev_t0, s));
     CK(cudaGraphLaunch(c->sgexec, s));
-    count_launches(5);
+    count_launches(enc ? 7 : 5);
     return CRAC_OK;
 }
 
 // Enqueue one segment of the checkpoint pass on s, reading the baseline
 // fp[fp_cur] and writing fingerprints to fp[out_fp]; the control block is
-// copied to the host at ctrl_dst after the pass, and ev_pass is recorded.
+// copied to the host at ctrl_dst after the pass, and ev_pass is recorded.  enc:
+// the coder's destination and tables, where the pass codes the image itself
+// (codes_in_pass); the streams' bytes are then in the control block's pad[1].
 crac_status_t launch_segment(crac_ctx *c, const Segment &sg, const CkptDesc *desc_dev,
                              const std::vector<uint64_t> &first, uint64_t *idx_d, uint64_t *off_d,
                              uint64_t idx_cap, uint8_t *staging, uint64_t staging_cap, int out_fp,
-                             void *ctrl_dst, cudaStream_t s) {
+                             void *ctrl_dst, cudaStream_t s, CodecParams *enc = nullptr) {
     const uint64_t nseg = sg.c1 - sg.c0;
     const uint64_t *fp_old = (const uint64_t *)c->fp[c->fp_cur].p;
     uint64_t *fp_new = (uint64_t *)c->fp[out_fp].p;
@@ -356,11 +389,13 @@ crac_status_t launch_segment(crac_ctx *c, const Segment &sg, const CkptDesc *des
         const uint64_t n_tiles = (nseg + cptF - 1) / cptF;
         if (n_tiles > 0x7fffffffull) return CRAC_ERR_UNSUPPORTED;
         const size_t status_bytes = sizeof(CkptCtrl) + 16 * n_tiles;
-        const size_t work_bytes = status_bytes + 8 * nseg;
+        size_t work_bytes = status_bytes + 8 * nseg;
+        const size_t enc_at = work_bytes;   // the coder's error word, ticket and look-back words
+        if (enc) work_bytes += 8 + 8 * crz_size_tiles(nseg);
         TRY(ensure_dev(c->work, work_bytes + 16));   // zeroed in 16-byte words
         // 512 B..4 KiB chunks: several whole chunks per warp iteration.
         const bool small = c->log2S >= 9 && c->log2S < 13;
-        const bool copies = staging && (c->full_copy_ok || c->sparse_ok);   // the hash kernel writes every chunk
+        const bool copies = staging && !enc && (c->full_copy_ok || c->sparse_ok);   // the hash kernel writes every chunk
         const uint32_t log2Seg = small ? c->log2S : split_hash_seg(sg.bytes, c->log2S, copies);
         // Coded contexts with chunks of 8 KiB and more: the kernel that writes a
         // chunk to staging (hash or gather) also writes its CRZ1 block headers
@@ -374,6 +409,7 @@ crac_status_t launch_segment(crac_ctx *c, const Segment &sg, const CkptDesc *des
                                       : split_hash_fn(crz_hdr != nullptr, c->all16);
         CkptParams P{};
         P.crz_hdr = crz_hdr;
+        P.hdr_only = enc ? 1u : 0u;
         P.desc = desc_dev;
         P.n_allocs = (uint32_t)c->allocs.size();
         P.log2_chunk = c->log2S;
@@ -413,7 +449,24 @@ crac_status_t launch_segment(crac_ctx *c, const Segment &sg, const CkptDesc *des
         const int gf = (int)std::min<uint64_t>(n_tiles, (uint64_t)c->sm_count * 2);
         const int gg = c->sm_count * 8;
         const int grids[3] = {gh, gf, gg};
-        TRY(launch_split_graph(c, P, work_bytes, acc, log2Seg, hash_fn, grids, ctrl_dst, s));
+        if (enc) {
+            enc->off = off_d;
+            enc->idx = idx_d;
+            enc->chdr = crz_hdr;
+            enc->log2_bpc = c->log2S - 9;
+            enc->segs_per_entry = crz_sized_segs(c->log2S);
+            enc->ctrl = P.ctrl;
+            enc->srcs = (uint64_t *)acc;   // the finalize kernel was their last reader
+            enc->desc = desc_dev;
+            enc->n_allocs = P.n_allocs;
+            enc->err = (unsigned int *)((uint8_t *)c->work.p + enc_at);
+            enc->ticket = (uint32_t *)enc->err + 1;
+            enc->status = (uint64_t *)((uint8_t *)c->work.p + enc_at + 8);
+            enc->pieces = 1;
+            enc->piece_off = (uint64_t *)P.ctrl->pad;   // 0 and the streams' bytes
+            enc->timeout_ns = c->cfg.timeout_ns;
+        }
+        TRY(launch_split_graph(c, P, work_bytes, acc, log2Seg, hash_fn, grids, enc, ctrl_dst, s));
         if (c->spec_now) {   // this pass's offsets predict the next one's
             c->ppos_cur ^= 1;
             c->ppos_ok = true;
@@ -422,7 +475,7 @@ crac_status_t launch_segment(crac_ctx *c, const Segment &sg, const CkptDesc *des
         c->last.grid = (uint32_t)gh;
         c->last.chunks_per_tile = cptF;
         c->last.warps_per_chunk = 0;
-        c->last.kernel_launches += 5;   // prologue, hash, finalize, gather, control-block report
+        c->last.kernel_launches += enc ? 7 : 5;   // prologue, hash, finalize, gather, [size, code,] report
         c->last.pass_kernel = P.sparse ? CRAC_PASS_SPARSE : CRAC_PASS_SPLIT;
     } else if (c->cfg.launch_mode == CRAC_LAUNCH_BATCHED) {
         const uint64_t S = 1ull << c->log2S;
@@ -508,6 +561,7 @@ crac_status_t launch_segment(crac_ctx *c, const Segment &sg, const CkptDesc *des
         c->last.kernel_launches += 1;
     }
     c->split_now = split;
+    c->enc_now = enc != nullptr;
     CK(cudaEventRecord(c->ev_t1, s));
     CK(cudaEventRecord(c->ev_pass, s));
     return CRAC_OK;
@@ -528,6 +582,10 @@ void pass_timings(crac_ctx *c, float *ms) {
             c->last.finalize_ms += b;
             c->last.gather_ms += d;
         }
+        if (c->enc_now && cudaEventElapsedTime(&t, c->sev[3], c->sev[4]) == cudaSuccess) {
+            c->last.codec_ms += t;   // not part of the pass's time
+            *ms -= t;
+        }
         cudaGetLastError();
     }
 }
@@ -537,8 +595,9 @@ void pass_timings(crac_ctx *c, float *ms) {
 crac_status_t run_segment(crac_ctx *c, const Segment &sg, const CkptDesc *desc_dev,
                           const std::vector<uint64_t> &first, uint64_t *idx_d, uint64_t *off_d,
                           uint64_t idx_cap, uint8_t *staging, uint64_t staging_cap, int out_fp,
-                          cudaStream_t s, CkptCtrl *ctrl_out, float *ms) {
-    TRY(launch_segment(c, sg, desc_dev, first, idx_d, off_d, idx_cap, staging, staging_cap, out_fp, c->ctrl_h.p, s));
+                          cudaStream_t s, CkptCtrl *ctrl_out, float *ms, CodecParams *enc = nullptr) {
+    TRY(launch_segment(c, sg, desc_dev, first, idx_d, off_d, idx_cap, staging, staging_cap, out_fp, c->ctrl_h.p, s,
+                       enc));
     CK(cudaEventSynchronize(c->ev_pass));
     pass_timings(c, ms);
     *ctrl_out = *(const CkptCtrl *)c->ctrl_h.p;
@@ -930,6 +989,23 @@ crac_status_t ctx_settle(crac_ctx *c, bool block) {
     return CRAC_OK;
 }
 
+// Whether a coded pass of `segments` segments codes the image in its own graph,
+// from the allocations themselves: one segment into a device image.  It takes
+// the worst case of the streams from the arena's regions as they are (as the
+// uncoded passes take theirs).  Where those have no room; for host images,
+// whose streams cross the link more slowly than any of this; and with
+// allocations in host memory, which would cross it twice: the pass gathers into
+// staging, and the host sizes the destination before the streams are coded.
+// 2 GiB of fp32: a FULL checkpoint 1400 us gathered -> 1200 so (nothing written
+// to staging, no round trips to the host), a delta of 10% 560 -> 470.  The
+// injected sizing fault counts tiles that only the host's form knows beforehand.
+bool codes_in_pass(const crac_ctx *c, size_t segments, bool host_res) {
+    if (!c->crz_hdr_now || host_res || segments != 1 || fault_armed(CRAC_FAULT_ENCODE_WAIT)) return false;
+    for (const AllocRec &r : c->allocs)
+        if (r.kind == CRAC_KIND_HOST) return false;
+    return true;
+}
+
 // The passes of a checkpoint that waits for each segment's dirty counts:
 // several staging segments, coded images or per-allocation launches.  Each
 // segment is enqueued, waited for, sized and drained (A2-A5) before the
@@ -977,8 +1053,16 @@ crac_status_t checkpoint_wait(crac_ctx *c, crac_image *im, const std::vector<Seg
             return cuda_status(cudaGetLastError());
         }
         CkptCtrl ctrl{};
+        CodecParams enc{};
+        const uint64_t zmax = sg.bytes + 16 * nseg;
+        const bool in_pass = codes_in_pass(c, segs.size(), host_res) && da.try_alloc(zmax, &pc.dev);
+        if (in_pass) {
+            enc.dst = pc.dev.p;
+            enc.zoff = (uint64_t *)pc.off_dev.p;
+            enc.zlen = (uint64_t *)pc.zlen_dev.p;
+        }
         st = run_segment(c, sg, (const CkptDesc *)c->desc.p, first, idx_d, off_d, nseg, stg, sg.bytes, out_fp, s,
-                         &ctrl, &ms);
+                         &ctrl, &ms, in_pass ? &enc : nullptr);
         if (st != CRAC_OK) {
             im->pieces.push_back(pc);
             return st;
@@ -992,7 +1076,14 @@ crac_status_t checkpoint_wait(crac_ctx *c, crac_image *im, const std::vector<Seg
         pc.bytes = sparse ? ctrl.payload : ctrl.D;
         pc.span = sparse ? ctrl.D : 0;
         bool zplaced = false;
-        if (coded && ctrl.k) {
+        if (in_pass) {
+            pc.bytes = ctrl.pad[1];
+            if (pc.bytes > ctrl.D + 16 * ctrl.k) {
+                im->pieces.push_back(pc);
+                return CRAC_ERR_CORRUPT;
+            }
+            if (ctrl.k == 0) da.free(pc.dev);
+        } else if (coded && ctrl.k) {
             uint64_t Z = 0;
             cudaEvent_t d0 = drain_started || !host_res ? nullptr : im->drain0;
             st = encode_segment(c, pc, ctrl, host_res, direct_flag, s, &Z, &zplaced, &d0);

@@ -94,7 +94,7 @@ __device__ __forceinline__ void block_headers(const uint4 q[8], uint32_t n, int 
 // have any alignment (else a multiple of 16, and the segment's length too).
 template <bool kHdr, bool kAny, class Dest>
 __device__ __forceinline__ uint64_t hash_seg(const uint8_t *__restrict__ src, uint32_t len, uint32_t j0, int lane,
-                                             Dest &&dest, uint64_t *__restrict__ hdr) {
+                                             Dest &&dest, uint64_t *__restrict__ hdr, bool store) {
     const uint4 *p = reinterpret_cast<const uint4 *>(src);
     const uint32_t nv = len >> 4;
     constexpr int U = 8;
@@ -112,7 +112,7 @@ __device__ __forceinline__ uint64_t hash_seg(const uint8_t *__restrict__ src, ui
             if (v0 + 32u * u + lane < nv) q[u] = __ldg(p + v0 + 32u * u + lane);
         if (v0 == 0) {
             copy_to = dest();
-            if (kAny) m = (uint32_t)(uintptr_t)copy_to & 15u;
+            if (kAny && store) m = (uint32_t)(uintptr_t)copy_to & 15u;
         }
         if (kAny && m) {   // warp-uniform
 #pragma unroll
@@ -121,7 +121,7 @@ __device__ __forceinline__ uint64_t hash_seg(const uint8_t *__restrict__ src, ui
                 store_shifted(copy_to, m, v0 + 32u * u + lane, nv, prev, q[u]);
             }
             last = q[U - 1];
-        } else if (copy_to) {   // the vectors also go straight to staging
+        } else if (copy_to && store) {   // the vectors also go straight to staging
             uint4 *to = reinterpret_cast<uint4 *>(copy_to) + v0 + lane;
 #pragma unroll
             for (int u = 0; u < U; ++u)
@@ -152,7 +152,7 @@ __device__ __forceinline__ uint64_t hash_seg(const uint8_t *__restrict__ src, ui
         acc += mixw(w0, kt);
         if (rem > 8) acc += mixw(w1, kt + kK1);
     }
-    if (kAny && copy_to && (m | rem)) store_ends(copy_to, src, m, nv, len, lane, 32);
+    if (kAny && copy_to && store && (m | rem)) store_ends(copy_to, src, m, nv, len, lane, 32);
     return acc;
 }
 
@@ -160,9 +160,10 @@ __device__ __forceinline__ uint64_t hash_seg(const uint8_t *__restrict__ src, ui
 // stores the CRZ1 header word of each whole 512-byte block b at hdr[b], in the
 // encoder's layout (lane l holds bytes 16l .. 16l+15 of the block).  A dst off
 // the 16-byte grid is copied by copy_group, which re-reads the (cached) source.
+// (!store: headers only).
 template <bool kAligned>
 __device__ __forceinline__ void copy_with_headers(uint8_t *__restrict__ dst, const uint8_t *__restrict__ src,
-                                                  uint64_t len, int lane, uint64_t *__restrict__ hdr) {
+                                                  uint64_t len, int lane, uint64_t *__restrict__ hdr, bool store) {
     const uint64_t nb = len >> 9;
     const uint4 *s = reinterpret_cast<const uint4 *>(src);
     uint4 *d = reinterpret_cast<uint4 *>(dst);
@@ -173,13 +174,14 @@ __device__ __forceinline__ void copy_with_headers(uint8_t *__restrict__ dst, con
 #pragma unroll
         for (int u = 0; u < U; ++u)
             if (b + u < nb) q[u] = __ldg(s + 32 * (b + u) + lane);
-        if (vec) {
+        if (vec && store) {
 #pragma unroll
             for (int u = 0; u < U; ++u)
                 if (b + u < nb) __stcs(d + 32 * (b + u) + lane, q[u]);
         }
         block_headers(q, (uint32_t)(nb - b), lane, hdr + b);
     }
+    if (!store) return;
     if (vec) copy_group<32, true>(dst + (nb << 9), src + (nb << 9), len - (nb << 9), lane);
     else copy_group<32>(dst, src, len, lane);
 }
@@ -232,7 +234,8 @@ split_hash_kernel(const CkptParams P, unsigned long long *__restrict__ acc, uint
         };
         const uint8_t *src = reinterpret_cast<const uint8_t *>(d.ptr) + (local << log2S) + off;
         uint64_t sum = hash_seg<kHdr, kAny>(src, len, off >> 3, lane, dest,
-                                            kHdr ? P.crz_hdr + (c << (log2S - 9)) + (off >> 9) : nullptr);
+                                            kHdr ? P.crz_hdr + (c << (log2S - 9)) + (off >> 9) : nullptr,
+                                            !kHdr || !P.hdr_only);
         sum = warp_sum(sum);
         if (lane == 0) {
             if (spc == 0) {
@@ -690,8 +693,8 @@ split_finalize_kernel(const CkptParams P, unsigned long long *__restrict__ acc, 
 template <bool kHdr, bool kAligned>
 __global__ void __launch_bounds__(kGatherNT, kHdr ? 2 : 4)
 split_gather_kernel(const CkptParams P, unsigned long long *, uint32_t) {
-    if (copies_all(P)) return;   // the hash kernel has already written every chunk
     wait_for_producer();         // the finalize kernel's list and counts
+    if (copies_all(P)) return;   // the hash kernel has already written every chunk
     const int lane = threadIdx.x & 31;
     const uint64_t kd = (uint64_t)P.ctrl->k;
     const uint64_t k = kd < P.idx_cap ? kd : P.idx_cap;
@@ -748,7 +751,7 @@ split_gather_kernel(const CkptParams P, unsigned long long *, uint32_t) {
             uint8_t *to = P.staging + __shfl_sync(kFull, dst, i);
             const uint8_t *from = reinterpret_cast<const uint8_t *>(__shfl_sync(kFull, src, i));
             const uint32_t n = __shfl_sync(kFull, len, i);
-            if (kHdr) copy_with_headers<kAligned>(to, from, n, lane, P.crz_hdr + __shfl_sync(kFull, blk, i));
+            if (kHdr) copy_with_headers<kAligned>(to, from, n, lane, P.crz_hdr + __shfl_sync(kFull, blk, i), !P.hdr_only);
             else copy_group<32, kAligned>(to, from, n, lane);
         }
     }

@@ -70,6 +70,7 @@ crac_status_t cuda_status(cudaError_t e);   // records e for crac_last_cuda_erro
     } while (0)
 
 bool fault_hit(int step);   // consumes one injected fault at `step`
+bool fault_armed(int step); // whether there is one
 
 inline uint64_t round_up(uint64_t x, uint64_t a) { return (x + a - 1) / a * a; }
 
@@ -476,8 +477,10 @@ struct crac_ctx {
     cudaGraph_t sgraph = nullptr;
     cudaGraphExec_t sgexec = nullptr;
     cudaGraphNode_t s_pro = nullptr, s_k[3] = {nullptr, nullptr, nullptr}, s_copy = nullptr;
-    cudaEvent_t sev[4] = {nullptr, nullptr, nullptr, nullptr};   // around each split-pass kernel
+    cudaEvent_t sev[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};   // around each split-pass kernel, and the coder
     const void *s_fns[3] = {nullptr, nullptr, nullptr};   // the kernels in it
+    cudaGraphNode_t s_enc[2] = {nullptr, nullptr};        // the coder's sizing and coding, if it codes too
+    bool s_codes = false, enc_now = false;                // (the graph; the pass just enqueued)
     crac_pass_info_t last{};
     crac_restart_info_t last_restart{};
     bool all16 = false;          // current pass: every size a multiple of 16 bytes
