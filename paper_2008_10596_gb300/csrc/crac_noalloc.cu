@@ -9,7 +9,9 @@
 // scratch -- the control block, the look-back status words and the regions'
 // payload offsets -- in a fixed array of this library's device memory instead
 // of a buffer obtained from cudaMalloc, and the caller's fingerprint table as
-// the chunks' accumulators.
+// the chunks' accumulators.  One kernel prepares all of that, and each later one
+// is launched as the one before it drains (six launches and memsets in a row
+// took 21 us more than the fused kernel's one on 22 MiB).
 // ---------------------------------------------------------------------------
 
 namespace {
@@ -23,26 +25,33 @@ void *g_noalloc_addr[kNoAllocMaxDevices];     // device address of the scratch, 
 int g_noalloc_grid[kNoAllocMaxDevices][2];   // SMs x occupancy of the fused kernel for warps-per-chunk 1 and 8
 int g_noalloc_sms[kNoAllocMaxDevices];
 
-constexpr int kPrefixNT = 1024;
+constexpr int kPrepareNT = 1024;
 
-// One CTA, before a pass without a baseline: the payload bytes before each
-// region, and the flag that the hash kernel may write every chunk there as it
-// reads it (there is room for them all).
-__global__ void __launch_bounds__(kPrefixNT)
-noalloc_prefix_kernel(const crac::CkptDesc *__restrict__ d, uint32_t n, uint64_t cap, uint64_t *__restrict__ prefix,
-                      uint32_t *__restrict__ flag) {
+// Before the pass: zeroed scratch and accumulators (na and nb words), and, where
+// there is no baseline (prefix), the payload bytes before each region and the
+// flag that the hash kernel may write every chunk there as it reads it (there
+// is room for them all), by CTA 0.
+__global__ void __launch_bounds__(kPrepareNT)
+noalloc_prepare_kernel(uint64_t *__restrict__ zero_a, uint32_t na, uint64_t *__restrict__ zero_b, uint32_t nb,
+                       const crac::CkptDesc *__restrict__ d, uint32_t n, uint64_t cap, uint64_t *__restrict__ prefix,
+                       uint32_t *__restrict__ flag) {
     using namespace crac;
-    __shared__ uint64_t s_sum[kPrefixNT / 32];
+    __shared__ uint64_t s_sum[kPrepareNT / 32];
+    for (uint32_t i = blockIdx.x * kPrepareNT + threadIdx.x; i < na + nb; i += gridDim.x * kPrepareNT) {
+        if (i < na) zero_a[i] = 0;
+        else zero_b[i - na] = 0;
+    }
+    if (blockIdx.x || !prefix) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t per = (n + kPrefixNT - 1) / kPrefixNT;
-    const uint32_t i0 = threadIdx.x * per, i1 = min(n, i0 + per);
+    const uint32_t per = (n + kPrepareNT - 1) / kPrepareNT;
+    const uint32_t i0 = min(n, threadIdx.x * per), i1 = min(n, i0 + per);
     uint64_t sum = 0;
     for (uint32_t i = i0; i < i1; ++i) sum += d[i].bytes;
     const uint64_t incl = warp_incl_scan(sum, lane);
     if (lane == 31) s_sum[warp] = incl;
     __syncthreads();
     uint64_t before = 0, total = 0;
-    for (int w = 0; w < kPrefixNT / 32; ++w) {
+    for (int w = 0; w < kPrepareNT / 32; ++w) {
         if (w < warp) before += s_sum[w];
         total += s_sum[w];
     }
@@ -59,6 +68,7 @@ noalloc_prefix_kernel(const crac::CkptDesc *__restrict__ d, uint32_t n, uint64_t
 // (tiles and CTAs of a ticket-driven pass).
 __global__ void noalloc_totals_kernel(const crac::CkptCtrl *ctrl, uint8_t *out, uint32_t reserved) {
     const uint32_t t = threadIdx.x;
+    crac::wait_for_producer();
     if (t >= sizeof(crac_pass_totals_t)) return;
     const uint64_t w = t < 8 ? (uint64_t)ctrl->err << 32 | reserved : t < 16 ? ctrl->k : ctrl->D;
     out[t] = (uint8_t)(w >> (8 * (t & 7u)));
@@ -135,12 +145,21 @@ extern "C" crac_status_t crac_pass_noalloc(const crac_region_t *regions_dev, uin
     }
     const uint32_t fin_tile = split_finalize_tile(n_chunks, g_noalloc_sms[dev]);
     const uint32_t fin_tiles = (uint32_t)((n_chunks + fin_tile - 1) / fin_tile);
-    const size_t used = sizeof(CkptCtrl) + 16 * (size_t)fin_tiles;   // at most 128 KiB + 64 B of the scratch
-    e = cudaMemsetAsync(scratch, 0, used, s);   // control block + status words start at zero
+    unsigned char *sc = static_cast<unsigned char *>(scratch);
+    const size_t used = sizeof(CkptCtrl) + 16 * (size_t)(fin_tiles > 32 ? fin_tiles : 32);   // at most 16.1 KiB
+    CkptCtrl *ctrl = reinterpret_cast<CkptCtrl *>(sc);
     uint32_t reserved = 0;
-    if (e == cudaSuccess && n_tiles) {
-        unsigned char *sc = static_cast<unsigned char *>(scratch);
+    if (n_tiles == 0) {
+        noalloc_prepare_kernel<<<1, kPrepareNT, 0, s>>>(reinterpret_cast<uint64_t *>(sc), (uint32_t)(used / 8), nullptr, 0,
+                                                        nullptr, 0, 0, nullptr, nullptr);
+        e = cudaGetLastError();
+        if (e == cudaSuccess) count_launches(1);
+    } else {
         CkptParams P{};
+        // A list that one CTA takes in a few rounds, too short for a chain of
+        // kernels: the fused one (4 chunks of 4 KiB: 19 us to the call's end, the
+        // chain 24; 512 chunks of 512 B 53 and 26).
+        const bool fused = n_chunks <= 32 && n_chunks * chunk_bytes <= (256u << 10);
         P.desc = reinterpret_cast<const CkptDesc *>(regions_dev);
         P.n_allocs = n_regions;
         uint32_t l = 0;
@@ -148,8 +167,8 @@ extern "C" crac_status_t crac_pass_noalloc(const crac_region_t *regions_dev, uin
         P.log2_chunk = l;
         P.c_begin = 0;
         P.c_end = n_chunks;
-        P.cpt = fin_tile;
-        P.n_tiles = fin_tiles;
+        P.cpt = fused ? cpt : fin_tile;
+        P.n_tiles = fused ? (uint32_t)n_tiles : fin_tiles;
         P.fp_old = fp_old_dev;
         P.fp_new = fp_new_dev;
         P.idx_out = idx_dev;
@@ -157,51 +176,56 @@ extern "C" crac_status_t crac_pass_noalloc(const crac_region_t *regions_dev, uin
         P.idx_cap = idx_cap;
         P.staging = staging_dev;
         P.staging_cap = staging_dev ? staging_cap : 0;
-        P.ctrl = reinterpret_cast<CkptCtrl *>(scratch);
+        P.ctrl = ctrl;
         P.tile_cnt = reinterpret_cast<uint64_t *>(sc + sizeof(CkptCtrl));
-        P.tile_bytes = P.tile_cnt + fin_tiles;
+        P.tile_bytes = P.tile_cnt + P.n_tiles;
         P.timeout_ns = 2000000000ull;
         // Without a baseline every chunk is dirty and its payload offset known
         // beforehand: the hash kernel writes it there as it reads it, if they
         // all fit (1 GiB in 64 KiB chunks: 486 us with the fused kernel, which
-        // reads every chunk twice, 340 us this way; with a baseline and 10%
-        // dirty 263 and 205 us).
+        // reads every chunk twice, 325 us this way; with a baseline and 10%
+        // dirty 263 and 200 us).
         const size_t at = (used + 255) / 256 * 256;
-        if (!fp_old_dev && staging_dev && n_regions <= (kNoAllocScratchBytes - at) / 8 - 1) {
-            uint64_t *prefix = reinterpret_cast<uint64_t *>(sc + at);
+        uint64_t *prefix = nullptr;
+        if (!fused && !fp_old_dev && staging_dev && n_regions <= (kNoAllocScratchBytes - at) / 8 - 1) {
+            prefix = reinterpret_cast<uint64_t *>(sc + at);
             P.full_copy = 1;
             P.full_flag = reinterpret_cast<const uint32_t *>(prefix + n_regions);
             P.alloc_prefix = prefix;
-            noalloc_prefix_kernel<<<1, kPrefixNT, 0, s>>>(P.desc, n_regions, P.staging_cap, prefix,
-                                                          reinterpret_cast<uint32_t *>(prefix + n_regions));
-            e = cudaGetLastError();
-            count_launches(1);
         }
         const bool small = l >= 9 && l < 13;
         const uint64_t most = n_chunks << l;   // the regions' bytes are in device memory only
         uint32_t log2Seg = small ? l : split_hash_seg(most, l, P.full_copy != 0);
         const uint32_t grid = split_hash_grid(n_chunks, most, l, log2Seg, &P.slots_per_warp);
         // Segmented chunks are summed up in the caller's table, in place.
-        unsigned long long *acc = log2Seg < l ? reinterpret_cast<unsigned long long *>(fp_new_dev) : nullptr;
-        if (e == cudaSuccess && acc) e = cudaMemsetAsync(fp_new_dev, 0, n_chunks * 8, s);
+        unsigned long long *acc = !fused && log2Seg < l ? reinterpret_cast<unsigned long long *>(fp_new_dev) : nullptr;
+        const uint32_t sms = (uint32_t)g_noalloc_sms[dev], na = (uint32_t)(used / 8), nb = acc ? (uint32_t)n_chunks : 0u;
+        const uint32_t want = (na + nb + kPrepareNT - 1) / kPrepareNT;
+        noalloc_prepare_kernel<<<want < sms ? want : sms, kPrepareNT, 0, s>>>(
+            reinterpret_cast<uint64_t *>(sc), na, fp_new_dev, nb, P.desc, n_regions, P.staging_cap, prefix,
+            prefix ? reinterpret_cast<uint32_t *>(prefix + n_regions) : nullptr);
+        e = cudaGetLastError();
+        if (e == cudaSuccess) count_launches(1);
         void *args[] = {&P, &acc, &log2Seg};
-        const int sms = g_noalloc_sms[dev];
-        if (e == cudaSuccess)
-            e = cudaLaunchKernel(small ? split_hash_small_fn(1 << (l - 7), false) : split_hash_fn(false, false), dim3(grid),
-                                 dim3(split_hash_threads()), args, 0, s);
-        if (e == cudaSuccess)
-            e = cudaLaunchKernel(split_finalize_fn(fin_tile), dim3(fin_tiles < 2u * sms ? fin_tiles : 2u * sms),
-                                 dim3(split_finalize_threads()), args, 0, s);
-        if (e == cudaSuccess)
-            e = cudaLaunchKernel(split_gather_fn(false, false), dim3(8 * sms), dim3(split_gather_threads()), args, 0, s);
-        if (e == cudaSuccess) count_launches(3);
+        if (e == cudaSuccess && fused) {
+            e = cudaLaunchKernel(ckpt_fused_fn(256, wpc), dim3((uint32_t)n_tiles), dim3(256), args, 0, s);
+            if (e == cudaSuccess) count_launches(1);
+        }
+        if (e == cudaSuccess && !fused)
+            e = launch_chained(small ? split_hash_small_fn(1 << (l - 7), false) : split_hash_fn(false, false), grid,
+                               split_hash_threads(), args, s);
+        if (e == cudaSuccess && !fused)
+            e = launch_chained(split_finalize_fn(fin_tile), fin_tiles < 2u * sms ? fin_tiles : 2u * sms,
+                               split_finalize_threads(), args, s);
+        if (e == cudaSuccess && !fused)
+            e = launch_chained(split_gather_fn(false, false), 8 * sms, split_gather_threads(), args, s);
         const uint64_t g = grid_per[wpc == 8 ? 1 : 0];
         reserved = (uint32_t)(n_tiles + (n_tiles < g ? n_tiles : g));
     }
     if (e == cudaSuccess) {
-        noalloc_totals_kernel<<<1, 32, 0, s>>>(reinterpret_cast<const CkptCtrl *>(scratch), reinterpret_cast<uint8_t *>(totals_dev), reserved);
-        e = cudaGetLastError();
-        if (e == cudaSuccess) count_launches(1);
+        uint8_t *out = reinterpret_cast<uint8_t *>(totals_dev);
+        void *args[] = {&ctrl, &out, &reserved};
+        e = launch_chained(reinterpret_cast<const void *>(&noalloc_totals_kernel), 1, 32, args, s);
     }
     if (e != cudaSuccess) {
         note_cuda_error((int)e);

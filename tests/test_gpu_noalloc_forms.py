@@ -53,10 +53,11 @@ def _expect(host, S, dirty):
 
 ALIGNED = [65536 * 3 + 48, 16, 4096, 8192 + 512, 131072, 262144 + 16]
 RAGGED = [65536 * 3 + 5, 3, 4097, 8191, 131072, 262144 + 1, 16]
+FEW = [4096 * 3 + 5, 3, 4097, 100, 70001]   # one short list with 4-16 KiB chunks
 
 
 @pytest.mark.parametrize("S", [64, 512, 4096, 8192, 16384, 65536, 262144])
-@pytest.mark.parametrize("sizes", [ALIGNED, RAGGED], ids=["aligned", "ragged"])
+@pytest.mark.parametrize("sizes", [ALIGNED, RAGGED, FEW], ids=["aligned", "ragged", "few"])
 @pytest.mark.parametrize("shift", [0, 8])
 def test_forms(S, sizes, shift):
     host = [W.host_contents("u32_xorshift", n, 70 + i) for i, n in enumerate(sizes)]
@@ -86,7 +87,7 @@ def test_forms(S, sizes, shift):
     check(_call(bufs, host, S, [i != 2 for i in range(len(sizes))], base, shift), dirty)
 
 
-@pytest.mark.parametrize("sizes", [ALIGNED, RAGGED], ids=["aligned", "ragged"])
+@pytest.mark.parametrize("sizes", [ALIGNED, RAGGED, FEW], ids=["aligned", "ragged", "few"])
 def test_too_small_buffers_are_reported(sizes):
     S = 4096
     host = [W.host_contents("u32_xorshift", n, 90 + i) for i, n in enumerate(sizes)]
