@@ -171,7 +171,11 @@ typedef struct crac_config {
  *   into device staging as usual and an encoder kernel writes the streams --
  *   into the device image, the staging drain, or, with
  *   CRAC_FLAG_DIRECT_DRAIN, straight into the image's pinned memory -- so
- *   only the coded bytes cross the host link.  Restores decode in the scatter
+ *   only the coded bytes cross the host link.  A pass of one segment into a
+ *   device image on chunks of 8 KiB and more codes straight from the
+ *   allocations, within the same graph, when the device arena has room for
+ *   the streams' worst case without growing (and no allocation is in host
+ *   memory).  Restores decode in the scatter
  *   kernel, reading host images in place; a context that has to stage its
  *   host restores (no unified addressing) cannot restore coded images
  *   (CRAC_ERR_UNSUPPORTED).  Images carry CRAC_IMAGE_CODED.  Not with
@@ -654,8 +658,9 @@ typedef struct crac_pass_totals {
  * addition of this library.
  *
  * It allocates nothing: no cudaMalloc, cudaFree, pinned memory or library
- * allocation.  Its only scratch (the pass control block and the look-back
- * status words, 64 + 16 * CRAC_NOALLOC_MAX_TILES bytes) is a fixed array in
+ * allocation.  Its only scratch (the pass control block, the look-back status
+ * words and the regions' payload offsets: 64 + 16 * CRAC_NOALLOC_MAX_TILES
+ * bytes; sums in progress are kept in fp_new_dev) is a fixed array in
  * the library's device memory, present on every device that loads the
  * library until the process exits.  The first call on a device looks up that
  * array's address (once per device); make that first call before any stream

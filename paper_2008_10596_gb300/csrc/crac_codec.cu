@@ -1,5 +1,6 @@
-// The CRZ1 encoder: a segment's raw payload (device staging) -> one stream
-// per entry, written to device memory or straight into mapped pinned memory.
+// The CRZ1 encoder: a segment's raw payload (in device staging, or where it
+// lies in the allocations) -> one stream per entry, written to device memory or
+// straight into mapped pinned memory.
 #include "crac_codec.cuh"
 
 namespace crac {
@@ -400,7 +401,8 @@ __global__ void __launch_bounds__(kCodecNT, 3) crz_encode_kernel(const CodecPara
 // With every block's header word already in P.chdr, a stream's length needs
 // only its headers' widths: crz_size_kernel sizes and places every stream
 // first, and crz_encode_sized_kernel then codes without any wait between
-// CTAs, one warp per 16 KiB segment of an entry, straight from staging.
+// CTAs, one warp per 16 KiB segment of an entry, straight from staging, or, as
+// nodes of the pass's graph, from the allocations.
 constexpr uint32_t kSizeTile = 64;         // entries per tile of the sizing kernel: eight a warp (with 256,
                                            // 2 GiB of 64 KiB entries kept 128 CTAs busy for 36 us)
 constexpr uint32_t kSegBlocks = 32;        // blocks per work item of the sized encoder: 16 KiB

@@ -69,7 +69,10 @@ __device__ __forceinline__ bool copies_all(const CkptParams &P) {
 // CRZ1 header words of the first n (at most 8) blocks of q (block u: q[u]
 // across the warp) to hdr[0 .. n).  Lane u keeps block u's ranges, so that the
 // header words are put together once for the eight, and stored together
-// (a FULL pass that makes them, 2 GiB: 739 -> 662 us, against 600 without).
+// (a FULL pass that makes them and writes staging, 2 GiB: 739 -> 662 us, against
+// 600 without headers; one that only makes them 535, against 312.  Reducing
+// several blocks' extremes together by shuffles, without reduction
+// instructions, gave 520 there and lost as much on deltas to its registers).
 __device__ __forceinline__ void block_headers(const uint4 q[8], uint32_t n, int lane, uint64_t *__restrict__ hdr) {
     uint32_t mins = 0, maxs = 0;
 #pragma unroll
