@@ -71,8 +71,8 @@ struct CkptParams {
     // dirty entry's offset points there, ctrl->D counts the segment's bytes
     // and ctrl->payload the dirty ones; nothing is gathered.
     uint32_t sparse;
-    // Split pass, hash kernel on chunks below 512 B and from 8 KiB: segments per
-    // warp.
+    // Split pass, hash kernel: segments per warp; on chunks of 512 B - 4 KiB
+    // iterations of 4 KiB.
     uint32_t slots_per_warp;
     // TMA pass: the allocations' first_chunk column fits in the CTA's shared
     // memory (n_allocs <= ckpt_tma_cached_allocs()) and is searched there.
@@ -170,9 +170,9 @@ int split_gather_threads();
 // log2 of the hash kernel's segment (at most the chunk) for `bytes` tracked
 // bytes; copy: every chunk is also written.  Not for chunks of 512 B - 4 KiB.
 uint32_t split_hash_seg(uint64_t bytes, uint32_t log2_chunk, bool copy);
-// Grid of the hash kernel over n_chunks chunks holding `bytes` bytes, and
-// CkptParams::slots_per_warp of that grid.
-uint32_t split_hash_grid(uint64_t n_chunks, uint64_t bytes, uint32_t log2_chunk, uint32_t log2_seg,
+// Grid of the hash kernel over n_chunks chunks holding `bytes` bytes (copy: as
+// for split_hash_seg), and CkptParams::slots_per_warp of that grid.
+uint32_t split_hash_grid(uint64_t n_chunks, uint64_t bytes, uint32_t log2_chunk, uint32_t log2_seg, bool copy,
                          uint32_t *slots_per_warp);
 const void *split_hash_small_dense_fn(int lanes_per_chunk);
 

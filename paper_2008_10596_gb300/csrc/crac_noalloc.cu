@@ -196,7 +196,7 @@ extern "C" crac_status_t crac_pass_noalloc(const crac_region_t *regions_dev, uin
         const bool small = l >= 9 && l < 13;
         const uint64_t most = n_chunks << l;   // the regions' bytes are in device memory only
         uint32_t log2Seg = small ? l : split_hash_seg(most, l, P.full_copy != 0);
-        const uint32_t grid = split_hash_grid(n_chunks, most, l, log2Seg, &P.slots_per_warp);
+        const uint32_t grid = split_hash_grid(n_chunks, most, l, log2Seg, P.full_copy != 0, &P.slots_per_warp);
         // Segmented chunks are summed up in the caller's table, in place.
         unsigned long long *acc = !fused && log2Seg < l ? reinterpret_cast<unsigned long long *>(fp_new_dev) : nullptr;
         const uint32_t sms = (uint32_t)g_noalloc_sms[dev], na = (uint32_t)(used / 8), nb = acc ? (uint32_t)n_chunks : 0u;

@@ -445,7 +445,7 @@ crac_status_t launch_segment(crac_ctx *c, const Segment &sg, const CkptDesc *des
             P.seg_base = pre + ((sg.c0 - first[a0]) << c->log2S);
         }
         unsigned long long *acc = (unsigned long long *)((uint8_t *)c->work.p + status_bytes);
-        const int gh = (int)split_hash_grid(nseg, sg.bytes, c->log2S, log2Seg, &P.slots_per_warp);
+        const int gh = (int)split_hash_grid(nseg, sg.bytes, c->log2S, log2Seg, copies, &P.slots_per_warp);
         const int gf = (int)std::min<uint64_t>(n_tiles, (uint64_t)c->sm_count * 2);
         const int gg = c->sm_count * 8;
         const int grids[3] = {gh, gf, gg};
@@ -1665,7 +1665,7 @@ crac_status_t fingerprint_against(crac_ctx *c, const uint64_t *fp_ref, cudaStrea
     P.tile_bytes = P.tile_cnt + n_tiles;
     P.timeout_ns = c->cfg.timeout_ns;
     unsigned long long *acc = (unsigned long long *)((uint8_t *)c->vwork.p + status_bytes);
-    const int gh = (int)split_hash_grid(n, bytes, log2S, log2Seg, &P.slots_per_warp);
+    const int gh = (int)split_hash_grid(n, bytes, log2S, log2Seg, false, &P.slots_per_warp);
     const int gf = (int)std::max<uint64_t>(1, std::min<uint64_t>(n_tiles, (uint64_t)c->sm_count * 2));
     void *args[] = {&P, &acc, &log2Seg};
     CK(launch_chained(hash_fn, gh, split_hash_threads(), args, s));

@@ -257,14 +257,18 @@ split_hash_kernel(const CkptParams P, unsigned long long *__restrict__ acc, uint
 
 // Hash kernel for chunks of 512 B..4 KiB: one warp iteration covers 4 KiB,
 // i.e. 4096/S whole chunks, one group of LPC = S/128 lanes per chunk (8
-// vectors per lane), so a warp keeps 4 KiB in flight whatever the chunk size; a
-// warp makes two iterations, a CTA 64 KiB, in the grid of split_hash_kernel
-// (8 GiB in 4 KiB chunks, every chunk written: 2741 -> 2407 us against one wave
-// of resident CTAs; one iteration per warp gives 2397, four 2453).
+// vectors per lane), so a warp keeps 4 KiB in flight whatever the chunk size, in
+// the grid of split_hash_kernel.  A warp makes two iterations where the pass
+// writes every chunk (8 GiB in 4 KiB chunks: 2741 -> 2407 us against one wave of
+// resident CTAs; one iteration gives 2397, four 2453).  Where it mostly reads,
+// the look-up that a warp starts with weighs more: up to sixteen, as long as
+// 4096 CTAs remain (32 GiB, clean: 5502 us in one wave, 5805 with two iterations,
+// 5349 with sixteen; 1 GiB 206, 212, 204 with eight).
 // Every chunk is finalized in place (direct mode: acc receives the dirty
 // length, and finalize only compacts).
 constexpr int kSmallVecs = 8;     // vectors per lane of one iteration
-constexpr int kSmallIters = 2;    // iterations per warp
+constexpr uint64_t kSmallIters = 2;        // iterations per warp,
+constexpr uint64_t kSmallItersRead = 16;   // ... at most, where the pass mostly reads
 
 template <int LPC, bool kAny>
 __device__ __forceinline__ void hash_small_iter(const CkptParams &P, unsigned long long *__restrict__ acc,
@@ -392,8 +396,8 @@ split_hash_small_kernel(const CkptParams P, unsigned long long *__restrict__ acc
     const int lane = threadIdx.x & 31;
     const uint64_t warp_g = ((uint64_t)blockIdx.x * kHashNT + threadIdx.x) >> 5;
     const uint64_t n_slots = (P.c_end - P.c_begin + CPS - 1) / CPS;
-    uint64_t q = warp_g * kSmallIters;
-    const uint64_t q_end = umin64(q + kSmallIters, n_slots);
+    uint64_t q = warp_g * P.slots_per_warp;
+    const uint64_t q_end = umin64(q + P.slots_per_warp, n_slots);
     CkptDesc d{};
     uint64_t a_next = 0;
     uint32_t a = 0;
@@ -441,8 +445,8 @@ split_hash_small_dense_kernel(const CkptParams P, unsigned long long *__restrict
     uint64_t a_next = 0;
     CkptDesc dw{};
 #pragma unroll 1
-    for (int it = 0; it < kSmallIters; ++it) {
-        const uint64_t c0 = P.c_begin + (warp_g * kSmallIters + it) * CPS;
+    for (uint32_t it = 0; it < P.slots_per_warp; ++it) {
+        const uint64_t c0 = P.c_begin + (warp_g * P.slots_per_warp + it) * CPS;
         if (c0 >= P.c_end) break;   // warp-uniform
         if (c0 >= a_next) {
             a = find_alloc_warp(P.desc, P.n_allocs, c0, lane);
@@ -824,12 +828,14 @@ uint32_t split_hash_seg(uint64_t bytes, uint32_t log2S, bool copy) {
 // A warp takes one segment, or as many as hold a segment's bytes on average
 // (chunks below 512 B; allocations mostly much shorter than a chunk, whose
 // segments past their end are empty).
-uint32_t split_hash_grid(uint64_t n_chunks, uint64_t bytes, uint32_t log2S, uint32_t log2Seg,
+uint32_t split_hash_grid(uint64_t n_chunks, uint64_t bytes, uint32_t log2S, uint32_t log2Seg, bool copy,
                          uint32_t *slots_per_warp) {
     constexpr uint64_t kWarps = kHashNT / 32;
     uint64_t per, n = n_chunks;   // items per warp, items
-    if (log2S >= 9 && log2S < 13) {   // chunks
-        per = (4096ull >> log2S) * kSmallIters;
+    if (log2S >= 9 && log2S < 13) {   // iterations of 4 KiB
+        n = (n << log2S) / 4096 + 1;
+        per = copy ? kSmallIters : n >> 15;
+        per = per < kSmallIters ? kSmallIters : umin64(per, kSmallItersRead);
     } else {                          // segments
         n <<= log2S - log2Seg;
         const uint32_t m = log2Seg < 13 ? 13 : log2Seg;

@@ -14,7 +14,8 @@ pytestmark = [pytest.mark.gpu, pytest.mark.usefixtures("oracle_lib")]
 
 
 @pytest.mark.parametrize("S,total,residency", [(64, 20 << 20, C.CRAC_RESIDENCY_HOST), (64, 40 << 20, C.CRAC_RESIDENCY_HOST),
-                                               (512, 170 << 20, C.CRAC_RESIDENCY_DEVICE)])
+                                               (512, 170 << 20, C.CRAC_RESIDENCY_DEVICE),
+                                               (2048, 420 << 20, C.CRAC_RESIDENCY_HOST)])   # three iterations a warp
 def test_many_chunks(S, total, residency):
     n_sm = torch.cuda.get_device_properties(0).multi_processor_count
     at = 2 * n_sm * 1024 * S if S == 64 and total < 30 << 20 else total   # just past the threshold, or well past it
