@@ -229,7 +229,8 @@ __device__ __forceinline__ void cp_async_wait() {
 // inconsistent (every caller checks the whole stream's), and the chunk may be
 // partly written when a plane value overflows a byte.  Bound by issue slots and
 // the latency of the shuffles, hence four blocks at a time: 2 GiB of fp32 in
-// device images 1264 -> 760 us (one block at a time 997, two 876 us).
+// device images 1264 -> 760 us (one block at a time 997, two 876 us).  dst is
+// 16-byte aligned.
 // kHost: the stream is in mapped host memory, where asynchronous copies into
 // shared memory reach 120 GB/s, ordinary loads the link's rate (190-200): the
 // units then come through registers, one step ahead of their use.
@@ -280,6 +281,13 @@ __device__ __forceinline__ bool crz_decode_warp(uint8_t *dst, const uint8_t *src
             tight |= ((uint32_t)(h >> (8 * p)) & 255u) + (1u << crz_width(h, p)) - 1u > 255u;
         const unsigned checked = __ballot_sync(kFull, tight);
         const int nblk = (int)min(32u, b_end - b0);
+        if (!__any_sync(kFull, ws != 0)) {   // constant planes only (zeros, say): a word repeated per block
+            for (int i = 0; i < nblk; ++i) {
+                const uint32_t w = crz_unrot(__shfl_sync(kFull, (uint32_t)h, i));
+                __stcs(reinterpret_cast<uint4 *>(dst + 512ull * (b0 + i)) + lane, make_uint4(w, w, w, w));
+            }
+            continue;
+        }
         // The units arrive in shared memory ahead of their use: one 16-byte
         // copy (kHost: load) per lane and block, lane k unit k.
         uint4 raw[kHost ? kG : 1];

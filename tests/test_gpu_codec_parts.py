@@ -23,6 +23,11 @@ def _contents(kind, n, seed):
         w[:, 1] = rng.integers(200, 203, size=w.shape[0])
         w[:, 2] = 0
         return w.reshape(-1)[:n].copy()
+    if kind == "half":   # windows of constant blocks before and between others
+        h = W.host_contents("f32_normal", n, seed)
+        h[: n // 2] = 0x7F
+        h[3 * n // 4: 3 * n // 4 + 20 * KIB] = 0
+        return h
     return W.host_contents(kind, n, seed)
 
 
@@ -32,7 +37,7 @@ def _contents(kind, n, seed):
 def test_coded_parts(S, residency, flags):
     edges = [512, 513, 16 * KIB - 512, 16 * KIB, 16 * KIB + 512 + 4, 32 * KIB - 16, 32 * KIB + 511, 48 * KIB + 1024,
              64 * KIB - 1, 2 * S, S + 16 * KIB + 3]
-    kinds = ["f32_normal", "zeros", "bf16", "wide", "u8"]
+    kinds = ["f32_normal", "zeros", "bf16", "half", "wide", "u8"]
     h = Harness(S, lineage=1900 + S % 97 + flags, image_residency=residency, flags=C.CRAC_FLAG_COMPRESS | flags)
     try:
         sizes = []
