@@ -663,8 +663,9 @@ typedef struct crac_pass_totals {
  * bytes; sums in progress are kept in fp_new_dev) is a fixed array in
  * the library's device memory, present on every device that loads the
  * library until the process exits.  The first call on a device looks up that
- * array's address (once per device); make that first call before any stream
- * capture.  Every call shares the array: calls whose work overlaps on the GPU
+ * array's address and loads every kernel that a call of any form may launch
+ * (once per device, which may allocate and synchronize); make that first call,
+ * of any form, before any stream capture.  Every call shares the array: calls whose work overlaps on the GPU
  * (different streams, or different host threads, without ordering) race and
  * give wrong results.  Each call clears the part it uses before the pass.
  *
