@@ -997,10 +997,13 @@ crac_status_t ctx_settle(crac_ctx *c, bool block) {
 // allocations in host memory, which would cross it twice: the pass gathers into
 // staging, and the host sizes the destination before the streams are coded.
 // 2 GiB of fp32: a FULL checkpoint 1400 us gathered -> 1200 so (nothing written
-// to staging, no round trips to the host), a delta of 10% 560 -> 470.  The
-// injected sizing fault counts tiles that only the host's form knows beforehand.
-bool codes_in_pass(const crac_ctx *c, size_t segments, bool host_res) {
-    if (!c->crz_hdr_now || host_res || segments != 1 || fault_armed(CRAC_FAULT_ENCODE_WAIT)) return false;
+// to staging, no round trips to the host), a delta of 10% 560 -> 470.  An
+// injected sizing fault skips a tile, which only a later tile's wait notices: it
+// is taken by a FULL pass, whose tiles are known beforehand (two or more);
+// while it is armed, other passes take the form that sizes from the counts.
+bool codes_in_pass(const crac_ctx *c, size_t segments, bool host_res, uint64_t n_chunks) {
+    if (!c->crz_hdr_now || host_res || segments != 1) return false;
+    if (fault_armed(CRAC_FAULT_ENCODE_WAIT) && !(c->full_copy_ok && crz_size_tiles(n_chunks) >= 2)) return false;
     for (const AllocRec &r : c->allocs)
         if (r.kind == CRAC_KIND_HOST) return false;
     return true;
@@ -1055,11 +1058,12 @@ crac_status_t checkpoint_wait(crac_ctx *c, crac_image *im, const std::vector<Seg
         CkptCtrl ctrl{};
         CodecParams enc{};
         const uint64_t zmax = sg.bytes + 16 * nseg;
-        const bool in_pass = codes_in_pass(c, segs.size(), host_res) && da.try_alloc(zmax, &pc.dev);
+        const bool in_pass = codes_in_pass(c, segs.size(), host_res, nseg) && da.try_alloc(zmax, &pc.dev);
         if (in_pass) {
             enc.dst = pc.dev.p;
             enc.zoff = (uint64_t *)pc.off_dev.p;
             enc.zlen = (uint64_t *)pc.zlen_dev.p;
+            enc.skip_first_ticket = fault_hit(CRAC_FAULT_ENCODE_WAIT) ? 1u : 0u;   // codes_in_pass: two or more tiles
         }
         st = run_segment(c, sg, (const CkptDesc *)c->desc.p, first, idx_d, off_d, nseg, stg, sg.bytes, out_fp, s,
                          &ctrl, &ms, in_pass ? &enc : nullptr);
