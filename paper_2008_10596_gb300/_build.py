@@ -35,7 +35,7 @@ def _deps_newer(target, sources):
     t = os.path.getmtime(target)
     extra = [os.path.join(INC, "crac.h"), os.path.join(CSRC, "crac_kernels.cuh"),
              os.path.join(CSRC, "crac_device.cuh"), os.path.join(CSRC, "crac_codec.cuh"),
-             os.path.join(CSRC, "crac_runtime.h")]
+             os.path.join(CSRC, "crac_grids.h"), os.path.join(CSRC, "crac_runtime.h")]
     return any(os.path.getmtime(s) > t for s in list(sources) + extra)
 
 

@@ -294,6 +294,15 @@ __device__ __forceinline__ uint32_t find_alloc_warp(const CkptDesc *__restrict__
     return lo;
 }
 
+// The same where c is past the first chunks of allocation a: usually one of the
+// next 32, in one load.
+__device__ __forceinline__ uint32_t find_alloc_near(const CkptDesc *__restrict__ d, uint32_t n, uint32_t a, uint64_t c,
+                                                    int lane) {
+    const uint32_t i = a + lane;
+    const unsigned m = __ballot_sync(kFull, i < n && d[i].first_chunk <= c);   // lane 0 always
+    return m == kFull ? find_alloc_warp(d, n, c, lane) : a + 31u - __clz(m);
+}
+
 __device__ __forceinline__ uint32_t find_scatter(const ScatterDesc *__restrict__ d, uint32_t n,
                                                  uint64_t c) {
     uint32_t lo = 0, hi = n;

@@ -167,13 +167,6 @@ const void *split_gather_fn(bool crz_headers, bool aligned);
 int split_hash_threads();
 int split_finalize_threads();
 int split_gather_threads();
-// log2 of the hash kernel's segment (at most the chunk) for `bytes` tracked
-// bytes; copy: every chunk is also written.  Not for chunks of 512 B - 4 KiB.
-uint32_t split_hash_seg(uint64_t bytes, uint32_t log2_chunk, bool copy);
-// Grid of the hash kernel over n_chunks chunks holding `bytes` bytes (copy: as
-// for split_hash_seg), and CkptParams::slots_per_warp of that grid.
-uint32_t split_hash_grid(uint64_t n_chunks, uint64_t bytes, uint32_t log2_chunk, uint32_t log2_seg, bool copy,
-                         uint32_t *slots_per_warp);
 const void *split_hash_small_dense_fn(int lanes_per_chunk);
 
 cudaError_t launch_fp_range(const CkptDesc *d, uint64_t c0, uint64_t c1, uint32_t log2_chunk,

@@ -2,6 +2,7 @@
 // (A1), the batched pass launched as one CUDA graph (A2-A4), the drain to
 // pinned host memory (A5) and the commit (A6); also the trial pass the
 // autotuner runs.
+#include "crac_grids.h"
 #include "crac_runtime.h"
 
 using namespace crac;
@@ -396,7 +397,7 @@ crac_status_t launch_segment(crac_ctx *c, const Segment &sg, const CkptDesc *des
         // 512 B..4 KiB chunks: several whole chunks per warp iteration.
         const bool small = c->log2S >= 9 && c->log2S < 13;
         const bool copies = staging && !enc && (c->full_copy_ok || c->sparse_ok);   // the hash kernel writes every chunk
-        const uint32_t log2Seg = small ? c->log2S : split_hash_seg(sg.bytes, c->log2S, copies);
+        const uint32_t log2Seg = small ? c->log2S : split_hash_seg(nseg, sg.bytes, c->log2S, copies);
         // Coded contexts with chunks of 8 KiB and more: the kernel that writes a
         // chunk to staging (hash or gather) also writes its CRZ1 block headers
         // for the encoder.
@@ -445,7 +446,7 @@ crac_status_t launch_segment(crac_ctx *c, const Segment &sg, const CkptDesc *des
             P.seg_base = pre + ((sg.c0 - first[a0]) << c->log2S);
         }
         unsigned long long *acc = (unsigned long long *)((uint8_t *)c->work.p + status_bytes);
-        const int gh = (int)split_hash_grid(nseg, sg.bytes, c->log2S, log2Seg, copies, &P.slots_per_warp);
+        const int gh = (int)split_hash_grid(nseg, sg.bytes, c->log2S, log2Seg, copies, c->sm_count, &P.slots_per_warp);
         const int gf = (int)std::min<uint64_t>(n_tiles, (uint64_t)c->sm_count * 2);
         const int gg = c->sm_count * 8;
         const int grids[3] = {gh, gf, gg};
@@ -1649,7 +1650,7 @@ crac_status_t fingerprint_against(crac_ctx *c, const uint64_t *fp_ref, cudaStrea
     CK(launch_prologue(c->vwork.p, (work_bytes + 15) / 16, c->vdesc.p, dh, c->uva ? na * sizeof(CkptDesc) / 16 : 0,
                        c->sm_count, s));
     const bool small = log2S >= 9 && log2S < 13;
-    uint32_t log2Seg = small ? log2S : split_hash_seg(bytes, log2S, false);
+    uint32_t log2Seg = small ? log2S : split_hash_seg(n, bytes, log2S, false);
     const void *hash_fn = small ? split_hash_small_fn(1 << (log2S - 7), true) : split_hash_fn(false, true);
     CkptParams P{};
     P.desc = (const CkptDesc *)c->vdesc.p;
@@ -1669,7 +1670,7 @@ crac_status_t fingerprint_against(crac_ctx *c, const uint64_t *fp_ref, cudaStrea
     P.tile_bytes = P.tile_cnt + n_tiles;
     P.timeout_ns = c->cfg.timeout_ns;
     unsigned long long *acc = (unsigned long long *)((uint8_t *)c->vwork.p + status_bytes);
-    const int gh = (int)split_hash_grid(n, bytes, log2S, log2Seg, false, &P.slots_per_warp);
+    const int gh = (int)split_hash_grid(n, bytes, log2S, log2Seg, false, c->sm_count, &P.slots_per_warp);
     const int gf = (int)std::max<uint64_t>(1, std::min<uint64_t>(n_tiles, (uint64_t)c->sm_count * 2));
     void *args[] = {&P, &acc, &log2Seg};
     CK(launch_chained(hash_fn, gh, split_hash_threads(), args, s));

@@ -1,6 +1,7 @@
 // The split pass (hash -> finalize + compaction -> gather, one graph) and its
 // sparse variant.
 #include "crac_codec.cuh"
+#include "crac_grids.h"
 
 namespace crac {
 
@@ -10,7 +11,7 @@ namespace {
 // Split pass: H (hash) -> F (finalize + dirty test + compaction) -> G (gather).
 //
 // H streams the tracked bytes with no inter-CTA dependency: every warp takes
-// one segment (8 or 16 KiB, or several short chunks), in rounds of eight
+// one segment (8 or 16 KiB, or several short chunks; crac_grids.h), in rounds of eight
 // 128-bit loads per lane, sums the per-word terms, and adds the warp's sum into
 // the chunk's accumulator with one 64-bit atomicAdd.  The CRAC-FP64 sum is
 // taken mod 2^64, so the order of these additions does not change a bit.  The
@@ -27,6 +28,7 @@ namespace {
 // dependency-free streaming phases.
 // ---------------------------------------------------------------------------
 constexpr int kHashNT = 256;
+static_assert(kHashNT / 32 == kHashWarps, "the grid's rule");
 constexpr int kFinNT = 1024;
 constexpr int kGatherNT = 256;
 
@@ -87,7 +89,7 @@ __device__ __forceinline__ void block_headers(const uint4 q[8], uint32_t n, int 
     if (lane < 8 && (uint32_t)lane < n) hdr[lane] = crz_header(mins, maxs);
 }
 
-// Partial CRAC-FP64 sum of a segment (<= 16 KiB) whose first word is word j0
+// Partial CRAC-FP64 sum of a segment (<= 64 KiB) whose first word is word j0
 // of its chunk, over the lanes of one warp.  dest(), asked for once the first
 // loads are on their way, says where the segment's bytes are also stored (null:
 // nowhere); then (kHdr) the CRZ1 header word of each whole 512-byte block of
@@ -197,26 +199,37 @@ split_hash_kernel(const CkptParams P, unsigned long long *__restrict__ acc, uint
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t log2S = P.log2_chunk;
     const uint32_t spc = log2S - log2Seg;   // log2 of segments per chunk
-    // The CTA's segments in turn to its warps, so that it streams through them.
-    const uint64_t per_cta = (uint64_t)kWarps * P.slots_per_warp;
-    const uint64_t q_end = umin64((blockIdx.x + 1) * per_cta, (P.c_end - P.c_begin) << spc);
+    // The CTA's segments in rows of one per warp, so that it streams through them.
+    // Which warp starts a row turns with the chunk (with the row, where a row
+    // holds whole chunks), so that allocations much shorter than a chunk, which
+    // fill only its first segments, keep all warps busy.
+    const uint32_t rsh = spc > 3 ? spc - 3 : 0;   // log2 of rows per chunk
     uint32_t a = 0;
     uint64_t a_next = 0;   // first chunk after allocation a
-    CkptDesc d{};
+    CkptDesc d{0, 1, ~0ull, 0};
     uint32_t writes = 0;   // chunks this warp wrote speculatively
-    for (uint64_t q = blockIdx.x * per_cta + warp; q < q_end; q += kWarps) {
+#pragma unroll 1
+    for (uint32_t r = 0; r < P.slots_per_warp; ++r) {
+        const uint64_t row = (uint64_t)blockIdx.x * P.slots_per_warp + r;
+        const uint64_t q = row * kWarps + ((warp + (uint32_t)(row >> rsh)) & (kWarps - 1));
         const uint64_t c = P.c_begin + (q >> spc);
-        if (c >= a_next) {
-            a = find_alloc_warp(P.desc, P.n_allocs, c, lane);
+        if (c >= P.c_end) break;
+        // past allocation a's chunks (kHdr: without a register for their end)
+        if (kHdr ? c - d.first_chunk > (d.bytes - 1) >> log2S : c >= a_next) {
+            a = r ? find_alloc_near(P.desc, P.n_allocs, a, c, lane) : find_alloc_warp(P.desc, P.n_allocs, c, lane);
             d = P.desc[a];
             a_next = d.first_chunk + ((d.bytes - 1) >> log2S) + 1;
         }
         const uint64_t local = c - d.first_chunk;
         const uint32_t clen = (uint32_t)umin64(d.bytes - (local << log2S), 1ull << log2S);
         const uint32_t off = (uint32_t)(q & ((1ull << spc) - 1)) << log2Seg;
-        if (off >= clen) continue;   // beyond the end of a short last chunk (warp-uniform)
+        if (off >= clen) {   // beyond the end of a short last chunk (warp-uniform): on to the next chunk's rows
+            const uint32_t last = (1u << rsh) - 1;
+            r += last - ((uint32_t)row & last);
+            continue;
+        }
         const uint32_t len = min(1u << log2Seg, clen - off);
-        // Direct mode (S <= 8 KiB, the warp sees the whole chunk): the baseline
+        // Direct mode (the chunk is one segment, so the warp sees all of it): the baseline
         // fingerprint is loaded before the chunk so that both latencies overlap.
         uint64_t fo = 0;
         const bool has = d.base_first != kNoBase && P.fp_old;
@@ -267,8 +280,6 @@ split_hash_kernel(const CkptParams P, unsigned long long *__restrict__ acc, uint
 // Every chunk is finalized in place (direct mode: acc receives the dirty
 // length, and finalize only compacts).
 constexpr int kSmallVecs = 8;     // vectors per lane of one iteration
-constexpr uint64_t kSmallIters = 2;        // iterations per warp,
-constexpr uint64_t kSmallItersRead = 16;   // ... at most, where the pass mostly reads
 
 template <int LPC, bool kAny>
 __device__ __forceinline__ void hash_small_iter(const CkptParams &P, unsigned long long *__restrict__ acc,
@@ -816,35 +827,6 @@ const void *split_hash_small_dense_fn(int lanes_per_chunk) {
     case 32: return reinterpret_cast<const void *>(&split_hash_small_dense_kernel<32>);
     default: return nullptr;
     }
-}
-// Bytes of a segment: 8 KiB; 16 KiB where the pass mostly reads and is large
-// enough that every SM still gets dozens of CTAs (4 GiB, read only: 623 -> 600
-// us), not where it writes every chunk (1211 -> 1234 us).
-uint32_t split_hash_seg(uint64_t bytes, uint32_t log2S, bool copy) {
-    const uint32_t m = copy || (bytes >> 14) < 32768 ? 13 : 14;
-    return log2S < m ? log2S : m;
-}
-
-// A warp takes one segment, or as many as hold a segment's bytes on average
-// (chunks below 512 B; allocations mostly much shorter than a chunk, whose
-// segments past their end are empty).
-uint32_t split_hash_grid(uint64_t n_chunks, uint64_t bytes, uint32_t log2S, uint32_t log2Seg, bool copy,
-                         uint32_t *slots_per_warp) {
-    constexpr uint64_t kWarps = kHashNT / 32;
-    uint64_t per, n = n_chunks;   // items per warp, items
-    if (log2S >= 9 && log2S < 13) {   // iterations of 4 KiB
-        n = (n << log2S) / 4096 + 1;
-        per = copy ? kSmallIters : n >> 15;
-        per = per < kSmallIters ? kSmallIters : umin64(per, kSmallItersRead);
-    } else {                          // segments
-        n <<= log2S - log2Seg;
-        const uint32_t m = log2Seg < 13 ? 13 : log2Seg;
-        per = n / ((bytes >> m) + 1);
-        per = per < 1 ? 1 : umin64(per, 1u << 20);
-    }
-    *slots_per_warp = (uint32_t)per;
-    const uint64_t g = (n + per * kWarps - 1) / (per * kWarps);
-    return (uint32_t)(g < 1 ? 1 : umin64(g, 0x7fffffffull));
 }
 
 }  // namespace crac
