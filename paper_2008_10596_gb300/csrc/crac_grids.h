@@ -51,4 +51,49 @@ inline uint32_t split_hash_grid(uint64_t n_chunks, uint64_t bytes, uint32_t log2
     return (uint32_t)(g < 1 ? 1 : g < 0x7fffffffull ? g : 0x7fffffffull);
 }
 
+// How a restore's scatter is cut: parts of 1 << log2_part bytes of the target's
+// chunks (a short chunk whole), and the grid that takes them.
+//   A plain chunk is cut into parts of 8 KiB, and a warp takes about 8 KiB of
+// short chunks.  Coded chunks are cut into parts of 32 KiB, and at most
+// sixteen, as every part checks the whole stream's headers (also in host
+// images, where the parts share them in L2: 16 MiB of bf16 in chunks of
+// 1 MiB 992 -> 107 us against a warp per chunk).  Where a chunk holds less than
+// 8 KiB on average (allocations much shorter than a chunk), both are up to 64 KiB.
+//   Parts past an allocation's end cost a look-up, a chain of dependent loads, and
+// no more, so where they are many a warp takes as many parts as hold a part's
+// bytes on average and looks up 32 at a time (at least 32 warps per SM; coded:
+// `lanes`, where most parts are empty or chunks short).  Whole restores, device
+// time: 1200 allocations of 64 bytes in 16 MiB chunks 775 us with a warp per part
+// of 8 KiB, 25 so; 20000 below 4 KiB in 1 MiB chunks 1205 and 74; 64 of 8 MiB and
+// 20000 below 512 B in 64 KiB chunks 371 and 242.
+//   An odd grid, where chunks have more parts than a CTA warps, so that the parts
+// with bytes, the first of a chunk, fall to all CTAs.
+struct RestoreCut {
+    uint32_t log2_part, ctas;
+    bool lanes;
+};
+inline RestoreCut restore_cut(uint64_t n_chunks, uint64_t bytes, uint32_t log2_chunk, bool coded, int sm_count,
+                              uint64_t max_ctas) {
+    const uint32_t l = log2_chunk, few = (bytes >> 13) < n_chunks ? 16 : coded ? 15 : 13;
+    uint32_t part = l < few ? l : few;
+    if (coded && part + 4 < l) part = l - 4;
+    const uint64_t items = n_chunks << (l - part), least = 32ull * (uint64_t)sm_count;
+    const bool lanes = coded && (l < 13 || items > 2 * ((bytes >> part) + 1));
+    uint64_t warps = items;
+    if (l < 13) {
+        const uint64_t some = n_chunks < least ? n_chunks : least;
+        warps = ((n_chunks - 1) >> (13 - (l < 8 ? 8 : l))) + 1;
+        warps = warps > some ? warps : some;
+    } else if (!coded || lanes) {
+        const uint64_t full = (bytes >> part) + (n_chunks >> 3);
+        warps = full > least ? full : least;
+        warps = warps < items ? warps : items;
+    }
+    uint64_t ctas = (warps + 7) / 8;
+    ctas = ctas < max_ctas ? ctas : max_ctas;
+    ctas = ctas < 0x7fffffffull ? ctas : 0x7fffffffull;
+    if (ctas * 8 < items && l - part > 3 && ctas > 1 && ctas % 2 == 0) --ctas;
+    return {part, (uint32_t)ctas, lanes};
+}
+
 }  // namespace crac

@@ -243,7 +243,8 @@ struct RestoreParams {
 // chunk from its owner (the scatter's grid follows the work, up to max_grid).
 cudaError_t launch_restore_mark(const RestoreParams &p, int grid, cudaStream_t s);
 cudaError_t launch_restore_check(const RestoreParams &p, int grid, cudaStream_t s);
-cudaError_t launch_restore_scatter(const RestoreParams &p, uint64_t max_grid, cudaStream_t s);
+cudaError_t launch_restore_scatter(const RestoreParams &p, uint64_t bytes, int sm_count, uint64_t max_grid,
+                                   cudaStream_t s);
 // Incremental restore, between check and scatter: clears the owner of every
 // chunk whose current fingerprint equals the target's, so it is not written.
 cudaError_t launch_restore_unmark(const RestoreParams &p, int grid, cudaStream_t s);

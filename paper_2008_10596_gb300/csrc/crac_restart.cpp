@@ -214,7 +214,7 @@ crac_status_t restart_device(crac_ctx *c, crac_image *img, const std::vector<cra
     if (incremental)
         CK(launch_restore_unmark(P, (int)std::max<uint64_t>(1, std::min<uint64_t>((nt + 255) / 256, grid)), s));
     P.host = any_host ? 1u : 0u;
-    CK(launch_restore_scatter(P, any_host || incremental ? grid : UINT64_MAX, s));
+    CK(launch_restore_scatter(P, ri.restored_bytes, c->sm_count, any_host || incremental ? grid : UINT64_MAX, s));
     CK(cudaEventRecord(c->ev_r1, s));
     if (incremental) CK(launch_report(vctrl, sizeof(CkptCtrl) / 8, nullptr, c->ctrl_h.p, s));
     CK(launch_report(nullptr, 0, P.err, c->serr_h.p, s));

@@ -1,6 +1,7 @@
 // Restart kernels: owner marks, coverage check and scatter over every piece of
 // a chain (device path), and the windowed scatter of the staged path.
 #include "crac_codec.cuh"
+#include "crac_grids.h"
 
 namespace crac {
 
@@ -11,6 +12,7 @@ namespace {
 // so that each target chunk is written once, by the newest image holding it.
 // ---------------------------------------------------------------------------
 constexpr int kScatterNT = 256;
+constexpr uint32_t kScatterWarps = kScatterNT / 32;
 
 __global__ void __launch_bounds__(kScatterNT, 4) scatter_kernel(const ScatterParams P) {
     constexpr int GT = 32;
@@ -106,7 +108,10 @@ __global__ void __launch_bounds__(256) restore_unmark_kernel(const RestoreParams
 // slowest (4 GiB in 64 KiB chunks: 1.32 ms in one wave of 5 CTAs per SM, 1.22 ms
 // with a CTA for every 64 KiB).  With a smaller grid (host images, whose link
 // one CTA per SM already paces; incremental restores, where most items are
-// skipped) a warp strides over the items, 32 at a time, a lane looking up each.
+// skipped; allocations much shorter than a chunk) a warp strides over the items,
+// 32 at a time, a lane looking up each, and its place in the CTA turns with each
+// step, so that the first parts of chunks, at times the only ones, keep all warps
+// busy.
 struct RestoreItem {
     uint64_t dst, src;   // raw: the item's bytes; coded: the whole chunk, its stream
     uint32_t len;        // bytes to write (0: nothing)
@@ -146,6 +151,11 @@ __device__ __forceinline__ RestoreItem restore_item(const RestoreParams &P, uint
     return r;
 }
 
+// A warp's item in step j of nw warps.
+__device__ __forceinline__ uint64_t restore_step(uint64_t j, uint64_t nw, int warp) {
+    return j * nw + (uint64_t)blockIdx.x * kScatterWarps + ((warp + (uint32_t)j) & (kScatterWarps - 1));
+}
+
 // kAligned: every allocation's size is a multiple of 16 bytes.
 template <bool kAligned>
 __device__ __forceinline__ void restore_scatter_body(const RestoreParams &P) {
@@ -153,10 +163,11 @@ __device__ __forceinline__ void restore_scatter_body(const RestoreParams &P) {
     if (*(volatile unsigned int *)P.err) return;   // uncovered or out of range: memory untouched
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint64_t n_items = P.n_owner << (P.log2_chunk - P.log2_part);
-    const uint64_t nw = (uint64_t)gridDim.x * (kScatterNT / 32);
-    for (uint64_t i0 = (uint64_t)blockIdx.x * (kScatterNT / 32) + warp; i0 < n_items; i0 += 32 * nw) {
+    const uint64_t nw = (uint64_t)gridDim.x * kScatterWarps;
+    for (uint64_t j = lane; (j - lane) * nw < n_items; j += 32) {   // warp-uniform
         RestoreItem r{};
-        if (i0 + lane * nw < n_items) r = restore_item<false>(P, i0 + lane * nw);
+        const uint64_t it = restore_step(j, nw, warp);
+        if (it < n_items) r = restore_item<false>(P, it);
         unsigned todo = __ballot_sync(kFull, r.len != 0);
         while (todo) {   // warp-uniform
             const int i = __ffs(todo) - 1;
@@ -177,30 +188,45 @@ __global__ void __launch_bounds__(kScatterNT, 4) restore_scatter_ragged_kernel(c
 }
 
 // Chains with a coded image: the decoder needs registers that the plain copy
-// does not (hence a kernel of its own), and an item, of 16 KiB or more, is
-// looked up by the whole warp: its decoding takes far longer than the look-up.
-template <bool kHost>
+// does not (hence kernels of their own).  An item of 16 KiB or more is looked up
+// by the whole warp, its decoding takes far longer; kLanes: short chunks, or mostly
+// empty items, 32 at a time, a lane each.
+template <bool kHost, bool kLanes>
 __global__ void __launch_bounds__(kScatterNT, 3) restore_scatter_coded_kernel(const RestoreParams P) {
     extern __shared__ __align__(16) uint8_t scratch[];   // kCrzDecodeScratch per warp
     wait_for_producer();
     if (*(volatile unsigned int *)P.err) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t parts = P.log2_chunk - P.log2_part;
-    const uint64_t n_items = P.n_owner << parts;
-    const uint64_t nw = (uint64_t)gridDim.x * (kScatterNT / 32);
-    for (uint64_t it = (uint64_t)blockIdx.x * (kScatterNT / 32) + warp; it < n_items; it += nw) {
-        const RestoreItem r = restore_item<true>(P, it);
-        if (r.len == 0) continue;
-        uint8_t *dst = reinterpret_cast<uint8_t *>(r.dst);
-        const uint8_t *src = reinterpret_cast<const uint8_t *>(r.src);
-        if (!r.z) {
-            copy_group<32>(dst, src, r.len, lane);
-            continue;
+    const uint64_t n_items = P.n_owner << (P.log2_chunk - P.log2_part);
+    const uint64_t nw = (uint64_t)gridDim.x * kScatterWarps;
+    for (uint64_t j = kLanes ? lane : 0; (kLanes ? j - lane : j) * nw < n_items; j += kLanes ? 32 : 1) {   // warp-uniform
+        RestoreItem mine{};
+        const uint64_t it = restore_step(j, nw, warp);
+        if (it < n_items) mine = restore_item<true>(P, it);
+        unsigned todo = kLanes ? __ballot_sync(kFull, mine.len != 0) : mine.len != 0;
+        while (todo) {   // warp-uniform
+            RestoreItem r = mine;
+            if (kLanes) {
+                const int i = __ffs(todo) - 1;
+                r.dst = __shfl_sync(kFull, mine.dst, i);
+                r.src = __shfl_sync(kFull, mine.src, i);
+                r.len = __shfl_sync(kFull, mine.len, i);
+                r.z = __shfl_sync(kFull, mine.z, i);
+                r.po = __shfl_sync(kFull, mine.po, i);
+                r.clen = __shfl_sync(kFull, mine.clen, i);
+            }
+            todo &= todo - 1;
+            uint8_t *dst = reinterpret_cast<uint8_t *>(r.dst);
+            const uint8_t *src = reinterpret_cast<const uint8_t *>(r.src);
+            if (!r.z) {
+                copy_group<32>(dst, src, r.len, lane);
+                continue;
+            }
+            const uint32_t b0 = r.po >> 9, b1 = (r.po + (1u << P.log2_part)) >> 9;   // the item's blocks of its chunk
+            if (!crz_decode_warp<kHost>(dst, src, r.clen, r.z, b0, b1, lane, scratch + kCrzDecodeScratch * warp) &&
+                lane == 0)
+                atomicOr(P.err, kErrCodec);
         }
-        const uint32_t b0 = r.po >> 9, b1 = (r.po + (1u << P.log2_part)) >> 9;   // the item's blocks of its chunk
-        if (!crz_decode_warp<kHost>(dst, src, r.clen, r.z, b0, b1, lane, scratch + kCrzDecodeScratch * warp) &&
-            lane == 0)
-            atomicOr(P.err, kErrCodec);
     }
 }
 
@@ -227,28 +253,23 @@ cudaError_t launch_restore_unmark(const RestoreParams &p, int grid, cudaStream_t
     return p.n_owner ? chain(restore_unmark_kernel, p, grid, 256, s) : cudaSuccess;
 }
 
-cudaError_t launch_restore_scatter(const RestoreParams &p, uint64_t max_grid, cudaStream_t s) {
+cudaError_t launch_restore_scatter(const RestoreParams &p, uint64_t bytes, int sm_count, uint64_t max_grid,
+                                   cudaStream_t s) {
     if (p.n_entries == 0 || p.n_owner == 0) return cudaSuccess;
-    constexpr uint64_t kWarps = kScatterNT / 32;
     RestoreParams q = p;
-    // A plain chunk is cut into parts of 8 KiB, and a warp takes about 8 KiB of
-    // short chunks.  Coded chunks are cut into parts of 32 KiB, and at most
-    // sixteen, as every part checks the whole stream's headers (also in host
-    // images, where the parts share them in L2: 16 MiB of bf16 in chunks of
-    // 1 MiB 992 -> 107 us against a warp per chunk).
-    if (p.coded) q.log2_part = p.log2_chunk < 15 ? p.log2_chunk : p.log2_chunk > 19 ? p.log2_chunk - 4 : 15;
-    else q.log2_part = p.log2_chunk < 13 ? p.log2_chunk : 13;
-    uint64_t warps = p.n_owner << (p.log2_chunk - q.log2_part);
-    if (p.log2_chunk < 13) warps = ((warps - 1) >> (13 - (p.log2_chunk < 8 ? 8 : p.log2_chunk))) + 1;
-    const uint64_t ctas = umin64((warps + kWarps - 1) / kWarps, umin64(max_grid, 0x7fffffffull));
+    const RestoreCut cut = restore_cut(p.n_owner, bytes, p.log2_chunk, p.coded != 0, sm_count, max_grid);
+    q.log2_part = cut.log2_part;
     if (p.coded) {
-        constexpr int kSmem = kCrzDecodeScratch * (int)kWarps;
+        static const void *const kFns[2][2] = {
+            {reinterpret_cast<const void *>(&restore_scatter_coded_kernel<false, false>),
+             reinterpret_cast<const void *>(&restore_scatter_coded_kernel<false, true>)},
+            {reinterpret_cast<const void *>(&restore_scatter_coded_kernel<true, false>),
+             reinterpret_cast<const void *>(&restore_scatter_coded_kernel<true, true>)}};
         void *args[] = {&q};
-        const void *fn = p.host ? reinterpret_cast<const void *>(&restore_scatter_coded_kernel<true>)
-                                : reinterpret_cast<const void *>(&restore_scatter_coded_kernel<false>);
-        return launch_chained(fn, (uint32_t)ctas, kScatterNT, args, s, kSmem);
+        return launch_chained(kFns[p.host ? 1 : 0][cut.lanes ? 1 : 0], cut.ctas, kScatterNT, args, s,
+                              kCrzDecodeScratch * kScatterWarps);
     }
-    return chain(p.ragged ? restore_scatter_ragged_kernel : restore_scatter_kernel, q, ctas, kScatterNT, s);
+    return chain(p.ragged ? restore_scatter_ragged_kernel : restore_scatter_kernel, q, cut.ctas, kScatterNT, s);
 }
 
 cudaError_t launch_scatter(const ScatterParams &p, int grid, cudaStream_t s) {

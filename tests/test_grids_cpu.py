@@ -19,6 +19,12 @@ uint32_t hash_seg(uint64_t n, uint64_t b, uint32_t l, int copy) { return split_h
 uint32_t hash_grid(uint64_t n, uint64_t b, uint32_t l, uint32_t s, int copy, int sm, uint32_t *per) {
     return split_hash_grid(n, b, l, s, copy, sm, per);
 }
+uint32_t restore_plan(uint64_t n, uint64_t b, uint32_t l, int coded, int sm, uint64_t most, uint32_t *out) {
+    const RestoreCut c = restore_cut(n, b, l, coded, sm, most);
+    out[0] = c.log2_part;
+    out[1] = c.lanes;
+    return c.ctas;
+}
 }
 """
 
@@ -34,6 +40,7 @@ def rules(tmp_path_factory):
     u64, u32 = ctypes.c_uint64, ctypes.c_uint32
     so.hash_seg.argtypes = [u64, u64, u32, ctypes.c_int]
     so.hash_grid.argtypes = [u64, u64, u32, u32, ctypes.c_int, ctypes.c_int, ctypes.POINTER(u32)]
+    so.restore_plan.argtypes = [u64, u64, u32, ctypes.c_int, ctypes.c_int, u64, ctypes.POINTER(u32)]
     return so
 
 
@@ -98,3 +105,47 @@ def test_the_hash_walk_takes_every_segment_once(rules, seed):
             seen = visit(len(lens), lens, log2S, seg, grid, per)
             assert set(seen.values()) <= {1}
             assert set(seen) == {(c, o) for c, ln in enumerate(lens) for o in range(0, ln, 1 << seg)}
+
+
+def restore_plan(so, n, nbytes, log2S, coded, sm=SM, most=(1 << 64) - 1):
+    out = (ctypes.c_uint32 * 2)()
+    return so.restore_plan(n, nbytes, log2S, coded, sm, most, out), out[0], bool(out[1])
+
+
+@pytest.mark.parametrize("log2S", range(13, 25))
+def test_restore_of_full_chunks_a_warp_a_part(rules, log2S):
+    n = (4 << 30) >> log2S
+    ctas, part, _ = restore_plan(rules, n, 4 << 30, log2S, 0)
+    assert part == 13 and ctas == (n << (log2S - 13)) // 8
+    ctas, part, lanes = restore_plan(rules, n, 4 << 30, log2S, 1)
+    assert part == max(min(15, log2S), log2S - 4) and ctas == ((n << (log2S - part)) + 7) // 8 and not lanes
+
+
+@pytest.mark.parametrize("coded", [0, 1])
+@pytest.mark.parametrize("log2S", [6, 9, 12, 13, 16, 18, 20, 24])
+@pytest.mark.parametrize("n,each", [(1200, 5), (1200, 64), (1200, 4096), (20000, 2000), (50000, 200)])
+def test_restore_of_short_allocations(rules, n, each, log2S, coded):
+    """Work for every SM, and no more than a look-up of 32 parts at a time per warp."""
+    each = min(each, 1 << log2S)
+    ctas, part, lanes = restore_plan(rules, n, n * each, log2S, coded)
+    items = n << (log2S - part)
+    assert ctas >= min(4 * SM, items // 8) - 1
+    assert ctas <= max(4 * SM, (n * each >> 13) + n // 8 + 1)
+    assert not coded or lanes or items <= 2 * ((n * each >> part) + 1)
+
+
+@pytest.mark.parametrize("seed", range(60))
+def test_the_restore_walk_takes_every_part_once(rules, seed):
+    rng = random.Random(seed)
+    log2S, sm = rng.choice([4, 9, 13, 16, 18, 20, 24]), rng.choice([1, 3, 16])
+    n, coded = rng.randrange(1, 400), rng.randrange(2)
+    nbytes = rng.randrange(n, (n << log2S) + 1)
+    ctas, part, lanes = restore_plan(rules, n, nbytes, log2S, coded, sm, rng.choice([1, 2, 5, 1 << 40]))
+    items, nw = n << (log2S - part), 8 * ctas
+    seen = [0] * items
+    for j in range((items + nw - 1) // nw):
+        for w in range(nw):
+            it = j * nw + w // 8 * 8 + ((w % 8 + j) & 7)
+            if it < items:
+                seen[it] += 1
+    assert set(seen) == {1}
