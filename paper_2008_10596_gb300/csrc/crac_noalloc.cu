@@ -29,39 +29,45 @@ int g_noalloc_sms[kNoAllocMaxDevices];
 constexpr int kPrepareNT = 1024;
 
 // Before the pass: zeroed scratch and accumulators (na and nb words), and, where
-// there is no baseline (prefix), the payload bytes before each region and the
-// flag that the hash kernel may write every chunk there as it reads it (there
-// is room for them all), by CTA 0.
+// there is no baseline (prefix), the payload bytes before each region, and by the
+// CTA of the last ones the flag that the hash kernel may write every chunk there as
+// it reads it (there is room for them all).  A CTA takes 1024 regions, a thread
+// each, and sums up those before them itself: bound by one SM's reads of the table
+// (75669 chunks of 256 bytes in 50000 regions, the whole pass: 170 us, 79 of them
+// here, with one CTA and a run of regions per thread; 122 with one CTA and
+// neighbouring regions on neighbouring lanes; 103 this way).
 __global__ void __launch_bounds__(kPrepareNT)
 noalloc_prepare_kernel(uint64_t *__restrict__ zero_a, uint32_t na, uint64_t *__restrict__ zero_b, uint32_t nb,
                        const crac::CkptDesc *__restrict__ d, uint32_t n, uint64_t cap, uint64_t *__restrict__ prefix,
                        uint32_t *__restrict__ flag) {
     using namespace crac;
-    __shared__ uint64_t s_sum[kPrepareNT / 32];
+    __shared__ uint64_t s_before[kPrepareNT / 32], s_sum[kPrepareNT / 32];
     for (uint32_t i = blockIdx.x * kPrepareNT + threadIdx.x; i < na + nb; i += gridDim.x * kPrepareNT) {
         if (i < na) zero_a[i] = 0;
         else zero_b[i - na] = 0;
     }
-    if (blockIdx.x || !prefix) return;
+    const uint32_t i0 = blockIdx.x * kPrepareNT, i = i0 + threadIdx.x;
+    if (!prefix || i0 >= n) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t per = (n + kPrepareNT - 1) / kPrepareNT;
-    const uint32_t i0 = min(n, threadIdx.x * per), i1 = min(n, i0 + per);
+    const uint64_t mine = i < n ? d[i].bytes : 0;
     uint64_t sum = 0;
-    for (uint32_t i = i0; i < i1; ++i) sum += d[i].bytes;
-    const uint64_t incl = warp_incl_scan(sum, lane);
-    if (lane == 31) s_sum[warp] = incl;
+#pragma unroll 8
+    for (uint32_t j = threadIdx.x; j < i0; j += kPrepareNT) sum += d[j].bytes;
+    sum = warp_sum(sum);
+    const uint64_t incl = warp_incl_scan(mine, lane);
+    if (lane == 31) {
+        s_before[warp] = sum;
+        s_sum[warp] = incl;
+    }
     __syncthreads();
-    uint64_t before = 0, total = 0;
+    uint64_t at = 0, total = 0;
     for (int w = 0; w < kPrepareNT / 32; ++w) {
-        if (w < warp) before += s_sum[w];
-        total += s_sum[w];
+        if (w < warp) at += s_sum[w];
+        at += s_before[w];
+        total += s_before[w] + s_sum[w];
     }
-    uint64_t at = before + incl - sum;
-    for (uint32_t i = i0; i < i1; ++i) {
-        prefix[i] = at;
-        at += d[i].bytes;
-    }
-    if (threadIdx.x == 0) *flag = total <= cap ? 1u : 0u;
+    if (i < n) prefix[i] = at + incl - mine;
+    if (threadIdx.x == 0 && n - i0 <= kPrepareNT) *flag = total <= cap ? 1u : 0u;
 }
 
 // The pass's results (a crac_pass_totals_t at any address) from its control
@@ -235,8 +241,9 @@ extern "C" crac_status_t crac_pass_noalloc(const crac_region_t *regions_dev, uin
         // Segmented chunks are summed up in the caller's table, in place.
         unsigned long long *acc = !fused && log2Seg < l ? reinterpret_cast<unsigned long long *>(fp_new_dev) : nullptr;
         const uint32_t sms = (uint32_t)g_noalloc_sms[dev], na = (uint32_t)(used / 8), nb = acc ? (uint32_t)n_chunks : 0u;
-        const uint32_t want = (na + nb + kPrepareNT - 1) / kPrepareNT;
-        noalloc_prepare_kernel<<<want < sms ? want : sms, kPrepareNT, 0, s>>>(
+        const uint32_t want = (na + nb + kPrepareNT - 1) / kPrepareNT, sums = prefix ? (n_regions - 1) / kPrepareNT + 1 : 1;
+        const uint32_t ctas = want < sms ? want : sms;
+        noalloc_prepare_kernel<<<ctas > sums ? ctas : sums, kPrepareNT, 0, s>>>(
             reinterpret_cast<uint64_t *>(sc), na, fp_new_dev, nb, P.desc, n_regions, P.staging_cap, prefix,
             prefix ? reinterpret_cast<uint32_t *>(prefix + n_regions) : nullptr);
         e = cudaGetLastError();
