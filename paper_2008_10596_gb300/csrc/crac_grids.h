@@ -51,6 +51,21 @@ inline uint32_t split_hash_grid(uint64_t n_chunks, uint64_t bytes, uint32_t log2
     return (uint32_t)(g < 1 ? 1 : g < 0x7fffffffull ? g : 0x7fffffffull);
 }
 
+// Whether the dense placement takes its room once per CTA instead of once per warp
+// and 4 KiB.  With a fraction f of the chunks dirty at random, 4 KiB of n chunks hold
+// a dirty one with probability p = 1 - (1 - f)^n, and the one counter takes about
+// 400 million additions a second once they queue up: from some p on they set the
+// pace, while the CTA's two barriers cost about 10%.  2 GiB, a delta's device time,
+// per warp and per CTA: 512 B chunks 5% dirty (p = 0.34) 619 and 474 us, 10% 841 and
+// 490, 20% 1024 and 511; 1 KiB 10% (0.34) 399 and 441, 20% 858 and 461; 2 KiB 20%
+// (0.36) 404 - 624 and 429.  4 KiB chunks, whose passes are the shortest, from
+// p = 0.22 (24%: 398 - 470 and 430).
+inline bool dense_by_cta(float f, uint32_t log2_chunk) {
+    float clean = 1.f;
+    for (uint32_t i = 0; i < (4096u >> log2_chunk); ++i) clean *= 1.f - f;
+    return clean < (log2_chunk < 12 ? 0.70f : 0.78f);
+}
+
 // How a restore's scatter is cut: parts of 1 << log2_part bytes of the target's
 // chunks (a short chunk whole), and the grid that takes them.
 //   A plain chunk is cut into parts of 8 KiB, and a warp takes about 8 KiB of

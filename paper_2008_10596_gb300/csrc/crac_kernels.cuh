@@ -167,7 +167,8 @@ const void *split_gather_fn(bool crz_headers, bool aligned);
 int split_hash_threads();
 int split_finalize_threads();
 int split_gather_threads();
-const void *split_hash_small_dense_fn(int lanes_per_chunk);
+// by_cta: the dirty chunks' room is taken once per CTA, not once per warp and 4 KiB.
+const void *split_hash_small_dense_fn(int lanes_per_chunk, bool by_cta);
 
 cudaError_t launch_fp_range(const CkptDesc *d, uint64_t c0, uint64_t c1, uint32_t log2_chunk,
                             const uint64_t *fp_old, uint64_t *fp_new, uint32_t *lens,

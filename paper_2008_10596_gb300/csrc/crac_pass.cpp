@@ -405,7 +405,7 @@ crac_status_t launch_segment(crac_ctx *c, const Segment &sg, const CkptDesc *des
         // The sparse pass on 512 B - 4 KiB chunks may place the dirty chunks
         // densely.
         const bool dense = small && c->sparse_ok && staging && c->dense_now;
-        const void *hash_fn = dense ? split_hash_small_dense_fn(1 << (c->log2S - 7))
+        const void *hash_fn = dense ? split_hash_small_dense_fn(1 << (c->log2S - 7), c->dense_cta)
                               : small ? split_hash_small_fn(1 << (c->log2S - 7), c->all16)
                                       : split_hash_fn(crz_hdr != nullptr, c->all16);
         CkptParams P{};
@@ -1389,10 +1389,11 @@ crac_status_t ctx_checkpoint(crac_ctx *c, cudaStream_t s, crac_image_t **out) {
         c->pass_now = resolve_pass_kernel(c, dev_res, all16);
         c->sparse_ok = c->pass_now == CRAC_PASS_SPARSE && dev_res && all16 &&
                        c->cfg.launch_mode == CRAC_LAUNCH_BATCHED;
-        // Dense placement takes one atomic on a single counter per warp
-        // iteration with dirty chunks, whose rate bounds it once many chunks
-        // are dirty: only after a delta that found under a quarter dirty.
+        // Dense placement takes its room from a single counter, whose rate bounds
+        // it once many chunks are dirty: only after a delta that found under a
+        // quarter dirty.
         c->dense_now = c->sparse_ok && any_base && c->delta_frac_valid && c->delta_frac < 0.25f;
+        c->dense_cta = c->dense_now && dense_by_cta(c->delta_frac, c->log2S);
         // Order after the previous operation of this context (drain / restore).
         if (cudaStreamWaitEvent(s, c->ev_last, 0) != cudaSuccess) return fail(cuda_status(cudaGetLastError()));
         c->desc_src = dh;   // copied by the pass
@@ -1579,7 +1580,8 @@ crac_status_t ctx_trial_pass(crac_ctx *c, cudaStream_t s, bool commit, float *ms
     c->pass_now = c->cfg.pass_kernel == CRAC_PASS_AUTO ? (uint32_t)CRAC_PASS_SPLIT : c->cfg.pass_kernel;
     c->sparse_ok = c->pass_now == CRAC_PASS_SPARSE && c->cfg.image_residency == CRAC_RESIDENCY_DEVICE &&
                    all16 && c->cfg.launch_mode == CRAC_LAUNCH_BATCHED;
-    c->dense_now = c->sparse_ok && any_base && c->dense_hint;
+    c->dense_now = c->sparse_ok && any_base && c->dense_hint >= 0.f;
+    c->dense_cta = c->dense_now && dense_by_cta(c->dense_hint, c->log2S);
     CK(cudaStreamWaitEvent(s, c->ev_last, 0));
     c->desc_src = dh;
     c->fp_copy_dst = nullptr;

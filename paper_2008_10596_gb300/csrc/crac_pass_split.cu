@@ -436,14 +436,15 @@ split_hash_small_kernel(const CkptParams P, unsigned long long *__restrict__ acc
 // leaders record each chunk's offset in its accumulator word.  Sizes are
 // multiples of 16 (a sparse pass requires it), so every offset is 16-byte
 // aligned.  8 GiB in 4 KiB chunks, 10% dirty: 1400 -> 1330 us against a form
-// that staged the dirty chunks in shared memory in one wave of resident CTAs;
-// one atomic per CTA, with two barriers for it, took 1505.
+// that staged the dirty chunks in shared memory in one wave of resident CTAs.
+// kCta: one atomicAdd for the CTA's eight warps, with two barriers for it, where
+// a warp's 4 KiB likely hold a dirty chunk (dense_by_cta).
 // ---------------------------------------------------------------------------
 constexpr uint64_t kAccLenMask = (1ull << 24) - 1;   // accumulator word: length in bits 0-23,
 constexpr int kAccPosShift = 24;                     // the chunk's offset in bits 24-62 (dense
 constexpr uint64_t kAccPosMask = (1ull << 39) - 1;   // sparse placement), kAccDirty in bit 63
 
-template <int LPC>
+template <int LPC, bool kCta>
 __global__ void __launch_bounds__(kHashNT, 4)
 split_hash_small_dense_kernel(const CkptParams P, unsigned long long *__restrict__ acc, uint32_t) {
     constexpr int CPS = 32 / LPC;   // chunks per iteration
@@ -452,14 +453,18 @@ split_hash_small_dense_kernel(const CkptParams P, unsigned long long *__restrict
     const int li = lane % LPC;
     const uint32_t log2S = P.log2_chunk;
     const uint64_t warp_g = ((uint64_t)blockIdx.x * kHashNT + threadIdx.x) >> 5;
+    __shared__ uint32_t s_total[2][kHashNT / 32];   // kCta: by turns
+    __shared__ uint64_t s_base[2];
     uint32_t a = 0;
     uint64_t a_next = 0;
     CkptDesc dw{};
 #pragma unroll 1
     for (uint32_t it = 0; it < P.slots_per_warp; ++it) {
         const uint64_t c0 = P.c_begin + (warp_g * P.slots_per_warp + it) * CPS;
-        if (c0 >= P.c_end) break;   // warp-uniform
-        if (c0 >= a_next) {
+        // kCta: all warps stay as long as the first, whose chunks come first, has any
+        const uint64_t c_go = kCta ? c0 - (uint64_t)(threadIdx.x >> 5) * P.slots_per_warp * CPS : c0;
+        if (c_go >= P.c_end) break;   // uniform over the warp (kCta: the CTA)
+        if (c0 >= a_next && (!kCta || c0 < P.c_end)) {
             a = find_alloc_warp(P.desc, P.n_allocs, c0, lane);
             dw = P.desc[a];
             a_next = dw.first_chunk + ((dw.bytes - 1) >> log2S) + 1;
@@ -501,7 +506,7 @@ split_hash_small_dense_kernel(const CkptParams P, unsigned long long *__restrict
             P.fp_new[c] = fp;
             if (!dirty) acc[c - P.c_begin] = len;
         }
-        if (!__any_sync(kFull, dirty)) continue;
+        if (!kCta && !__any_sync(kFull, dirty)) continue;
         const uint32_t mine = (li == 0 && dirty) ? len : 0u;
         uint32_t incl = mine;
         if (LPC < 32) {
@@ -514,8 +519,24 @@ split_hash_small_dense_kernel(const CkptParams P, unsigned long long *__restrict
         const uint32_t total = __shfl_sync(kFull, incl, 32 - LPC);   // the last leader
         const uint32_t loc = __shfl_sync(kFull, incl - mine, lane - li);
         uint64_t base = 0;
-        if (lane == 0) base = atomicAdd(&P.ctrl->pad[0], (unsigned long long)total);
-        base = __shfl_sync(kFull, base, 0);
+        if (kCta) {
+            const int warp = threadIdx.x >> 5, turn = it & 1;
+            if (lane == 0) s_total[turn][warp] = total;
+            __syncthreads();
+            uint32_t before = 0, all = 0;
+#pragma unroll
+            for (int w = 0; w < kHashNT / 32; ++w) {
+                const uint32_t t = s_total[turn][w];
+                if (w < warp) before += t;
+                all += t;
+            }
+            if (threadIdx.x == 0 && all) s_base[turn] = atomicAdd(&P.ctrl->pad[0], (unsigned long long)all);
+            __syncthreads();
+            base = all ? s_base[turn] + before : 0;
+        } else {
+            if (lane == 0) base = atomicAdd(&P.ctrl->pad[0], (unsigned long long)total);
+            base = __shfl_sync(kFull, base, 0);
+        }
         const bool fits = base + total <= P.staging_cap;
         if (!fits && lane == 0) atomicOr(&P.ctrl->err, kErrBounds);
         if (dirty) {
@@ -819,14 +840,18 @@ const void *split_gather_fn(bool crz_headers, bool aligned) {
 int split_hash_threads() { return kHashNT; }
 int split_finalize_threads() { return kFinNT; }
 int split_gather_threads() { return kGatherNT; }
-const void *split_hash_small_dense_fn(int lanes_per_chunk) {
+template <bool kCta>
+static const void *hash_small_dense_fn(int lanes_per_chunk) {
     switch (lanes_per_chunk) {
-    case 4: return reinterpret_cast<const void *>(&split_hash_small_dense_kernel<4>);
-    case 8: return reinterpret_cast<const void *>(&split_hash_small_dense_kernel<8>);
-    case 16: return reinterpret_cast<const void *>(&split_hash_small_dense_kernel<16>);
-    case 32: return reinterpret_cast<const void *>(&split_hash_small_dense_kernel<32>);
+    case 4: return reinterpret_cast<const void *>(&split_hash_small_dense_kernel<4, kCta>);
+    case 8: return reinterpret_cast<const void *>(&split_hash_small_dense_kernel<8, kCta>);
+    case 16: return reinterpret_cast<const void *>(&split_hash_small_dense_kernel<16, kCta>);
+    case 32: return reinterpret_cast<const void *>(&split_hash_small_dense_kernel<32, kCta>);
     default: return nullptr;
     }
+}
+const void *split_hash_small_dense_fn(int lanes_per_chunk, bool by_cta) {
+    return by_cta ? hash_small_dense_fn<true>(lanes_per_chunk) : hash_small_dense_fn<false>(lanes_per_chunk);
 }
 
 }  // namespace crac

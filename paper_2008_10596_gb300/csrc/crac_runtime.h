@@ -487,7 +487,9 @@ struct crac_ctx {
     bool full_copy_ok = false;   // current pass: no baseline anywhere
     bool sparse_ok = false;      // current pass: CRAC_PASS_SPARSE, device images, 16-byte sizes
     bool dense_now = false;      // ... and, on 512 B - 4 KiB chunks, dense placement of the dirty chunks
-    bool dense_hint = false;     // trial passes: dense placement (set by the tuner for a sparse timing)
+    bool dense_cta = false;      // ... taking its room once per CTA
+    float dense_hint = -1.f;     // trial passes: dense placement, for this fraction of dirty chunks (set by the
+                                 // tuner for a sparse timing; below 0: none)
     uint32_t pass_now = CRAC_PASS_SPLIT;   // kernel of the current pass (CRAC_PASS_AUTO resolved)
     bool split_now = false;      // the current pass is the split graph (per-kernel timing events)
     bool prefetch_now = false;   // the current pass prefetched managed memory (ev_p0 / ev_p1)

@@ -6,6 +6,7 @@ import os
 import random
 import subprocess
 
+import numpy as np
 import pytest
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
@@ -19,6 +20,7 @@ uint32_t hash_seg(uint64_t n, uint64_t b, uint32_t l, int copy) { return split_h
 uint32_t hash_grid(uint64_t n, uint64_t b, uint32_t l, uint32_t s, int copy, int sm, uint32_t *per) {
     return split_hash_grid(n, b, l, s, copy, sm, per);
 }
+int dense(float f, uint32_t l) { return dense_by_cta(f, l); }
 uint32_t restore_plan(uint64_t n, uint64_t b, uint32_t l, int coded, int sm, uint64_t most, uint32_t *out) {
     const RestoreCut c = restore_cut(n, b, l, coded, sm, most);
     out[0] = c.log2_part;
@@ -40,6 +42,7 @@ def rules(tmp_path_factory):
     u64, u32 = ctypes.c_uint64, ctypes.c_uint32
     so.hash_seg.argtypes = [u64, u64, u32, ctypes.c_int]
     so.hash_grid.argtypes = [u64, u64, u32, u32, ctypes.c_int, ctypes.c_int, ctypes.POINTER(u32)]
+    so.dense.argtypes = [ctypes.c_float, u32]
     so.restore_plan.argtypes = [u64, u64, u32, ctypes.c_int, ctypes.c_int, u64, ctypes.POINTER(u32)]
     return so
 
@@ -149,3 +152,13 @@ def test_the_restore_walk_takes_every_part_once(rules, seed):
             if it < items:
                 seen[it] += 1
     assert set(seen) == {1}
+
+
+def test_dense_placement_by_cta_where_the_counter_would_set_the_pace(rules):
+    """Once per CTA from about three in ten 4 KiB with a dirty chunk, on 4 KiB chunks from 22%."""
+    for log2S in (9, 10, 11, 12):
+        n, least = 4096 >> log2S, 0.3 if log2S < 12 else 0.22
+        for f in np.linspace(0, 0.25, 251):
+            p = 1 - (1 - f) ** n
+            if abs(p - least) > 1e-3:
+                assert bool(rules.dense(f, log2S)) == (p > least), (f, log2S)
