@@ -404,7 +404,9 @@ __global__ void __launch_bounds__(kCodecNT, 3) crz_encode_kernel(const CodecPara
 // CTAs, one warp per 16 KiB segment of an entry, straight from staging, or, as
 // nodes of the pass's graph, from the allocations.
 constexpr uint32_t kSizeTile = 64;         // entries per tile of the sizing kernel: eight a warp (with 256,
-                                           // 2 GiB of 64 KiB entries kept 128 CTAs busy for 36 us)
+                                           // 2 GiB of 64 KiB entries kept 128 CTAs busy for 36 us),
+constexpr uint32_t kSizeTileLong = 8;      // one a warp for chunks of 1 MiB and more (256 MiB in 4 MiB chunks
+                                           // were one tile: 300 -> 90 us for sizing and coding)
 constexpr uint32_t kSegBlocks = 32;        // blocks per work item of the sized encoder: 16 KiB
 
 // The entries to code: P.k, or in the pass's graph what the pass found (none
@@ -414,11 +416,26 @@ __device__ __forceinline__ uint64_t entry_count(const CodecParams &P) {
     return P.ctrl->err ? 0 : (uint64_t)P.ctrl->k;
 }
 
+__host__ __device__ __forceinline__ uint32_t size_tile(uint32_t log2_bpc) {
+    return log2_bpc < 11 ? kSizeTile : kSizeTileLong;
+}
+
+// The upper 16 bits of a header word, zero in a stream, carry a tag in chdr.
+__device__ __forceinline__ uint64_t crz_tag(uint64_t h, uint32_t tag) {
+    return (h & 0x0000FFFFFFFFFFFFull) | (uint64_t)tag << 48;
+}
+__device__ __forceinline__ uint32_t crz_tag_of(uint64_t h) { return (uint32_t)(h >> 48); }
+
 // zlen and zoff of every entry (and zoff[k]) from the header widths: one warp
-// per entry sums them; a tile's padded lengths are scanned and placed by a
-// decoupled look-back over the earlier tiles (tiles are taken in ticket
-// order, so every predecessor has started).  piece_off[i] receives zoff of
-// entry k * i / pieces, for i = 0 .. pieces.
+// per entry sums them, and leaves the units before each segment but the first as
+// the tags of the two headers in front of it; a tile's padded lengths are scanned
+// and placed by a decoupled look-back over the earlier tiles (tiles are taken in
+// ticket order, so every predecessor has started).  piece_off[i] receives zoff of
+// entry k * i / pieces, for i = 0 .. pieces.  (Without the tags every warp of the
+// coder sums up its entry's widths so far once more, which was most of its time on
+// long chunks: 256 MiB of fp32, FULL, in chunks of 1 MiB 413 -> 225 us, of 4 MiB 881
+// -> 239, of 16 MiB 1003 -> 307.)
+static_assert(kSegBlocks == 32, "a segment's headers, a lane each");
 __global__ void __launch_bounds__(kCodecNT) crz_size_kernel(const CodecParams P) {
     __shared__ uint32_t s_tile;
     __shared__ uint64_t s_z[kSizeTile];
@@ -427,6 +444,7 @@ __global__ void __launch_bounds__(kCodecNT) crz_size_kernel(const CodecParams P)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     wait_for_producer();   // in the pass's graph: its list, counts and headers
     const uint64_t k = entry_count(P);
+    const uint32_t n_tile = size_tile(P.log2_bpc);
     for (;;) {
         __syncthreads();   // the previous tile's shared state is consumed
         if (tid == 0) {
@@ -437,20 +455,32 @@ __global__ void __launch_bounds__(kCodecNT) crz_size_kernel(const CodecParams P)
             s_tile = t;
         }
         __syncthreads();
-        const uint64_t e0 = (uint64_t)s_tile * kSizeTile;
+        const uint32_t tile = s_tile;
+        const uint64_t e0 = (uint64_t)tile * n_tile;
         if (e0 >= k) return;
-        const uint32_t ne = (uint32_t)umin64(kSizeTile, k - e0);
+        const uint32_t ne = (uint32_t)umin64(n_tile, k - e0);
         for (uint32_t t = warp; t < ne; t += kCodecWarps) {
             const uint64_t e = e0 + t;
             const uint64_t L = P.off[e + 1] - P.off[e], nb = L >> 9, c = P.idx[e];
-            const uint64_t *h = P.chdr + (c << P.log2_bpc);
+            uint64_t *h = P.chdr + (c << P.log2_bpc);
             if (P.srcs) {   // where the encoder finds the entry
                 const CkptDesc a = P.desc[find_alloc_warp(P.desc, P.n_allocs, c, lane)];
                 if (lane == 0) P.srcs[e] = a.ptr + ((c - a.first_chunk) << (P.log2_bpc + 9));
             }
-            uint32_t w = 0;
-            for (uint64_t b = lane; b < nb; b += 32) w += crz_width_sum(h[b]);
-            w = __reduce_add_sync(kFull, w);   // <= 32 per block, nb <= 2^15
+            uint32_t w = 0;   // units so far: <= 32 per block, nb <= 2^15
+            for (uint64_t b0 = 0; b0 < nb; b0 += 32 * 8) {
+                uint64_t v[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) v[u] = b0 + 32 * u + lane < nb ? h[b0 + 32 * u + lane] : 0;
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    if (b0 + 32 * u >= nb) break;   // warp-uniform
+                    w += __reduce_add_sync(kFull, crz_width_sum(v[u]));
+                    // for the segment that begins after these blocks
+                    if (lane >= 30 && b0 + 32 * (u + 1) < nb)
+                        h[b0 + 32 * u + lane] = crz_tag(v[u], lane == 30 ? w & 0xFFFFu : w >> 16);
+                }
+            }
             if (lane == 0) {
                 const uint64_t zc = crz_head_bytes(nb) + 16ull * w + (L & 511u);
                 const uint64_t z = (nb && zc < L) ? zc : L;
@@ -461,7 +491,6 @@ __global__ void __launch_bounds__(kCodecNT) crz_size_kernel(const CodecParams P)
         __syncthreads();
         uint64_t tile_bytes;
         const uint64_t ex = cta_excl_scan<uint64_t>((uint32_t)tid < ne ? s_z[tid] : 0ull, s_w64, &tile_bytes);
-        const uint32_t tile = (uint32_t)(e0 / kSizeTile);
         if (warp == 0) {
             uint64_t base = 0;
             if (tile == 0) {
@@ -492,9 +521,9 @@ __global__ void __launch_bounds__(kCodecNT) crz_size_kernel(const CodecParams P)
 // Entries [e_begin, e_end) -> their streams at zoff (made by crz_size_kernel):
 // work item = (entry, segment of kSegBlocks blocks), one warp each, in entry
 // order.  A coded segment writes its blocks' header words and units (unit
-// offsets: the widths of the entry's earlier blocks, then a warp scan over the
-// segment's, a lane per block), and the segment holding the entry's last block
-// also the header pad, the raw tail and the stream pad; a raw entry is copied
+// offsets: the units before the segment, from the sizing kernel, then a warp scan
+// over the segment's widths, a lane per block), and the segment holding the
+// entry's last block also the header pad, the raw tail and the stream pad; a raw entry is copied
 // segment by segment.  Coding is integer work (about 146 warp instructions per
 // block, 76% of the issue slots used), so the raw blocks arrive in a ring of
 // shared memory by asynchronous copies, kAhead blocks a step, three steps
@@ -543,13 +572,11 @@ __global__ void __launch_bounds__(kCodecNT, 4) crz_encode_sized_kernel(const Cod
         uint64_t *dh = reinterpret_cast<uint64_t *>(d);
         src += 512ull * b0;
         // units of the entry's blocks before this segment
-        uint32_t before = 0;
-        for (uint32_t b = lane; b < b0; b += 32) before += crz_width_sum(h[b]);
-        before = __reduce_add_sync(kFull, before);
+        const uint32_t before = b0 ? crz_tag_of(h[b0 - 2]) | crz_tag_of(h[b0 - 1]) << 16 : 0u;
         // lane l: block b0 + l's header word, and its units' place in the stream
         uint64_t hw = 0;
         if ((uint32_t)lane < nseg) {
-            hw = h[b0 + lane];
+            hw = crz_tag(h[b0 + lane], 0);
             dh[b0 + lane] = hw;
         }
         const uint32_t ends = crz_ends(hw), mine = ends >> 24;
@@ -615,7 +642,10 @@ __global__ void __launch_bounds__(kCodecNT, 4) crz_encode_sized_kernel(const Cod
 
 uint32_t crz_tile_max() { return kCodecTileMax; }
 
-uint64_t crz_size_tiles(uint64_t k) { return (k + kSizeTile - 1) / kSizeTile; }
+uint64_t crz_size_tiles(uint64_t k, uint32_t log2S) {
+    const uint32_t tile = size_tile(log2S - 9);
+    return (k + tile - 1) / tile;
+}
 
 uint32_t crz_sized_segs(uint32_t log2S) { return log2S > 14 ? 1u << (log2S - 14) : 1u; }
 

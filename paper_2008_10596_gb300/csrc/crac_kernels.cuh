@@ -277,8 +277,9 @@ struct CodecParams {
     uint64_t timeout_ns;
     uint32_t skip_first_ticket;   // fault injection: tile 0 is never processed
     // Block header words made by the pass (CkptParams::crz_hdr), or null:
-    // entry e's block b has chdr[(idx[e] << log2_bpc) + b].
-    const uint64_t *chdr;
+    // entry e's block b has chdr[(idx[e] << log2_bpc) + b] (bits 0 - 47; the sizing
+    // kernel leaves the segments' places in the upper 16).
+    uint64_t *chdr;
     const uint64_t *idx;          // the entries' global chunk ids
     uint32_t log2_bpc;            // log2 of 512-byte blocks per chunk
     // With chdr, the streams are sized and placed first (crz_size_kernel:
@@ -303,7 +304,7 @@ const void *crz_encode_sized_fn();   // streams to device memory
 int crz_threads();
 cudaError_t launch_crz_encode(const CodecParams &p, int grid, cudaStream_t s);
 cudaError_t launch_crz_size(const CodecParams &p, int grid, cudaStream_t s);
-uint64_t crz_size_tiles(uint64_t k);   // look-back words it needs
+uint64_t crz_size_tiles(uint64_t k, uint32_t log2S);   // look-back words it needs
 cudaError_t launch_crz_encode_sized(const CodecParams &p, bool to_host, int sm_count, cudaStream_t s);
 uint32_t crz_sized_segs(uint32_t log2S);   // work items per entry of the sized encoder
 uint32_t crz_tile_max();

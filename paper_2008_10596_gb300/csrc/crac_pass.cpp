@@ -297,7 +297,7 @@ crac_status_t launch_split_graph(crac_ctx *c, const CkptParams &P, size_t work_b
         Ec = *enc;
         const uint64_t n = P.c_end - P.c_begin, items = n * Ec.segs_per_entry, warps = crz_threads() / 32;
         ek[0].func = const_cast<void *>(crz_size_fn());
-        ek[0].gridDim = dim3((unsigned)std::min<uint64_t>(crz_size_tiles(n), (uint64_t)c->sm_count * 4));
+        ek[0].gridDim = dim3((unsigned)std::min<uint64_t>(crz_size_tiles(n, c->log2S), (uint64_t)c->sm_count * 4));
         // A FULL pass codes every item: a CTA for every eight.  A delta's count
         // is not known yet: up to four waves of resident CTAs stride over it.
         ek[1].func = const_cast<void *>(crz_encode_sized_fn());
@@ -392,7 +392,7 @@ crac_status_t launch_segment(crac_ctx *c, const Segment &sg, const CkptDesc *des
         const size_t status_bytes = sizeof(CkptCtrl) + 16 * n_tiles;
         size_t work_bytes = status_bytes + 8 * nseg;
         const size_t enc_at = work_bytes;   // the coder's error word, ticket and look-back words
-        if (enc) work_bytes += 8 + 8 * crz_size_tiles(nseg);
+        if (enc) work_bytes += 8 + 8 * crz_size_tiles(nseg, c->log2S);
         TRY(ensure_dev(c->work, work_bytes + 16));   // zeroed in 16-byte words
         // 512 B..4 KiB chunks: several whole chunks per warp iteration.
         const bool small = c->log2S >= 9 && c->log2S < 13;
@@ -655,7 +655,7 @@ crac_status_t encode_segment_sized(crac_ctx *c, Piece &pc, const CkptCtrl &ctrl,
     *zplaced = false;
     TRY(ensure_dev(c->zwork, crz_work_bytes(k, D, c->log2S)));
     uint8_t *w = (uint8_t *)c->zwork.p;
-    const uint64_t size_tiles = crz_size_tiles(k);
+    const uint64_t size_tiles = crz_size_tiles(k, c->log2S);
     const uint32_t spe = crz_sized_segs(c->log2S);
     // staged host images: launches of at least 32 MiB of raw payload each (the
     // copy of a piece's streams takes far longer than its encoding)
@@ -666,7 +666,7 @@ crac_status_t encode_segment_sized(crac_ctx *c, Piece &pc, const CkptCtrl &ctrl,
     P.src = (const uint8_t *)c->staging.p;
     P.off = (const uint64_t *)c->off.p;
     P.k = k;
-    P.chdr = (const uint64_t *)c->chdr.p;
+    P.chdr = (uint64_t *)c->chdr.p;
     P.idx = host_res ? (const uint64_t *)c->idx.p : (const uint64_t *)pc.idx_dev.p;
     P.log2_bpc = c->log2S - 9;
     P.zoff = host_res ? (uint64_t *)c->zoff.p : (uint64_t *)pc.off_dev.p;
@@ -780,7 +780,7 @@ crac_status_t encode_segment(crac_ctx *c, Piece &pc, const CkptCtrl &ctrl, bool 
     P.src = (const uint8_t *)c->staging.p;
     P.off = (const uint64_t *)c->off.p;
     if (c->crz_hdr_now) {   // the pass made the block headers
-        P.chdr = (const uint64_t *)c->chdr.p;
+        P.chdr = (uint64_t *)c->chdr.p;
         P.idx = host_res ? (const uint64_t *)c->idx.p : (const uint64_t *)pc.idx_dev.p;
         P.log2_bpc = c->log2S - 9;
     }
@@ -1004,7 +1004,8 @@ crac_status_t ctx_settle(crac_ctx *c, bool block) {
 // while it is armed, other passes take the form that sizes from the counts.
 bool codes_in_pass(const crac_ctx *c, size_t segments, bool host_res, uint64_t n_chunks) {
     if (!c->crz_hdr_now || host_res || segments != 1) return false;
-    if (fault_armed(CRAC_FAULT_ENCODE_WAIT) && !(c->full_copy_ok && crz_size_tiles(n_chunks) >= 2)) return false;
+    const bool tiles_known = c->full_copy_ok && crz_size_tiles(n_chunks, c->log2S) >= 2;
+    if (fault_armed(CRAC_FAULT_ENCODE_WAIT) && !tiles_known) return false;
     for (const AllocRec &r : c->allocs)
         if (r.kind == CRAC_KIND_HOST) return false;
     return true;
