@@ -13,15 +13,18 @@ constexpr uint64_t kSmallItersRead = 16;   // ... at most, where the pass mostly
 // log2 of the hash kernel's segment (at most the chunk) for n_chunks chunks of
 // `bytes` tracked bytes; copy: every chunk is also written.  Not for chunks of
 // 512 B - 4 KiB.
-//   8 KiB; 16 KiB where the pass mostly reads and is large enough that every SM
-// still gets dozens of CTAs (4 GiB, read only: 623 -> 600 us), not where it writes
-// every chunk (1211 -> 1234 us).  Where a chunk holds less than 8 KiB on average
+//   8 KiB; 16 KiB where the pass is large enough that every SM still gets dozens of
+// CTAs, and mostly reads (4 GiB, read only: 623 -> 600 us; writing every chunk 1211
+// -> 1234) or writes chunks of 2 MiB and more: with fewer chunks than CTAs, all of
+// them add to the same few sums, one after another (4 GiB in chunks of 16 MiB: 1557
+// -> 1272 us, of 4 MiB 1351 -> 1272).  Where a chunk holds less than 8 KiB on average
 // (allocations much shorter than a chunk), up to 64 KiB, so that the segments past
 // an allocation's end, whose look-up costs as much as any other's, are few (50000
 // allocations below 512 B in 64 KiB chunks, hash kernel: 469 us in segments of
 // 8 KiB, 49 whole).
 inline uint32_t split_hash_seg(uint64_t n_chunks, uint64_t bytes, uint32_t log2_chunk, bool copy) {
-    const uint32_t m = (bytes >> 13) < n_chunks ? 16 : copy || (bytes >> 14) < 32768 ? 13 : 14;
+    const bool brief = (copy && log2_chunk < 21) || (bytes >> 14) < 32768;
+    const uint32_t m = (bytes >> 13) < n_chunks ? 16 : brief ? 13 : 14;
     return log2_chunk < m ? log2_chunk : m;
 }
 
