@@ -136,15 +136,17 @@ crac_status_t restart_device(crac_ctx *c, crac_image *img, const std::vector<cra
     ScatterDesc *sdh = (ScatterDesc *)c->sdesc_h.p;
     RestorePiece *rph = (RestorePiece *)((uint8_t *)c->sdesc_h.p + desc_bytes);
     size_t dpos = 0, ppos = 0;
-    uint64_t entries = 0;
+    uint64_t entries = 0, sizes = 0;   // sizes: all of them, ored
     for (size_t i = 0; i < chain.size(); ++i) {
         const crac_image *im = chain[i];
         const std::vector<int64_t> m = allocs.of(im);
         const size_t d0 = dpos;
-        for (size_t a = 0; a < im->allocs.size(); ++a, ++dpos)
+        for (size_t a = 0; a < im->allocs.size(); ++a, ++dpos) {
             sdh[dpos] = ScatterDesc{im->allocs[a].first_chunk, im->allocs[a].bytes,
                                     m[a] < 0 ? 0 : img->allocs[m[a]].first_chunk, m[a] < 0 ? 0 : c->allocs[m[a]].ptr,
                                     0, {0, 0, 0}};
+            sizes |= im->allocs[a].bytes;
+        }
         const bool host = im->residency != CRAC_RESIDENCY_DEVICE;
         const bool coded = (im->flags & CRAC_IMAGE_CODED) != 0;
         for (const Piece &pc : im->pieces) {
@@ -161,6 +163,11 @@ crac_status_t restart_device(crac_ctx *c, crac_image *img, const std::vector<cra
             entries += pc.k;
         }
     }
+    crac_restart_info_t ri{};
+    ri.chain_length = ri.images_used = (uint32_t)chain.size();
+    for (const ImgAlloc &a : img->allocs) ri.restored_bytes += a.bytes;
+    ri.entries_scanned = entries;
+    ri.scatter_launches = entries ? 1 : 0;
     for (crac_image *im : chain)   // deserialized images have no event: complete from the start
         if (im->done) CK(cudaStreamWaitEvent(s, im->done, 0));
     CK(cudaStreamWaitEvent(s, c->ev_last, 0));
@@ -171,11 +178,6 @@ crac_status_t restart_device(crac_ctx *c, crac_image *img, const std::vector<cra
     if (!c->uva)
         CK(cudaMemcpyAsync(c->sdesc.p, c->sdesc_h.p, sdesc16 * 16, cudaMemcpyHostToDevice, s));
     CK(launch_prologue(c->owner.p, owner16 + 1, c->sdesc.p, c->sdesc_h.p, c->uva ? sdesc16 : 0, c->sm_count, s));
-    crac_restart_info_t ri{};
-    ri.chain_length = ri.images_used = (uint32_t)chain.size();
-    for (const ImgAlloc &a : img->allocs) ri.restored_bytes += a.bytes;
-    ri.entries_scanned = entries;
-    ri.scatter_launches = entries ? 1 : 0;
     RestoreParams P{};
     P.pieces = (const RestorePiece *)((uint8_t *)c->sdesc.p + desc_bytes);
     P.n_pieces = (uint32_t)ppos;
@@ -187,10 +189,8 @@ crac_status_t restart_device(crac_ctx *c, crac_image *img, const std::vector<cra
     P.owner = (unsigned long long *)c->owner.p;
     P.n_owner = nt;
     P.err = (unsigned int *)((uint8_t *)c->owner.p + owner16 * 16);
-    for (const crac_image *im : chain) {
-        P.coded |= (im->flags & CRAC_IMAGE_CODED) ? 1u : 0u;
-        for (const ImgAlloc &a : im->allocs) P.ragged |= (a.bytes & 15) ? 1u : 0u;
-    }
+    for (const crac_image *im : chain) P.coded |= (im->flags & CRAC_IMAGE_CODED) ? 1u : 0u;
+    P.ragged = (sizes & 15) ? 1u : 0u;
     // Reads of host images are paced by the host link, which one CTA per SM
     // already saturates (4 KiB in flight per warp); a bigger grid would only
     // keep SMs from other streams' work for the length of the transfer.
