@@ -4,6 +4,12 @@
 
 #include <cstdint>
 
+#ifdef __CUDACC__
+#define CRAC_HD __host__ __device__
+#else
+#define CRAC_HD
+#endif
+
 namespace crac {
 
 constexpr uint64_t kHashWarps = 8;         // warps of a hash CTA
@@ -67,6 +73,22 @@ inline bool dense_by_cta(float f, uint32_t log2_chunk) {
     float clean = 1.f;
     for (uint32_t i = 0; i < (4096u >> log2_chunk); ++i) clean *= 1.f - f;
     return clean < (log2_chunk < 12 ? 0.70f : 0.78f);
+}
+
+// log2 of the items of each of n chunks (2^log2_parts parts of 2^log2_part bytes)
+// that hold `bytes` bytes together; item s takes parts s, s + items, ... of what its
+// chunk holds.
+//   An item per part; where nearly all parts lie past the end of an allocation, as many
+// (at least 8, or as take four parts each) as `lanes` lanes look up in one round: empty
+// items cost as much of a look-up as others, while a chunk's parts in one item are
+// copied or coded one after another.  20000 allocations below 4 KiB, all dirty,
+// a delta: 481 -> 134 us in chunks of 1 MiB, 1448 -> 135 in chunks of 4 MiB; coded
+// 2267 -> 276 in the latter.
+CRAC_HD inline uint32_t chunk_items(uint64_t n, uint64_t bytes, uint32_t log2_part, uint32_t log2_parts, uint64_t lanes) {
+    if ((n << log2_parts) <= 32 * (bytes >> log2_part) + 3 * n) return log2_parts;
+    uint32_t s = log2_parts < 5 ? (log2_parts < 2 ? 0 : log2_parts - 2) : 3;
+    while (s < log2_parts && (n << (s + 1)) <= lanes) ++s;
+    return s;
 }
 
 // How a restore's scatter is cut: parts of 1 << log2_part bytes of the target's

@@ -163,7 +163,8 @@ const void *split_hash_fn(bool crz_headers, bool aligned);
 const void *split_hash_small_fn(int lanes_per_chunk, bool aligned);
 uint32_t split_finalize_tile(uint64_t n_chunks, int sm_count);   // chunks per tile of the finalize kernel
 const void *split_finalize_fn(uint32_t tile);
-const void *split_gather_fn(bool crz_headers, bool aligned);
+// for passes over n_chunks chunks of 2^log2_chunk holding `bytes` bytes
+const void *split_gather_fn(bool crz_headers, bool aligned, uint64_t n_chunks, uint64_t bytes, uint32_t log2_chunk);
 int split_hash_threads();
 int split_finalize_threads();
 int split_gather_threads();

@@ -109,7 +109,7 @@ cudaError_t load_kernels() {
                          split_hash_small_fn(32, false),
                          split_finalize_fn(split_finalize_tile(1, 1)),
                          split_finalize_fn(split_finalize_tile(UINT64_MAX, 1)),
-                         split_gather_fn(false, false)};
+                         split_gather_fn(false, false, 1, 1, 0)};
     cudaError_t e = cudaSuccess;
     cudaFuncAttributes a;
     for (const void *f : fns)
@@ -260,7 +260,7 @@ extern "C" crac_status_t crac_pass_noalloc(const crac_region_t *regions_dev, uin
             e = launch_chained(split_finalize_fn(fin_tile), fin_tiles < 2u * sms ? fin_tiles : 2u * sms,
                                split_finalize_threads(), args, s);
         if (e == cudaSuccess && !fused)
-            e = launch_chained(split_gather_fn(false, false), 8 * sms, split_gather_threads(), args, s);
+            e = launch_chained(split_gather_fn(false, false, n_chunks, full, l), 8 * sms, split_gather_threads(), args, s);
         const uint64_t g = grid_per[wpc == 8 ? 1 : 0];
         reserved = (uint32_t)(n_tiles + (n_tiles < g ? n_tiles : g));
     }

@@ -729,7 +729,8 @@ split_finalize_kernel(const CkptParams P, unsigned long long *__restrict__ acc, 
 // too (a separate instance, so that the plain gather keeps its registers low).
 // kAligned: every allocation's size, so every payload offset, is a multiple of
 // 16 bytes.
-template <bool kHdr, bool kAligned>
+// kMulti: an item takes several parts of its entry (chunk_items).
+template <bool kHdr, bool kAligned, bool kMulti>
 __global__ void __launch_bounds__(kGatherNT, kHdr ? 2 : 4)
 split_gather_kernel(const CkptParams P, unsigned long long *, uint32_t) {
     wait_for_producer();         // the finalize kernel's list and counts
@@ -752,15 +753,16 @@ split_gather_kernel(const CkptParams P, unsigned long long *, uint32_t) {
     // that a small payload still spreads over the chip; a warp strides over the
     // items, 32 at a time, a lane looking up each (a chain of dependent loads).
     // 96 MiB in 1200 ragged allocations, 64 KiB chunks: all of them 545 -> 36 us.
-    const uint32_t log2P = log2S < 13 ? log2S : 13, parts = log2S - log2P;   // parts: log2 of the items per entry
-    const uint64_t n_items = k << parts;
+    const uint32_t log2P = log2S < 13 ? log2S : 13;
+    const uint32_t items = kMulti ? chunk_items(k, P.ctrl->D, log2P, log2S - log2P, 32 * nw) : log2S - log2P;   // log2 per entry
+    const uint64_t n_items = k << items;
     for (uint64_t i0 = ((uint64_t)blockIdx.x * kGatherNT + threadIdx.x) >> 5; i0 < n_items; i0 += 32 * nw) {
         const uint64_t it = i0 + lane * nw;
         uint64_t dst = 0, src = 0, blk = 0;
-        uint32_t len = 0;   // bytes to copy
+        uint32_t len = 0;   // bytes to copy (kMulti: of the chunk, from the item's first part on)
         if (it < n_items) {
-            const uint64_t j = it >> parts;
-            const uint64_t po = (it & ((1ull << parts) - 1)) << log2P;   // the item's offset in its entry
+            const uint64_t j = it >> items;
+            const uint64_t po = (it & ((1ull << items) - 1)) << log2P;   // the item's offset in its entry
             const uint64_t c = P.idx_out[j];
             const uint64_t o = P.off_out[j];
             if (next && po == 0) next[c - P.c_begin] = o;
@@ -778,7 +780,7 @@ split_gather_kernel(const CkptParams P, unsigned long long *, uint32_t) {
                 } else if (po < clen) {   // a short last chunk has fewer items
                     dst = o + po;
                     src = d.ptr + at + po;
-                    len = (uint32_t)umin64(1ull << log2P, clen - po);
+                    len = (uint32_t)(kMulti ? clen - po : umin64(1ull << log2P, clen - po));
                     if (kHdr) blk = (c << (log2S - 9)) + (po >> 9);
                 }
             }
@@ -790,8 +792,13 @@ split_gather_kernel(const CkptParams P, unsigned long long *, uint32_t) {
             uint8_t *to = P.staging + __shfl_sync(kFull, dst, i);
             const uint8_t *from = reinterpret_cast<const uint8_t *>(__shfl_sync(kFull, src, i));
             const uint32_t n = __shfl_sync(kFull, len, i);
-            if (kHdr) copy_with_headers<kAligned>(to, from, n, lane, P.crz_hdr + __shfl_sync(kFull, blk, i), !P.hdr_only);
-            else copy_group<32, kAligned>(to, from, n, lane);
+            uint64_t *hdr = kHdr ? P.crz_hdr + __shfl_sync(kFull, blk, i) : nullptr;
+            for (uint32_t at = 0; at < n; at += 1u << (log2P + items)) {
+                const uint32_t part = kMulti ? min(1u << log2P, n - at) : n;
+                if (kHdr) copy_with_headers<kAligned>(to + at, from + at, part, lane, hdr + (at >> 9), !P.hdr_only);
+                else copy_group<32, kAligned>(to + at, from + at, part, lane);
+                if (!kMulti) break;
+            }
         }
     }
     hits = __reduce_add_sync(kFull, hits);
@@ -830,12 +837,16 @@ const void *split_finalize_fn(uint32_t tile) {
     return tile == kFinNT ? reinterpret_cast<const void *>(&split_finalize_kernel<1>)
                           : reinterpret_cast<const void *>(&split_finalize_kernel<8>);
 }
-const void *split_gather_fn(bool crz_headers, bool aligned) {
-    if (crz_headers)
-        return aligned ? reinterpret_cast<const void *>(&split_gather_kernel<true, true>)
-                       : reinterpret_cast<const void *>(&split_gather_kernel<true, false>);
-    return aligned ? reinterpret_cast<const void *>(&split_gather_kernel<false, true>)
-                   : reinterpret_cast<const void *>(&split_gather_kernel<false, false>);
+template <bool kHdr>
+static const void *gather_fn(bool aligned, bool multi) {
+    if (multi) return reinterpret_cast<const void *>(&split_gather_kernel<kHdr, false, true>);
+    return aligned ? reinterpret_cast<const void *>(&split_gather_kernel<kHdr, true, false>)
+                   : reinterpret_cast<const void *>(&split_gather_kernel<kHdr, false, false>);
+}
+const void *split_gather_fn(bool crz_headers, bool aligned, uint64_t n_chunks, uint64_t bytes, uint32_t log2S) {
+    const uint32_t parts = log2S > 13 ? log2S - 13 : 0;
+    const bool multi = chunk_items(n_chunks, bytes, 13, parts, 0) != parts;
+    return crz_headers ? gather_fn<true>(aligned, multi) : gather_fn<false>(aligned, multi);
 }
 int split_hash_threads() { return kHashNT; }
 int split_finalize_threads() { return kFinNT; }
