@@ -2,6 +2,7 @@
 // lies in the allocations) -> one stream per entry, written to device memory or
 // straight into mapped pinned memory.
 #include "crac_codec.cuh"
+#include "crac_grids.h"
 
 namespace crac {
 
@@ -519,11 +520,12 @@ __global__ void __launch_bounds__(kCodecNT) crz_size_kernel(const CodecParams P)
 }
 
 // Entries [e_begin, e_end) -> their streams at zoff (made by crz_size_kernel):
-// work item = (entry, segment of kSegBlocks blocks), one warp each, in entry
-// order.  A coded segment writes its blocks' header words and units (unit
-// offsets: the units before the segment, from the sizing kernel, then a warp scan
-// over the segment's widths, a lane per block), and the segment holding the
-// entry's last block also the header pad, the raw tail and the stream pad; a raw entry is copied
+// work item = (entry, segment of kSegBlocks blocks; several of them where most
+// entries hold few, see crz_log2_items), one warp each, in entry order.  A coded
+// segment writes its blocks' header words and units (unit offsets: the units before
+// the segment, from the sizing kernel, then a warp scan over the segment's widths,
+// a lane per block), and the segment holding the entry's last block also the
+// header pad, the raw tail and the stream pad; a raw entry is copied
 // segment by segment.  Coding is integer work (about 146 warp instructions per
 // block, 76% of the issue slots used), so the raw blocks arrive in a ring of
 // shared memory by asynchronous copies, kAhead blocks a step, three steps
@@ -539,101 +541,102 @@ __global__ void __launch_bounds__(kCodecNT, 4) crz_encode_sized_kernel(const Cod
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const CrzLane LT = crz_lane(lane);
     wait_for_producer();   // in the pass's graph: the sizing kernel
-    const uint32_t spe = P.segs_per_entry;
-    uint64_t items = (P.e_end - P.e_begin) * spe;
+    const uint32_t per = 1u << P.log2_items;   // items per entry
+    uint64_t items = (P.e_end - P.e_begin) << P.log2_items;
     if (P.ctrl) {
         const unsigned int err = *P.err;   // of the sizing: offsets are missing
         if (err && blockIdx.x == 0 && tid == 0) atomicOr(&P.ctrl->err, err);
-        items = err ? 0 : entry_count(P) * spe;
+        items = err ? 0 : entry_count(P) << P.log2_items;
     }
     const uint64_t nw = ((uint64_t)gridDim.x * kCodecNT) >> 5;
     for (uint64_t it = ((uint64_t)blockIdx.x * kCodecNT + tid) >> 5; it < items; it += nw) {
-        const uint64_t e = P.e_begin + it / spe;
-        const uint32_t sg = (uint32_t)(it % spe);
+        const uint64_t e = P.e_begin + (it >> P.log2_items);
         const uint64_t o = P.off[e], L = P.off[e + 1] - o;
         const uint64_t z = P.zlen[e];
         uint8_t *d = P.dst + P.zoff[e];
-        const uint8_t *src = P.srcs ? reinterpret_cast<const uint8_t *>(P.srcs[e]) : P.src + o;
-        if (z == L) {   // stored raw
-            const uint64_t x0 = (uint64_t)sg * (512ull * kSegBlocks);
-            if (x0 >= L) continue;
-            const uint64_t x1 = umin64(L, x0 + 512ull * kSegBlocks);
-            copy_group<32>(d + x0, src + x0, x1 - x0, lane);
-            if (x1 == L)
-                for (uint64_t i = L + lane; i < ((L + 15) & ~15ull); i += 32) d[i] = 0;
-            continue;
-        }
-        const uint32_t nb = (uint32_t)(L >> 9);   // >= 1: a coded stream is shorter than its entry
-        const uint32_t last = (nb - 1) / kSegBlocks;
-        if (sg > last) continue;
-        const uint32_t b0 = sg * kSegBlocks;
-        const uint32_t nseg = min(kSegBlocks, nb - b0);
-        const uint64_t *h = P.chdr + (P.idx[e] << P.log2_bpc);
-        uint64_t *dh = reinterpret_cast<uint64_t *>(d);
-        src += 512ull * b0;
-        // units of the entry's blocks before this segment
-        const uint32_t before = b0 ? crz_tag_of(h[b0 - 2]) | crz_tag_of(h[b0 - 1]) << 16 : 0u;
-        // lane l: block b0 + l's header word, and its units' place in the stream
-        uint64_t hw = 0;
-        if ((uint32_t)lane < nseg) {
-            hw = crz_tag(h[b0 + lane], 0);
-            dh[b0 + lane] = hw;
-        }
-        const uint32_t ends = crz_ends(hw), mine = ends >> 24;
-        uint32_t inc = mine;
+        const uint8_t *entry = P.srcs ? reinterpret_cast<const uint8_t *>(P.srcs[e]) : P.src + o;
+        for (uint32_t sg = (uint32_t)it & (per - 1);; sg += per) {   // the item's segments, mostly one
+            if (z == L) {   // stored raw
+                const uint64_t x0 = (uint64_t)sg * (512ull * kSegBlocks);
+                if (x0 >= L) break;
+                const uint64_t x1 = umin64(L, x0 + 512ull * kSegBlocks);
+                copy_group<32>(d + x0, entry + x0, x1 - x0, lane);
+                if (x1 == L)
+                    for (uint64_t i = L + lane; i < ((L + 15) & ~15ull); i += 32) d[i] = 0;
+                continue;
+            }
+            const uint32_t nb = (uint32_t)(L >> 9);   // >= 1: a coded stream is shorter than its entry
+            const uint32_t last = (nb - 1) / kSegBlocks;
+            if (sg > last) break;
+            const uint32_t b0 = sg * kSegBlocks;
+            const uint32_t nseg = min(kSegBlocks, nb - b0);
+            const uint64_t *h = P.chdr + (P.idx[e] << P.log2_bpc);
+            uint64_t *dh = reinterpret_cast<uint64_t *>(d);
+            const uint8_t *src = entry + 512ull * b0;
+            // units of the entry's blocks before this segment
+            const uint32_t before = b0 ? crz_tag_of(h[b0 - 2]) | crz_tag_of(h[b0 - 1]) << 16 : 0u;
+            // lane l: block b0 + l's header word, and its units' place in the stream
+            uint64_t hw = 0;
+            if ((uint32_t)lane < nseg) {
+                hw = crz_tag(h[b0 + lane], 0);
+                dh[b0 + lane] = hw;
+            }
+            const uint32_t ends = crz_ends(hw), mine = ends >> 24;
+            uint32_t inc = mine;
 #pragma unroll
-        for (int s = 1; s < 32; s <<= 1) {
-            const uint32_t t = __shfl_up_sync(kFull, inc, s);
-            if (lane >= s) inc += t;
-        }
-        const uint32_t first = before + inc - mine;
-        uint8_t *units = d + crz_head_bytes(nb);
-        if (sg == last && lane == 0 && (nb & 1)) dh[nb] = 0;   // header pad
-        auto code = [&](uint32_t j, const uint32_t w[4]) {
-            const uint32_t mins = __shfl_sync(kFull, (uint32_t)hw, j);
-            const uint32_t be = __shfl_sync(kFull, ends, j);
-            const uint32_t u = __shfl_sync(kFull, first, j);
-            crz_block_units<kScratch>(mins, be, w, units + 16ull * u, lane, LT, s_units[kScratch ? warp : 0]);
-        };
-        if (((uintptr_t)src & 15u) == 0) {
-            constexpr int kG = kAhead, kN = 4;   // blocks a step, steps in the ring
-            uint8_t *ring = s_ring[warp];
-            auto fetch = [&](uint32_t j) {
-#pragma unroll
-                for (int g = 0; g < kG; ++g)
-                    if (j + g < nseg)
-                        cp_async16(ring + 512 * ((j + g) % (kG * kN)) + 16 * lane, src + 512ull * (j + g) + 16 * lane);
-                cp_async_commit();
+            for (int s = 1; s < 32; s <<= 1) {
+                const uint32_t t = __shfl_up_sync(kFull, inc, s);
+                if (lane >= s) inc += t;
+            }
+            const uint32_t first = before + inc - mine;
+            uint8_t *units = d + crz_head_bytes(nb);
+            if (sg == last && lane == 0 && (nb & 1)) dh[nb] = 0;   // header pad
+            auto code = [&](uint32_t j, const uint32_t w[4]) {
+                const uint32_t mins = __shfl_sync(kFull, (uint32_t)hw, j);
+                const uint32_t be = __shfl_sync(kFull, ends, j);
+                const uint32_t u = __shfl_sync(kFull, first, j);
+                crz_block_units<kScratch>(mins, be, w, units + 16ull * u, lane, LT, s_units[kScratch ? warp : 0]);
             };
-            __syncwarp();
+            if (((uintptr_t)src & 15u) == 0) {
+                constexpr int kG = kAhead, kN = 4;   // blocks a step, steps in the ring
+                uint8_t *ring = s_ring[warp];
+                auto fetch = [&](uint32_t j) {
 #pragma unroll
-            for (int i = 0; i < kG * (kN - 1); i += kG) fetch(i);
-            const uint32_t *rd = reinterpret_cast<const uint32_t *>(ring) + 4 * (lane & 7) + (lane >> 3);
+                    for (int g = 0; g < kG; ++g)
+                        if (j + g < nseg)
+                            cp_async16(ring + 512 * ((j + g) % (kG * kN)) + 16 * lane, src + 512ull * (j + g) + 16 * lane);
+                    cp_async_commit();
+                };
+                __syncwarp();
+#pragma unroll
+                for (int i = 0; i < kG * (kN - 1); i += kG) fetch(i);
+                const uint32_t *rd = reinterpret_cast<const uint32_t *>(ring) + 4 * (lane & 7) + (lane >> 3);
 #pragma unroll 1
-            for (uint32_t j = 0; j < nseg; j += kG) {
-                fetch(j + kG * (kN - 1));
-                cp_async_wait<kN - 1>();
-                __syncwarp();
+                for (uint32_t j = 0; j < nseg; j += kG) {
+                    fetch(j + kG * (kN - 1));
+                    cp_async_wait<kN - 1>();
+                    __syncwarp();
 #pragma unroll
-                for (int g = 0; g < kG; ++g) {
-                    if (j + g >= nseg) break;   // warp-uniform
-                    const uint32_t *n = rd + 128 * ((j + g) % (kG * kN));
-                    const uint32_t v[4] = {n[0], n[32], n[64], n[96]};
-                    code(j + g, v);
+                    for (int g = 0; g < kG; ++g) {
+                        if (j + g >= nseg) break;   // warp-uniform
+                        const uint32_t *n = rd + 128 * ((j + g) % (kG * kN));
+                        const uint32_t v[4] = {n[0], n[32], n[64], n[96]};
+                        code(j + g, v);
+                    }
+                    __syncwarp();
                 }
-                __syncwarp();
+            } else {   // a payload off the 16-byte grid (allocations of any byte size)
+                for (uint32_t j = 0; j < nseg; ++j) {
+                    uint32_t w[4];
+                    crz_load_words(src + 512 * j, lane, w);
+                    code(j, w);
+                }
             }
-        } else {   // a payload off the 16-byte grid (allocations of any byte size)
-            for (uint32_t j = 0; j < nseg; ++j) {
-                uint32_t w[4];
-                crz_load_words(src + 512 * j, lane, w);
-                code(j, w);
+            if (sg == last) {   // the raw tail, then the stream pad
+                const uint64_t tl = L & 511u;
+                copy_group<32>(d + z - tl, src + 512ull * nseg, tl, lane);
+                for (uint64_t i = z + lane; i < ((z + 15) & ~15ull); i += 32) d[i] = 0;
             }
-        }
-        if (sg == last) {   // the raw tail, then the stream pad
-            const uint64_t tl = L & 511u;
-            copy_group<32>(d + z - tl, src + 512ull * nseg, tl, lane);
-            for (uint64_t i = z + lane; i < ((z + 15) & ~15ull); i += 32) d[i] = 0;
         }
     }
 }
@@ -647,7 +650,13 @@ uint64_t crz_size_tiles(uint64_t k, uint32_t log2S) {
     return (k + tile - 1) / tile;
 }
 
-uint32_t crz_sized_segs(uint32_t log2S) { return log2S > 14 ? 1u << (log2S - 14) : 1u; }
+// A warp of the coder finds out about an empty item by itself, a chain of three
+// loads, so where nearly all are empty only as many are kept as give every SM 256 warps
+// (20000 allocations below 4 KiB in chunks of 1 MiB, host images, all dirty: 965 -> 386
+// us with the gather).
+uint32_t crz_log2_items(uint64_t k, uint64_t bytes, uint32_t log2S, int sm_count) {
+    return chunk_items(k, bytes, 14, log2S > 14 ? log2S - 14 : 0, 256ull * sm_count);
+}
 
 const void *crz_size_fn() { return reinterpret_cast<const void *>(&crz_size_kernel); }
 const void *crz_encode_sized_fn() { return reinterpret_cast<const void *>(&crz_encode_sized_kernel<false>); }
@@ -667,7 +676,7 @@ cudaError_t launch_crz_size(const CodecParams &p, int grid, cudaStream_t s) {
 // three CTAs per SM, and 16-byte stores.
 cudaError_t launch_crz_encode_sized(const CodecParams &p, bool to_host, int sm_count, cudaStream_t s) {
     if (p.e_end <= p.e_begin) return cudaSuccess;
-    const uint64_t want = ((p.e_end - p.e_begin) * p.segs_per_entry + kCodecWarps - 1) / kCodecWarps;
+    const uint64_t want = (((p.e_end - p.e_begin) << p.log2_items) + kCodecWarps - 1) / kCodecWarps;
     if (to_host)
         crz_encode_sized_kernel<true><<<(unsigned)umin64(want, 3ull * sm_count), kCodecNT, 0, s>>>(p);
     else

@@ -286,10 +286,10 @@ struct CodecParams {
     // With chdr, the streams are sized and placed first (crz_size_kernel:
     // zlen, zoff; piece_off[i] = zoff[k * i / pieces], i = 0 .. pieces), then
     // coded by crz_encode_sized_kernel over entries [e_begin, e_end), each
-    // entry as segs_per_entry work items of 16 KiB.
+    // entry as 1 << log2_items work items of a 16 KiB segment or several.
     uint64_t *piece_off;
     uint32_t pieces;
-    uint32_t segs_per_entry;
+    uint32_t log2_items;
     uint64_t e_begin, e_end;
     // Coded in the pass's own graph, straight from the allocations (the pass
     // then writes block headers but no payload): the entry count and the pass's
@@ -307,7 +307,8 @@ cudaError_t launch_crz_encode(const CodecParams &p, int grid, cudaStream_t s);
 cudaError_t launch_crz_size(const CodecParams &p, int grid, cudaStream_t s);
 uint64_t crz_size_tiles(uint64_t k, uint32_t log2S);   // look-back words it needs
 cudaError_t launch_crz_encode_sized(const CodecParams &p, bool to_host, int sm_count, cudaStream_t s);
-uint32_t crz_sized_segs(uint32_t log2S);   // work items per entry of the sized encoder
+// log2 of the sized encoder's work items per entry, for k entries of `bytes` bytes.
+uint32_t crz_log2_items(uint64_t k, uint64_t bytes, uint32_t log2S, int sm_count);
 uint32_t crz_tile_max();
 int crz_encode_max_ctas_per_sm();
 

@@ -295,7 +295,7 @@ crac_status_t launch_split_graph(crac_ctx *c, const CkptParams &P, size_t work_b
     cudaKernelNodeParams ek[2] = {};
     if (enc) {
         Ec = *enc;
-        const uint64_t n = P.c_end - P.c_begin, items = n * Ec.segs_per_entry, warps = crz_threads() / 32;
+        const uint64_t n = P.c_end - P.c_begin, items = n << Ec.log2_items, warps = crz_threads() / 32;
         ek[0].func = const_cast<void *>(crz_size_fn());
         ek[0].gridDim = dim3((unsigned)std::min<uint64_t>(crz_size_tiles(n, c->log2S), (uint64_t)c->sm_count * 4));
         // A FULL pass codes every item: a CTA for every eight.  A delta's count
@@ -455,7 +455,7 @@ crac_status_t launch_segment(crac_ctx *c, const Segment &sg, const CkptDesc *des
             enc->idx = idx_d;
             enc->chdr = crz_hdr;
             enc->log2_bpc = c->log2S - 9;
-            enc->segs_per_entry = crz_sized_segs(c->log2S);
+            enc->log2_items = crz_log2_items(nseg, sg.bytes, c->log2S, c->sm_count);
             enc->ctrl = P.ctrl;
             enc->srcs = (uint64_t *)acc;   // the finalize kernel was their last reader
             enc->desc = desc_dev;
@@ -656,7 +656,6 @@ crac_status_t encode_segment_sized(crac_ctx *c, Piece &pc, const CkptCtrl &ctrl,
     TRY(ensure_dev(c->zwork, crz_work_bytes(k, D, c->log2S)));
     uint8_t *w = (uint8_t *)c->zwork.p;
     const uint64_t size_tiles = crz_size_tiles(k, c->log2S);
-    const uint32_t spe = crz_sized_segs(c->log2S);
     // staged host images: launches of at least 32 MiB of raw payload each (the
     // copy of a piece's streams takes far longer than its encoding)
     uint32_t pieces = 1;
@@ -676,7 +675,7 @@ crac_status_t encode_segment_sized(crac_ctx *c, Piece &pc, const CkptCtrl &ctrl,
     P.status = (uint64_t *)(w + kZworkHead);
     P.piece_off = (uint64_t *)(w + kZworkPieceOff);
     P.pieces = pieces;
-    P.segs_per_entry = spe;
+    P.log2_items = crz_log2_items(k, D, c->log2S, c->sm_count);
     P.timeout_ns = c->cfg.timeout_ns;
     P.skip_first_ticket = (size_tiles >= 2 && fault_hit(CRAC_FAULT_ENCODE_WAIT)) ? 1u : 0u;
     uint64_t *out_h = (uint64_t *)((uint8_t *)c->ctrl_h.p + sizeof(CkptCtrl));

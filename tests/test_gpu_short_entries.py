@@ -49,10 +49,11 @@ def test_entries_of_several_parts(S, n, form):
         h.close()
 
 
-@pytest.mark.parametrize("form", ["device"])
+@pytest.mark.parametrize("form", ["device", "coded"])
 def test_empty_parts_do_not_set_the_pace(form):
     """20000 allocations below 4 KiB, all dirty, in chunks of 4 MiB against 16 KiB: the
-    gather (eight times as long and more where every part of a chunk was looked up)."""
+    gather and the coder (eight times as long and more where every part of a chunk was
+    looked up)."""
     r = random.Random(5)
     sizes = [r.randrange(1, 4096) for _ in range(20000)]
     mem = torch.zeros(20000 * 4096 // 4, dtype=torch.float32, device="cuda").normal_()
