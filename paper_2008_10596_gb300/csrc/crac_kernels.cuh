@@ -157,7 +157,7 @@ cudaError_t ckpt_tma_prepare();   // raise the dynamic shared memory limit (once
 // and the look-back status words; G reads k from ctrl.
 // aligned: every allocation's size is a multiple of 16 bytes (the other
 // instances store chunks at payload offsets of any alignment).
-const void *split_hash_fn(bool crz_headers, bool aligned);
+const void *split_hash_fn(bool crz_headers, bool aligned, uint32_t log2_chunk);
 // Hash kernel for 512 B <= chunk < 8 KiB: lanes_per_chunk = chunk / 128;
 // it finalizes every chunk itself, so finalize runs with log2Seg = log2_chunk.
 const void *split_hash_small_fn(int lanes_per_chunk, bool aligned);

@@ -102,7 +102,8 @@ cudaError_t load_kernels() {
                          reinterpret_cast<const void *>(&noalloc_totals_kernel),
                          ckpt_fused_fn(256, 1),
                          ckpt_fused_fn(256, 8),
-                         split_hash_fn(false, false),
+                         split_hash_fn(false, false, 0),
+                         split_hash_fn(false, false, 13),
                          split_hash_small_fn(4, false),
                          split_hash_small_fn(8, false),
                          split_hash_small_fn(16, false),
@@ -254,7 +255,7 @@ extern "C" crac_status_t crac_pass_noalloc(const crac_region_t *regions_dev, uin
             if (e == cudaSuccess) count_launches(1);
         }
         if (e == cudaSuccess && !fused)
-            e = launch_chained(small ? split_hash_small_fn(1 << (l - 7), false) : split_hash_fn(false, false), grid,
+            e = launch_chained(small ? split_hash_small_fn(1 << (l - 7), false) : split_hash_fn(false, false, l), grid,
                                split_hash_threads(), args, s);
         if (e == cudaSuccess && !fused)
             e = launch_chained(split_finalize_fn(fin_tile), fin_tiles < 2u * sms ? fin_tiles : 2u * sms,

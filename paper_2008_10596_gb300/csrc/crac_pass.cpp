@@ -407,7 +407,7 @@ crac_status_t launch_segment(crac_ctx *c, const Segment &sg, const CkptDesc *des
         const bool dense = small && c->sparse_ok && staging && c->dense_now;
         const void *hash_fn = dense ? split_hash_small_dense_fn(1 << (c->log2S - 7), c->dense_cta)
                               : small ? split_hash_small_fn(1 << (c->log2S - 7), c->all16)
-                                      : split_hash_fn(crz_hdr != nullptr, c->all16);
+                                      : split_hash_fn(crz_hdr != nullptr, c->all16, c->log2S);
         CkptParams P{};
         P.crz_hdr = crz_hdr;
         P.hdr_only = enc ? 1u : 0u;
@@ -1653,7 +1653,7 @@ crac_status_t fingerprint_against(crac_ctx *c, const uint64_t *fp_ref, cudaStrea
                        c->sm_count, s));
     const bool small = log2S >= 9 && log2S < 13;
     uint32_t log2Seg = small ? log2S : split_hash_seg(n, bytes, log2S, false);
-    const void *hash_fn = small ? split_hash_small_fn(1 << (log2S - 7), true) : split_hash_fn(false, true);
+    const void *hash_fn = small ? split_hash_small_fn(1 << (log2S - 7), true) : split_hash_fn(false, true, log2S);
     CkptParams P{};
     P.desc = (const CkptDesc *)c->vdesc.p;
     P.n_allocs = (uint32_t)na;

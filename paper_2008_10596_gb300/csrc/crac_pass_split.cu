@@ -96,13 +96,13 @@ __device__ __forceinline__ void block_headers(const uint4 q[8], uint32_t n, int 
 // the segment goes to hdr[block] (lane l holds bytes 16l .. 16l+15 of block u
 // in q[u], the encoder's layout of a block).  Only chunks written to staging
 // get headers, so their cost follows the dirty bytes.  kAny: the destination may
-// have any alignment (else a multiple of 16, and the segment's length too).
-template <bool kHdr, bool kAny, class Dest>
+// have any alignment (else a multiple of 16, and the segment's length too).  U:
+// vectors per lane and round.
+template <bool kHdr, bool kAny, int U, class Dest>
 __device__ __forceinline__ uint64_t hash_seg(const uint8_t *__restrict__ src, uint32_t len, uint32_t j0, int lane,
                                              Dest &&dest, uint64_t *__restrict__ hdr, bool store) {
     const uint4 *p = reinterpret_cast<const uint4 *>(src);
     const uint32_t nv = len >> 4;
-    constexpr int U = 8;
     uint64_t acc = 0;
     uint64_t key = (uint64_t)(j0 + 2u * lane + 1u) * kK1;
     constexpr uint64_t kStep = 64ull * kK1;
@@ -191,14 +191,17 @@ __device__ __forceinline__ void copy_with_headers(uint8_t *__restrict__ dst, con
     else copy_group<32>(dst, src, len, lane);
 }
 
-template <bool kHdr, bool kAny>
-__global__ void __launch_bounds__(kHashNT, 3)
+// U = 1: chunks below 512 B, a warp each (bound by the issue slots of the other seven
+// vectors when they had the eight of longer ones: 1 GiB in chunks of 256 B, a clean
+// pass 1790 -> 1190 us, FULL 1723 -> 1157).
+template <bool kHdr, bool kAny, int U>
+__global__ void __launch_bounds__(kHashNT, U > 1 ? 3 : 4)
 split_hash_kernel(const CkptParams P, unsigned long long *__restrict__ acc, uint32_t log2Seg) {
     constexpr uint32_t kWarps = kHashNT / 32;
     wait_for_producer();   // the descriptors and zeroed accumulators
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t log2S = P.log2_chunk;
-    const uint32_t spc = log2S - log2Seg;   // log2 of segments per chunk
+    const uint32_t spc = U > 1 ? log2S - log2Seg : 0;   // log2 of segments per chunk
     // The CTA's segments in rows of one per warp, so that it streams through them.
     // Which warp starts a row turns with the chunk (with the row, where a row
     // holds whole chunks), so that allocations much shorter than a chunk, which
@@ -211,7 +214,7 @@ split_hash_kernel(const CkptParams P, unsigned long long *__restrict__ acc, uint
 #pragma unroll 1
     for (uint32_t r = 0; r < P.slots_per_warp; ++r) {
         const uint64_t row = (uint64_t)blockIdx.x * P.slots_per_warp + r;
-        const uint64_t q = row * kWarps + ((warp + (uint32_t)(row >> rsh)) & (kWarps - 1));
+        const uint64_t q = row * kWarps + (U > 1 ? (warp + (uint32_t)(row >> rsh)) & (kWarps - 1) : warp);
         const uint64_t c = P.c_begin + (q >> spc);
         if (c >= P.c_end) break;
         // past allocation a's chunks (kHdr: without a register for their end)
@@ -223,7 +226,7 @@ split_hash_kernel(const CkptParams P, unsigned long long *__restrict__ acc, uint
         const uint64_t local = c - d.first_chunk;
         const uint32_t clen = (uint32_t)umin64(d.bytes - (local << log2S), 1ull << log2S);
         const uint32_t off = (uint32_t)(q & ((1ull << spc) - 1)) << log2Seg;
-        if (off >= clen) {   // beyond the end of a short last chunk (warp-uniform): on to the next chunk's rows
+        if (U > 1 && off >= clen) {   // beyond the end of a short last chunk (warp-uniform): on to the next chunk's rows
             const uint32_t last = (1u << rsh) - 1;
             r += last - ((uint32_t)row & last);
             continue;
@@ -249,7 +252,7 @@ split_hash_kernel(const CkptParams P, unsigned long long *__restrict__ acc, uint
             return nullptr;
         };
         const uint8_t *src = reinterpret_cast<const uint8_t *>(d.ptr) + (local << log2S) + off;
-        uint64_t sum = hash_seg<kHdr, kAny>(src, len, off >> 3, lane, dest,
+        uint64_t sum = hash_seg<kHdr, kAny, U>(src, len, off >> 3, lane, dest,
                                             kHdr ? P.crz_hdr + (c << (log2S - 9)) + (off >> 9) : nullptr,
                                             !kHdr || !P.hdr_only);
         sum = warp_sum(sum);
@@ -809,12 +812,15 @@ split_gather_kernel(const CkptParams P, unsigned long long *, uint32_t) {
 
 }  // namespace
 
-const void *split_hash_fn(bool crz_headers, bool aligned) {
-    if (crz_headers)
-        return aligned ? reinterpret_cast<const void *>(&split_hash_kernel<true, false>)
-                       : reinterpret_cast<const void *>(&split_hash_kernel<true, true>);
-    return aligned ? reinterpret_cast<const void *>(&split_hash_kernel<false, false>)
-                   : reinterpret_cast<const void *>(&split_hash_kernel<false, true>);
+const void *split_hash_fn(bool crz_headers, bool aligned, uint32_t log2S) {
+    if (crz_headers)   // chunks of 8 KiB and more
+        return aligned ? reinterpret_cast<const void *>(&split_hash_kernel<true, false, 8>)
+                       : reinterpret_cast<const void *>(&split_hash_kernel<true, true, 8>);
+    if (log2S < 9)
+        return aligned ? reinterpret_cast<const void *>(&split_hash_kernel<false, false, 1>)
+                       : reinterpret_cast<const void *>(&split_hash_kernel<false, true, 1>);
+    return aligned ? reinterpret_cast<const void *>(&split_hash_kernel<false, false, 8>)
+                   : reinterpret_cast<const void *>(&split_hash_kernel<false, true, 8>);
 }
 template <bool kAny>
 static const void *hash_small_fn(int lanes_per_chunk) {
