@@ -136,8 +136,8 @@ struct PerAllocCarry {
 // ---- launchers (return cudaGetLastError() of the launch) ----------------
 // Kernel entry of the fused pass for a (threads, warps_per_chunk) variant, for
 // building a graph kernel node; nullptr if the variant does not exist.
-const void *ckpt_fused_fn(int threads, int warps_per_chunk);
-int ckpt_fused_max_ctas_per_sm(int threads, int warps_per_chunk);
+const void *ckpt_fused_fn(int threads, int warps_per_chunk, bool aligned);
+int ckpt_fused_max_ctas_per_sm(int threads, int warps_per_chunk, bool aligned);
 
 
 // TMA-staged variant of the fused pass (chunk sizes 1-64 KiB): one CTA per

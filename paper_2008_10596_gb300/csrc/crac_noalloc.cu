@@ -23,7 +23,6 @@ constexpr size_t kNoAllocScratchBytes =
 constexpr int kNoAllocMaxDevices = 64;
 std::mutex g_noalloc_mu;
 void *g_noalloc_addr[kNoAllocMaxDevices];     // device address of the scratch, per device
-int g_noalloc_grid[kNoAllocMaxDevices][2];   // SMs x occupancy of the fused kernel for warps-per-chunk 1 and 8
 int g_noalloc_sms[kNoAllocMaxDevices];
 
 constexpr int kPrepareNT = 1024;
@@ -72,7 +71,7 @@ noalloc_prepare_kernel(uint64_t *__restrict__ zero_a, uint32_t na, uint64_t *__r
 
 // The pass's results (a crac_pass_totals_t at any address) from its control
 // block.  `reserved` keeps the value that earlier versions left in that word
-// (tiles and CTAs of a ticket-driven pass).
+// (tiles, and CTAs at five per SM, of a ticket-driven pass).
 __global__ void noalloc_totals_kernel(const crac::CkptCtrl *ctrl, uint8_t *out, uint32_t reserved) {
     const uint32_t t = threadIdx.x;
     crac::wait_for_producer();
@@ -100,8 +99,8 @@ cudaError_t load_kernels() {
     using namespace crac;
     const void *fns[] = {reinterpret_cast<const void *>(&noalloc_prepare_kernel),
                          reinterpret_cast<const void *>(&noalloc_totals_kernel),
-                         ckpt_fused_fn(256, 1),
-                         ckpt_fused_fn(256, 8),
+                         ckpt_fused_fn(256, 1, false),
+                         ckpt_fused_fn(256, 8, false),
                          split_hash_fn(false, false, 0),
                          split_hash_fn(false, false, 13),
                          split_hash_small_fn(4, false),
@@ -149,7 +148,6 @@ extern "C" crac_status_t crac_pass_noalloc(const crac_region_t *regions_dev, uin
         return CRAC_ERR_CUDA;
     }
     void *scratch = nullptr;
-    int grid_per[2] = {0, 0};
     {
         std::lock_guard<std::mutex> lk(g_noalloc_mu);
         if (!g_noalloc_addr[dev]) {
@@ -169,13 +167,9 @@ extern "C" crac_status_t crac_pass_noalloc(const crac_region_t *regions_dev, uin
                 return CRAC_ERR_CUDA;
             }
             g_noalloc_sms[dev] = sms;
-            g_noalloc_grid[dev][0] = sms * (ckpt_fused_max_ctas_per_sm(256, 1) > 0 ? ckpt_fused_max_ctas_per_sm(256, 1) : 1);
-            g_noalloc_grid[dev][1] = sms * (ckpt_fused_max_ctas_per_sm(256, 8) > 0 ? ckpt_fused_max_ctas_per_sm(256, 8) : 1);
             g_noalloc_addr[dev] = p;
         }
         scratch = g_noalloc_addr[dev];
-        grid_per[0] = g_noalloc_grid[dev][0];
-        grid_per[1] = g_noalloc_grid[dev][1];
     }
     const uint32_t fin_tile = split_finalize_tile(n_chunks, g_noalloc_sms[dev]);
     const uint32_t fin_tiles = (uint32_t)((n_chunks + fin_tile - 1) / fin_tile);
@@ -251,7 +245,7 @@ extern "C" crac_status_t crac_pass_noalloc(const crac_region_t *regions_dev, uin
         if (e == cudaSuccess) count_launches(1);
         void *args[] = {&P, &acc, &log2Seg};
         if (e == cudaSuccess && fused) {
-            e = cudaLaunchKernel(ckpt_fused_fn(256, wpc), dim3((uint32_t)n_tiles), dim3(256), args, 0, s);
+            e = cudaLaunchKernel(ckpt_fused_fn(256, wpc, false), dim3((uint32_t)n_tiles), dim3(256), args, 0, s);
             if (e == cudaSuccess) count_launches(1);
         }
         if (e == cudaSuccess && !fused)
@@ -262,7 +256,7 @@ extern "C" crac_status_t crac_pass_noalloc(const crac_region_t *regions_dev, uin
                                split_finalize_threads(), args, s);
         if (e == cudaSuccess && !fused)
             e = launch_chained(split_gather_fn(false, false, n_chunks, full, l), 8 * sms, split_gather_threads(), args, s);
-        const uint64_t g = grid_per[wpc == 8 ? 1 : 0];
+        const uint64_t g = 5ull * sms;
         reserved = (uint32_t)(n_tiles + (n_tiles < g ? n_tiles : g));
     }
     if (e == cudaSuccess) {

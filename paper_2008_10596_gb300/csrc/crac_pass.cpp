@@ -500,10 +500,10 @@ crac_status_t launch_segment(crac_ctx *c, const Segment &sg, const CkptDesc *des
             per_sm = 1;
         } else {
             pick_split(c, &wpc, &cpt);
-            fn = ckpt_fused_fn(256, wpc);
+            fn = ckpt_fused_fn(256, wpc, c->all16);
             threads = 256;
             per_sm = (int)c->cfg.ctas_per_sm;
-            if (!per_sm) per_sm = std::max(1, ckpt_fused_max_ctas_per_sm(256, wpc));
+            if (!per_sm) per_sm = std::max(1, ckpt_fused_max_ctas_per_sm(256, wpc, c->all16));
         }
         const uint64_t n_tiles = (nseg + cpt - 1) / cpt;
         if (n_tiles > 0x7fffffffull) return CRAC_ERR_UNSUPPORTED;
