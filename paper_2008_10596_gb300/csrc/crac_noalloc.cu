@@ -49,21 +49,26 @@ noalloc_prepare_kernel(uint64_t *__restrict__ zero_a, uint32_t na, uint64_t *__r
     if (!prefix || i0 >= n) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint64_t mine = i < n ? d[i].bytes : 0;
-    uint64_t sum = 0;
+    if (i0) {
+        uint64_t sum = 0;
 #pragma unroll 8
-    for (uint32_t j = threadIdx.x; j < i0; j += kPrepareNT) sum += d[j].bytes;
-    sum = warp_sum(sum);
-    const uint64_t incl = warp_incl_scan(mine, lane);
-    if (lane == 31) {
-        s_before[warp] = sum;
-        s_sum[warp] = incl;
+        for (uint32_t j = threadIdx.x; j < i0; j += kPrepareNT) sum += d[j].bytes;
+        sum = warp_sum(sum);
+        if (lane == 0) s_before[warp] = sum;
     }
+    const uint64_t incl = warp_incl_scan(mine, lane);
+    if (lane == 31) s_sum[warp] = incl;
     __syncthreads();
     uint64_t at = 0, total = 0;
     for (int w = 0; w < kPrepareNT / 32; ++w) {
         if (w < warp) at += s_sum[w];
-        at += s_before[w];
-        total += s_before[w] + s_sum[w];
+        total += s_sum[w];
+    }
+    if (i0) {
+        uint64_t before = 0;
+        for (int w = 0; w < kPrepareNT / 32; ++w) before += s_before[w];
+        at += before;
+        total += before;
     }
     if (i < n) prefix[i] = at + incl - mine;
     if (threadIdx.x == 0 && n - i0 <= kPrepareNT) *flag = total <= cap ? 1u : 0u;
