@@ -181,7 +181,7 @@ cudaError_t launch_compact_range(const uint32_t *lens, uint64_t lens_base, uint6
 cudaError_t launch_gather_range(const CkptDesc *d, uint32_t log2_chunk, const uint64_t *idx,
                                 const uint64_t *off, PerAllocCarry *carry, uint64_t max_entries,
                                 uint64_t idx_cap, uint8_t *staging, uint64_t staging_cap,
-                                CkptCtrl *ctrl, int grid, cudaStream_t s);
+                                CkptCtrl *ctrl, bool aligned, int grid, cudaStream_t s);
 
 cudaError_t launch_scatter(const ScatterParams &p, int grid, cudaStream_t s);
 

@@ -555,7 +555,7 @@ crac_status_t launch_segment(crac_ctx *c, const Segment &sg, const CkptDesc *des
             CK(launch_compact_range((const uint32_t *)c->lens.p, sg.c0, u0, u1, idx_d, off_d, idx_cap,
                                     (PerAllocCarry *)c->carry.p, ctrl, s));
             CK(launch_gather_range(desc_dev + a, c->log2S, idx_d, off_d, (PerAllocCarry *)c->carry.p,
-                                   u1 - u0, idx_cap, staging, staging_cap, ctrl, g, s));
+                                   u1 - u0, idx_cap, staging, staging_cap, ctrl, c->all16, g, s));
             c->last.kernel_launches += 3;
         }
         CK(launch_report(ctrl, sizeof(CkptCtrl) / 8, nullptr, ctrl_dst, s));

@@ -111,6 +111,9 @@ compact_range_kernel(const uint32_t *__restrict__ lens, uint64_t lens_base, uint
 }
 
 // K3: copy the dirty chunks listed by the last K2 of this allocation.
+// kAligned: every allocation's size is a multiple of 16 bytes (the shifted copy's
+// registers cost the others occupancy: 1 GiB in 4 KiB chunks, FULL, 1377 -> 1214 us).
+template <bool kAligned>
 __global__ void __launch_bounds__(kRangeNT)
 gather_range_kernel(const CkptDesc *__restrict__ dp, uint32_t log2S,
                     const uint64_t *__restrict__ idx, const uint64_t *__restrict__ off,
@@ -130,8 +133,8 @@ gather_range_kernel(const CkptDesc *__restrict__ dp, uint32_t log2S,
             if (threadIdx.x == 0) atomicOr(&ctrl->err, kErrBounds);
             continue;
         }
-        copy_group<GT>(staging + o, reinterpret_cast<const uint8_t *>(d.ptr) + (local << log2S),
-                       len, threadIdx.x);
+        copy_group<GT, kAligned>(staging + o, reinterpret_cast<const uint8_t *>(d.ptr) + (local << log2S),
+                                 len, threadIdx.x);
     }
 }
 
@@ -160,10 +163,10 @@ cudaError_t launch_compact_range(const uint32_t *lens, uint64_t lens_base, uint6
 cudaError_t launch_gather_range(const CkptDesc *d, uint32_t log2S, const uint64_t *idx,
                                 const uint64_t *off, PerAllocCarry *carry, uint64_t max_entries,
                                 uint64_t idx_cap, uint8_t *staging, uint64_t staging_cap,
-                                CkptCtrl *ctrl, int grid, cudaStream_t s) {
+                                CkptCtrl *ctrl, bool aligned, int grid, cudaStream_t s) {
     if (max_entries == 0) return cudaSuccess;
-    gather_range_kernel<<<grid, kRangeNT, 0, s>>>(d, log2S, idx, off, carry, idx_cap, staging,
-                                                  staging_cap, ctrl);
+    const auto kernel = aligned ? gather_range_kernel<true> : gather_range_kernel<false>;
+    kernel<<<grid, kRangeNT, 0, s>>>(d, log2S, idx, off, carry, idx_cap, staging, staging_cap, ctrl);
     const cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) count_launches(1);
     return e;
