@@ -64,11 +64,11 @@ inline uint32_t split_hash_grid(uint64_t n_chunks, uint64_t bytes, uint32_t log2
 // and 4 KiB.  With a fraction f of the chunks dirty at random, 4 KiB of n chunks hold
 // a dirty one with probability p = 1 - (1 - f)^n, and the one counter takes about
 // 400 million additions a second once they queue up: from some p on they set the
-// pace, while the CTA's two barriers cost about 10%.  2 GiB, a delta's device time,
-// per warp and per CTA: 512 B chunks 5% dirty (p = 0.34) 619 and 474 us, 10% 841 and
-// 490, 20% 1024 and 511; 1 KiB 10% (0.34) 399 and 441, 20% 858 and 461; 2 KiB 20%
-// (0.36) 404 - 624 and 429.  4 KiB chunks, whose passes are the shortest, from
-// p = 0.22 (24%: 398 - 470 and 430).
+// pace, while the CTA's two barriers cost 7 - 10%.  A delta's device time, per warp and
+// per CTA: 512 B chunks 4.5% dirty (p = 0.31) 2 GiB 430 and 469 us, 8 GiB 2190 and 1801,
+// 10% 2 GiB 840 and 485; 1 KiB 10% (0.34) 398 and 439, 13% 682 and 446; 2 KiB 20% (0.36)
+// 401 - 619 and 427.  4 KiB chunks, whose passes are the shortest, from p = 0.22 (24.5%:
+// 2 GiB 402 and 430, 8 GiB 1723 and 1628).
 inline bool dense_by_cta(float f, uint32_t log2_chunk) {
     float clean = 1.f;
     for (uint32_t i = 0; i < (4096u >> log2_chunk); ++i) clean *= 1.f - f;
@@ -84,7 +84,8 @@ inline bool dense_by_cta(float f, uint32_t log2_chunk) {
 // copied or coded one after another.  20000 allocations below 4 KiB, all dirty,
 // a delta: 481 -> 134 us in chunks of 1 MiB, 1448 -> 135 in chunks of 4 MiB; coded
 // 2267 -> 276 in the latter.
-CRAC_HD inline uint32_t chunk_items(uint64_t n, uint64_t bytes, uint32_t log2_part, uint32_t log2_parts, uint64_t lanes) {
+CRAC_HD inline uint32_t chunk_items(uint64_t n, uint64_t bytes, uint32_t log2_part, uint32_t log2_parts,
+                                    uint64_t lanes) {
     if ((n << log2_parts) <= 32 * (bytes >> log2_part) + 3 * n) return log2_parts;
     uint32_t s = log2_parts < 5 ? (log2_parts < 2 ? 0 : log2_parts - 2) : 3;
     while (s < log2_parts && (n << (s + 1)) <= lanes) ++s;

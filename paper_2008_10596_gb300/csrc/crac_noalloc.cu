@@ -215,9 +215,9 @@ extern "C" crac_status_t crac_pass_noalloc(const crac_region_t *regions_dev, uin
         P.timeout_ns = 2000000000ull;
         // Without a baseline every chunk is dirty and its payload offset known
         // beforehand: the hash kernel writes it there as it reads it, if they
-        // all fit (1 GiB in 64 KiB chunks: 486 us with the fused kernel, which
-        // reads every chunk twice, 325 us this way; with a baseline and 10%
-        // dirty 263 and 200 us).
+        // all fit (1 GiB in 64 KiB chunks, the whole call: 513 us with the fused
+        // kernel, which reads every chunk twice, 330 us this way; with a baseline
+        // and 10% dirty 283 and 215 us).
         const size_t at = (used + 255) / 256 * 256;
         uint64_t *prefix = nullptr;
         if (!fused && !fp_old_dev && staging_dev && n_regions <= (kNoAllocScratchBytes - at) / 8 - 1) {

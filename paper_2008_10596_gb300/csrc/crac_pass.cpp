@@ -266,7 +266,8 @@ crac_status_t launch_fused_graph(crac_ctx *c, const CkptParams &P, size_t work_b
 crac_status_t launch_split_graph(crac_ctx *c, const CkptParams &P, size_t work_bytes, unsigned long long *acc,
                                  uint32_t log2Seg, uint64_t bytes, const void *hash_fn, const int grids[3],
                                  const CodecParams *enc, void *ctrl_dst, cudaStream_t s) {
-    const void *fns[3] = {hash_fn, split_finalize_fn(P.cpt), split_gather_fn(P.crz_hdr != nullptr, c->all16, P.c_end - P.c_begin, bytes, c->log2S)};
+    const void *fns[3] = {hash_fn, split_finalize_fn(P.cpt),
+                          split_gather_fn(P.crz_hdr != nullptr, c->all16, P.c_end - P.c_begin, bytes, c->log2S)};
     const int thr[3] = {split_hash_threads(), split_finalize_threads(), split_gather_threads()};
     CkptParams Pc = P;
     unsigned long long *accv = acc;
@@ -864,8 +865,8 @@ crac_status_t encode_segment(crac_ctx *c, Piece &pc, const CkptCtrl &ctrl, bool 
 // CRAC_PASS_AUTO: the split pass, unless the last pass with a baseline found
 // more than half of the chunks dirty (or, on 512 B - 4 KiB chunks of device
 // images, under a quarter); then a pass that reads every byte once
-// (at 100% dirty 4 KiB pages and 64 KiB chunks: sparse 0.94, TMA 0.72, LDG
-// 0.69, split 0.66 of the HBM peak), the best one the images and sizes allow,
+// (at 100% dirty 4 KiB pages and 64 KiB chunks: sparse 1.04, TMA 0.72, LDG
+// 0.69, split 0.67 of the measured copy rate), the best one the images and sizes allow,
 // except for coded images on chunks of 8 KiB and more.
 uint32_t resolve_pass_kernel(const crac_ctx *c, bool dev_res, bool all16) {
     const bool coded = (c->cfg.flags & CRAC_FLAG_COMPRESS) != 0;
@@ -875,14 +876,14 @@ uint32_t resolve_pass_kernel(const crac_ctx *c, bool dev_res, bool all16) {
     // 512 B - 4 KiB chunks of device images, after a delta with under a
     // quarter of the chunks dirty: the sparse pass places the dirty chunks
     // densely and reads every byte once (32 GiB at 4 KiB chunks, 10% dirty
-    // pages: 0.93 of the HBM peak against the split pass's 0.84).
+    // pages: 1.03 of the measured copy rate against the split pass's 0.87).
     if (c->delta_frac_valid && c->delta_frac < 0.25f && dev_res && all16 && !coded && c->log2S >= 9 &&
         c->log2S <= 12 && c->cfg.launch_mode == CRAC_LAUNCH_BATCHED)
         return CRAC_PASS_SPARSE;
     if (!c->delta_frac_valid || c->delta_frac <= 0.5f) return CRAC_PASS_SPLIT;
     // coded images on chunks of 8 KiB and more: the split pass makes the block
     // headers of the two-launch encoder (4 GiB fp32, every chunk dirty: split
-    // 2.0 + 2.1 ms, TMA 1.7 + 3.8 ms for the one-launch encoder)
+    // 1.5 + 1.3 ms, TMA 1.7 + 3.4 ms for the one-launch encoder)
     if (coded && c->log2S >= 13 && c->cfg.launch_mode == CRAC_LAUNCH_BATCHED) return CRAC_PASS_SPLIT;
     if (dev_res && all16 && !coded) return CRAC_PASS_SPARSE;
     if (c->log2S >= 10 && c->log2S <= 16) return CRAC_PASS_TMA;

@@ -226,7 +226,7 @@ split_hash_kernel(const CkptParams P, unsigned long long *__restrict__ acc, uint
         const uint64_t local = c - d.first_chunk;
         const uint32_t clen = (uint32_t)umin64(d.bytes - (local << log2S), 1ull << log2S);
         const uint32_t off = (uint32_t)(q & ((1ull << spc) - 1)) << log2Seg;
-        if (U > 1 && off >= clen) {   // beyond the end of a short last chunk (warp-uniform): on to the next chunk's rows
+        if (U > 1 && off >= clen) {   // beyond the end of a short last chunk (warp-uniform): to the next chunk's rows
             const uint32_t last = (1u << rsh) - 1;
             r += last - ((uint32_t)row & last);
             continue;
@@ -253,8 +253,8 @@ split_hash_kernel(const CkptParams P, unsigned long long *__restrict__ acc, uint
         };
         const uint8_t *src = reinterpret_cast<const uint8_t *>(d.ptr) + (local << log2S) + off;
         uint64_t sum = hash_seg<kHdr, kAny, U>(src, len, off >> 3, lane, dest,
-                                            kHdr ? P.crz_hdr + (c << (log2S - 9)) + (off >> 9) : nullptr,
-                                            !kHdr || !P.hdr_only);
+                                               kHdr ? P.crz_hdr + (c << (log2S - 9)) + (off >> 9) : nullptr,
+                                               !kHdr || !P.hdr_only);
         sum = warp_sum(sum);
         if (lane == 0) {
             if (spc == 0) {
@@ -757,7 +757,8 @@ split_gather_kernel(const CkptParams P, unsigned long long *, uint32_t) {
     // items, 32 at a time, a lane looking up each (a chain of dependent loads).
     // 96 MiB in 1200 ragged allocations, 64 KiB chunks: all of them 545 -> 36 us.
     const uint32_t log2P = log2S < 13 ? log2S : 13;
-    const uint32_t items = kMulti ? chunk_items(k, P.ctrl->D, log2P, log2S - log2P, 32 * nw) : log2S - log2P;   // log2 per entry
+    const uint32_t parts = log2S - log2P;   // log2 of the parts of an entry, and of its items:
+    const uint32_t items = kMulti ? chunk_items(k, P.ctrl->D, log2P, parts, 32 * nw) : parts;
     const uint64_t n_items = k << items;
     for (uint64_t i0 = ((uint64_t)blockIdx.x * kGatherNT + threadIdx.x) >> 5; i0 < n_items; i0 += 32 * nw) {
         const uint64_t it = i0 + lane * nw;

@@ -196,7 +196,7 @@ crac_status_t restart_device(crac_ctx *c, crac_image *img, const std::vector<cra
     // keep SMs from other streams' work for the length of the transfer.
     // Decoding coded images is compute-heavy, and chunks that code to almost
     // nothing are bound by their stores: up to sixteen CTAs per SM, handed out
-    // as they end (1 GiB of zeros in host images: 412 us with four, 346).
+    // as they end (1 GiB of zeros in host images: 250 us with four, 167).
     bool any_host = false;
     for (const crac_image *im : chain) any_host = any_host || im->residency != CRAC_RESIDENCY_DEVICE;
     const uint64_t grid = (uint64_t)c->sm_count * (any_host ? (P.coded ? 16 : 1) : 8);
