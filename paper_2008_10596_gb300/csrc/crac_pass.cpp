@@ -264,10 +264,10 @@ crac_status_t launch_fused_graph(crac_ctx *c, const CkptParams &P, size_t work_b
 // runs in it after the gather, so that a coded image too is of one point in the
 // stream's order.
 crac_status_t launch_split_graph(crac_ctx *c, const CkptParams &P, size_t work_bytes, unsigned long long *acc,
-                                 uint32_t log2Seg, uint64_t bytes, const void *hash_fn, const int grids[3],
+                                 uint32_t log2Seg, const void *hash_fn, const int grids[3],
                                  const CodecParams *enc, void *ctrl_dst, cudaStream_t s) {
     const void *fns[3] = {hash_fn, split_finalize_fn(P.cpt),
-                          split_gather_fn(P.crz_hdr != nullptr, c->all16, P.c_end - P.c_begin, bytes, c->log2S)};
+                          split_gather_fn(P.crz_hdr != nullptr, c->all16, c->pass_chunks, c->pass_bytes, c->log2S)};
     const int thr[3] = {split_hash_threads(), split_finalize_threads(), split_gather_threads()};
     CkptParams Pc = P;
     unsigned long long *accv = acc;
@@ -468,7 +468,7 @@ crac_status_t launch_segment(crac_ctx *c, const Segment &sg, const CkptDesc *des
             enc->piece_off = (uint64_t *)P.ctrl->pad;   // 0 and the streams' bytes
             enc->timeout_ns = c->cfg.timeout_ns;
         }
-        TRY(launch_split_graph(c, P, work_bytes, acc, log2Seg, sg.bytes, hash_fn, grids, enc, ctrl_dst, s));
+        TRY(launch_split_graph(c, P, work_bytes, acc, log2Seg, hash_fn, grids, enc, ctrl_dst, s));
         if (c->spec_now) {   // this pass's offsets predict the next one's
             c->ppos_cur ^= 1;
             c->ppos_ok = true;
@@ -1387,6 +1387,8 @@ crac_status_t ctx_checkpoint(crac_ctx *c, cudaStream_t s, crac_image_t **out) {
         }
         c->all16 = all16;
         c->full_copy_ok = !any_base;
+        c->pass_chunks = n;
+        c->pass_bytes = tracked;
         c->pass_now = resolve_pass_kernel(c, dev_res, all16);
         c->sparse_ok = c->pass_now == CRAC_PASS_SPARSE && dev_res && all16 &&
                        c->cfg.launch_mode == CRAC_LAUNCH_BATCHED;
@@ -1576,6 +1578,8 @@ crac_status_t ctx_trial_pass(crac_ctx *c, cudaStream_t s, bool commit, float *ms
     }
     c->all16 = all16;
     c->full_copy_ok = !any_base;
+    c->pass_chunks = n;
+    c->pass_bytes = tracked;
     // Trial passes run the configured kernel; AUTO is the split pass here, so
     // that the tuner's observations of different sizes are comparable.
     c->pass_now = c->cfg.pass_kernel == CRAC_PASS_AUTO ? (uint32_t)CRAC_PASS_SPLIT : c->cfg.pass_kernel;

@@ -485,6 +485,7 @@ struct crac_ctx {
     crac_restart_info_t last_restart{};
     bool all16 = false;          // current pass: every size a multiple of 16 bytes
     bool full_copy_ok = false;   // current pass: no baseline anywhere
+    uint64_t pass_chunks = 0, pass_bytes = 0;   // current pass: all segments' chunks and bytes (one graph for all)
     bool sparse_ok = false;      // current pass: CRAC_PASS_SPARSE, device images, 16-byte sizes
     bool dense_now = false;      // ... and, on 512 B - 4 KiB chunks, dense placement of the dirty chunks
     bool dense_cta = false;      // ... taking its room once per CTA

@@ -17,6 +17,7 @@ pytestmark = [pytest.mark.gpu, pytest.mark.usefixtures("oracle_lib")]
 KIB, MIB = 1024, 1 << 20
 FORMS = {"device": dict(image_residency=C.CRAC_RESIDENCY_DEVICE),
          "host": dict(image_residency=C.CRAC_RESIDENCY_HOST),
+         "segments": dict(image_residency=C.CRAC_RESIDENCY_DEVICE, staging_bytes=18 * MIB),   # one long chunk in each
          "coded": dict(image_residency=C.CRAC_RESIDENCY_DEVICE, flags=C.CRAC_FLAG_COMPRESS),
          "coded host": dict(image_residency=C.CRAC_RESIDENCY_HOST, flags=C.CRAC_FLAG_COMPRESS),
          "coded direct": dict(image_residency=C.CRAC_RESIDENCY_HOST,
