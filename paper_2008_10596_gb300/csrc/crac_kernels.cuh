@@ -301,7 +301,7 @@ struct CodecParams {
     uint32_t n_allocs;
 };
 const void *crz_size_fn();
-const void *crz_encode_sized_fn();   // streams to device memory
+const void *crz_encode_sized_fn(const CodecParams &p);   // streams to device memory
 int crz_threads();
 cudaError_t launch_crz_encode(const CodecParams &p, int grid, cudaStream_t s);
 cudaError_t launch_crz_size(const CodecParams &p, int grid, cudaStream_t s);

@@ -301,7 +301,7 @@ crac_status_t launch_split_graph(crac_ctx *c, const CkptParams &P, size_t work_b
         ek[0].gridDim = dim3((unsigned)std::min<uint64_t>(crz_size_tiles(n, c->log2S), (uint64_t)c->sm_count * 4));
         // A FULL pass codes every item: a CTA for every eight.  A delta's count
         // is not known yet: up to four waves of resident CTAs stride over it.
-        ek[1].func = const_cast<void *>(crz_encode_sized_fn());
+        ek[1].func = const_cast<void *>(crz_encode_sized_fn(Ec));
         ek[1].gridDim = dim3((unsigned)std::min<uint64_t>(
             (items + warps - 1) / warps, c->full_copy_ok ? 0x7fffffffull : (uint64_t)c->sm_count * 16));
         for (cudaKernelNodeParams &k : ek) {
@@ -312,7 +312,7 @@ crac_status_t launch_split_graph(crac_ctx *c, const CkptParams &P, size_t work_b
     ReportNode rep(P.ctrl, ctrl_dst, c->fp_copy_dst, c->fp_copy_dst ? P.fp_new : nullptr,
                    c->fp_copy_dst ? P.c_end : 0, c->sm_count);
     bool ok = c->sgexec != nullptr && c->s_fns[0] == fns[0] && c->s_fns[1] == fns[1] && c->s_fns[2] == fns[2] &&
-              c->s_codes == (enc != nullptr);
+              c->s_enc_fn == ek[1].func;
     if (ok) {
         ok = cudaGraphExecKernelNodeSetParams(c->sgexec, c->s_pro, &pro) == cudaSuccess;
         for (int i = 0; ok && i < 3; ++i)
@@ -356,7 +356,7 @@ crac_status_t launch_split_graph(crac_ctx *c, const CkptParams &P, size_t work_b
         CK(cudaGraphAddDependencies(c->sgraph, last, &c->s_copy, &pe, 1));
         CK(cudaGraphInstantiate(&c->sgexec, c->sgraph, 0));
         std::copy(fns, fns + 3, c->s_fns);
-        c->s_codes = enc != nullptr;
+        c->s_enc_fn = ek[1].func;
     }
     if (!c->uva) CK(link_copy(c, c->desc.p, c->desc_src, c->allocs.size() * kDescBytes, cudaMemcpyHostToDevice, s));
     CK(cudaEventRecord(c->ev_t0, s));

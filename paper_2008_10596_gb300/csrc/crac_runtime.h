@@ -480,7 +480,8 @@ struct crac_ctx {
     cudaEvent_t sev[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};   // around each split-pass kernel, and the coder
     const void *s_fns[3] = {nullptr, nullptr, nullptr};   // the kernels in it
     cudaGraphNode_t s_enc[2] = {nullptr, nullptr};        // the coder's sizing and coding, if it codes too
-    bool s_codes = false, enc_now = false;                // (the graph; the pass just enqueued)
+    const void *s_enc_fn = nullptr;                       // ... the coding kernel (null: it does not code)
+    bool enc_now = false;                                 // the pass just enqueued codes
     crac_pass_info_t last{};
     crac_restart_info_t last_restart{};
     bool all16 = false;          // current pass: every size a multiple of 16 bytes
