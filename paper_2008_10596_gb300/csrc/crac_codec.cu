@@ -535,7 +535,7 @@ __global__ void __launch_bounds__(kCodecNT) crz_size_kernel(const CodecParams P)
 constexpr int kAhead = 2;
 
 // kMulti: an item holds several segments (an instance of its own: the loop over them
-// cost the others 1% of their time: 2 GiB of fp32, 628 -> 636 us).
+// cost the others 2% of their time: 2 GiB of fp32, 629 -> 641 us with the sizing).
 template <bool kScratch, bool kMulti>
 __global__ void __launch_bounds__(kCodecNT, 4) crz_encode_sized_kernel(const CodecParams P) {
     __shared__ __align__(16) uint8_t s_units[kScratch ? kCodecWarps : 1][512];
